@@ -180,7 +180,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_MISC + 4);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const MaskSpec ms{p.S, p.causal, p.window, p.skip_rows};
     const int b = blockIdx.x / p.Hkv, xh = blockIdx.x - b * p.Hkv;
     // heaviest key tiles first under a causal mask; with block lists the caller's order
@@ -229,7 +229,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
 #ifdef AF_TRACE
     long long* const trc = (blockIdx.x == 0 && blockIdx.y == 0) ? g_trace : nullptr;
 #endif
@@ -242,7 +242,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     if (warp < 4) setmaxnreg_dec<kFusedLightRegs>();
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tm_x); prefetch_tmap(&tm_y); prefetch_tmap(&tm_a); prefetch_tmap(&tm_b);
             mbar_arrive_expect_tx(&bars[L::B_XFULL], TILE);
             mbar_arrive_expect_tx(&bars[L::B_YFULL], TILE);
@@ -251,11 +251,13 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                 tma_load_4d(sX + bx * BOX_BYTES, &tm_x, &bars[L::B_XFULL], bx * BOX_COLS, x0, xh, b);
                 tma_load_4d(sY + bx * BOX_BYTES, &tm_y, &bars[L::B_YFULL], bx * BOX_COLS, x0, xh, b);
             }
-            Cursor cur = first;
-            for (int n = 0; n < n_it; ++n) {
-                const int st = n % NST, ah = cur.head, a0 = row0_of(cur);
-                advance(cur);
-                if (!mbar_wait(&bars[L::B_EMPTY + st], ((n / NST) & 1) ^ 1, abort_flag, 41)) break;
+        }
+        Cursor cur = first;
+        for (int n = 0; n < n_it; ++n) {
+            const int st = n % NST, ah = cur.head, a0 = row0_of(cur);
+            advance(cur);
+            if (!mbar_wait_warp(&bars[L::B_EMPTY + st], ((n / NST) & 1) ^ 1, abort_flag, 41)) break;
+            if (elect_one()) {
                 mbar_arrive_expect_tx(&bars[L::B_AFULL + st], TILE);
                 mbar_arrive_expect_tx(&bars[L::B_BFULL + st], TILE);
 #pragma unroll
@@ -269,14 +271,15 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         // ------------------------------------------------------------ MMA issuers 0 and 1
         //   issuer 0: T1 = K' Q'^T  and dV  += P^T dO    (A from TMEM)
         //   issuer 1: T2 = V dO^T   and dK' += dS^T Q'   (A from shared memory)
-        if (lane == 0) {
+        {
             const int who = warp - 1;
-            bool ok = mbar_wait(&bars[who == 0 ? L::B_XFULL : L::B_YFULL], 0, abort_flag, 42);
+            bool ok = mbar_wait_warp(&bars[who == 0 ? L::B_XFULL : L::B_YFULL], 0, abort_flag, 42);
             const uint32_t dhi = desc_hi(1024);
             const uint32_t s_lo = desc_lo(smem_u32(who == 0 ? sX : sY), 16);
             const uint32_t t_dst = tmem_base + (who == 0 ? T1 : T2);
             const uint32_t acc_dst = tmem_base + (who == 0 ? ACC1 : ACC2);
             auto issue_T = [&](int n, int hf) {
+                if (!elect_one()) return;
                 const int st = n % NST;
                 const uint32_t r_lo = desc_lo(smem_u32((who == 0 ? sA : sB) + st * TILE) + hf * 64 * 128, 16);
 #pragma unroll 2   // (partly rolled: loop code against issue slots per MMA)
@@ -288,8 +291,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             };
             auto wait_stream = [&](int n) {
                 const int st = n % NST;
-                bool r = mbar_wait(&bars[L::B_AFULL + st], (n / NST) & 1, abort_flag, 43);
-                if (r) r = mbar_wait(&bars[L::B_BFULL + st], (n / NST) & 1, abort_flag, 44);
+                bool r = mbar_wait_warp(&bars[L::B_AFULL + st], (n / NST) & 1, abort_flag, 43);
+                if (r) r = mbar_wait_warp(&bars[L::B_BFULL + st], (n / NST) & 1, abort_flag, 44);
                 tc_fence_after_sync();
                 return r;
             };
@@ -307,11 +310,12 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                 for (int hf = 0; hf < 2; ++hf) {
                     AF_FSTAMP(who, n, hf * 4);
                     // issuer 0 goes on when P^T of the half is in TMEM, issuer 1 when dS^T is in shared memory
-                    ok = mbar_wait(&bars[(who == 0 ? L::B_PRDY : L::B_PDS) + hf], n & 1, abort_flag, 45);
+                    ok = mbar_wait_warp(&bars[(who == 0 ? L::B_PRDY : L::B_PDS) + hf], n & 1, abort_flag, 45);
                     if (!ok) break;
                     AF_FSTAMP(who, n, hf * 4 + 1);
                     tc_fence_after_sync();
-                    if (who == 0) {
+                    if (!elect_one()) {
+                    } else if (who == 0) {
 #pragma unroll
                         for (int k4 = 0; k4 < 4; ++k4) {
                             const int kk = hf * 4 + k4;
@@ -327,11 +331,11 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                         }
                         mma_commit(&bars[L::B_DSFREE + hf]);
                     }
-                    if (hf == 1) mma_commit(&bars[L::B_EMPTY + st]);
+                    if (hf == 1) elect_commit(&bars[L::B_EMPTY + st]);
                     if (next) {
                         if (hf == 0) ok = wait_stream(n + 1);
                         // T2's half is free once the dQ'^T partial of the same rows has been read out of it
-                        if (ok && who == 1 && !kOwnDq) ok = mbar_wait(&bars[L::B_T2FREE + hf], n & 1, abort_flag, 46);
+                        if (ok && who == 1 && !kOwnDq) ok = mbar_wait_warp(&bars[L::B_T2FREE + hf], n & 1, abort_flag, 46);
                         if (!ok) break;
                         tc_fence_after_sync();
                         AF_FSTAMP(who, n, hf * 4 + 2);
@@ -340,33 +344,35 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                     AF_FSTAMP(who, n, hf * 4 + 3);
                 }
                 if (!ok) break;
-                if (!next) mma_commit(&bars[L::B_DONE]);
+                if (!next) elect_commit(&bars[L::B_DONE]);
             }
         }
     } else if (warp == 3) {
         // ------------------------------------------------------------ MMA issuer 2: dQ'^T half = K'^T dS^T half -> T2 half
-        if (lane == 0) {
-            bool ok = mbar_wait(&bars[L::B_XFULL], 0, abort_flag, 47);
+        {
+            bool ok = mbar_wait_warp(&bars[L::B_XFULL], 0, abort_flag, 47);
             const uint32_t dhi = desc_hi(1024);
             const uint32_t a_lo = desc_lo(smem_u32(sX), BOX_BYTES);   // MN-major: 16 key rows (2 KB) per K step
             for (int n = 0; ok && n < n_it; ++n) {
 #pragma unroll 1   // (rolled: half the issuer's loop code; the instruction path is the tightest resource of this kernel)
                 for (int hf = 0; hf < 2; ++hf) {
                     AF_FSTAMP(6, n, hf * 4);
-                    ok = mbar_wait(&bars[L::B_PDS + hf], n & 1, abort_flag, 48);
+                    ok = mbar_wait_warp(&bars[L::B_PDS + hf], n & 1, abort_flag, 48);
                     AF_FSTAMP(6, n, hf * 4 + 1);
                     // (own buffers: the previous tile's partial of this half must have been read out)
-                    if (ok && kOwnDq && n > 0) ok = mbar_wait(&bars[L::B_T2FREE + hf], (n - 1) & 1, abort_flag, 54);
+                    if (ok && kOwnDq && n > 0) ok = mbar_wait_warp(&bars[L::B_T2FREE + hf], (n - 1) & 1, abort_flag, 54);
                     if (!ok) break;
                     AF_FSTAMP(6, n, hf * 4 + 2);
                     tc_fence_after_sync();
-                    const uint32_t b_lo = desc_lo(smem_u32(sDS + hf * L::DS_HALF), 16);
-                    const uint32_t dst = tmem_base + TDQ + hf * 64;
+                    if (elect_one()) {
+                        const uint32_t b_lo = desc_lo(smem_u32(sDS + hf * L::DS_HALF), 16);
+                        const uint32_t dst = tmem_base + TDQ + hf * 64;
 #pragma unroll 2
-                    for (int kk = 0; kk < 8; ++kk)
-                        mma_ss_lo_rt(dst, a_lo + kk * 128, b_lo + kk * 128, dhi, IDESC_DQ, kk > 0 ? 1u : 0u);
-                    mma_commit(&bars[L::B_DQFULL + hf]);
-                    mma_commit(&bars[L::B_DSFREE + hf]);
+                        for (int kk = 0; kk < 8; ++kk)
+                            mma_ss_lo_rt(dst, a_lo + kk * 128, b_lo + kk * 128, dhi, IDESC_DQ, kk > 0 ? 1u : 0u);
+                        mma_commit(&bars[L::B_DQFULL + hf]);
+                        mma_commit(&bars[L::B_DSFREE + hf]);
+                    }
                     AF_FSTAMP(6, n, hf * 4 + 3);
                 }
             }

@@ -336,7 +336,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_MISC + 4);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const MaskSpec ms{p.S, p.causal, p.window, p.skip_rows};
     // stationary tile: DKV -> key tile of kv head (b, hk); DQ -> query tile of head (b, h)
     const int xh_count = DKV ? p.Hkv : p.Hq;
@@ -394,7 +394,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
     // Programmatic dependent launch: this grid may have been scheduled while its predecessor in the backward
     // sequence (delta, RoPE pass or the other gradient kernel) was still running; from here on it reads what
     // they wrote.  The next kernel of the sequence may in turn be scheduled from now on.
@@ -404,7 +404,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tm_x); prefetch_tmap(&tm_y); prefetch_tmap(&tm_a); prefetch_tmap(&tm_b);
             mbar_arrive_expect_tx(&bars[L::B_XFULL], TILE);
             mbar_arrive_expect_tx(&bars[L::B_YFULL], TILE);
@@ -413,11 +413,13 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                 tma_load_4d(sX + bx * BOX_BYTES, &tm_x, &bars[L::B_XFULL], bx * BOX_COLS, x0, xh, b);
                 tma_load_4d(sY + bx * BOX_BYTES, &tm_y, &bars[L::B_YFULL], bx * BOX_COLS, x0, xh, b);
             }
-            Cursor cur = first;
-            for (int n = 0; n < n_it; ++n) {
-                const int st = n % NST, ah = cur.head, a0 = row0_of(cur);
-                advance(cur);
-                if (!mbar_wait(&bars[L::B_EMPTY + st], ((n / NST) & 1) ^ 1, abort_flag, 21)) break;
+        }
+        Cursor cur = first;
+        for (int n = 0; n < n_it; ++n) {
+            const int st = n % NST, ah = cur.head, a0 = row0_of(cur);
+            advance(cur);
+            if (!mbar_wait_warp(&bars[L::B_EMPTY + st], ((n / NST) & 1) ^ 1, abort_flag, 21)) break;
+            if (elect_one()) {
                 mbar_arrive_expect_tx(&bars[L::B_AFULL + st], TILE);
                 mbar_arrive_expect_tx(&bars[L::B_BFULL + st], TILE);
 #pragma unroll
@@ -434,21 +436,21 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
         //   issuer 0: T1 = X A^T and acc1 (DKV: dV += P^T dO;  DQ: dQ' += dS K')
         //   issuer 1: T2 = Y Bc^T and, in the DKV role, acc2 (dK' += dS^T Q')
         // A single thread issuing all 48 MMAs of a tile pair was the bottleneck of this kernel.
-        if (lane == 0) {
+        {
             constexpr int B_XREADY = ROT_X ? L::B_XROT : L::B_XFULL;
             constexpr int B_AREADY = ROT_A ? L::B_AROT : L::B_AFULL;
             const int who = warp - 1;
             bool ok = true;
             if (who == 0) {
-                ok = mbar_wait(&bars[B_XREADY], 0, abort_flag, 22);
-                if (ok && ROT_X && p.store_x) {
+                ok = mbar_wait_warp(&bars[B_XREADY], 0, abort_flag, 22);
+                if (ok && ROT_X && p.store_x && elect_one()) {
                     // publish the rotated stationary tile (rows past S are clipped by the tensor map)
 #pragma unroll
                     for (int bx = 0; bx < NBOX; ++bx) tma_store_4d(&tm_s, sX + bx * BOX_BYTES, bx * BOX_COLS, x0, xh, b);
                     tma_store_commit();
                 }
             } else {
-                ok = mbar_wait(&bars[L::B_YFULL], 0, abort_flag, 23);
+                ok = mbar_wait_warp(&bars[L::B_YFULL], 0, abort_flag, 23);
             }
             const uint32_t xa = smem_u32(sX), ya = smem_u32(sY);
             constexpr uint32_t IDESC_TH = idesc_bf16_f32(128, 64, 0, 0);   // half tile: 64 streamed rows
@@ -456,25 +458,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             const uint32_t s_lo = desc_lo(who == 0 ? xa : ya, 16);          // this issuer's stationary operand
             const uint32_t t_dst = tmem_base + (who == 0 ? T1 : T2);
             // T1 or T2, half hf of streamed tile n: rows [64 hf, 64 hf + 64) of A (or Bc) are the N index
-#ifndef AF_BWD_TFULL
-#define AF_BWD_TFULL 0
-#endif
-            constexpr bool kTFull = AF_BWD_TFULL != 0;   // T1/T2 as one N = 128 MMA group per tile instead of two N = 64 halves
             auto issue_T = [&](int n, int hf) {
+                if (!elect_one()) return;
                 const int st = n % NST;
-                if (kTFull) {
-                    if (hf == 0) return;   // issued once per tile, at the second half's turn
-                    const uint32_t r_lo = desc_lo(smem_u32((who == 0 ? sA : sB) + st * TILE), 16);
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) {
-                        const uint32_t off = ((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4;
-                        if (kk == 0) mma_ss_lo<false>(t_dst, s_lo + off, r_lo + off, dhi, IDESC_T);
-                        else mma_ss_lo<true>(t_dst, s_lo + off, r_lo + off, dhi, IDESC_T);
-                    }
-                    mma_commit(&bars[L::B_TFULL + 0]);
-                    mma_commit(&bars[L::B_TFULL + 1]);
-                    return;
-                }
                 const uint32_t r_lo = desc_lo(smem_u32((who == 0 ? sA : sB) + st * TILE) + hf * 64 * 128, 16);
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
@@ -486,9 +472,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             };
             auto wait_stream = [&](int n) {
                 const int st = n % NST;
-                bool r = mbar_wait(&bars[(who == 0 ? B_AREADY : L::B_BFULL) + st], (n / NST) & 1, abort_flag, 24);
+                bool r = mbar_wait_warp(&bars[(who == 0 ? B_AREADY : L::B_BFULL) + st], (n / NST) & 1, abort_flag, 24);
                 // the accumulator MMAs of issuer 1 (DKV) read A as well, those of issuer 0 (DKV) read Bc
-                if (r && DKV) r = mbar_wait(&bars[(who == 0 ? L::B_BFULL : B_AREADY) + st], (n / NST) & 1, abort_flag, 25);
+                if (r && DKV) r = mbar_wait_warp(&bars[(who == 0 ? L::B_BFULL : B_AREADY) + st], (n / NST) & 1, abort_flag, 25);
                 tc_fence_after_sync();
                 return r;
             };
@@ -511,11 +497,11 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     // this half: 4 K = 16 steps over its 64 streamed rows; the bf16 operands sit at the start of
                     // the half's own columns of T1 (issuer 0) or T2 (issuer 1)
                     AF_BSTAMP(who, n, 3 * hf);
-                    ok = mbar_wait(&bars[L::B_PDS + hf], n & 1, abort_flag, 26);
+                    ok = mbar_wait_warp(&bars[L::B_PDS + hf], n & 1, abort_flag, 26);
                     AF_BSTAMP(who, n, 3 * hf + 1);
                     if (!ok) break;
                     tc_fence_after_sync();
-                    if (has_acc) {
+                    if (has_acc && elect_one()) {
 #pragma unroll
                         for (int k4 = 0; k4 < 4; ++k4) {
                             const int kk = hf * 4 + k4;
@@ -524,8 +510,8 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     }
                     if (hf == 1) {
                         // the stage is free once both issuers have consumed both halves
-                        if (has_acc) mma_commit(&bars[L::B_EMPTY + st]);
-                        else mbar_arrive(&bars[L::B_EMPTY + st]);   // DQ, issuer 1: its T2 MMAs of this stage were complete at TFULL
+                        if (has_acc) elect_commit(&bars[L::B_EMPTY + st]);
+                        else if (elect_one()) mbar_arrive(&bars[L::B_EMPTY + st]);   // DQ, issuer 1: its T2 MMAs of this stage were complete at TFULL
                     }
                     // the same half of the next streamed tile may overwrite T1/T2 right behind (in-order per issuer)
                     if (next) {
@@ -537,11 +523,11 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                 }
                 if (!ok) break;
                 if (!next) {
-                    if (has_acc) mma_commit(&bars[L::B_DONE]);
-                    else mbar_arrive(&bars[L::B_DONE]);
+                    if (has_acc) elect_commit(&bars[L::B_DONE]);
+                    else if (elect_one()) mbar_arrive(&bars[L::B_DONE]);
                 }
             }
-            if (who == 0 && ROT_X && p.store_x) tma_store_wait_all();   // the tile must stay in place until it has been read
+            if (who == 0 && ROT_X && p.store_x && elect_one()) tma_store_wait_all();   // the tile must stay in place until it has been read
         }
     } else if (warp >= 4 && warp < 8) {
         // ------------------------------------------------------------ rotation warpgroup: X once, every A tile

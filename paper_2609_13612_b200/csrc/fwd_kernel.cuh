@@ -327,7 +327,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_MISC + 4);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     // blockIdx.x: a head, or with pair_heads (even GQA group) a pair of adjacent heads that share a kv head.
     // Pairing heads gives both query tiles the same key range, so the two softmax warpgroups stay in
     // step down to the last tile; without it the tiles are rows [256 rb, +128) and [256 rb + 128, +128).
@@ -416,7 +416,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
     // Register budget: the softmax warpgroups hold a full row of 128 scores; the others need little, but the
     // MMA issuer must not spill (it is the most latency-sensitive thread of the CTA: at 64 registers it spilled
@@ -427,18 +427,22 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (warp < 4) setmaxnreg_dec<kIssuerRegs>();
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            prefetch_tmap(&tm_q);
-            prefetch_tmap(&tm_k);
-            prefetch_tmap(&tm_v);
-            if (tab_tiles) prefetch_tmap(&tm_t);
+        {
+            if (elect_one()) {
+                prefetch_tmap(&tm_q);
+                prefetch_tmap(&tm_k);
+                prefetch_tmap(&tm_v);
+                if (tab_tiles) prefetch_tmap(&tm_t);
+            }
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
                 if (jhi[q] < jlo[q]) continue;
-                mbar_arrive_expect_tx(&bars[L::B_QFULL + q], TILE);
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&bars[L::B_QFULL + q], TILE);
 #pragma unroll
-                for (int bx = 0; bx < NBOX; ++bx)
-                    tma_load_4d(sQ + q * TILE + bx * BOX_BYTES, &tm_q, &bars[L::B_QFULL + q], bx * BOX_COLS, i0[q], hq[q], b);
+                    for (int bx = 0; bx < NBOX; ++bx)
+                        tma_load_4d(sQ + q * TILE + bx * BOX_BYTES, &tm_q, &bars[L::B_QFULL + q], bx * BOX_COLS, i0[q], hq[q], b);
+                }
             }
             // hybrid arm: the keys are written by the RoPE pass launched just before this grid, which may still be
             // running (programmatic dependent launch); everything above overlaps with its tail
@@ -446,22 +450,28 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             for (int it = 0; it < n_it; ++it) {
                 const int j0 = tile_at(jlo_c + it) * BN;
                 const int ks = it % KS, vs = it % VS;
-                if (!mbar_wait(&bars[L::B_KEMPTY + ks], ((it / KS) & 1) ^ 1, abort_flag, 1)) break;
-                mbar_arrive_expect_tx(&bars[L::B_KFULL + ks], TILE);
+                if (!mbar_wait_warp(&bars[L::B_KEMPTY + ks], ((it / KS) & 1) ^ 1, abort_flag, 1)) break;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&bars[L::B_KFULL + ks], TILE);
 #pragma unroll
-                for (int bx = 0; bx < NBOX; ++bx)
-                    tma_load_4d(sK + ks * TILE + bx * BOX_BYTES, &tm_k, &bars[L::B_KFULL + ks], bx * BOX_COLS, j0, hk, b);
+                    for (int bx = 0; bx < NBOX; ++bx)
+                        tma_load_4d(sK + ks * TILE + bx * BOX_BYTES, &tm_k, &bars[L::B_KFULL + ks], bx * BOX_COLS, j0, hk, b);
+                }
                 if (tab_tiles) {
                     // the single table stage is free once the previous tile has been rotated
-                    if (!mbar_wait(&bars[L::B_TEMPTY], (it & 1) ^ 1, abort_flag, 12)) break;
-                    mbar_arrive_expect_tx(&bars[L::B_TFULL], 256u * p.R);
-                    tma_load_2d(sT, &tm_t, &bars[L::B_TFULL], 0, j0);
+                    if (!mbar_wait_warp(&bars[L::B_TEMPTY], (it & 1) ^ 1, abort_flag, 12)) break;
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(&bars[L::B_TFULL], 256u * p.R);
+                        tma_load_2d(sT, &tm_t, &bars[L::B_TFULL], 0, j0);
+                    }
                 }
-                if (!mbar_wait(&bars[L::B_VEMPTY + vs], ((it / VS) & 1) ^ 1, abort_flag, 2)) break;
-                mbar_arrive_expect_tx(&bars[L::B_VFULL + vs], TILE);
+                if (!mbar_wait_warp(&bars[L::B_VEMPTY + vs], ((it / VS) & 1) ^ 1, abort_flag, 2)) break;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&bars[L::B_VFULL + vs], TILE);
 #pragma unroll
-                for (int bx = 0; bx < NBOX; ++bx)
-                    tma_load_4d(sV + vs * TILE + bx * BOX_BYTES, &tm_v, &bars[L::B_VFULL + vs], bx * BOX_COLS, j0, hk, b);
+                    for (int bx = 0; bx < NBOX; ++bx)
+                        tma_load_4d(sV + vs * TILE + bx * BOX_BYTES, &tm_v, &bars[L::B_VFULL + vs], bx * BOX_COLS, j0, hk, b);
+                }
             }
         }
     } else if (warp == 1) {
@@ -488,7 +498,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             fence_proxy_async_smem();
             __syncwarp();
         }
-        if (lane == 0) {
+        {
             const int B_KREADY = (ROPE && p.rot_k) ? L::B_KROT : L::B_KFULL;
             constexpr int B_QREADY = ROPE ? L::B_QROT : L::B_QFULL;
             int cnt[NQ];
@@ -499,6 +509,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // descriptors differ only in their low word: one add per operand and step
             const uint32_t dhi = desc_hi(1024);
             auto issue_S = [&](int q, int ks) {
+                if (!elect_one()) return;
                 const uint32_t q_lo = desc_lo(smem_u32(sQ + q * TILE), 16), k_lo = desc_lo(smem_u32(sK + ks * TILE), 16);
                 const uint32_t d = tmem_base + q * BN;
 #pragma unroll
@@ -515,6 +526,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             };
             // part pt of O += P V: its 8 / kPParts K-steps; that part of P starts at its own score columns
             auto issue_O_part = [&](int q, int vs, bool acc, int pt) {
+                if (!elect_one()) return;
                 constexpr int KPP = 8 / kPParts;
                 const uint32_t v_lo = desc_lo(smem_u32(sV + vs * TILE), BOX_BYTES);
                 const uint32_t d = tmem_base + NQ * BN + q * D, a = tmem_base + q * BN + pt * (BN / kPParts);
@@ -526,31 +538,31 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // prologue: S of the first key tile, each query tile as soon as it is ready (the softmax
             // warpgroups rotate their Q tiles while the rotation warpgroup rotates K tile 0)
             if (BS && n_it <= 0) ok = false;   // a row block without active blocks: nothing to issue
-            if (ok) ok = mbar_wait(&bars[B_KREADY + 0], 0, abort_flag, 4);
+            if (ok) ok = mbar_wait_warp(&bars[B_KREADY + 0], 0, abort_flag, 4);
             AF_STAMP(0, 63, 3);  // first K ready
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
                 if (ok && jhi[q] >= jlo[q]) {
-                    ok = mbar_wait(&bars[B_QREADY + q], 0, abort_flag, 3);
+                    ok = mbar_wait_warp(&bars[B_QREADY + q], 0, abort_flag, 3);
                     tc_fence_after_sync();
                     if (ok && active(q, jlo_c)) issue_S(q, 0);
                 }
             }
             AF_STAMP(0, 63, 2);  // Q ready
-            if (ok) mma_commit(&bars[L::B_KEMPTY + 0]);
+            if (ok) elect_commit(&bars[L::B_KEMPTY + 0]);
             for (int it = 0; ok && it < n_it; ++it) {
                 const int j = jlo_c + it, vs = it % VS, ks1 = (it + 1) % KS;
                 const bool next = it + 1 < n_it;
                 bool kwaited = false;
                 AF_STAMP(0, it, 0);
-                ok = mbar_wait(&bars[L::B_VFULL + vs], (it / VS) & 1, abort_flag, 5);
+                ok = mbar_wait_warp(&bars[L::B_VFULL + vs], (it / VS) & 1, abort_flag, 5);
                 AF_STAMP(0, it, 1);
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
                     if (ok && active(q, j)) {
 #pragma unroll
                         for (int pt = 0; pt < kPParts; ++pt) {
-                            if (ok) ok = mbar_wait(&bars[L::B_PREADY + 4 * q + pt], cnt[q] & 1, abort_flag, 6);
+                            if (ok) ok = mbar_wait_warp(&bars[L::B_PREADY + 4 * q + pt], cnt[q] & 1, abort_flag, 6);
                             if (pt == 0) AF_STAMP(0, it, 2 + 3 * q);
                             if (ok) {
                                 tc_fence_after_sync();
@@ -560,12 +572,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         if (ok) {
                             AF_STAMP(0, it, 3 + 3 * q);
                             ++cnt[q];
-                            if (is_last(q, j)) mma_commit(&bars[L::B_ODONE + q]);
+                            if (is_last(q, j)) elect_commit(&bars[L::B_ODONE + q]);
                         }
                     }
                     if (ok && next && active(q, j + 1)) {
                         if (!kwaited) {
-                            ok = mbar_wait(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7);
+                            ok = mbar_wait_warp(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7);
                             tc_fence_after_sync();
                             kwaited = true;
                         }
@@ -574,8 +586,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     }
                 }
                 if (ok) {
-                    mma_commit(&bars[L::B_VEMPTY + vs]);
-                    if (next) mma_commit(&bars[L::B_KEMPTY + ks1]);
+                    elect_commit(&bars[L::B_VEMPTY + vs]);
+                    if (next) elect_commit(&bars[L::B_KEMPTY + ks1]);
                 }
             }
         }

@@ -93,6 +93,21 @@ __global__ void wait_timeout_selftest_kernel(long long limit_cycles) {
     __syncthreads();
 }
 
+// One lane of a converged warp.  The roles that issue MMAs and TMA copies run with all 32 lanes and guard only the issuing
+// instructions with this: control flow and operands then stay warp-uniform, which is what those instructions need
+// (their descriptors and addresses live in uniform registers).  A role run by lane 0 alone pays for every operand of
+// every MMA: forward without rotation at 32 q / 8 kv heads, S = 16384, D = 128: 2142 -> 1923 us, S = 4096 with rotation
+// 169.6 -> 164.0 us, hybrid 188.7 -> 175.6 us (B = 4, S = 2048); one-pass backward 525 -> 508 us (B = 4, 12 heads,
+// S = 4096, D = 64), two-kernel backward 653 -> 641 us (B = 4, 32 / 8 heads, S = 2048).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+// A value that is the same in all lanes, in a form the compiler can keep in a uniform register.
+template <typename T>
+__device__ __forceinline__ T warp_uniform(T v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 // ---------------------------------------------------------------- proxies and fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -249,6 +264,11 @@ __device__ __forceinline__ uint32_t desc_hi_noswizzle(uint32_t sbo_bytes) {
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
+}
+
+// The same from a converged warp.  (elect.sync picks the same lane every time, so the commit sees that lane's MMAs.)
+__device__ __forceinline__ void elect_commit(uint64_t* bar) {
+    if (elect_one()) mma_commit(bar);
 }
 
 // ---------------------------------------------------------------- TMEM <-> registers (32 lanes x 32-bit, one row per thread)
