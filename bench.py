@@ -706,7 +706,7 @@ def main():
             "fwd": host_us(lambda i: af.fwd(st_["q"], st_["k"], st_["v"], rt, tt_, mt, wt.scale, out=ot, lse=lt)),
             "bwd": host_us(lambda i: af.bwd(st_["q"], st_["k"], st_["v"], ot, lt, st_["do"], rt, tt_, mt, wt.scale, workspace=wst)),
             "decode": ex["flash_decoding"][0]["c_abi_call_from_host_us"],
-            "note": "Python ctypes binding included; small shapes so that the device never back-pressures the host"}
+            "note": "Python binding included; small shapes so that the device never back-pressures the host"}
         line["extras"] = ex
         # the three arms of the fuse-or-not experiment on the headline workload, side by side (TFLOP/s)
         c2 = ex[synth.CONFIGS[1].name]

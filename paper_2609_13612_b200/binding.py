@@ -1,4 +1,8 @@
-"""ctypes binding with the same names as the C entry points (see include/attnfuse.h)."""
+"""Python binding with the same names as the C entry points (see include/attnfuse.h).
+
+The calls of a training or serving loop (fwd, fwd_hybrid, fwd_blocks, fwd_fp8, bwd, decode) go through a small native
+module (csrc/torch_binding.cpp), because for small problems the host time of a call is what bounds it; set-up, status
+and the less frequent entry points use ctypes."""
 from __future__ import annotations
 
 import ctypes
@@ -145,6 +149,30 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native = None
+
+
+def _bind(native, L) -> None:
+    """Hand the native module the entry points of the loaded library."""
+    native.bind({n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in (
+        "attnfuse_strerror", "attnfuse_fwd", "attnfuse_fwd_hybrid", "attnfuse_fwd_hybrid_workspace_bytes", "attnfuse_fwd_blocks",
+        "attnfuse_fwd_fp8", "attnfuse_bwd", "attnfuse_bwd_blocks", "attnfuse_bwd_onepass_workspace_bytes", "attnfuse_decode",
+        "attnfuse_decode_splits", "attnfuse_decode_workspace_bytes")}, AttnFuseError)
+
+
+def _load_native():
+    global _native
+    L = lib()
+    if _native is None:
+        try:
+            from . import _torch_binding
+        except ImportError as e:
+            raise AttnFuseError(-1, "_torch_binding.so is not built (%s); run `python -m paper_2609_13612_b200.build`" % e)
+        _bind(_torch_binding, L)
+        _native = _torch_binding   # (last: another thread may call through it as soon as it is set)
+    return _native
+
+
 def _check(code: int):
     if code != 0:
         raise AttnFuseError(code, lib().attnfuse_strerror(code).decode())
@@ -256,26 +284,7 @@ def fwd(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: RopeSpec, 
         mask: MaskSpec, softmax_scale: float, out: Optional[torch.Tensor] = None,
         lse: Optional[torch.Tensor] = None, out_dtype: torch.dtype = torch.bfloat16, want_lse: bool = True):
     """Fused forward.  q [B,Hq,S,D], k/v [B,Hkv,S,D] bf16 (last dim contiguous).  Returns (o, lse)."""
-    _need_cuda(q, k, v, table, out, lse)
-    assert q.dtype == k.dtype == v.dtype == torch.bfloat16
-    B, Hq, S, D = q.shape
-    Hkv = k.shape[1]
-    assert k.shape == v.shape == (B, Hkv, S, D) and k.stride() == v.stride()
-    if out is None:
-        out = torch.empty((B, Hq, S, D), dtype=out_dtype, device=q.device)
-    if lse is None and want_lse:
-        lse = torch.empty((B, Hq, S), dtype=torch.float32, device=q.device)
-    assert out.is_contiguous() and out.dtype in (torch.bfloat16, torch.float32)
-    sh = _Shape(B, Hq, Hkv, S, D)
-    sq, skv = _strides(q), _strides(k)
-    r = _Rope(rope_spec.theta, rope_spec.rotary_dim, rope_spec.pos_offset)
-    m = _mask_struct(mask)
-    _check(lib().attnfuse_fwd(ctypes.byref(sh), q.data_ptr(), k.data_ptr(), v.data_ptr(), ctypes.byref(sq),
-                              ctypes.byref(skv), ctypes.byref(r), table.data_ptr() if table is not None else None,
-                              ctypes.byref(m), Hq // Hkv, float(softmax_scale), out.data_ptr(),
-                              AF_F32 if out.dtype == torch.float32 else AF_BF16,
-                              lse.data_ptr() if lse is not None else None, _stream()))
-    return out, lse
+    return (_native or _load_native()).fwd(q, k, v, rope_spec, table, mask, softmax_scale, out, lse, out_dtype, want_lse)
 
 
 def fwd_variant(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: RopeSpec, table: Optional[torch.Tensor],
@@ -350,20 +359,7 @@ def fwd_fp8(q8: torch.Tensor, k8: torch.Tensor, vt8: torch.Tensor, mask: MaskSpe
             scale_q: float = 1.0, scale_k: float = 1.0, scale_v: float = 1.0, out_dtype: torch.dtype = torch.bfloat16):
     """Forward with E4M3 operands: q8 [B,Hq,S,D], k8 [B,Hkv,S,D], vt8 [B,Hkv,D,S] (V transposed) as uint8 codes (or
     torch.float8_e4m3fn tensors) on the device, value = code x scale.  Returns (o, lse)."""
-    _need_cuda(q8, k8, vt8)
-    q8, k8, vt8 = (t.view(torch.uint8) if t.dtype != torch.uint8 else t for t in (q8, k8, vt8))
-    assert q8.is_contiguous() and k8.is_contiguous() and vt8.is_contiguous()
-    B, Hq, S, D = q8.shape
-    Hkv = k8.shape[1]
-    assert k8.shape == (B, Hkv, S, D) and vt8.shape == (B, Hkv, D, S)
-    out = torch.empty((B, Hq, S, D), dtype=out_dtype, device=q8.device)
-    lse = torch.empty((B, Hq, S), dtype=torch.float32, device=q8.device)
-    sh = _Shape(B, Hq, Hkv, S, D)
-    m = _mask_struct(mask)
-    _check(lib().attnfuse_fwd_fp8(ctypes.byref(sh), q8.data_ptr(), k8.data_ptr(), vt8.data_ptr(), ctypes.byref(m), Hq // Hkv,
-                                  float(softmax_scale), float(scale_q), float(scale_k), float(scale_v), out.data_ptr(),
-                                  AF_F32 if out.dtype == torch.float32 else AF_BF16, lse.data_ptr(), _stream()))
-    return out, lse
+    return (_native or _load_native()).fwd_fp8(q8, k8, vt8, mask, softmax_scale, scale_q, scale_k, scale_v, out_dtype)
 
 
 def fwd_hybrid(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: RopeSpec, table: Optional[torch.Tensor],
@@ -372,31 +368,8 @@ def fwd_hybrid(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: Rop
                workspace: Optional[torch.Tensor] = None):
     """Hybrid forward (Section 5.3): K rotated once by a RoPE pass into `workspace` (uint8, at least
     attnfuse_fwd_hybrid_workspace_bytes; allocated when None), Q rotated inside the kernel.  Returns (o, lse)."""
-    _need_cuda(q, k, v, table, out, lse, workspace)
-    assert q.dtype == k.dtype == v.dtype == torch.bfloat16
-    B, Hq, S, D = q.shape
-    Hkv = k.shape[1]
-    assert k.shape == v.shape == (B, Hkv, S, D) and k.stride() == v.stride()
-    if out is None:
-        out = torch.empty((B, Hq, S, D), dtype=out_dtype, device=q.device)
-    if lse is None and want_lse:
-        lse = torch.empty((B, Hq, S), dtype=torch.float32, device=q.device)
-    assert out.is_contiguous() and out.dtype in (torch.bfloat16, torch.float32)
-    sh = _Shape(B, Hq, Hkv, S, D)
-    if workspace is None:
-        workspace = torch.empty(lib().attnfuse_fwd_hybrid_workspace_bytes(ctypes.byref(sh)), dtype=torch.uint8,
-                                device=q.device)
-    sq, skv = _strides(q), _strides(k)
-    r = _Rope(rope_spec.theta, rope_spec.rotary_dim, rope_spec.pos_offset)
-    m = _mask_struct(mask)
-    _check(lib().attnfuse_fwd_hybrid(ctypes.byref(sh), q.data_ptr(), k.data_ptr(), v.data_ptr(), ctypes.byref(sq),
-                                     ctypes.byref(skv), ctypes.byref(r),
-                                     table.data_ptr() if table is not None else None, ctypes.byref(m), Hq // Hkv,
-                                     float(softmax_scale), out.data_ptr(),
-                                     AF_F32 if out.dtype == torch.float32 else AF_BF16,
-                                     lse.data_ptr() if lse is not None else None, workspace.data_ptr(),
-                                     workspace.numel() * workspace.element_size(), _stream()))
-    return out, lse
+    return (_native or _load_native()).fwd_hybrid(q, k, v, rope_spec, table, mask, softmax_scale, out, lse, out_dtype, want_lse,
+                                                  workspace)
 
 
 class BlockMask:
@@ -445,26 +418,7 @@ def fwd_blocks(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: Rop
                mask: MaskSpec, softmax_scale: float, blocks: BlockMask, out: Optional[torch.Tensor] = None,
                lse: Optional[torch.Tensor] = None, out_dtype: torch.dtype = torch.bfloat16):
     """Block-sparse forward: `fwd` restricted to the active blocks of `blocks`.  Returns (o, lse)."""
-    _need_cuda(q, k, v, table, out, lse)
-    assert q.dtype == k.dtype == v.dtype == torch.bfloat16
-    B, Hq, S, D = q.shape
-    Hkv = k.shape[1]
-    assert k.shape == v.shape == (B, Hkv, S, D) and k.stride() == v.stride()
-    assert blocks.nb == (S + 127) // 128
-    if out is None:
-        out = torch.empty((B, Hq, S, D), dtype=out_dtype, device=q.device)
-    if lse is None:
-        lse = torch.empty((B, Hq, S), dtype=torch.float32, device=q.device)
-    sh = _Shape(B, Hq, Hkv, S, D)
-    sq, skv = _strides(q), _strides(k)
-    r = _Rope(rope_spec.theta, rope_spec.rotary_dim, rope_spec.pos_offset)
-    m = _mask_struct(mask)
-    bl = blocks.struct()
-    _check(lib().attnfuse_fwd_blocks(ctypes.byref(sh), q.data_ptr(), k.data_ptr(), v.data_ptr(), ctypes.byref(sq),
-                                     ctypes.byref(skv), ctypes.byref(r), table.data_ptr() if table is not None else None,
-                                     ctypes.byref(m), Hq // Hkv, float(softmax_scale), ctypes.byref(bl), out.data_ptr(),
-                                     AF_F32 if out.dtype == torch.float32 else AF_BF16, lse.data_ptr(), _stream()))
-    return out, lse
+    return (_native or _load_native()).fwd_blocks(q, k, v, rope_spec, table, mask, softmax_scale, blocks, out, lse, out_dtype)
 
 
 def fwd_host(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: RopeSpec, table: Optional[torch.Tensor],
@@ -506,37 +460,8 @@ def bwd(q, k, v, o, lse, d_o, rope_spec: RopeSpec, table, mask: MaskSpec, softma
         blocks: Optional[BlockMask] = None):
     """Fused backward (over the active blocks of `blocks`, if given).  Returns (dq, dk, dv).
     Without a workspace of the caller's, one of the largest useful size is allocated (`bwd_workspace_bytes`)."""
-    _need_cuda(q, k, v, o, lse, d_o, table, workspace)
-    B, Hq, S, D = q.shape
-    Hkv = k.shape[1]
-    assert o.is_contiguous() and d_o.is_contiguous() and lse.is_contiguous()
-    assert o.dtype == d_o.dtype == torch.bfloat16 and lse.dtype == torch.float32
-    sh = _Shape(B, Hq, Hkv, S, D)
-    if workspace is None:
-        workspace = torch.empty(bwd_workspace_bytes(B, Hq, Hkv, S, D), dtype=torch.uint8, device=q.device)
-    dq = torch.empty((B, Hq, S, D), dtype=dq_dtype, device=q.device)
-    dk = torch.empty((B, Hkv, S, D), dtype=dkv_dtype, device=q.device)
-    dv = torch.empty((B, Hkv, S, D), dtype=dkv_dtype, device=q.device)
-    sq, skv = _strides(q), _strides(k)
-    r = _Rope(rope_spec.theta, rope_spec.rotary_dim, rope_spec.pos_offset)
-    m = _mask_struct(mask)
-    code = lambda dt: AF_F32 if dt == torch.float32 else AF_BF16
-    if blocks is not None:
-        assert blocks.nb == (S + 127) // 128
-        bl = blocks.struct()
-        _check(lib().attnfuse_bwd_blocks(ctypes.byref(sh), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
-                                         lse.data_ptr(), d_o.data_ptr(), ctypes.byref(sq), ctypes.byref(skv),
-                                         ctypes.byref(r), table.data_ptr() if table is not None else None,
-                                         ctypes.byref(m), Hq // Hkv, float(softmax_scale), ctypes.byref(bl),
-                                         dq.data_ptr(), code(dq_dtype), dk.data_ptr(), dv.data_ptr(), code(dkv_dtype),
-                                         workspace.data_ptr(), workspace.numel(), _stream()))
-        return dq, dk, dv
-    _check(lib().attnfuse_bwd(ctypes.byref(sh), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
-                              lse.data_ptr(), d_o.data_ptr(), ctypes.byref(sq), ctypes.byref(skv), ctypes.byref(r),
-                              table.data_ptr() if table is not None else None, ctypes.byref(m), Hq // Hkv,
-                              float(softmax_scale), dq.data_ptr(), code(dq_dtype), dk.data_ptr(), dv.data_ptr(),
-                              code(dkv_dtype), workspace.data_ptr(), workspace.numel(), _stream()))
-    return dq, dk, dv
+    return (_native or _load_native()).bwd(q, k, v, o, lse, d_o, rope_spec, table, mask, softmax_scale, dq_dtype, dkv_dtype,
+                                           workspace, blocks)
 
 
 BWD_STATIC_MAX_ROWS = 1 << 20
@@ -547,28 +472,7 @@ def decode(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, mask: MaskSpec, so
            workspace: Optional[torch.Tensor] = None, want_lse: bool = True):
     """Flash Decoding: q [B,Hq,D] (one position per head, the last one) against the cache k/v [B,Hkv,N,D].
     Returns (o [B,Hq,D] bf16, lse [B,Hq])."""
-    _need_cuda(q, k, v, out, lse, workspace)
-    assert q.dtype == k.dtype == v.dtype == torch.bfloat16 and q.is_contiguous()
-    B, Hq, D = q.shape
-    Hkv, N = k.shape[1], k.shape[2]
-    assert k.shape == v.shape == (B, Hkv, N, D) and k.stride() == v.stride()
-    if out is None:
-        out = torch.empty((B, Hq, D), dtype=torch.bfloat16, device=q.device)
-    if lse is None and want_lse:
-        lse = torch.empty((B, Hq), dtype=torch.float32, device=q.device)
-    sh = _Shape(B, Hq, Hkv, N, D)
-    if n_splits <= 0:
-        n_splits = lib().attnfuse_decode_splits(ctypes.byref(sh))
-    if workspace is None:   # (a caller's own workspace must have been cleared once: decode_workspace)
-        workspace = torch.zeros(lib().attnfuse_decode_workspace_bytes(ctypes.byref(sh), n_splits), dtype=torch.uint8,
-                                device=q.device)
-    skv = _strides(k)
-    m = _mask_struct(mask)
-    _check(lib().attnfuse_decode(ctypes.byref(sh), q.data_ptr(), k.data_ptr(), v.data_ptr(), ctypes.byref(skv),
-                                 ctypes.byref(m), Hq // Hkv, float(softmax_scale), out.data_ptr(),
-                                 lse.data_ptr() if lse is not None else None, int(n_splits), workspace.data_ptr(),
-                                 workspace.numel() * workspace.element_size(), _stream()))
-    return out, lse
+    return (_native or _load_native()).decode(q, k, v, mask, softmax_scale, n_splits, out, lse, workspace, want_lse)
 
 
 def decode_workspace(B: int, Hq: int, Hkv: int, N: int, D: int, n_splits: int = 0, device="cuda") -> torch.Tensor:

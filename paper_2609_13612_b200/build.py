@@ -1,13 +1,16 @@
-"""Build libattnfuse.so (sm_100a) in-tree with nvcc.  `python -m paper_2609_13612_b200.build`."""
+"""Build libattnfuse.so (sm_100a, nvcc) and the torch binding (g++) in-tree.  `python -m paper_2609_13612_b200.build`."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libattnfuse.so")
+BINDING = os.path.join(PKG, "_torch_binding.so")
+BINDING_SRC = os.path.join(CSRC, "torch_binding.cpp")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC"]
 
@@ -24,7 +27,27 @@ def is_stale() -> bool:
     return any(os.path.getmtime(s) > t for s in _sources())
 
 
+def build_binding(force: bool = False) -> str:
+    """The native side of the Python binding: a CPython module over torch's C++ headers, host code only."""
+    deps = [BINDING_SRC, os.path.join(os.path.dirname(PKG), "include", "attnfuse.h")]
+    if not force and os.path.exists(BINDING) and all(os.path.getmtime(d) <= os.path.getmtime(BINDING) for d in deps):
+        return BINDING
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    tmp = BINDING + ".tmp.%d" % os.getpid()
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++20", "-shared", "-fPIC", "-fvisibility=hidden",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] +
+                          ["-isystem" + d for d in inc] + ["-o", tmp, BINDING_SRC, "-L" + os.path.join(root, "lib"),
+                           "-Wl,-rpath," + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+    os.replace(tmp, BINDING)
+    return BINDING
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_binding(force)
     if not force and not is_stale():
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")

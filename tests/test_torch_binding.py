@@ -1,0 +1,29 @@
+"""Argument checks of the native side of the Python binding (no GPU needed: nothing here reaches a launch)."""
+import pytest
+import torch
+
+import paper_2609_13612_b200 as af
+
+CPU = torch.zeros(1, 2, 128, 64, dtype=torch.bfloat16)
+CODES = torch.zeros(1, 2, 128, 128, dtype=torch.uint8)
+ROPE, MASK = af.RopeSpec(rotary_dim=0), af.MaskSpec()
+
+
+@pytest.mark.parametrize("call", [
+    lambda: af.fwd(CPU, CPU, CPU, ROPE, None, MASK, 0.1),
+    lambda: af.fwd_hybrid(CPU, CPU, CPU, ROPE, None, MASK, 0.1),
+    lambda: af.fwd_blocks(CPU, CPU, CPU, ROPE, None, MASK, 0.1, af.BlockMask([[True]], device="cpu")),
+    lambda: af.fwd_fp8(CODES, CODES, CODES, MASK, 0.1),
+    lambda: af.bwd(CPU, CPU, CPU, CPU, CPU, CPU, ROPE, None, MASK, 0.1),
+    lambda: af.decode(CPU[:, :, 0], CPU, CPU, MASK, 0.1),
+], ids=["fwd", "fwd_hybrid", "fwd_blocks", "fwd_fp8", "bwd", "decode"])
+def test_tensors_off_the_device_are_refused(call):
+    with pytest.raises(af.AttnFuseError) as e:
+        call()
+    assert e.value.code == -2
+
+
+@pytest.mark.parametrize("bad", [None, 3.0, "q"])
+def test_arguments_of_another_kind_are_refused(bad):
+    with pytest.raises(TypeError):
+        af.fwd(bad, CPU, CPU, ROPE, None, MASK, 0.1)
