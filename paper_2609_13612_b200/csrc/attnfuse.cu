@@ -405,6 +405,30 @@ af_status launch_rope(const void* x_in, const af_strides& st, void* x_out, int B
                          static_cast<long long>(st.b), static_cast<long long>(st.h), static_cast<long long>(st.s));
 }
 
+// The set-up pass of a backward sequence (bwd_prologue_kernel): delta always, the rest as the parameters say.
+template <int D>
+af_status launch_prologue(const af_shape* sh, const void* o, const void* d_o, float* delta, BwdPrologueParams p, cudaStream_t stream) {
+    p.B = sh->B; p.Hq = sh->Hq; p.Hkv = sh->Hkv; p.S = sh->S;
+    p.o = static_cast<const uint4*>(o);
+    p.d_o = static_cast<const uint4*>(d_o);
+    p.delta = delta;
+    p.rows = static_cast<long long>(sh->B) * sh->Hq * sh->S;
+    auto blocks = [](long long n, long long per) { return (n + per - 1) / per; };
+    const long long per_head = p.R > 0 ? blocks(static_cast<long long>(sh->S) * ((p.R >> 4) + ((D - p.R) >> 3)), 256) : 0;
+    const long long bq = p.q_out ? per_head * blocks(static_cast<long long>(sh->B) * sh->Hq, kPrologueHeads) : 0;
+    const long long bk = p.k_out ? per_head * blocks(static_cast<long long>(sh->B) * sh->Hkv, kPrologueHeads) : 0;
+    const long long bd = blocks(p.rows * (D / 8), 256 * kPrologueRows);
+    p.acc_quads = p.acc ? p.rows * (D / 4) : 0;
+    const long long ba = blocks(p.acc_quads, 256 * kPrologueAccQuads);
+    const long long bf = p.first_rows > 0 ? static_cast<long long>(sh->B) * sh->Hkv : 0;
+    const long long total = bq + bk + bd + ba + bf;
+    if (total > 0x7fffffffll) return AF_ERR_SHAPE;
+    p.blocks_q = static_cast<unsigned>(bq); p.blocks_k = static_cast<unsigned>(bk); p.blocks_delta = static_cast<unsigned>(bd);
+    p.blocks_acc = static_cast<unsigned>(ba); p.blocks_first = static_cast<unsigned>(bf);
+    bwd_prologue_kernel<D><<<static_cast<unsigned>(total), 256, 0, stream>>>(p);
+    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+}
+
 // delta, then the two gradient kernels.  tkp / tqp: tensor maps over the rotated-K and rotated-Q caches in
 // the workspace, or nullptr when the workspace has no room for them (see bwd_kernel.cuh for the three set-ups).
 // k / stkv / kcache: the caller's K, its strides and the K' cache, for the RoPE pass of the two-cache set-up.
@@ -430,8 +454,8 @@ template <int D>
 af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                              const CUtensorMap& tdo, const CUtensorMap& tkp, const CUtensorMap& tqp, const void* k,
                              const af_strides& stkv, void* kcache, const void* o, const void* d_o, BwdParams p, void* dq,
-                             int dq_f32, void* dk, void* dv, int dkv_f32, float* delta, const OnePassArgs& a,
-                             cudaStream_t stream);
+                             int dq_f32, void* dk, void* dv, int dkv_f32, float* delta, const FirstRowsParams& fp,
+                             const OnePassArgs& a, cudaStream_t stream);
 
 template <int D>
 af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
@@ -442,15 +466,16 @@ af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMa
     p.skip_rows = fp.rows;
     af_status st;
     st = onepass ? launch_bwd_onepass<D>(sh, tq, tk, tv, tdo, tkp ? *tkp : tk, tqp ? *tqp : tq, k, stkv, kcache, o, d_o, p, dq, dq_f32,
-                                         dk, dv, dkv_f32, delta, *onepass, stream)
+                                         dk, dv, dkv_f32, delta, fp, *onepass, stream)
                  : launch_bwd_mma<D>(sh, tq, tk, tv, tdo, tkp, tqp, k, stkv, kcache, o, d_o, p, dq, dq_f32, dk, dv,
                                      dkv_f32, delta, blocks, stream);
-    if (st != AF_OK || fp.rows == 0) return st;
+    // (the one-pass kernel runs them in its own grid when dK and dV are fp32)
+    if (st != AF_OK || fp.rows == 0 || (onepass && dkv_f32)) return st;
     return launch_first_rows<D>(fp, stream);
 }
 
-// One-pass sequence (bwd_fused_kernel.cuh): zero the fp32 dQ' accumulator, delta, RoPE passes on K and Q into the
-// caches, the one-pass kernel (dK, dV, dQ' partials), then scale / rotate back / convert dQ.
+// One-pass sequence (bwd_fused_kernel.cuh): the set-up pass (zeroed fp32 dQ' accumulator, delta, rotated K and Q in the
+// caches), the one-pass kernel (dK, dV, dQ' partials), then scale / rotate back / convert dQ.
 struct OnePassArgs {
     const void* q;
     af_strides stq;
@@ -463,20 +488,26 @@ template <int D>
 af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                              const CUtensorMap& tdo, const CUtensorMap& tkp, const CUtensorMap& tqp, const void* k,
                              const af_strides& stkv, void* kcache, const void* o, const void* d_o, BwdParams p, void* dq,
-                             int dq_f32, void* dk, void* dv, int dkv_f32, float* delta, const OnePassArgs& a,
-                             cudaStream_t stream) {
+                             int dq_f32, void* dk, void* dv, int dkv_f32, float* delta, const FirstRowsParams& fp,
+                             const OnePassArgs& a, cudaStream_t stream) {
     using L = BwdFusedSmem<D>;
-    if (cudaMemsetAsync(a.dq_acc, 0, a.dq_acc_bytes, stream) != cudaSuccess) return AF_ERR_CUDA;
-    const long long rows = static_cast<long long>(sh->B) * sh->Hq * sh->S;
-    const long long threads = rows * (D / 8);
-    bwd_delta_kernel<D><<<static_cast<unsigned>((threads + 255) / 256), 256, 0, stream>>>(
-        static_cast<const uint4*>(o), static_cast<const uint4*>(d_o), delta, rows);
-    if (cudaGetLastError() != cudaSuccess) return AF_ERR_CUDA;
-    af_status st;
+    const bool first = fp.rows > 0 && dkv_f32;   // the first query rows in the one-pass kernel's own grid
+    BwdPrologueParams pp = {};
+    pp.R = p.R;
+    pp.table = p.table;
     if (p.R > 0) {
-        if ((st = launch_rope(k, stkv, kcache, sh->B, sh->Hkv, sh->S, D, p.R, p.table, 0, stream, true)) != AF_OK) return st;
-        if ((st = launch_rope(a.q, a.stq, a.qcache, sh->B, sh->Hq, sh->S, D, p.R, p.table, 0, stream, true)) != AF_OK) return st;
+        pp.q = static_cast<const uint4*>(a.q); pp.q_out = static_cast<uint4*>(a.qcache);
+        pp.qb = a.stq.b; pp.qh = a.stq.h; pp.qs = a.stq.s;
+        pp.k = static_cast<const uint4*>(k); pp.k_out = static_cast<uint4*>(kcache);
+        pp.kb = stkv.b; pp.kh = stkv.h; pp.ks = stkv.s;
     }
+    pp.acc = reinterpret_cast<float4*>(a.dq_acc);
+    if (first) {
+        pp.dk = static_cast<float*>(dk); pp.dv = static_cast<float*>(dv);
+        pp.first_rows = fp.rows;
+    }
+    af_status st = launch_prologue<D>(sh, o, d_o, delta, pp, stream);
+    if (st != AF_OK) return st;
     p.delta = delta;
     p.out1 = dv; p.out2 = dk; p.out_f32 = dkv_f32; p.store_x = 0;
     p.dq_acc = a.dq_acc;
@@ -488,13 +519,17 @@ af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CU
     static std::atomic<unsigned long long> configured[2];
     if (allow_dynamic_smem(kern, L::BYTES, configured[a.blocks ? 1 : 0]) != AF_OK) return AF_ERR_CUDA;
     const unsigned tiles = static_cast<unsigned>((sh->S + 127) / 128);
-    dim3 grid(sh->B * sh->Hkv, tiles, 1);
-    st = p.R > 0 ? launch_kernel(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, tkp, tv, tqp, tdo, p)
-                 : launch_kernel(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, tk, tv, tq, tdo, p);
+    const int first_ctas = first ? 1 : 0;   // rows of the grid
+    dim3 grid(sh->B * sh->Hkv, tiles + first_ctas, 1);
+    st = p.R > 0 ? launch_kernel(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, tkp, tv, tqp, tdo, p, fp, first_ctas)
+                 : launch_kernel(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, tk, tv, tq, tdo, p, fp, first_ctas);
     if (st != AF_OK) return st;
-    const long long fthreads = rows * (D / 4);
-    return launch_kernel(bwd_dq_finish_kernel<D>, dim3(static_cast<unsigned>((fthreads + 255) / 256), 1, 1), dim3(256, 1, 1), 0,
-                         stream, true, static_cast<const float*>(a.dq_acc), dq, dq_f32, p.table, sh->S, p.R, p.scale, rows);
+    const long long fthreads = static_cast<long long>(sh->S) * (D / 8);
+    const int nh = sh->B * sh->Hq;
+    const unsigned fy = static_cast<unsigned>((nh + kFinishHeads - 1) / kFinishHeads);
+    if (fy > 65535) return AF_ERR_SHAPE;
+    return launch_kernel(bwd_dq_finish_kernel<D>, dim3(static_cast<unsigned>((fthreads + 255) / 256), fy, 1), dim3(256, 1, 1), 0,
+                         stream, true, static_cast<const float*>(a.dq_acc), dq, dq_f32, p.table, nh, sh->S, p.R, p.scale, first ? fp.rows : 0);
 }
 
 template <int D>
@@ -509,14 +544,19 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
         p.bs_idx = blocks ? (dkv_role ? blocks->row_idx : blocks->col_idx) : nullptr;
         p.bs_order = blocks ? (dkv_role ? blocks->col_order : blocks->row_order) : nullptr;
     };
-    const long long rows = static_cast<long long>(sh->B) * sh->Hq * sh->S;
-    const long long threads = rows * (D / 8);
-    bwd_delta_kernel<D><<<static_cast<unsigned>((threads + 255) / 256), 256, 0, stream>>>(
-        static_cast<const uint4*>(o), static_cast<const uint4*>(d_o), delta, rows);
-    if (cudaGetLastError() != cudaSuccess) return AF_ERR_CUDA;
+    // with room for both caches K' comes from the set-up pass (and Q' from the dQ kernel)
+    const bool k_cached = p.R > 0 && tkp && tqp;
+    BwdPrologueParams pp = {};
+    pp.R = p.R;
+    pp.table = p.table;
+    if (k_cached) {
+        pp.k = static_cast<const uint4*>(k); pp.k_out = static_cast<uint4*>(kcache);
+        pp.kb = stkv.b; pp.kh = stkv.h; pp.ks = stkv.s;
+    }
+    af_status st = launch_prologue<D>(sh, o, d_o, delta, pp, stream);
+    if (st != AF_OK) return st;
     p.delta = delta;
     const unsigned tiles = static_cast<unsigned>((sh->S + 127) / 128);
-    af_status st;
 #ifdef AF_TRACE
     // tracing builds only: 1 = dK/dV kernel only, 2 = dQ kernel only (the skipped outputs stay unwritten)
     const int only = getenv("AF_BWD_ONLY") ? atoi(getenv("AF_BWD_ONLY")) : 0;
@@ -527,8 +567,7 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
     if (p.bias || p.relu) {
         // additive_bias / relu_attention: the both-caches set-up with rotation, the plain one without
         if (p.R > 0) {
-            if (!tkp || !tqp) return AF_ERR_WORKSPACE;
-            if ((st = launch_rope(k, stkv, kcache, sh->B, sh->Hkv, sh->S, D, p.R, p.table, 0, stream, true)) != AF_OK) return st;
+            if (!k_cached) return AF_ERR_WORKSPACE;
             p.out1 = dq; p.out2 = nullptr; p.out_f32 = dq_f32; p.store_x = 1;
             if ((st = launch_bwd_gen<D, false, true>(tq, tdo, *tkp, tv, *tqp, p, gq, stream)) != AF_OK) return st;
             p.out1 = dv; p.out2 = dk; p.out_f32 = dkv_f32; p.store_x = 0;
@@ -539,9 +578,8 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
         p.out1 = dv; p.out2 = dk; p.out_f32 = dkv_f32; p.store_x = 0;
         return launch_bwd_gen<D, true, false>(tk, tv, tq, tdo, tk, p, gkv, stream);
     }
-    if (p.R > 0 && tkp && tqp && only == 0) {
-        // both caches: K' by the RoPE pass, Q' by the dQ kernel, no on-chip rotation in the dK/dV loop
-        if ((st = launch_rope(k, stkv, kcache, sh->B, sh->Hkv, sh->S, D, p.R, p.table, 0, stream, true)) != AF_OK) return st;
+    if (k_cached && only == 0) {
+        // both caches: K' by the set-up pass, Q' by the dQ kernel, no on-chip rotation in the dK/dV loop
         p.out1 = dq; p.out2 = nullptr; p.out_f32 = dq_f32; p.store_x = 1;
         role_lists(false);
         if ((st = launch_bwd_variant<D, false, true, false>(tq, tdo, *tkp, tv, *tqp, p, gq, stream)) != AF_OK) return st;

@@ -12,8 +12,12 @@
 // One CTA per (batch, kv head).  The query rows of up to four heads of the group are stacked into one
 // [4 * kFirstRows, D] panel, so every product below is a small dense contraction over shared memory and the
 // sums over the heads of the group happen in a fixed order: the result is run-to-run deterministic.
-// The kernel runs after the two MMA kernels: it overwrites rows i < kFirstRows of dQ (which the dQ kernel
-// wrote as zeros) and adds its part to rows j < kFirstRows of dK and dV.
+// Two ways to run it.  SHARED = true: as extra CTAs of the one-pass backward kernel's grid (fp32 dK and dV).  Both sides
+// add to rows j < kFirstRows of dK and dV, which the set-up pass zeroed (two addends: the sum does not depend on
+// their order), and the last pass of dQ leaves rows i < kFirstRows to these CTAs.  The chain of latencies that this
+// computation is then runs beside the MMA work instead of behind it.  SHARED = false: as a kernel of its own after the
+// MMA kernels (two-kernel sequence, bf16 dK and dV): it overwrites rows i < kFirstRows of dQ and adds its part to rows
+// j < kFirstRows of dK and dV.
 #pragma once
 #include "common.cuh"
 
@@ -55,11 +59,11 @@ __device__ __forceinline__ void first_rows_rotate(float* row, int R, const float
     }
 }
 
-template <int D>
-__global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsParams p) {
+// NT threads of one CTA on the (batch, kv head) `unit`; all of the CTA's threads call it.
+template <int D, int NT, bool SHARED>
+__device__ __forceinline__ void first_rows_unit(const FirstRowsParams& p, int unit, float* fr_smem) {
     using L = FirstRowsSmem<D>;
     constexpr int NR = kFirstRows, PANEL = L::PANEL, LDK = L::LDK;
-    extern __shared__ float fr_smem[];
     float* Kp = fr_smem;                  // [NR][LDK] rotated keys
     float* Vs = Kp + NR * LDK;            // [NR][LDK]
     float* dKp = Vs + NR * LDK;           // [NR][D] gradient w.r.t. rotated keys
@@ -74,22 +78,21 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
     float2* cs = reinterpret_cast<float2*>(dl + PANEL);   // [NR][R/2] {cos, sin} of positions 0 .. NR - 1
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int b = blockIdx.x / p.Hkv, hk = blockIdx.x % p.Hkv;
+    const int b = unit / p.Hkv, hk = unit % p.Hkv;
     const int rows = p.rows;              // query rows per head here = key rows they can see
     const __nv_bfloat16* kbase = p.k + b * p.kb + hk * p.kh;
     const __nv_bfloat16* vbase = p.v + b * p.kb + hk * p.kh;
 
-    grid_dep_launch();
     // Every global read below is a 16-byte load issued in a batch before its first use: with one CTA per
     // (batch, kv head) the kernel is a chain of memory latencies, not of arithmetic.
     // {cos, sin} of the first positions (the table rows of positions 0 .. rows - 1 are contiguous)
     if (p.R > 0) {
         const int n4 = rows * (p.R >> 1) / 2;   // float4 = two {cos, sin} pairs; R / 2 is a multiple of 8
-        for (int idx = tid; idx < n4; idx += 256)
+        for (int idx = tid; idx < n4; idx += NT)
             reinterpret_cast<float4*>(cs)[idx] = __ldg(reinterpret_cast<const float4*>(p.table) + idx);
     }
     // keys and values of the first rows (8 bf16 per load); gradients start at zero
-    static_assert(NR * D / 8 == 256 || NR * D / 8 == 128, "one 16-byte chunk of K and of V per thread");
+    static_assert(NR * D / 8 <= NT, "at most one 16-byte chunk of K and of V per thread");
     if (tid < NR * D / 8) {
         const int j = tid / (D / 8), d = (tid % (D / 8)) * 8;
         uint4 kw = make_uint4(0u, 0u, 0u, 0u), vw = kw;
@@ -106,13 +109,13 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
             Vs[j * LDK + d + 2 * u + 1] = bf16hi_to_f32(va[u]);
         }
     }
-    for (int idx = tid; idx < NR * D; idx += 256) {
+    for (int idx = tid; idx < NR * D; idx += NT) {
         dKp[idx] = 0.f;
         dVs[idx] = 0.f;
     }
     __syncthreads();
     if (p.R > 0)
-        for (int j = warp; j < rows; j += 8) first_rows_rotate(Kp + j * LDK, p.R, cs, j, 1.f, lane);
+        for (int j = warp; j < rows; j += NT / 32) first_rows_rotate(Kp + j * LDK, p.R, cs, j, 1.f, lane);
     __syncthreads();
 
     for (int h0 = 0; h0 < p.group; h0 += kFirstHeads) {
@@ -120,11 +123,11 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         const int prow = nh * NR;          // panel rows in use: r = hh * NR + i
         // 1. queries (rotated) and upstream gradients of the panel
         {
-            constexpr int CH = PANEL * D / 8 / 256;   // 16-byte chunks per thread and array
+            constexpr int CH = PANEL * D / 8 / NT;   // 16-byte chunks per thread and array
             uint4 qw[CH], gw[CH];
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
-                const int idx = (tid + c * 256) * 8;
+                const int idx = (tid + c * NT) * 8;
                 const int r = idx / D, d = idx - r * D, hh = r / NR, i = r - hh * NR;
                 const int h = hk * p.group + h0 + hh;
                 qw[c] = make_uint4(0u, 0u, 0u, 0u);
@@ -136,7 +139,7 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
             }
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
-                const int idx = (tid + c * 256) * 8;
+                const int idx = (tid + c * NT) * 8;
                 const uint32_t qa[4] = {qw[c].x, qw[c].y, qw[c].z, qw[c].w}, ga[4] = {gw[c].x, gw[c].y, gw[c].z, gw[c].w};
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -149,11 +152,11 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         }
         __syncthreads();
         if (p.R > 0)
-            for (int r = warp; r < prow; r += 8)
+            for (int r = warp; r < prow; r += NT / 32)
                 if (r % NR < rows) first_rows_rotate(Qp + r * D, p.R, cs, r % NR, 1.f, lane);
         __syncthreads();
         // 2. scores s_rj = c <q'_r, k'_j> + slope (j - i) for the kept pairs (j <= i, i - j <= window), and dP_rj = <dO_r, v_j>
-        for (int idx = tid; idx < PANEL * NR; idx += 256) {
+        for (int idx = tid; idx < PANEL * NR; idx += NT) {
             const int r = idx / NR, j = idx - r * NR, hh = r / NR, i = r - hh * NR;
             float s = -INFINITY, dp = 0.f;
             if (hh < nh && i < rows && j <= i && (p.window < 0 || i - j <= p.window)) {
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         }
         __syncthreads();
         // 4. delta_r = <dO_r, O_r> with O_r = sum_j P_rj v_j recomputed here; one warp per row
-        for (int r = warp; r < PANEL; r += 8) {
+        for (int r = warp; r < PANEL; r += NT / 32) {
             float part = 0.f;
             for (int d = lane; d < D; d += 32) {
                 float o = 0.f;
@@ -198,10 +201,10 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         }
         __syncthreads();
         // 5. dS_rj = P_rj (dP_rj - delta_r)
-        for (int idx = tid; idx < PANEL * NR; idx += 256) dSs[idx] = Ps[idx] * (dPs[idx] - dl[idx / NR]);
+        for (int idx = tid; idx < PANEL * NR; idx += NT) dSs[idx] = Ps[idx] * (dPs[idx] - dl[idx / NR]);
         __syncthreads();
         // 6. dV_j += sum_r P_rj dO_r,  dK'_j += c sum_r dS_rj q'_r   (panel rows in order: fixed summation order)
-        for (int idx = tid; idx < NR * D; idx += 256) {
+        for (int idx = tid; idx < NR * D; idx += NT) {
             const int j = idx / D, d = idx - j * D;
             float av = 0.f, ak = 0.f;
             for (int r = 0; r < prow; ++r) {
@@ -212,7 +215,7 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
             dKp[idx] += ak * p.scale;
         }
         //    dQ'_r = c sum_j dS_rj k'_j
-        for (int idx = tid; idx < PANEL * D; idx += 256) {
+        for (int idx = tid; idx < PANEL * D; idx += NT) {
             const int r = idx / D, d = idx - r * D;
             float a = 0.f;
             for (int j = 0; j < NR; ++j) a = fmaf(dSs[r * NR + j], Kp[j * LDK + d], a);
@@ -221,11 +224,11 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         __syncthreads();
         // 7. dQ_r = R(i)^T dQ'_r, written over the zeros the dQ kernel left in these rows
         if (p.R > 0)
-            for (int r = warp; r < prow; r += 8)
+            for (int r = warp; r < prow; r += NT / 32)
                 if (r % NR < rows) first_rows_rotate(dQp + r * D, p.R, cs, r % NR, -1.f, lane);
         __syncthreads();
-        grid_dep_wait();   // (first use of an output: the MMA kernels before this one in the stream are complete)
-        for (int idx = tid * 4; idx < PANEL * D; idx += 256 * 4) {
+        if (!SHARED) grid_dep_wait();   // (first use of an output: the MMA kernels before this one in the stream are complete)
+        for (int idx = tid * 4; idx < PANEL * D; idx += NT * 4) {
             const int r = idx / D, d = idx - r * D, hh = r / NR, i = r - hh * NR;
             if (hh < nh && i < rows) {
                 const size_t off = ((static_cast<size_t>(b) * p.Hq + hk * p.group + h0 + hh) * p.S + i) * D + d;
@@ -238,17 +241,25 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
     }
     // dK_j = R(j)^T dK'_j; both gradients are added to what the dK/dV kernel wrote for the later query rows
     if (p.R > 0)
-        for (int j = warp; j < rows; j += 8) first_rows_rotate(dKp + j * D, p.R, cs, j, -1.f, lane);
+        for (int j = warp; j < rows; j += NT / 32) first_rows_rotate(dKp + j * D, p.R, cs, j, -1.f, lane);
     __syncthreads();
-    grid_dep_wait();
-    // four columns per thread and pass; both passes' loads are issued before the first add
-    constexpr int PASSES = NR * D / 4 / 256;
     const size_t out_base = (static_cast<size_t>(b) * p.Hkv + hk) * p.S * D;   // rows j of this kv head are contiguous
+    if constexpr (SHARED) {
+        for (int idx = tid * 4; idx < rows * D; idx += NT * 4) {
+            const float4 a = *reinterpret_cast<const float4*>(dKp + idx), g = *reinterpret_cast<const float4*>(dVs + idx);
+            red_add4(static_cast<float*>(p.dk) + out_base + idx, a);
+            red_add4(static_cast<float*>(p.dv) + out_base + idx, g);
+        }
+        return;
+    }
+    if (!SHARED) grid_dep_wait();
+    // four columns per thread and pass; both passes' loads are issued before the first add
+    constexpr int PASSES = NR * D / 4 / NT > 0 ? NR * D / 4 / NT : 1;
     if (p.dkv_f32) {
         float4 ok[PASSES], ov[PASSES];
 #pragma unroll
         for (int c = 0; c < PASSES; ++c) {
-            const int idx = (tid + c * 256) * 4;
+            const int idx = (tid + c * NT) * 4;
             if (idx / D < rows) {
                 ok[c] = *reinterpret_cast<const float4*>(static_cast<float*>(p.dk) + out_base + idx);
                 ov[c] = *reinterpret_cast<const float4*>(static_cast<float*>(p.dv) + out_base + idx);
@@ -256,7 +267,7 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         }
 #pragma unroll
         for (int c = 0; c < PASSES; ++c) {
-            const int idx = (tid + c * 256) * 4;
+            const int idx = (tid + c * NT) * 4;
             if (idx / D < rows) {
                 const float4 a = *reinterpret_cast<const float4*>(dKp + idx), g = *reinterpret_cast<const float4*>(dVs + idx);
                 *reinterpret_cast<float4*>(static_cast<float*>(p.dk) + out_base + idx) =
@@ -269,7 +280,7 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         uint2 ok[PASSES], ov[PASSES];
 #pragma unroll
         for (int c = 0; c < PASSES; ++c) {
-            const int idx = (tid + c * 256) * 4;
+            const int idx = (tid + c * NT) * 4;
             if (idx / D < rows) {
                 ok[c] = *reinterpret_cast<const uint2*>(static_cast<__nv_bfloat16*>(p.dk) + out_base + idx);
                 ov[c] = *reinterpret_cast<const uint2*>(static_cast<__nv_bfloat16*>(p.dv) + out_base + idx);
@@ -277,7 +288,7 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
         }
 #pragma unroll
         for (int c = 0; c < PASSES; ++c) {
-            const int idx = (tid + c * 256) * 4;
+            const int idx = (tid + c * NT) * 4;
             if (idx / D < rows) {
                 const float4 a = *reinterpret_cast<const float4*>(dKp + idx), g = *reinterpret_cast<const float4*>(dVs + idx);
                 *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.dk) + out_base + idx) =
@@ -289,6 +300,13 @@ __global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsPara
             }
         }
     }
+}
+
+template <int D>
+__global__ void __launch_bounds__(256) bwd_first_rows_kernel(const FirstRowsParams p) {
+    extern __shared__ float fr_smem[];
+    grid_dep_launch();
+    first_rows_unit<D, 256, false>(p, blockIdx.x, fr_smem);
 }
 
 }  // namespace af

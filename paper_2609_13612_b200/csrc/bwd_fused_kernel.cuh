@@ -42,6 +42,7 @@
 // working out the next tile's mask and addresses between the two phases (the warpgroups fall into step and the
 // shared exponential unit stretches phase P: 4.9 k).
 #pragma once
+#include "bwd_first_rows.cuh"
 #include "bwd_kernel.cuh"
 
 namespace af {
@@ -151,7 +152,8 @@ __device__ __forceinline__ void grad_phase_ds32(const uint32_t* dp, int col0, co
 template <int D, bool BS = false>
 __global__ void __launch_bounds__(512, 1)
 attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_y,
-                      const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const BwdParams p) {
+                      const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const BwdParams p,
+                      const FirstRowsParams fr, int first_ctas) {
     static_assert(D == 128 || D == 64, "head dimension");
     using L = BwdFusedSmem<D>;
     constexpr int TILE = L::TILE, NST = L::NST;
@@ -173,6 +175,14 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         if (threadIdx.x == 0) atomicCAS(&g_device_status, 0u, (kFusedSmemCode << 16) | (blockIdx.x & 0xffffu));
         return;
     }
+    if (static_cast<int>(blockIdx.y) < first_ctas) {
+        // the first row of the grid: the pairs of the first query rows, in fp32 (see bwd_first_rows.cuh)
+        grid_dep_wait();
+        grid_dep_launch();
+        static_assert(FirstRowsSmem<D>::BYTES <= L::NEEDED, "the panels of the first rows must fit");
+        first_rows_unit<D, 512, true>(fr, blockIdx.x, reinterpret_cast<float*>(smem));
+        return;
+    }
     uint8_t *sX = smem + L::OFF_X, *sY = smem + L::OFF_Y, *sA = smem + L::OFF_A, *sB = smem + L::OFF_B;
     uint8_t* sDS = smem + L::OFF_DS;
     float* sStats = reinterpret_cast<float*>(smem + L::OFF_STATS);
@@ -184,7 +194,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     const MaskSpec ms{p.S, p.causal, p.window, p.skip_rows};
     const int b = blockIdx.x / p.Hkv, xh = blockIdx.x - b * p.Hkv;
     // heaviest key tiles first under a causal mask; with block lists the caller's order
-    const int x0 = ((BS && p.bs_order) ? __ldg(p.bs_order + blockIdx.y) : static_cast<int>(blockIdx.y)) * 128;
+    const int by = static_cast<int>(blockIdx.y) - first_ctas;
+    const int x0 = ((BS && p.bs_order) ? __ldg(p.bs_order + by) : by) * 128;
     int lo, hi;
     qtile_range(ms, x0, lo, hi);
     int bs_base = 0;
@@ -549,8 +560,9 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             tc_fence_after_sync();
             float* stg = reinterpret_cast<float*>(sA);
             const size_t out_row0 = (static_cast<size_t>(b) * p.Hkv + xh) * p.S + x0;
-            store_acc_rotated<D>(tb + ACC1, stg, gtid, 1.f, 0, p.table, x0, p.S, p.out1, out_row0, p.out_f32);
-            store_acc_rotated<D>(tb + ACC2, stg, gtid, p.scale, p.R, p.table, x0, p.S, p.out2, out_row0, p.out_f32);
+            const int add_rows = first_ctas ? fr.rows : 0;
+            store_acc_rotated<D>(tb + ACC1, stg, gtid, 1.f, 0, p.table, x0, p.S, p.out1, out_row0, p.out_f32, add_rows);
+            store_acc_rotated<D>(tb + ACC2, stg, gtid, p.scale, p.R, p.table, x0, p.S, p.out2, out_row0, p.out_f32, add_rows);
         }
     }
 
@@ -562,39 +574,57 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     }
 }
 
-// dQ = c * R^T(accumulated dQ'): fp32 accumulator [rows][D] -> the caller's dQ (bf16 or fp32), rows = B * Hq * S in
-// [B, Hq, S] order.  One thread per four columns below R / 2 together with their partners above (or four
-// unrotated columns).  HBM bound: 4 + 2 (or 4) bytes per element.
+// dQ = c * R^T(accumulated dQ'): fp32 accumulator [B * Hq, S, D] -> the caller's dQ (bf16 or fp32).  A thread owns columns
+// 4 c .. 4 c + 3 below R / 2 and their partners above (or eight unrotated columns) of one sequence row for
+// kFinishHeads heads: every element is read once, and the cos/sin of the row once for all of them.  HBM bound: 4 + 2
+// (or 4) bytes per element.  Rows i < skip_rows belong to the first-rows CTAs.
+constexpr int kFinishHeads = 4;
 template <int D>
 __global__ void __launch_bounds__(256) bwd_dq_finish_kernel(const float* __restrict__ acc, void* __restrict__ out, int out_f32,
-                                                            const float2* __restrict__ table, int S, int R, float scale,
-                                                            long long rows) {
+                                                            const float2* __restrict__ table, int NH, int S, int R, float scale,
+                                                            int skip_rows) {
     grid_dep_wait();
     grid_dep_launch();
-    constexpr int TPR = D / 4;
-    const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    const long long row = idx / TPR;
-    if (row >= rows) return;
-    const int d = static_cast<int>(idx % TPR) * 4;
-    const int half = R >> 1;
-    const float4 a = __ldcs(reinterpret_cast<const float4*>(acc + row * D + d));
-    float4 y = make_float4(a.x * scale, a.y * scale, a.z * scale, a.w * scale);
-    if (d < R) {
-        const bool upper = d >= half;
-        const int partner = upper ? d - half : d + half, fi = upper ? d - half : d;
-        const float4 o = __ldcs(reinterpret_cast<const float4*>(acc + row * D + partner));
-        const int pos = static_cast<int>(row % S);
-        const float4 t01 = __ldg(reinterpret_cast<const float4*>(table + static_cast<size_t>(pos) * half + fi));
-        const float4 t23 = __ldg(reinterpret_cast<const float4*>(table + static_cast<size_t>(pos) * half + fi + 2));
-        const float sg = upper ? -scale : scale;   // transpose rotation: y c + other s below R / 2, y c - other s above
-        y.x = fmaf(y.x, t01.x, o.x * sg * t01.y);
-        y.y = fmaf(y.y, t01.z, o.y * sg * t01.w);
-        y.z = fmaf(y.z, t23.x, o.z * sg * t23.y);
-        y.w = fmaf(y.w, t23.z, o.w * sg * t23.w);
+    constexpr int SPR = D / 8;   // slots per row
+    const long long idx = blockIdx.x * 256ll + threadIdx.x;
+    const int s = static_cast<int>(idx / SPR), c = static_cast<int>(idx % SPR);
+    if (s >= S || s < skip_rows) return;
+    const int half = R >> 1, rslots = R >> 3, h0 = blockIdx.y * kFinishHeads;
+    const bool rot = c < rslots;
+    const int d0 = rot ? 4 * c : R + 8 * (c - rslots), d1 = rot ? d0 + half : d0 + 4;
+    float4 a[kFinishHeads], b[kFinishHeads];
+#pragma unroll
+    for (int u = 0; u < kFinishHeads; ++u)
+        if (h0 + u < NH) {
+            const float* row = acc + (static_cast<size_t>(h0 + u) * S + s) * D;
+            a[u] = __ldcs(reinterpret_cast<const float4*>(row + d0));
+            b[u] = __ldcs(reinterpret_cast<const float4*>(row + d1));
+        }
+    float4 cs = make_float4(scale, scale, scale, scale), sn = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (rot) {
+        const float4 t01 = __ldg(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0));
+        const float4 t23 = __ldg(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0 + 2));
+        cs = make_float4(t01.x * scale, t01.z * scale, t23.x * scale, t23.z * scale);
+        sn = make_float4(t01.y * scale, t01.w * scale, t23.y * scale, t23.w * scale);
     }
-    const size_t oi = static_cast<size_t>(row) * D + d;
-    if (out_f32) *reinterpret_cast<float4*>(static_cast<float*>(out) + oi) = y;
-    else *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + oi) = make_uint2(pack_bf16x2(y.x, y.y), pack_bf16x2(y.z, y.w));
+#pragma unroll
+    for (int u = 0; u < kFinishHeads; ++u)
+        if (h0 + u < NH) {
+            // transpose rotation: a c + b s below R / 2, b c - a s above
+            const float4 y0 = make_float4(fmaf(a[u].x, cs.x, b[u].x * sn.x), fmaf(a[u].y, cs.y, b[u].y * sn.y),
+                                          fmaf(a[u].z, cs.z, b[u].z * sn.z), fmaf(a[u].w, cs.w, b[u].w * sn.w));
+            const float4 y1 = make_float4(fmaf(b[u].x, cs.x, -a[u].x * sn.x), fmaf(b[u].y, cs.y, -a[u].y * sn.y),
+                                          fmaf(b[u].z, cs.z, -a[u].z * sn.z), fmaf(b[u].w, cs.w, -a[u].w * sn.w));
+            const size_t row = (static_cast<size_t>(h0 + u) * S + s) * D;
+            if (out_f32) {
+                *reinterpret_cast<float4*>(static_cast<float*>(out) + row + d0) = y0;
+                *reinterpret_cast<float4*>(static_cast<float*>(out) + row + d1) = y1;
+            } else {
+                __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + row;
+                *reinterpret_cast<uint2*>(o + d0) = make_uint2(pack_bf16x2(y0.x, y0.y), pack_bf16x2(y0.z, y0.w));
+                *reinterpret_cast<uint2*>(o + d1) = make_uint2(pack_bf16x2(y1.x, y1.y), pack_bf16x2(y1.z, y1.w));
+            }
+        }
 }
 
 }  // namespace af

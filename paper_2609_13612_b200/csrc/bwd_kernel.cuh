@@ -1,5 +1,5 @@
 // Backward kernels (Section 4.4, FlashAttention-2 decomposition):
-//   1. bwd_delta_kernel      delta_i = sum_d dO_id * O_id             (row-reduced gradients)
+//   1. bwd_prologue_kernel   delta_i = sum_d dO_id * O_id, rotated copies    (row-reduced gradients)
 //   2. attn_bwd_kernel<DKV>  per key tile: dV += P^T dO, dK' += dS^T Q'   (no atomics: one CTA owns the tile)
 //   3. attn_bwd_kernel<DQ>   per query tile: dQ' += dS K'
 // Both MMA kernels recompute P from the saved L, recompute the RoPE rotation on chip, and rotate
@@ -21,6 +21,7 @@
 #include <cuda.h>
 #include <type_traits>
 #include "common.cuh"
+#include "rope_kernels.cuh"
 
 namespace af {
 
@@ -53,25 +54,94 @@ struct BwdParams {
     int relu;
 };
 
-// delta[row] = <dO[row], O[row]>; one 16-byte chunk per thread, D/8 threads per row.
+// Set-up pass of the backward sequences, one launch: delta, the rotated copies of K and Q that the sequence asked for, and
+// zeros where it accumulates.  The parts are independent; each takes a range of blocks.  All of them are HBM-bound copies,
+// so for large problems one launch costs what the parts cost, and for small ones (a launch each, of 3 to 7 us) it is
+// one latency instead of four.  Backward as a whole with this pass, the first query rows inside the one-pass grid
+// and the single-read last pass: 83.1 -> 51.8 us at B = 2, 6 q / 2 kv heads, S = 777, D = 128; 144 -> 124 us at B = 4,
+// 16 heads, S = 1024, D = 128; 564 -> 522 us at B = 4, 32 / 8 heads, S = 2048; 508 -> 476 us at B = 4, 12 heads, S = 4096, D = 64.
+struct BwdPrologueParams {
+    const uint4 *o, *d_o;       // [rows][D] bf16
+    float* delta;               // delta[row] = <dO[row], O[row]>
+    long long rows;
+    const uint4 *q, *k;         // rotated copies (blocks_q / blocks_k > 0): strided input, contiguous output
+    uint4 *q_out, *k_out;
+    long long qb, qh, qs, kb, kh, ks;
+    const float2* table;
+    int B, Hq, Hkv, S, R;
+    float4* acc;                // fp32 accumulator of dQ', zeroed (blocks_acc > 0)
+    long long acc_quads;
+    float *dk, *dv;             // rows j < first_rows of dK and dV (fp32), zeroed (blocks_first > 0)
+    int first_rows;
+    unsigned blocks_q, blocks_k, blocks_delta, blocks_acc, blocks_first;
+};
+constexpr int kPrologueHeads = 4;       // heads per thread of the rotation (one table read for all)
+constexpr int kPrologueRows = 4;        // rows per thread of delta
+constexpr int kPrologueAccQuads = 4;    // 16-byte stores per thread of the zeroing
+
 template <int D>
-__global__ void __launch_bounds__(256) bwd_delta_kernel(const uint4* __restrict__ o, const uint4* __restrict__ d_o,
-                                                        float* __restrict__ delta, long long rows) {
-    constexpr int TPR = D / 8;
-    grid_dep_launch();   // the next kernel of the backward sequence may be scheduled while this one runs
-    const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    const long long row = idx / TPR;
-    float acc = 0.f;
-    if (row < rows) {
-        const uint4 a = __ldg(o + idx), b = __ldg(d_o + idx);
-        const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            acc += bf16lo_to_f32(aw[u]) * bf16lo_to_f32(bw[u]) + bf16hi_to_f32(aw[u]) * bf16hi_to_f32(bw[u]);
+__global__ void __launch_bounds__(256) bwd_prologue_kernel(const BwdPrologueParams p) {
+    grid_dep_wait();
+    grid_dep_launch();   // the gradient kernel may be scheduled (and run its set-up) while this pass runs
+    unsigned blk = blockIdx.x;
+    if (blk < p.blocks_q + p.blocks_k) {
+        const bool is_q = blk < p.blocks_q;
+        if (!is_q) blk -= p.blocks_q;
+        const int H = is_q ? p.Hq : p.Hkv;
+        const int per_row = (p.R >> 4) + ((D - p.R) >> 3);
+        const unsigned per_head = static_cast<unsigned>((static_cast<long long>(p.S) * per_row + 255) / 256);
+        rope_apply_heads<kPrologueHeads>(static_cast<long long>(blk % per_head) * 256 + threadIdx.x,
+                                         static_cast<int>(blk / per_head) * kPrologueHeads, is_q ? p.q : p.k, is_q ? p.q_out : p.k_out,
+                                         p.table, p.B * H, H, p.S, D, p.R, 1.f, is_q ? p.qb : p.kb, is_q ? p.qh : p.kh,
+                                         is_q ? p.qs : p.ks);
+        return;
     }
+    blk -= p.blocks_q + p.blocks_k;
+    if (blk < p.blocks_delta) {
+        // D / 8 threads per row, kPrologueRows rows per thread (the rotation's registers leave few blocks per SM, so every
+        // thread keeps several loads in flight)
+        constexpr int TPR = D / 8;
+        uint4 a[kPrologueRows], b[kPrologueRows];
+        const long long idx0 = blk * (256ll * kPrologueRows) + threadIdx.x;
 #pragma unroll
-    for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (row < rows && (threadIdx.x % TPR) == 0) delta[row] = acc;
+        for (int u = 0; u < kPrologueRows; ++u) {
+            const long long idx = idx0 + u * 256;
+            a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (idx / TPR < p.rows) {
+                a[u] = __ldg(p.o + idx);
+                b[u] = __ldg(p.d_o + idx);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kPrologueRows; ++u) {
+            const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
+            float acc = 0.f;
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+                acc += bf16lo_to_f32(aw[w]) * bf16lo_to_f32(bw[w]) + bf16hi_to_f32(aw[w]) * bf16hi_to_f32(bw[w]);
+#pragma unroll
+            for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            const long long row = (idx0 + u * 256) / TPR;
+            if (row < p.rows && (threadIdx.x % TPR) == 0) p.delta[row] = acc;
+        }
+        return;
+    }
+    blk -= p.blocks_delta;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (blk < p.blocks_acc) {
+#pragma unroll
+        for (int u = 0; u < kPrologueAccQuads; ++u) {
+            const long long i = (static_cast<long long>(blk) * kPrologueAccQuads + u) * 256 + threadIdx.x;
+            if (i < p.acc_quads) p.acc[i] = zero;
+        }
+        return;
+    }
+    blk -= p.blocks_acc;   // one block per (batch, kv head)
+    for (int i = threadIdx.x; i < p.first_rows * (D / 4); i += 256) {
+        const size_t at = static_cast<size_t>(blk) * p.S * (D / 4) + i;
+        reinterpret_cast<float4*>(p.dk)[at] = zero;
+        reinterpret_cast<float4*>(p.dv)[at] = zero;
+    }
 }
 
 template <int D>
@@ -113,10 +183,11 @@ __device__ __forceinline__ bool wg_all(bool v) { return bar_all(v, 3, 256); }
 // (gradients w.r.t. rotated rows are rotated back).  Global writes are coalesced along D.  (Writing each
 // thread's TMEM row straight to global memory - no staging, no barriers, cos/sin read per row - measured
 // slower: a warp's store then touches 32 rows, and the store rate is what bounds this epilogue.)
+// Rows below add_rows (fp32 output only) are added to what is there instead of stored.
 template <int D>
 __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, int gtid, float mul, int R,
                                                   const float2* table, int row0, int S, void* out, size_t out_row0,
-                                                  int out_f32) {
+                                                  int out_f32, int add_rows = 0) {
     constexpr int STRIDE = BwdSmem<D>::STG_STRIDE;
     // (set-up of the second phase first: its table reads are in flight while the first phase runs)
     // Second phase: thread (rsub, d4) writes the four columns 4 d4 .. 4 d4 + 3 of rows rsub, rsub + RPP, ...
@@ -171,7 +242,9 @@ __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, in
                 y.w = fmaf(y.w, c[3], o.w * sn[3]);
             }
             const size_t oi = (out_row0 + r) * D + d;
-            if (out_f32) {
+            if (row0 + r < add_rows) {
+                red_add4(static_cast<float*>(out) + oi, y);
+            } else if (out_f32) {
                 *reinterpret_cast<float4*>(static_cast<float*>(out) + oi) = y;
             } else {
                 *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + oi) =

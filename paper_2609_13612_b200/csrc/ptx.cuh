@@ -325,6 +325,11 @@ __device__ __forceinline__ void setmaxnreg_dec() {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// four fp32 values added to global memory (16-byte aligned)
+__device__ __forceinline__ void red_add4(float* at, float4 v) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 // ---------------------------------------------------------------- small math helpers
 __device__ __forceinline__ float ex2(float x) {
     float y;

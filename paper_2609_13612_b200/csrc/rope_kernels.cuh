@@ -29,22 +29,16 @@ __global__ void rope_table_kernel(float2* __restrict__ table, __nv_bfloat16* __r
 // (columns 8cp.., R/2+8cp..) of sequence row s for HPT consecutive heads, so the table entry is
 // read once and reused; consecutive threads touch consecutive 16-byte chunks (coalesced).
 // Chunks past R are copied when y != x.  sgn = -1 applies the transpose rotation.
+// idx: (row, chunk) of this thread, h0: its first head
 template <int HPT>
-__global__ void __launch_bounds__(256)
-rope_apply_kernel(const uint4* x, uint4* y, const float2* __restrict__ table, int NH, int H, int S,
-                  int D, int R, float sgn, long long xb, long long xh, long long xs) {
-    // programmatic dependent launch, both ways: as a dependent (inside the backward sequence) wait for the
-    // predecessor before touching memory; as a predecessor (of the hybrid forward or of a gradient kernel) let
-    // the next grid be scheduled and run its set-up while this pass runs
-    grid_dep_wait();
-    grid_dep_launch();
+__device__ __forceinline__ void rope_apply_heads(long long idx, int h0, const uint4* x, uint4* y, const float2* __restrict__ table,
+                                                 int NH, int H, int S, int D, int R, float sgn, long long xb, long long xh,
+                                                 long long xs) {
     const int CP = R >> 4;                 // rotated chunk pairs per row
     const int PT = (D - R) >> 3;           // pass-through chunks per row
     const int per_row = CP + PT;
-    const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
     if (idx >= static_cast<long long>(S) * per_row) return;
     const int s = static_cast<int>(idx / per_row), c = static_cast<int>(idx - static_cast<long long>(s) * per_row);
-    const int h0 = blockIdx.y * HPT;
     const int row_chunks = D >> 3;
     // 16-byte chunk index of row s of flattened head h in the (possibly strided) input
     auto in_base = [&](int h) {
@@ -86,6 +80,19 @@ rope_apply_kernel(const uint4* x, uint4* y, const float2* __restrict__ table, in
             }
         }
     }
+}
+
+template <int HPT>
+__global__ void __launch_bounds__(256)
+rope_apply_kernel(const uint4* x, uint4* y, const float2* __restrict__ table, int NH, int H, int S,
+                  int D, int R, float sgn, long long xb, long long xh, long long xs) {
+    // programmatic dependent launch, both ways: as a dependent (inside this library's sequences) wait for the
+    // predecessor before touching memory; as a predecessor (of the hybrid forward) let the next grid be scheduled
+    // and run its set-up while this pass runs
+    grid_dep_wait();
+    grid_dep_launch();
+    rope_apply_heads<HPT>(blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x, blockIdx.y * HPT, x, y, table, NH, H, S, D,
+                          R, sgn, xb, xh, xs);
 }
 
 }  // namespace af

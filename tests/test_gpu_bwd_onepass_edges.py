@@ -1,0 +1,28 @@
+"""One-pass backward at the edges of its parts: the first query rows (fp32, beside the MMA work when dK and dV are fp32,
+behind it when they are bf16), the set-up pass and the last pass of dQ - sequences shorter than, equal to and one past
+the 16 first rows and the 128-row tile, every panel remainder of the query group, partial rotary widths."""
+import pytest
+import torch
+
+import oracle
+import paper_2609_13612_b200 as af
+from paper_2609_13612_b200 import synth
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+W = synth.Workload
+
+
+@pytest.mark.parametrize("dkv", [torch.float32, torch.bfloat16], ids=["fp32", "bf16"])
+@pytest.mark.parametrize("S,group,D,R", [(7, 1, 128, 128), (16, 3, 64, 64), (17, 5, 128, 64), (129, 4, 64, 32), (300, 2, 128, 48), (260, 1, 64, 0)])
+def test_onepass_edges(S, group, D, R, dkv):
+    w = W("onepass_edge", 2, 2 * group, 2, S, D, theta=1e4, rotary_dim=R, backward=True, sigma=0.5, seed_id=700 + S + group)
+    t = synth.draw_all(w)
+    dev = {k: pu.to_dev(v) for k, v in t.items()}
+    o, lse = pu.gpu_fwd(w, dev)
+    with af.option(af.OPT_BWD_ONEPASS, 2):
+        got = pu.gpu_bwd(w, dev, o, lse, dkv_dtype=dkv)
+    want = oracle.run_workload(w, t, backward=True)
+    for name, g, ref in zip(("dQ", "dK", "dV"), got, want):
+        # (the bound of the parity tests; a bf16 dK or dV adds two roundings of half an ulp, 2^-8 of its value in all)
+        pu.assert_close_scaled("%s %s" % (w.name, name), pu.to_np(g), ref)
