@@ -1,7 +1,6 @@
 // Host side of the C-ABI declared in include/attnfuse.h: argument validation, tensor-map
 // encoding, variant selection and launches.  All arithmetic of the path runs in the kernels.
 #include <cuda.h>
-#include <algorithm>
 #include <atomic>
 #include <utility>
 #include <cuda_runtime.h>
@@ -1179,19 +1178,14 @@ af_status bwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     const size_t off_k = bwd_delta_bytes(shape), off_q = off_k + bwd_kcache_bytes(shape);
     const size_t off_acc = off_q + bwd_qcache_bytes(shape);
     // One-pass sequence: dense, room for both caches and the fp32 dQ' accumulator, and not switched off.
-    // Left to itself (option value 1) the choice goes by the average number of kept key tiles per query tile: the
-    // one-pass kernel costs more per tile pair than the two roles of the two-kernel sequence together, but the dQ
-    // role pays a fixed set-up and epilogue per query tile, which dominates while rows are short (measured: ahead at
-    // 8.5 and 9.5 tiles per query tile, behind at 16.5).
+    // Left to itself (option value 1) it is taken wherever it measured faster than the two-kernel sequence: for every
+    // dense mask (D = 64: 1.2-1.4 times on every shape tried; D = 128: 522 against 622 us at B = 4, 32 / 8 heads, S = 2048,
+    // 447 against 487 us at S = 4096, B = 1, 808 against 879 us at 16 / 4 heads, S = 8192, 428 against 479 us without a
+    // causal mask at 16 / 8 heads, S = 4096), and over block lists at D = 64.  Over block lists at D = 128 the key block
+    // that every query block lists makes one CTA the critical path (376 against 455 us at 16 / 4 heads, S = 4096, B = 2).
     const int mode = opt(AF_OPT_BWD_ONEPASS);
-    const double n_tiles = (shape->S + 127) / 128;
-    double avg_tiles = p.causal ? 0.5 * (n_tiles + 1) : n_tiles;
-    if (p.window >= 0) avg_tiles = std::min(avg_tiles, (p.causal ? 1.0 : 2.0) * p.window / 128.0 + 1.5);
-    // At D = 64 the one-pass sequence measured 1.2-1.3 times faster on every shape tried (short and long rows,
-    // grouped queries, window, no causal mask): shared-memory traffic per tile pair is half that of D = 128.
-    // Over block lists (short lists are the rule there) it is taken at D = 64 and, at D = 128, only on request.
     const bool onepass = !gen && workspace_bytes >= off_acc + bwd_dqacc_bytes(shape) &&
-                         (mode >= 2 || (mode == 1 && (shape->D == 64 || (!blocks && avg_tiles <= 12.0))));
+                         (mode >= 2 || (mode == 1 && (shape->D == 64 || !blocks)));
     const bool have_k = p.R > 0 && workspace_bytes >= off_q;
     const bool have_q = have_k && workspace_bytes >= off_acc;
     void* kc = static_cast<uint8_t*>(workspace) + off_k;
