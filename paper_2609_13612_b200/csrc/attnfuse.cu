@@ -201,20 +201,33 @@ af_status allow_dynamic_smem(Kernel kern, int bytes, std::atomic<unsigned long l
 // Launch as a programmatic dependent of the kernel that precedes it in the stream: the grid may be scheduled
 // while that kernel drains and runs its set-up, then waits (griddepcontrol.wait in the kernel) for the
 // predecessor's completion before it touches global memory.  dependent = false: a plain launch.
+// cluster_z: CTAs per cluster along the grid's z dimension.
 template <typename... KArgs, typename... Args>
-af_status launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool dependent,
-                        Args&&... args) {
+af_status launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool dependent,
+                         unsigned cluster_z, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = dependent ? 1 : 0;
+    if (dependent) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster_z > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = 1;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = cluster_z;
+    }
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...) == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+}
+template <typename... KArgs, typename... Args>
+af_status launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool dependent,
+                        Args&&... args) {
+    return launch_cluster(kern, grid, block, smem, stream, dependent, 1u, std::forward<Args>(args)...);
 }
 
 // Internal streams and events of attnfuse_fwd_host, per device, created on first use and kept.
@@ -473,6 +486,47 @@ af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMa
     return launch_first_rows<D>(fp, stream);
 }
 
+// CTAs per key tile of the one-pass kernel: 1, 2, 4 or 8 (a cluster that shares out the key tile's query tiles and sums dK
+// and dV over distributed shared memory).  The number with the smallest estimated time, from a model with three
+// measured constants: a tile pair (2.9 us at D = 128, 2.3 us at D = 64), set-up and epilogue of a CTA (6 us) and what
+// every further CTA of a cluster costs the SMs (18 us: its own set-up, waiting for the others, and SMs held free until
+// a whole cluster fits).  The time is the longer of the longest CTA and the total work over the SMs.
+// Measured, whole backward, 1 / 2 / 4 / 8 CTAs: 52 / 38 / 36 / 43 us (B = 2, 6 q / 2 kv heads, S = 777, window 300, D = 128),
+// 129 / 76 / 65 / 65 us (B = 2, 16 / 2 heads, S = 596), 124 / 188 / 232 / 288 us (B = 4, 16 heads, S = 1024).
+// The lengths of block lists are not known here.  They are taken to be those of a pattern with one global key block and
+// four query blocks for each other key block: 449 / 260 / 247 / 319 us (B = 2, 16 / 4 heads, S = 4096, D = 128, such a list).
+int onepass_splits(int D, int units, int S, int group, int causal, int window, bool blocks) {
+    const double pair = D == 128 ? 2.9 : 2.3, cta = 6.0, extra = 18.0, sms = sm_count() > 0 ? sm_count() : 148;
+    const int tiles = (S + 127) / 128;
+    double longest = 0.0, sum = 0.0;   // query tiles that see a key tile: the most, and over all key tiles
+    if (blocks) {
+        longest = tiles;
+        sum = tiles + 4.0 * (tiles - 1);
+    } else {
+        const int reach = window < 0 ? tiles : (window + 127) / 128 + 1;   // query tiles from the diagonal on
+        for (int j = 0; j < tiles; ++j) {
+            const int below = reach < tiles - j ? reach : tiles - j, above = causal ? 0 : (reach - 1 < j ? reach - 1 : j);
+            const double n = below + above;
+            longest = n > longest ? n : longest;
+            sum += n;
+        }
+    }
+    longest *= group;
+    sum *= static_cast<double>(group) * units;
+    int best = 1;
+    double best_time = 0.0;
+    for (int n = 1; n <= 8; n *= 2) {
+        const double a = longest / n * pair + cta;
+        const double b = (sum * pair + static_cast<double>(units) * tiles * (cta + (n - 1) * extra)) / sms;
+        const double t = a > b ? a : b;
+        if (n == 1 || t < 0.95 * best_time) {
+            best = n;
+            best_time = t;
+        }
+    }
+    return best;
+}
+
 // One-pass sequence (bwd_fused_kernel.cuh): the set-up pass (zeroed fp32 dQ' accumulator, delta, rotated K and Q in the
 // caches), the one-pass kernel (dK, dV, dQ' partials), then scale / rotate back / convert dQ.
 struct OnePassArgs {
@@ -514,14 +568,16 @@ af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CU
     p.bs_ptr = a.blocks ? a.blocks->col_ptr : nullptr;
     p.bs_idx = a.blocks ? a.blocks->row_idx : nullptr;
     p.bs_order = a.blocks ? a.blocks->col_order : nullptr;
-    auto kern = a.blocks ? attn_bwd_fused_kernel<D, true> : attn_bwd_fused_kernel<D, false>;
-    static std::atomic<unsigned long long> configured[2];
-    if (allow_dynamic_smem(kern, L::BYTES, configured[a.blocks ? 1 : 0]) != AF_OK) return AF_ERR_CUDA;
+    const int splits = onepass_splits(D, sh->B * sh->Hkv, sh->S, p.group, p.causal, p.window, a.blocks != nullptr);
+    auto kern = a.blocks ? (splits > 1 ? attn_bwd_fused_kernel<D, true, true> : attn_bwd_fused_kernel<D, true, false>)
+                         : (splits > 1 ? attn_bwd_fused_kernel<D, false, true> : attn_bwd_fused_kernel<D, false, false>);
+    static std::atomic<unsigned long long> configured[4];
+    if (allow_dynamic_smem(kern, L::BYTES, configured[(a.blocks ? 2 : 0) + (splits > 1 ? 1 : 0)]) != AF_OK) return AF_ERR_CUDA;
     const unsigned tiles = static_cast<unsigned>((sh->S + 127) / 128);
     const int first_ctas = first ? 1 : 0;   // rows of the grid
-    dim3 grid(sh->B * sh->Hkv, tiles + first_ctas, 1);
-    st = p.R > 0 ? launch_kernel(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, tkp, tv, tqp, tdo, p, fp, first_ctas)
-                 : launch_kernel(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, tk, tv, tq, tdo, p, fp, first_ctas);
+    dim3 grid(sh->B * sh->Hkv, tiles + first_ctas, splits);
+    st = p.R > 0 ? launch_cluster(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, splits, tkp, tv, tqp, tdo, p, fp, first_ctas, splits)
+                 : launch_cluster(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, splits, tk, tv, tq, tdo, p, fp, first_ctas, splits);
     if (st != AF_OK) return st;
     const long long fthreads = static_cast<long long>(sh->S) * (D / 8);
     const int nh = sh->B * sh->Hq;
@@ -1177,15 +1233,13 @@ af_status bwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     CUtensorMap tkp, tqp;
     const size_t off_k = bwd_delta_bytes(shape), off_q = off_k + bwd_kcache_bytes(shape);
     const size_t off_acc = off_q + bwd_qcache_bytes(shape);
-    // One-pass sequence: dense, room for both caches and the fp32 dQ' accumulator, and not switched off.
-    // Left to itself (option value 1) it is taken wherever it measured faster than the two-kernel sequence: for every
-    // dense mask (D = 64: 1.2-1.4 times on every shape tried; D = 128: 522 against 622 us at B = 4, 32 / 8 heads, S = 2048,
-    // 447 against 487 us at S = 4096, B = 1, 808 against 879 us at 16 / 4 heads, S = 8192, 428 against 479 us without a
-    // causal mask at 16 / 8 heads, S = 4096), and over block lists at D = 64.  Over block lists at D = 128 the key block
-    // that every query block lists makes one CTA the critical path (376 against 455 us at 16 / 4 heads, S = 4096, B = 2).
-    const int mode = opt(AF_OPT_BWD_ONEPASS);
-    const bool onepass = !gen && workspace_bytes >= off_acc + bwd_dqacc_bytes(shape) &&
-                         (mode >= 2 || (mode == 1 && (shape->D == 64 || !blocks)));
+    // One-pass sequence: room for both caches and the fp32 dQ' accumulator, and not switched off.
+    // It measured faster than the two-kernel sequence wherever it applies: D = 64 1.2-1.4 times on every shape tried;
+    // D = 128 522 against 622 us at B = 4, 32 / 8 heads, S = 2048, 447 against 487 us at S = 4096, B = 1, 808 against 879 us
+    // at 16 / 4 heads, S = 8192, 428 against 479 us without a causal mask at 16 / 8 heads, S = 4096; over block lists
+    // 684 against 830 us (B = 4, 32 / 8 heads, S = 4096), 84 against 97 us (B = 2, 12 heads, S = 2000), 259 against 370 us
+    // (B = 2, 16 / 4 heads, S = 4096).
+    const bool onepass = !gen && workspace_bytes >= off_acc + bwd_dqacc_bytes(shape) && opt(AF_OPT_BWD_ONEPASS) >= 1;
     const bool have_k = p.R > 0 && workspace_bytes >= off_q;
     const bool have_q = have_k && workspace_bytes >= off_acc;
     void* kc = static_cast<uint8_t*>(workspace) + off_k;

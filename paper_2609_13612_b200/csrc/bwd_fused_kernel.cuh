@@ -70,6 +70,7 @@ struct BwdFusedSmem {
     static constexpr int STG_STRIDE = BwdSmem<D>::STG_STRIDE;
     static_assert(NEEDED <= 232448, "shared-memory layout exceeds one CTA's limit");
     static_assert(128 * STG_STRIDE * 4 <= 2 * NST * TILE, "staging buffer must fit in the stream stages");
+    static_assert(2 * 128 * STG_STRIDE * 4 <= OFF_STATS, "both staging buffers must fit in the operand tiles");
 };
 
 // timeline stamps for tuning (compiled out unless AF_TRACE): as AF_BSTAMP, with the buffer's address read once per
@@ -84,6 +85,7 @@ struct BwdFusedSmem {
 #endif
 
 constexpr int kFusedLightRegs = 64, kFusedReduceRegs = 96, kFusedGradRegs = 176;
+constexpr int kFusedMinTiles = 2;           // streamed tiles per CTA below which a key tile is not shared out further
 constexpr uint32_t kFusedSmemCode = 0x40;   // status code: dynamic shared memory too misaligned for the layout
 
 // The gradient warpgroups work on a half tile (64 streamed rows) in two phases, so that each of the two products
@@ -147,13 +149,17 @@ __device__ __forceinline__ void grad_phase_ds32(const uint32_t* dp, int col0, co
     }
 }
 
+// SPLIT: the grid's z dimension is a cluster of `splits` CTAs that share out the streamed tiles of a key tile; their partial dV
+// and dK' are summed through distributed shared memory, in rank order.  For problems with fewer key tiles than SMs, or
+// with key tiles that many more query tiles see than the average: see onepass_splits (attnfuse.cu) for where it is
+// taken.  Its own instantiation, because the extra epilogue costs the plain kernel 2-3 % through register allocation.
 // BS: block-sparse attention (Section 4.3) - the streamed query tiles of a key block come from its list of active
 // blocks (p.bs_ptr / p.bs_idx by key block, p.bs_order the launch order) instead of a contiguous range.
-template <int D, bool BS = false>
+template <int D, bool BS = false, bool SPLIT = false>
 __global__ void __launch_bounds__(512, 1)
 attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_y,
                       const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const BwdParams p,
-                      const FirstRowsParams fr, int first_ctas) {
+                      const FirstRowsParams fr, int first_ctas, int splits) {
     static_assert(D == 128 || D == 64, "head dimension");
     using L = BwdFusedSmem<D>;
     constexpr int TILE = L::TILE, NST = L::NST;
@@ -177,6 +183,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     }
     if (static_cast<int>(blockIdx.y) < first_ctas) {
         // the first row of the grid: the pairs of the first query rows, in fp32 (see bwd_first_rows.cuh)
+        if (blockIdx.z != 0) return;
         grid_dep_wait();
         grid_dep_launch();
         static_assert(FirstRowsSmem<D>::BYTES <= L::NEEDED, "the panels of the first rows must fit");
@@ -186,6 +193,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     uint8_t *sX = smem + L::OFF_X, *sY = smem + L::OFF_Y, *sA = smem + L::OFF_A, *sB = smem + L::OFF_B;
     uint8_t* sDS = smem + L::OFF_DS;
     float* sStats = reinterpret_cast<float*>(smem + L::OFF_STATS);
+    // staging of the two accumulators when they are summed over a cluster (all operand tiles are idle by then)
+    float *stg0 = reinterpret_cast<float*>(smem), *stg1 = stg0 + 128 * L::STG_STRIDE;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_MISC + 4);
@@ -205,13 +214,23 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         hi = __ldg(p.bs_ptr + x0 / 128 + 1) - bs_base - 1;
     }
     const int per_head = hi - lo + 1;
-    const int n_it = per_head > 0 ? per_head * p.group : 0;
+    const int n_all = per_head > 0 ? per_head * p.group : 0;
+    // The streamed tiles are shared out among `parts` CTAs of the cluster (a power of two, at least kFusedMinTiles each);
+    // CTAs beyond that have nothing to do.
+    int parts = 1, rank = 0, n_first = 0, n_it = n_all;
+    if constexpr (SPLIT) {
+        rank = static_cast<int>(blockIdx.z);
+        while (parts < splits && n_all >= 2 * parts * kFusedMinTiles) parts *= 2;
+        if (rank >= parts) return;
+        n_first = n_all * rank / parts;
+        n_it = n_all * (rank + 1) / parts - n_first;
+    }
     // Streamed tile n = (query head xh * group + n / per_head, position lo + n % per_head): every role walks the
     // sequence with a cursor of its own (a division per tile sat on the gradient warpgroups' loop-carried chain).
     struct Cursor {
         int pos, head;
     };
-    const Cursor first{0, xh * p.group};
+    const Cursor first{SPLIT && parts > 1 ? n_first % per_head : 0, xh * p.group + (SPLIT && parts > 1 ? n_first / per_head : 0)};
     auto advance = [&](Cursor& c) {
         if (++c.pos == per_head) {
             c.pos = 0;
@@ -556,7 +575,17 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                 }
             }
         }
-        if (ok && n_it > 0) {
+        if (SPLIT && ok && parts > 1) {
+            // (the staging buffers cover the stationary tile and dS^T, which the last dQ'^T products read)
+            ok = wg_all(mbar_wait(&bars[L::B_DQFULL], (n_it - 1) & 1, abort_flag, 55) &&
+                        mbar_wait(&bars[L::B_DQFULL + 1], (n_it - 1) & 1, abort_flag, 56));
+        }
+        if (SPLIT && ok && parts > 1) {
+            tc_fence_after_sync();
+            stage_acc<D>(tb + ACC1, stg0, gtid, 1.f);
+            stage_acc<D>(tb + ACC2, stg1, gtid, p.scale);
+        }
+        if (ok && n_it > 0 && (!SPLIT || parts == 1)) {
             tc_fence_after_sync();
             float* stg = reinterpret_cast<float*>(sA);
             const size_t out_row0 = (static_cast<size_t>(b) * p.Hkv + xh) * p.S + x0;
@@ -566,6 +595,19 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         }
     }
 
+    if (SPLIT && parts > 1) {
+        // (every thread of every working CTA takes both barriers, also after a wait that gave up)
+        __syncwarp();
+        cluster_sync();
+        if (warp >= 8 && !*abort_flag) {
+            const int gtid = threadIdx.x - 256, add_rows = first_ctas ? fr.rows : 0;
+            const size_t out_row0 = (static_cast<size_t>(b) * p.Hkv + xh) * p.S + x0;
+            store_shared_rows<D>(stg0, rank, parts, gtid, 0, p.table, x0, p.S, p.out1, out_row0, p.out_f32, add_rows);
+            store_shared_rows<D>(stg1, rank, parts, gtid, p.R, p.table, x0, p.S, p.out2, out_row0, p.out_f32, add_rows);
+        }
+        __syncwarp();
+        cluster_sync();   // nobody leaves while its shared memory is being read
+    }
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 1) {

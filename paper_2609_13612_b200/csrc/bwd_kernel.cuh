@@ -264,6 +264,65 @@ __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, in
     wg_sync();
 }
 
+// The same epilogue for a key tile whose query tiles were shared out among the CTAs of a cluster: every CTA stages its partial
+// accumulator (stage_acc), and after a cluster barrier CTA `rank` of `n` sums rows [128 rank / n, 128 (rank + 1) / n) over
+// the cluster, in rank order (reproducible), and stores them (store_shared_rows).
+template <int D>
+__device__ __forceinline__ void stage_acc(uint32_t t_acc, float* stg, int gtid, float mul) {
+    constexpr int STRIDE = BwdSmem<D>::STG_STRIDE;
+    const int lane_row = gtid & 127, chalf = gtid >> 7;
+#pragma unroll 1
+    for (int cc = 0; cc < D / 64; ++cc) {
+        const int col = chalf * (D / 2) + cc * 32;
+        uint32_t v[32];
+        tmem_ld32(t_acc + col, v);
+        tmem_wait_ld();
+        float4* dst = reinterpret_cast<float4*>(stg + lane_row * STRIDE + col);
+#pragma unroll
+        for (int e = 0; e < 32; e += 4)
+            dst[e >> 2] = make_float4(__uint_as_float(v[e]) * mul, __uint_as_float(v[e + 1]) * mul,
+                                      __uint_as_float(v[e + 2]) * mul, __uint_as_float(v[e + 3]) * mul);
+    }
+}
+template <int D>
+__device__ __forceinline__ void store_shared_rows(const float* stg, int rank, int n, int gtid, int R, const float2* table, int row0,
+                                                  int S, void* out, size_t out_row0, int out_f32, int add_rows) {
+    constexpr int STRIDE = BwdSmem<D>::STG_STRIDE, TPR = D / 4, RPP = 256 / TPR;
+    const int d = (gtid % TPR) * 4, half = R >> 1;
+    const bool rot = d < R, upper = d >= half;
+    const int partner = upper ? d - half : d + half;
+    const uint32_t base = smem_u32(stg);
+#pragma unroll 1
+    for (int r = 128 * rank / n + gtid / TPR; r < 128 * (rank + 1) / n && row0 + r < S; r += RPP) {
+        float4 y = make_float4(0.f, 0.f, 0.f, 0.f), o = y;
+        float4 t01 = y, t23 = y;
+        if (rot) {
+            const float4* t = reinterpret_cast<const float4*>(table + static_cast<size_t>(row0 + r) * half + (upper ? d - half : d));
+            t01 = __ldg(t);
+            t23 = __ldg(t + 1);
+        }
+        for (int c = 0; c < n; ++c) {
+            const float4 v = ld_cluster4(base + (r * STRIDE + d) * 4, c);
+            y.x += v.x; y.y += v.y; y.z += v.z; y.w += v.w;
+            if (rot) {
+                const float4 w = ld_cluster4(base + (r * STRIDE + partner) * 4, c);
+                o.x += w.x; o.y += w.y; o.z += w.z; o.w += w.w;
+            }
+        }
+        if (rot) {
+            const float sg = upper ? -1.f : 1.f;   // transpose rotation
+            y.x = fmaf(y.x, t01.x, o.x * sg * t01.y);
+            y.y = fmaf(y.y, t01.z, o.y * sg * t01.w);
+            y.z = fmaf(y.z, t23.x, o.z * sg * t23.y);
+            y.w = fmaf(y.w, t23.z, o.w * sg * t23.w);
+        }
+        const size_t oi = (out_row0 + r) * D + d;
+        if (row0 + r < add_rows) red_add4(static_cast<float*>(out) + oi, y);
+        else if (out_f32) *reinterpret_cast<float4*>(static_cast<float*>(out) + oi) = y;
+        else *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + oi) = make_uint2(pack_bf16x2(y.x, y.y), pack_bf16x2(y.z, y.w));
+    }
+}
+
 // One 32-column pass of a gradient warpgroup over its lane's row of T1 (scores) and T2 (dP):
 //   p = 2^(c2 * s + bias - L2),  ds = p * (dP - delta),  masked entries give 0;
 // p (DKV role only) and ds go back to TMEM as bf16 pairs at `out_col` of T1 / T2.

@@ -26,3 +26,24 @@ def test_onepass_edges(S, group, D, R, dkv):
     for name, g, ref in zip(("dQ", "dK", "dV"), got, want):
         # (the bound of the parity tests; a bf16 dK or dV adds two roundings of half an ulp, 2^-8 of its value in all)
         pu.assert_close_scaled("%s %s" % (w.name, name), pu.to_np(g), ref)
+
+
+@pytest.mark.parametrize("B,Hkv,group,S,D,causal,window", [
+    (1, 1, 8, 600, 128, True, -1),      # clusters of 8; the last key tiles share out fewer than 8 ways
+    (2, 2, 3, 777, 128, True, 300),     # 4, odd group: parts begin in the middle of a head
+    (1, 1, 1, 640, 64, False, 100),     # few tiles per key tile, first ones not at the diagonal
+    (1, 8, 4, 1530, 128, True, -1),     # 2
+    (1, 4, 2, 1000, 64, False, -1),     # no mask at all
+])
+def test_key_tiles_shared_out_over_a_cluster(B, Hkv, group, S, D, causal, window):
+    w = W("onepass_cluster", B, Hkv * group, Hkv, S, D, theta=1e4, causal=causal, window=window, alibi=causal, backward=True, seed_id=760 + S)
+    t = synth.draw_all(w)
+    dev = {k: pu.to_dev(v) for k, v in t.items()}
+    o, lse = pu.gpu_fwd(w, dev)
+    got = pu.gpu_bwd(w, dev, o, lse)
+    again = pu.gpu_bwd(w, dev, o, lse)
+    want = oracle.run_workload(w, t, backward=True)
+    for name, g, ref in zip(("dQ", "dK", "dV"), got, want):
+        pu.assert_close_scaled("%s %s" % (w.name, name), pu.to_np(g), ref)
+    # the sums over the cluster run in rank order
+    assert torch.equal(got[1], again[1]) and torch.equal(got[2], again[2])
