@@ -200,7 +200,8 @@ af_status allow_dynamic_smem(Kernel kern, int bytes, std::atomic<unsigned long l
 
 // Launch as a programmatic dependent of the kernel that precedes it in the stream: the grid may be scheduled
 // while that kernel drains and runs its set-up, then waits (griddepcontrol.wait in the kernel) for the
-// predecessor's completion before it touches global memory.  dependent = false: a plain launch.
+// predecessor's completion before it touches global memory.  The predecessor may be anybody's kernel: one that does not
+// signal its dependents early just completes first.  dependent = false: a plain launch.
 // cluster_z: CTAs per cluster along the grid's z dimension.
 template <typename... KArgs, typename... Args>
 af_status launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool dependent,
@@ -310,13 +311,8 @@ af_status launch_fwd_variant(const CUtensorMap& tq, const CUtensorMap& tk, const
     const int rows_per_cta = p.pair_heads ? BM : BM * NQ;
     p.n_row_blocks = (p.S + rows_per_cta - 1) / rows_per_cta;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
-    if (ROPE && !p.rot_k) {
-        // hybrid arm: launched as a programmatic dependent of the RoPE pass on K that precedes it in the stream;
-        // the kernel waits for that pass only before its first key-tile load
-        return launch_kernel(kern, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
-    }
-    kern<<<grid, 128 * (2 + NQ), L::BYTES, stream>>>(tq, tk, tv, to, tt, p);
-    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+    // (hybrid arm: the kernel waits for the RoPE pass on K that precedes it only before its first key-tile load)
+    return launch_kernel(kern, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
 }
 
 // Block-sparse variant (Section 4.3): the grid is (heads or head pairs, 128-row blocks); every CTA walks the
@@ -336,8 +332,7 @@ af_status launch_fwd_blocks_variant(const CUtensorMap& tq, const CUtensorMap& tk
     p.n_row_blocks = (p.S + BM - 1) / BM;
     if (p.bs_rowpair) p.n_row_blocks = (p.n_row_blocks + 1) / 2;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
-    kern<<<grid, 128 * (2 + NQ), L::BYTES, stream>>>(tq, tk, tv, to, tt, p);
-    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+    return launch_kernel(kern, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
 }
 template <int D>
 af_status launch_fwd_blocks(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt,
@@ -402,16 +397,15 @@ af_status launch_bwd_gen(const CUtensorMap& tx, const CUtensorMap& ty, const CUt
 }
 
 // RoPE pass x [B, H, S, D] (strided) -> x_out (contiguous); R > 0.
-// dependent: launch as a programmatic dependent of the preceding kernel (only inside this library's own sequences).
 af_status launch_rope(const void* x_in, const af_strides& st, void* x_out, int B, int H, int S, int D, int R,
-                      const void* rope_table, int inverse, cudaStream_t stream, bool dependent = false) {
+                      const void* rope_table, int inverse, cudaStream_t stream) {
     constexpr int HPT = 4;
     const long long NH = static_cast<long long>(B) * H;
     const int per_row = (R >> 4) + ((D - R) >> 3);
     const long long items = static_cast<long long>(S) * per_row;
     dim3 grid(static_cast<unsigned>((items + 255) / 256), static_cast<unsigned>((NH + HPT - 1) / HPT), 1);
     if (grid.y > 65535) return AF_ERR_SHAPE;
-    return launch_kernel(rope_apply_kernel<HPT>, grid, dim3(256, 1, 1), 0, stream, dependent,
+    return launch_kernel(rope_apply_kernel<HPT>, grid, dim3(256, 1, 1), 0, stream, true,
                          static_cast<const uint4*>(x_in), static_cast<uint4*>(x_out),
                          static_cast<const float2*>(rope_table), static_cast<int>(NH), H, S, D, R, inverse ? -1.f : 1.f,
                          static_cast<long long>(st.b), static_cast<long long>(st.h), static_cast<long long>(st.s));
@@ -437,8 +431,7 @@ af_status launch_prologue(const af_shape* sh, const void* o, const void* d_o, fl
     if (total > 0x7fffffffll) return AF_ERR_SHAPE;
     p.blocks_q = static_cast<unsigned>(bq); p.blocks_k = static_cast<unsigned>(bk); p.blocks_delta = static_cast<unsigned>(bd);
     p.blocks_acc = static_cast<unsigned>(ba); p.blocks_first = static_cast<unsigned>(bf);
-    bwd_prologue_kernel<D><<<static_cast<unsigned>(total), 256, 0, stream>>>(p);
-    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+    return launch_kernel(bwd_prologue_kernel<D>, dim3(static_cast<unsigned>(total), 1, 1), dim3(256, 1, 1), 0, stream, true, p);
 }
 
 // delta, then the two gradient kernels.  tkp / tqp: tensor maps over the rotated-K and rotated-Q caches in
@@ -925,8 +918,8 @@ af_status attnfuse_fwd_fp8(const af_shape* shape, const void* q8, const void* k8
     static std::atomic<unsigned long long> configured{0};
     if (allow_dynamic_smem(attn_fwd_fp8_kernel, Fp8Smem::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
-    attn_fwd_fp8_kernel<<<grid, 512, Fp8Smem::BYTES, static_cast<cudaStream_t>(cuda_stream)>>>(tq, tk, tv, p);
-    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+    return launch_kernel(attn_fwd_fp8_kernel, grid, dim3(512, 1, 1), Fp8Smem::BYTES, static_cast<cudaStream_t>(cuda_stream), true, tq,
+                         tk, tv, p);
 }
 
 size_t attnfuse_fwd_hybrid_workspace_bytes(const af_shape* shape) {
@@ -1156,13 +1149,11 @@ af_status attnfuse_decode(const af_shape* shape, const void* q, const void* k, c
     if (shape->D == 128) {
         static std::atomic<unsigned long long> configured{0};
         if (allow_dynamic_smem(decode_split_kernel<128>, DecodeSmem<128>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
-        decode_split_kernel<128><<<grid, kDecWarps * 32, DecodeSmem<128>::BYTES, stream>>>(tk, tv, p);
-    } else {
-        static std::atomic<unsigned long long> configured{0};
-        if (allow_dynamic_smem(decode_split_kernel<64>, DecodeSmem<64>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
-        decode_split_kernel<64><<<grid, kDecWarps * 32, DecodeSmem<64>::BYTES, stream>>>(tk, tv, p);
+        return launch_kernel(decode_split_kernel<128>, grid, dim3(kDecWarps * 32, 1, 1), DecodeSmem<128>::BYTES, stream, true, tk, tv, p);
     }
-    return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+    static std::atomic<unsigned long long> configured{0};
+    if (allow_dynamic_smem(decode_split_kernel<64>, DecodeSmem<64>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
+    return launch_kernel(decode_split_kernel<64>, grid, dim3(kDecWarps * 32, 1, 1), DecodeSmem<64>::BYTES, stream, true, tk, tv, p);
 }
 
 size_t attnfuse_bwd_workspace_bytes(const af_shape* shape) {

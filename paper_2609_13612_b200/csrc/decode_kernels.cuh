@@ -110,7 +110,13 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         *abort_flag = 0;
         fence_mbar_init();
     }
+    if (lane == 0) {
+        prefetch_tmap(&tm_k);
+        prefetch_tmap(&tm_v);
+    }
     __syncthreads();
+    grid_dep_launch();   // programmatic dependent launch: the set-up above overlaps with the end of the previous kernel
+    grid_dep_wait();
 
     uint8_t* wbase = smem + warp * L::WARP_BYTES;
     uint64_t* wbar = bars + warp * kDecStages;
@@ -127,10 +133,6 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
             }
         }
     };
-    if (lane == 0 && nt > 0) {
-        prefetch_tmap(&tm_k);
-        prefetch_tmap(&tm_v);
-    }
 #pragma unroll
     for (int i = 0; i < kDecStages; ++i)
         if (nt > i) issue(i);

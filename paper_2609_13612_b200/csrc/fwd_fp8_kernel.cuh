@@ -205,6 +205,8 @@ attn_fwd_fp8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    grid_dep_launch();   // programmatic dependent launch: the set-up above overlaps with the end of the previous kernel
+    grid_dep_wait();
 
     if (warp < 8) setmaxnreg_dec<80>();
     if (warp == 0) {

@@ -357,6 +357,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     // Block-sparse: the loops below run over positions in the row block's list (jlo = 0, jhi = length - 1, the
     // same for both query tiles, which share the row block); tile_at() gives the key tile of a position.
+    if constexpr (BS) grid_dep_wait();   // the lists are read here
     int bs_base = 0;
     int last_act[NQ];   // row-pair mode: last list position that is active for query tile q (-1: none)
 #pragma unroll
@@ -417,6 +418,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = warp_uniform(*tmem_slot);
+    // Programmatic dependent launch: everything up to here overlaps with the end of the kernel before this one in the
+    // stream, whose results (and buffers) may be touched from here on.  The hybrid arm waits later, in the producer:
+    // its Q, table and outputs are settled before the RoPE pass that precedes it starts.
+    grid_dep_launch();
+    if (!(ROPE && !p.rot_k)) grid_dep_wait();
 
     // Register budget: the softmax warpgroups hold a full row of 128 scores; the others need little, but the
     // MMA issuer must not spill (it is the most latency-sensitive thread of the CTA: at 64 registers it spilled
