@@ -287,7 +287,8 @@ af_status attnfuse_fwd_host(const af_shape* shape, const void* q_host, const voi
  * rows need 16-byte alignment and strides that are multiples of 8 elements); lse (nullable): [B,Hq] fp32.
  * gqa_group <= 16; D in {64, 128}.  n_splits <= 0: attnfuse_decode_splits(shape), the largest count that keeps the
  * grid of n_splits x B x Hkv CTAs within one CTA per SM of the current device (one wave) with at least 128 keys
- * per split.  Larger requests are clamped to ceil(S / 128) and to 256 splits.
+ * per split, and one split for up to 640 keys.  Larger requests are clamped to that many per kept (not windowed
+ * away) keys and to 256 splits.
  * workspace: attnfuse_decode_workspace_bytes(shape, n_splits) device bytes: a ticket counter per (batch, kv head)
  * at its head, then the partials.  Both phases run in ONE launch: the CTA that finishes last for a kv head merges
  * that head group's partials (in split order: the result does not depend on which CTA is last).  The counters must

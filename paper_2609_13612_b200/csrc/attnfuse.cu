@@ -649,6 +649,14 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
                  : launch_bwd_variant<D, false, true, true>(tq, tdo, tk, tv, tk, p, gq, stream);
 }
 
+template <int D, int NT>
+af_status launch_decode(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t stream) {
+    static std::atomic<unsigned long long> configured{0};
+    if (allow_dynamic_smem(decode_split_kernel<D, NT>, DecodeSmem<D>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
+    return launch_kernel(decode_split_kernel<D, NT>, dim3(p.n_splits, p.B * p.Hkv, 1), dim3(kDecWarps * 32, 1, 1),
+                         DecodeSmem<D>::BYTES, stream, true, tk, tv, p);
+}
+
 size_t bwd_delta_bytes(const af_shape* sh) {
     return (static_cast<size_t>(sh->B) * sh->Hq * sh->S * sizeof(float) + 255) / 256 * 256;
 }
@@ -1085,10 +1093,15 @@ int attnfuse_decode_splits(const af_shape* shape) {
     if (!shape || shape->B < 1 || shape->Hkv < 1 || shape->S < 1) return 0;
     // one CTA per SM fits (its stages take most of the shared memory): as many splits as give at most one
     // CTA per SM of the current device in a single wave, at least 128 keys (one tile per warp) per split
+    if (shape->S <= kDecOneSplitKeys) return 1;
     const int ctas_per_split = shape->B * shape->Hkv;
     int sms = sm_count();
     if (sms < 1) sms = 148;   // no device to ask (host-only callers sizing a workspace): the B200 count
-    const int want = sms / ctas_per_split;
+    int want = sms / ctas_per_split;
+    // Many splits stream faster (45 GB/s each) but are merged kDecBatch at a time by one CTA (0.9 us a batch): past the
+    // optimum of the sum more splits lose (one kv head, 20000 keys, D = 128: 9.3 us with 74 splits, 11.0 us with 148).
+    const double best = sqrt(4.0 * shape->D * shape->S / 45e3 * kDecBatch / 0.9);
+    if (want > kDecBatch && want > best) want = best > kDecBatch ? static_cast<int>(best) : kDecBatch;
     const int most = (shape->S + 127) / 128;
     return want < 1 ? 1 : (want > most ? most : want);
 }
@@ -1122,7 +1135,9 @@ af_status attnfuse_decode(const af_shape* shape, const void* q, const void* k, c
     if (!(softmax_scale > 0.f) || !isfinite(softmax_scale)) return AF_ERR_SPEC;
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !aligned16(workspace)) return AF_ERR_ALIGN;
     if (n_splits <= 0) n_splits = attnfuse_decode_splits(shape);
-    if (n_splits > (shape->S + 127) / 128) n_splits = (shape->S + 127) / 128;
+    const int kept = mask->window >= 0 && mask->window < shape->S ? mask->window + 1 : shape->S;   // keys the window leaves
+    if (n_splits > (kept + 127) / 128) n_splits = (kept + 127) / 128;
+    if (kept <= kDecOneSplitKeys) n_splits = 1;
     if (n_splits > kCombineMaxSplits) n_splits = kCombineMaxSplits;
     if (workspace_bytes < attnfuse_decode_workspace_bytes(shape, n_splits)) return AF_ERR_WORKSPACE;
     af_status st;
@@ -1145,15 +1160,8 @@ af_status attnfuse_decode(const af_shape* shape, const void* q, const void* k, c
     p.o = static_cast<__nv_bfloat16*>(o);
     p.lse = lse;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    dim3 grid(n_splits, shape->B * shape->Hkv, 1);
-    if (shape->D == 128) {
-        static std::atomic<unsigned long long> configured{0};
-        if (allow_dynamic_smem(decode_split_kernel<128>, DecodeSmem<128>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
-        return launch_kernel(decode_split_kernel<128>, grid, dim3(kDecWarps * 32, 1, 1), DecodeSmem<128>::BYTES, stream, true, tk, tv, p);
-    }
-    static std::atomic<unsigned long long> configured{0};
-    if (allow_dynamic_smem(decode_split_kernel<64>, DecodeSmem<64>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
-    return launch_kernel(decode_split_kernel<64>, grid, dim3(kDecWarps * 32, 1, 1), DecodeSmem<64>::BYTES, stream, true, tk, tv, p);
+    if (shape->D == 128) return gqa_group <= 8 ? launch_decode<128, 1>(tk, tv, p, stream) : launch_decode<128, 2>(tk, tv, p, stream);
+    return gqa_group <= 8 ? launch_decode<64, 1>(tk, tv, p, stream) : launch_decode<64, 2>(tk, tv, p, stream);
 }
 
 size_t attnfuse_bwd_workspace_bytes(const af_shape* shape) {

@@ -2,16 +2,22 @@
 //
 // Phase 1 (decode_split_kernel): the cache is cut into splits; a CTA takes one split of one kv head
 // and computes, for the g query heads of that kv head, a partial (m, l, acc) triple with the online
-// softmax.  The g heads are the rows of a 16-row MMA tile (padded by cyclic replication, as the paper
-// does), so K and V are read exactly once per CTA.  Phase 2 merges the partials with a log-sum-exp; it runs in
-// the same launch, in the CTA that finishes last for its kv head (a ticket counter tells which).
+// softmax.  The g heads are the columns of 8-wide MMA tiles, so K and V are read exactly once per CTA.  Phase 2 merges
+// the partials with a log-sum-exp; it runs in the same launch, in the CTA that finishes last for its kv head (a ticket
+// counter tells which).
 //
 // The path is bound by HBM (every K and V byte is read once and used for 4 g flops), so the kernel is
 // built around the memory system: each of the 4 warps of a CTA streams its own 32-key tiles through
 // its own ring of shared-memory stages with TMA (128-byte swizzle, an mbarrier per stage, no
-// CTA-wide synchronisation in the loop), 128 KB in flight per SM.  The two small contractions per
-// tile run on the warp-level tensor-core path (mma.sync m16n8k16 with ldmatrix fragments): at M = 16
-// rows a tcgen05 tile of 128 rows would be 7/8 padding, and the arithmetic is far from the bound.
+// CTA-wide synchronisation in the loop), 192 KB in flight per SM.  The two small contractions per
+// tile run on the warp-level tensor-core path (mma.sync m16n8k16 with ldmatrix fragments): with at most 16 heads a
+// tcgen05 tile of 128 rows would be 7/8 padding, and the arithmetic is far from the bound.
+// Timeline of a call at 8 kv heads, 4096 keys, D = 128 (18 splits, L2-cold caches): first tile 1.0 us after the start, two tiles
+// per warp 1.2 us, the CTA's partial 0.6 us, fence and ticket 0.9 us, the last CTA's merge 1.6 us.  For short caches
+// the parts behind the loop are what matters, so they are written as few dependent memory accesses and little code
+// (it runs once per launch, so every instruction is fetched cold).  Replayed graph, before and after the merges were
+// rewritten and the heads became the N dimension: 8.5 -> 6.5 us (4096 keys, 32 / 8 heads), 31.1 -> 27.3 us (32768 keys,
+// 64 / 8 heads: 4.9 TB/s; the loop alone runs at 7), 26.9 -> 23.2 us (B = 16, 2048 keys), 22.6 -> 14.3 us (64 / 4 heads, 5000).
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"
@@ -35,14 +41,15 @@ struct DecodeParams {
     float* lse;                 // [B, Hq] or nullptr
 };
 
-constexpr int kCombineThreads = 128;
-constexpr int kCombineMaxSplits = 1024;
+constexpr int kCombineMaxSplits = 256;
+constexpr int kDecBatch = 20;   // partial rows the merging CTA requests at once (one CTA per SM: 18 splits at 8 kv heads)
 constexpr int kDecTile = 32;    // keys per warp tile
 constexpr int kDecWarps = 4;
-#ifndef AF_DEC_STAGES
-#define AF_DEC_STAGES 3
-#endif
-constexpr int kDecStages = AF_DEC_STAGES;   // tiles in flight per warp
+constexpr int kDecStages = 3;   // tiles in flight per warp
+
+// Up to here one CTA takes all keys of a kv head: a tile of each warp takes 0.6 us, publishing partials and merging them
+// 2.8 us (5.1 us against 5.4 us with four splits and 6.1 us with two at 512 keys).
+constexpr int kDecOneSplitKeys = 640;
 
 template <int D>
 struct DecodeSmem {
@@ -51,9 +58,8 @@ struct DecodeSmem {
     static constexpr int OFF_BAR = kDecWarps * WARP_BYTES;
     static constexpr int OFF_MISC = OFF_BAR + kDecWarps * kDecStages * 8;
     static constexpr int BYTES = OFF_MISC + 16 + 1024;
-    static constexpr int MERGE_STRIDE = D + 4;                               // floats per merged row
-    static_assert(kDecWarps * 16 * (MERGE_STRIDE + 2) * 4 <= OFF_BAR, "merge buffer must fit in the stages");
-    static_assert((16 * kCombineMaxSplits + 32) * 4 <= OFF_BAR, "combine weights (up to 16 heads) must fit in the stages");
+    static constexpr int PART_STRIDE = D + 4;                                // floats per partial row: acc[D], m, l, padding
+    static_assert(16 * PART_STRIDE * 4 <= WARP_BYTES, "the partials of a warp must fit in its stages");
 };
 
 // 16-byte chunk `chunk` of key row r in a tile of D/64 boxes [32 rows][64 cols], 128-byte swizzle
@@ -70,6 +76,12 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t* r) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
 }
+// 8x8 matrix of bf16 (a word = two adjacent columns of row lane / 4) -> its transpose in the same layout
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t v) {
+    uint32_t r;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+    return r;
+}
 // D (16x8, fp32) += A (16x16, bf16, row) * B (16x8, bf16, col)
 __device__ __forceinline__ void mma_16816(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -79,13 +91,30 @@ __device__ __forceinline__ void mma_16816(float* d, const uint32_t* a, uint32_t 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void dec_accumulate(float4& acc, float& lsum, float4 v, float l, float f) {
+    acc.x = fmaf(v.x, f, acc.x);
+    acc.y = fmaf(v.y, f, acc.y);
+    acc.z = fmaf(v.z, f, acc.z);
+    acc.w = fmaf(v.w, f, acc.w);
+    lsum = fmaf(l, f, lsum);
+}
+// four head dims of row `bh` of the output, and its log-sum-exp
 template <int D>
+__device__ __forceinline__ void dec_store(const DecodeParams& p, size_t bh, int d4, float4 acc, float M, float lsum) {
+    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+    *reinterpret_cast<uint2*>(p.o + bh * D + d4 * 4) =
+        make_uint2(pack_bf16x2(acc.x * inv, acc.y * inv), pack_bf16x2(acc.z * inv, acc.w * inv));
+    if (d4 == 0 && p.lse) p.lse[bh] = lsum > 0.f ? (M + log2f(lsum)) * 0.6931471805599453f : -INFINITY;
+}
+
+// NT: 8-head column tiles, ceil(g / 8).
+template <int D, int NT>
 __global__ void __launch_bounds__(kDecWarps * 32)
 decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                     const DecodeParams p) {
     using L = DecodeSmem<D>;
     constexpr int TILE_BYTES = L::TILE_BYTES;
-    constexpr int NBOX = D / 64, KSTEPS = D / 16, DT = D / 8;
+    constexpr int NBOX = D / 64, KSTEPS = D / 16, MT = kDecTile / 16, DT = D / 16;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -103,7 +132,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     const int t_hi = static_cast<int>(static_cast<long long>(split + 1) * tiles_all / p.n_splits);
     const int k_lo = (tile0 + t_lo) * kDecTile;
     const int n_tiles = t_hi - t_lo;
-    const int nt = n_tiles > warp ? (n_tiles - warp + kDecWarps - 1) / kDecWarps : 0;   // this warp's tiles
+    const int nt_tiles = n_tiles > warp ? (n_tiles - warp + kDecWarps - 1) / kDecWarps : 0;   // this warp's tiles
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kDecWarps * kDecStages; ++i) mbar_init(&bars[i], 1);
@@ -135,192 +164,201 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     };
 #pragma unroll
     for (int i = 0; i < kDecStages; ++i)
-        if (nt > i) issue(i);
+        if (nt_tiles > i) issue(i);
 
-    // the g query heads of this kv head as the 16 rows of the A operand (row r <-> head r mod g)
-    const int r0 = lane >> 2, r1 = r0 + 8;
-    const int h0 = hk * p.group + r0 % p.group, h1 = hk * p.group + r1 % p.group;
-    uint32_t qa[KSTEPS][4];
-    {
-        const uint32_t* q0 = reinterpret_cast<const uint32_t*>(p.q + (static_cast<size_t>(b) * p.Hq + h0) * D);
-        const uint32_t* q1 = reinterpret_cast<const uint32_t*>(p.q + (static_cast<size_t>(b) * p.Hq + h1) * D);
+    // The heads are the N dimension of both products, S^T = K Q^T and O^T = V^T P^T (keys and head dims are M): 8 heads
+    // fill an MMA, where with the heads as rows half of a 16-row tile would be copies for g <= 8.
+    // Column c of tile nt of a result belongs to head hk * g + 8 nt + c (columns beyond g repeat heads and are dropped).
+    uint32_t qb[NT][KSTEPS][2];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        const int h = hk * p.group + (nt * 8 + (lane >> 2)) % p.group;
+        const uint32_t* qr = reinterpret_cast<const uint32_t*>(p.q + (static_cast<size_t>(b) * p.Hq + h) * D) + (lane & 3);
 #pragma unroll
         for (int ks = 0; ks < KSTEPS; ++ks) {
-            const int w = ks * 8 + (lane & 3);   // 32-bit word index: columns 16 ks + 2 (lane % 4)
-            qa[ks][0] = __ldg(q0 + w);
-            qa[ks][1] = __ldg(q1 + w);
-            qa[ks][2] = __ldg(q0 + w + 4);
-            qa[ks][3] = __ldg(q1 + w + 4);
+            qb[nt][ks][0] = __ldg(qr + ks * 8);
+            qb[nt][ks][1] = __ldg(qr + ks * 8 + 4);
         }
     }
-    const float sl0 = p.slopes ? p.slopes[h0] * 1.4426950408889634f : 0.f;
-    const float sl1 = p.slopes ? p.slopes[h1] * 1.4426950408889634f : 0.f;
-
-    float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
-    float o[DT][4];
+    // this lane's result columns: heads 8 nt + 2 (lane % 4) + {0, 1}
+    float slope[NT][2], m[NT][2], l[NT][2];
+    float o[NT][DT][4];
 #pragma unroll
-    for (int i = 0; i < DT; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+    for (int nt = 0; nt < NT; ++nt) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            slope[nt][e] = p.slopes ? p.slopes[hk * p.group + (nt * 8 + 2 * (lane & 3) + e) % p.group] * 1.4426950408889634f : 0.f;
+            m[nt][e] = -INFINITY;
+            l[nt][e] = 0.f;
+        }
+#pragma unroll
+        for (int dt = 0; dt < DT; ++dt) o[nt][dt][0] = o[nt][dt][1] = o[nt][dt][2] = o[nt][dt][3] = 0.f;
+    }
 
     bool ok = true;
-    for (int i = 0; i < nt; ++i) {
+    for (int i = 0; i < nt_tiles; ++i) {
         const int st = i % kDecStages;
         const int key0 = k_lo + kDecTile * (warp + kDecWarps * i);
         ok = mbar_wait_warp(&wbar[st], (i / kDecStages) & 1, abort_flag, 40);
         if (!ok) break;
         const uint32_t sk = smem_u32(wbase + st * 2 * TILE_BYTES), sv = sk + TILE_BYTES;
+        const int mi = lane >> 3;
 
-        // scores S[16 heads][32 keys] = Q K^T.  The fragment loads of the next step are issued before the
-        // MMAs of the current one (the asm statements keep their order, so the overlap is written out).
-        float s[4][4];
+        // scores: A = K (16 keys x 16 dims per load), the loads of the next step issued before the MMAs of this one (the
+        // asm statements keep their order, so the overlap is written out); two accumulators per tile, for even and odd
+        // steps, halve the chain of dependent MMAs
+        float s[NT][MT][4], s2[NT][MT][4];
 #pragma unroll
-        for (int n8 = 0; n8 < 4; ++n8) s[n8][0] = s[n8][1] = s[n8][2] = s[n8][3] = 0.f;
-        uint32_t kf[2][4][4];
-        auto load_k = [&](int k2, uint32_t (*dst)[4]) {
-            // per 8-key tile four 8x8 matrices: keys 8 n8 .. +7 (rows) x 32 head dims (four 16-byte chunks)
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int n8 = 0; n8 < 4; ++n8)
-                ldmatrix_x4(sk + dec_chunk_offset(n8 * 8 + (lane & 7), k2 * 4 + (lane >> 3)), dst[n8]);
+            for (int mt = 0; mt < MT; ++mt) {
+                s[nt][mt][0] = s[nt][mt][1] = s[nt][mt][2] = s[nt][mt][3] = 0.f;
+                s2[nt][mt][0] = s2[nt][mt][1] = s2[nt][mt][2] = s2[nt][mt][3] = 0.f;
+            }
+        uint32_t kf[2][2][MT][4];   // [buffer][even / odd step][16 keys]
+        auto load_k = [&](int k2, uint32_t (*dst)[MT][4]) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+                    ldmatrix_x4(sk + dec_chunk_offset(mt * 16 + (mi & 1) * 8 + (lane & 7), (2 * k2 + u) * 2 + (mi >> 1)), dst[u][mt]);
         };
         load_k(0, kf[0]);
 #pragma unroll
         for (int k2 = 0; k2 < KSTEPS / 2; ++k2) {
             if (k2 + 1 < KSTEPS / 2) load_k(k2 + 1, kf[(k2 + 1) & 1]);
 #pragma unroll
-            for (int n8 = 0; n8 < 4; ++n8) {
-                mma_16816(s[n8], qa[2 * k2], kf[k2 & 1][n8][0], kf[k2 & 1][n8][1]);
-                mma_16816(s[n8], qa[2 * k2 + 1], kf[k2 & 1][n8][2], kf[k2 & 1][n8][3]);
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    mma_16816(s[nt][mt], kf[k2 & 1][0][mt], qb[nt][2 * k2][0], qb[nt][2 * k2][1]);
+                    mma_16816(s2[nt][mt], kf[k2 & 1][1][mt], qb[nt][2 * k2 + 1][0], qb[nt][2 * k2 + 1][1]);
+                }
+        }
+        uint32_t pb[NT][MT][2];   // P^T as B operands
+        bool grown = false;
+        float f[NT][2];
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            // log2-domain scores with bias and mask: rows = keys lane / 4 (e = 0, 1) and + 8 (e = 2, 3), columns = heads
+            float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int j = key0 + mt * 16 + (lane >> 2) + (e >> 1) * 8;
+                    float t = fmaf(s[nt][mt][e] + s2[nt][mt][e], p.scale_log2, slope[nt][e & 1] * static_cast<float>(j - qpos));
+                    t = (j < p.N && j >= jmin) ? t : -INFINITY;
+                    s[nt][mt][e] = t;
+                    mx[e & 1] = fmaxf(mx[e & 1], t);
+                }
+            float ref[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                for (int off = 4; off < 32; off <<= 1) mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], off));
+                const float mn = fmaxf(m[nt][e], mx[e]);
+                ref[e] = mn == -INFINITY ? 0.f : mn;
+                f[nt][e] = ex2(m[nt][e] - ref[e]);   // m = -inf -> 0
+                grown = grown || f[nt][e] != 1.f;
+                m[nt][e] = mn;
+                l[nt][e] *= f[nt][e];
+            }
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    s[nt][mt][e] = ex2(s[nt][mt][e] - ref[e & 1]);
+                    l[nt][e & 1] += s[nt][mt][e];   // per-lane partial sums; reduced over the key lanes at the end
+                }
+                // (keys x heads) -> (heads x keys): the B operand wants a head's adjacent keys in one word
+                pb[nt][mt][0] = movmatrix_trans(pack_bf16x2(s[nt][mt][0], s[nt][mt][1]));
+                pb[nt][mt][1] = movmatrix_trans(pack_bf16x2(s[nt][mt][2], s[nt][mt][3]));
             }
         }
-        // log2-domain scores with bias and mask; thread holds rows r0 (e = 0, 1) and r1 (e = 2, 3)
-        float mx0 = -INFINITY, mx1 = -INFINITY;
+        if (i > 0 && __any_sync(0xffffffffu, grown)) {   // a new maximum somewhere in the warp
 #pragma unroll
-        for (int n8 = 0; n8 < 4; ++n8) {
+            for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int j = key0 + n8 * 8 + 2 * (lane & 3) + (e & 1);
-                const float rel = static_cast<float>(j - qpos);
-                float t = fmaf(s[n8][e], p.scale_log2, (e < 2 ? sl0 : sl1) * rel);
-                t = (j < p.N && j >= jmin) ? t : -INFINITY;
-                s[n8][e] = t;
-                if (e < 2) mx0 = fmaxf(mx0, t);
-                else mx1 = fmaxf(mx1, t);
-            }
+                for (int dt = 0; dt < DT; ++dt) {
+                    o[nt][dt][0] *= f[nt][0];
+                    o[nt][dt][1] *= f[nt][1];
+                    o[nt][dt][2] *= f[nt][0];
+                    o[nt][dt][3] *= f[nt][1];
+                }
         }
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-        const float mn0 = fmaxf(m[0], mx0), mn1 = fmaxf(m[1], mx1);
-        const float ms0 = mn0 == -INFINITY ? 0.f : mn0, ms1 = mn1 == -INFINITY ? 0.f : mn1;
-        const float a0 = ex2(m[0] - ms0), a1 = ex2(m[1] - ms1);   // m = -inf -> 0
-        m[0] = mn0;
-        m[1] = mn1;
-        float ps0 = 0.f, ps1 = 0.f;
+        // O^T += V^T P^T: A = V^T (16 dims x 16 keys per load, transposed on the way), again one step ahead
+        uint32_t vf[2][MT][4];
+        auto load_v = [&](int dt, uint32_t (*dst)[4]) {
 #pragma unroll
-        for (int n8 = 0; n8 < 4; ++n8) {
-            s[n8][0] = ex2(s[n8][0] - ms0);
-            s[n8][1] = ex2(s[n8][1] - ms0);
-            s[n8][2] = ex2(s[n8][2] - ms1);
-            s[n8][3] = ex2(s[n8][3] - ms1);
-            ps0 += s[n8][0] + s[n8][1];
-            ps1 += s[n8][2] + s[n8][3];
-        }
-        l[0] = l[0] * a0 + ps0;   // per-thread partial sums; reduced over the quad at the end
-        l[1] = l[1] * a1 + ps1;
-#pragma unroll
-        for (int i2 = 0; i2 < DT; ++i2) {
-            o[i2][0] *= a0;
-            o[i2][1] *= a0;
-            o[i2][2] *= a1;
-            o[i2][3] *= a1;
-        }
-        // O += P V: the score fragments of two adjacent 8-key tiles form the A operand of a 16-key step
-        uint32_t pa[2][4];
-#pragma unroll
-        for (int kb = 0; kb < 2; ++kb) {
-            pa[kb][0] = pack_bf16x2(s[2 * kb][0], s[2 * kb][1]);
-            pa[kb][1] = pack_bf16x2(s[2 * kb][2], s[2 * kb][3]);
-            pa[kb][2] = pack_bf16x2(s[2 * kb + 1][0], s[2 * kb + 1][1]);
-            pa[kb][3] = pack_bf16x2(s[2 * kb + 1][2], s[2 * kb + 1][3]);
-        }
-        // V fragments in groups of four loads (group gi: 16-key step gi / NG, head dims 64 (gi % NG) .. +63),
-        // again one group ahead of the MMAs
-        constexpr int NG = DT / 8;          // groups per 16-key step
-        uint32_t vf[2][4][4];
-        auto load_v = [&](int gi, uint32_t (*dst)[4]) {
-            const int kb = gi / NG, dp0 = (gi % NG) * 4, mi = lane >> 3;
-            // transposed 8x8 matrices: keys 16 kb + {0..7, 8..15} (rows) x head dims 16 dp + {0..7, 8..15}
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                ldmatrix_x4_trans(sv + dec_chunk_offset(kb * 16 + (mi & 1) * 8 + (lane & 7), (dp0 + u) * 2 + (mi >> 1)), dst[u]);
+            for (int mt = 0; mt < MT; ++mt)
+                ldmatrix_x4_trans(sv + dec_chunk_offset(mt * 16 + (mi >> 1) * 8 + (lane & 7), dt * 2 + (mi & 1)), dst[mt]);
         };
         load_v(0, vf[0]);
 #pragma unroll
-        for (int gi = 0; gi < 2 * NG; ++gi) {
-            if (gi + 1 < 2 * NG) load_v(gi + 1, vf[(gi + 1) & 1]);
-            const int kb = gi / NG, dp0 = (gi % NG) * 4;
+        for (int dt = 0; dt < DT; ++dt) {
+            if (dt + 1 < DT) load_v(dt + 1, vf[(dt + 1) & 1]);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                mma_16816(o[2 * (dp0 + u)], pa[kb], vf[gi & 1][u][0], vf[gi & 1][u][1]);
-                mma_16816(o[2 * (dp0 + u) + 1], pa[kb], vf[gi & 1][u][2], vf[gi & 1][u][3]);
-            }
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) mma_16816(o[nt][dt], vf[dt & 1][mt], pb[nt][mt][0], pb[nt][mt][1]);
         }
         __syncwarp();
-        if (i + kDecStages < nt) {
+        if (i + kDecStages < nt_tiles) {
             fence_proxy_async_smem();   // the stage was read through the generic proxy; TMA writes it next
             issue(i + kDecStages);
         }
     }
 
-    // merge the four warps' partials in shared memory (the stages are idle now) and write one partial per head
-    l[0] += __shfl_xor_sync(0xffffffffu, l[0], 1);
-    l[0] += __shfl_xor_sync(0xffffffffu, l[0], 2);
-    l[1] += __shfl_xor_sync(0xffffffffu, l[1], 1);
-    l[1] += __shfl_xor_sync(0xffffffffu, l[1], 2);
-    __syncthreads();
-    float* mo = reinterpret_cast<float*>(smem);                                  // [warp][16][MERGE_STRIDE]
-    float* mml = mo + kDecWarps * 16 * L::MERGE_STRIDE;                          // [warp][16][2]
-    {
-        float* w0 = mo + (warp * 16 + r0) * L::MERGE_STRIDE + 2 * (lane & 3);
-        float* w1 = mo + (warp * 16 + r1) * L::MERGE_STRIDE + 2 * (lane & 3);
+    // Merge the four warps' partials and write one partial per head.  A warp's partials go to its own stages (idle now):
+    // row h = (acc[D], m, l) of query head h.
 #pragma unroll
-        for (int i2 = 0; i2 < DT; ++i2) {
-            *reinterpret_cast<float2*>(w0 + i2 * 8) = make_float2(o[i2][0], o[i2][1]);
-            *reinterpret_cast<float2*>(w1 + i2 * 8) = make_float2(o[i2][2], o[i2][3]);
-        }
-        if ((lane & 3) == 0) {
-            mml[(warp * 16 + r0) * 2] = m[0];
-            mml[(warp * 16 + r0) * 2 + 1] = l[0];
-            mml[(warp * 16 + r1) * 2] = m[1];
-            mml[(warp * 16 + r1) * 2 + 1] = l[1];
-        }
-    }
-    __syncthreads();
-    if (*abort_flag) return;
-    for (int idx = threadIdx.x; idx < p.group * D; idx += kDecWarps * 32) {
-        const int h = idx / D, d = idx - h * D;
-        float mw[kDecWarps], M = -INFINITY;
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int w = 0; w < kDecWarps; ++w) {
-            mw[w] = mml[(w * 16 + h) * 2];
-            M = fmaxf(M, mw[w]);
-        }
-        float acc = 0.f, lsum = 0.f;
-        if (M != -INFINITY) {
+        for (int e = 0; e < 2; ++e) {
 #pragma unroll
-            for (int w = 0; w < kDecWarps; ++w) {
-                const float f = ex2(mw[w] - M);
-                acc = fmaf(mo[(w * 16 + h) * L::MERGE_STRIDE + d], f, acc);
-                lsum = fmaf(mml[(w * 16 + h) * 2 + 1], f, lsum);
+            for (int off = 4; off < 32; off <<= 1) l[nt][e] += __shfl_xor_sync(0xffffffffu, l[nt][e], off);
+            const int h = nt * 8 + 2 * (lane & 3) + e;
+            if (h < p.group) {
+                float* row = reinterpret_cast<float*>(wbase) + h * L::PART_STRIDE;
+#pragma unroll
+                for (int dt = 0; dt < DT; ++dt) {
+                    row[dt * 16 + (lane >> 2)] = o[nt][dt][e];
+                    row[dt * 16 + (lane >> 2) + 8] = o[nt][dt][e + 2];
+                }
+                if (lane < 4) *reinterpret_cast<float2*>(row + D) = make_float2(m[nt][e], l[nt][e]);
             }
         }
-        const size_t row = (static_cast<size_t>(b) * p.Hq + hk * p.group + h) * p.n_splits + split;
-        p.part_o[row * D + d] = acc;
-        if (d == 0) {
-            p.part_ml[row * 2] = M;
-            p.part_ml[row * 2 + 1] = lsum;
+    __syncthreads();
+    if (*abort_flag) return;
+    // one thread per (head, four head dims): every load is independent of the others
+    constexpr int D4 = D / 4;
+    const size_t bh0 = static_cast<size_t>(b) * p.Hq + hk * p.group;
+    for (int idx = threadIdx.x; idx < p.group * D4; idx += kDecWarps * 32) {
+        const int h = idx / D4, d4 = idx - h * D4;
+        const float* row = reinterpret_cast<const float*>(smem) + h * L::PART_STRIDE;
+        float2 ml[kDecWarps];
+        float4 v[kDecWarps];
+#pragma unroll
+        for (int w = 0; w < kDecWarps; ++w) {
+            ml[w] = *reinterpret_cast<const float2*>(row + w * (L::WARP_BYTES / 4) + D);
+            v[w] = *reinterpret_cast<const float4*>(row + w * (L::WARP_BYTES / 4) + d4 * 4);
+        }
+        const float M = fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x));
+        const float ref = M == -INFINITY ? 0.f : M;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float lsum = 0.f;
+#pragma unroll
+        for (int w = 0; w < kDecWarps; ++w) dec_accumulate(acc, lsum, v[w], ml[w].y, ex2(ml[w].x - ref));   // m = -inf -> 0
+        if (p.n_splits == 1) {
+            dec_store<D>(p, bh0 + h, d4, acc, M, lsum);
+        } else {
+            const size_t at = (bh0 + h) * p.n_splits + split;
+            *reinterpret_cast<float4*>(p.part_o + at * D + d4 * 4) = acc;
+            if (d4 == 0) *reinterpret_cast<float2*>(p.part_ml + at * 2) = make_float2(M, lsum);
         }
     }
+    if (p.n_splits == 1) return;
 
     // ---- phase 2 in the same launch (Section 4.2: log-sum-exp combine of the partials).  Every CTA publishes its
     // partials (fence), then draws a ticket; the CTA with the last ticket of its kv head sees all of them.  The sums
@@ -331,63 +369,53 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     if (threadIdx.x == 0) {
         const unsigned int t = atomicAdd(p.tickets + blockIdx.y, 1u);
         s_last = (t == static_cast<unsigned int>(p.n_splits) - 1u) ? 1 : 0;
+        if (s_last) p.tickets[blockIdx.y] = 0u;   // ready for the next call on this workspace
     }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    // weights 2^(m_s - M) of every head and split (the stages are idle): one warp per head, lanes over the splits
-    float* wgt = reinterpret_cast<float*>(smem);          // [group][n_splits]
-    float* stat = wgt + 16 * kCombineMaxSplits;            // [group][2]: M, L
-    const int tid = threadIdx.x, n = p.n_splits;
-    const size_t bh0 = static_cast<size_t>(b) * p.Hq + hk * p.group;
-    for (int h = warp; h < p.group; h += kDecWarps) {
-        const float* ml = p.part_ml + (bh0 + h) * n * 2;
-        float mloc = -INFINITY;
-        for (int sidx = lane; sidx < n; sidx += 32) mloc = fmaxf(mloc, __ldcg(ml + sidx * 2));
+    // The last CTA is a chain of memory latencies, so it makes as few of them as it can: a group of D / 4 lanes (one per
+    // four head dims) takes a head, requests up to kDecBatch partial rows at once beside the statistics of all splits
+    // (one lane per split), and only then forms the weights, which it hands round by shuffles.
+    constexpr int GROUPS = 32 / D4 > 0 ? 32 / D4 : 1, LANES = D4;   // heads per warp, lanes per head
+    static_assert(LANES == 32 || LANES == 16, "a head's four-dim columns are a warp or half of one");
+    const int n = p.n_splits, gl = lane % LANES, gbase = lane - gl;
+    for (int h0w = warp * GROUPS; h0w < p.group; h0w += kDecWarps * GROUPS) {   // (uniform over the warp)
+        const int h = min(h0w + lane / LANES, p.group - 1);
+        const float4* po = reinterpret_cast<const float4*>(p.part_o + (bh0 + h) * n * D) + gl;
+        const float2* pm = reinterpret_cast<const float2*>(p.part_ml) + (bh0 + h) * n;
+        constexpr int ROUNDS = (kDecBatch + LANES - 1) / LANES;   // statistics per lane and batch
+        float4 v[kDecBatch];
+        float2 ml[ROUNDS];
+        auto load_batch = [&](int s0) {   // (short straight code: every instruction of this part is fetched cold)
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, off));
-        float lloc = 0.f;
-        for (int sidx = lane; sidx < n; sidx += 32) {
-            const float2 v2 = __ldcg(reinterpret_cast<const float2*>(ml + sidx * 2));
-            const float f = mloc == -INFINITY ? 0.f : ex2(v2.x - mloc);
-            wgt[h * n + sidx] = f;
-            lloc = fmaf(v2.y, f, lloc);
-        }
-        // (fixed tree: the sum does not depend on which CTA runs this)
+            for (int r = 0; r < ROUNDS; ++r)
+                ml[r] = (r * LANES + gl < kDecBatch && s0 + r * LANES + gl < n) ? __ldcg(pm + s0 + r * LANES + gl) : make_float2(-INFINITY, 0.f);
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) lloc += __shfl_xor_sync(0xffffffffu, lloc, off);
-        if (lane == 0) {
-            stat[2 * h] = mloc;
-            stat[2 * h + 1] = lloc;
-        }
-    }
-    __syncthreads();
-    // weighted sums: one thread per (head, four head dims), the splits in index order, 16-byte loads several in flight
-    constexpr int D4 = D / 4;
-    for (int idx = tid; idx < p.group * D4; idx += kDecWarps * 32) {
-        const int h = idx / D4, d4 = idx - h * D4;
-        const float4* po = reinterpret_cast<const float4*>(p.part_o + (bh0 + h) * n * D) + d4;
-        const float* wh = wgt + h * n;
+            for (int u = 0; u < kDecBatch; ++u) v[u] = __ldcg(po + static_cast<size_t>(min(s0 + u, n - 1)) * D4);
+        };
+        load_batch(0);
+        float M = ml[0].x;
+#pragma unroll
+        for (int r = 1; r < ROUNDS; ++r) M = fmaxf(M, ml[r].x);
+        for (int s = kDecBatch + gl; s < n; s += LANES) M = fmaxf(M, __ldcg(pm + s).x);
+#pragma unroll
+        for (int off = LANES / 2; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+        const float ref = M == -INFINITY ? 0.f : M;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-        for (int sidx = 0; sidx < n; ++sidx) {
-            const float4 v4 = __ldcg(po + static_cast<size_t>(sidx) * D4);
-            const float f = wh[sidx];
-            acc.x = fmaf(v4.x, f, acc.x);
-            acc.y = fmaf(v4.y, f, acc.y);
-            acc.z = fmaf(v4.z, f, acc.z);
-            acc.w = fmaf(v4.w, f, acc.w);
+        float lsum = 0.f;
+        for (int s0 = 0; s0 < n; s0 += kDecBatch) {
+            if (s0 > 0) load_batch(s0);
+            float f[ROUNDS];
+#pragma unroll
+            for (int r = 0; r < ROUNDS; ++r) f[r] = ex2(ml[r].x - ref);   // m = -inf, or no such split -> 0
+#pragma unroll
+            for (int u = 0; u < kDecBatch; ++u)
+                dec_accumulate(acc, lsum, v[u], __shfl_sync(0xffffffffu, ml[u / LANES].y, gbase + u % LANES),
+                               __shfl_sync(0xffffffffu, f[u / LANES], gbase + u % LANES));
         }
-        const float Lsum = stat[2 * h + 1];
-        const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
-        *reinterpret_cast<uint2*>(p.o + (bh0 + h) * D + d4 * 4) =
-            make_uint2(pack_bf16x2(acc.x * inv, acc.y * inv), pack_bf16x2(acc.z * inv, acc.w * inv));
+        if (h0w + lane / LANES < p.group) dec_store<D>(p, bh0 + h, gl, acc, M, lsum);
     }
-    if (p.lse && tid < p.group) {
-        const float M = stat[2 * tid], Lsum = stat[2 * tid + 1];
-        p.lse[bh0 + tid] = Lsum > 0.f ? (M + log2f(Lsum)) * 0.6931471805599453f : -INFINITY;
-    }
-    if (tid == 0) p.tickets[blockIdx.y] = 0u;   // ready for the next call on this workspace
 }
 
 }  // namespace af
