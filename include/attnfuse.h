@@ -71,7 +71,8 @@ const char* attnfuse_strerror(af_status st);
  * calls that start later.  attnfuse_set_option returns AF_ERR_SPEC for an unknown option;
  * attnfuse_get_option returns -1 for one. */
 typedef enum {
-    AF_OPT_FWD_QTILES = 0,     /* AF_FWD_NQ, default 2: query tiles per CTA of the forward kernel (1 or 2) */
+    AF_OPT_FWD_QTILES = 0,     /* AF_FWD_NQ, default 2: query tiles per CTA of the forward kernel: 2 = two, or one where two
+                                  would leave SMs idle; 1 = one; 3 = always two */
     AF_OPT_FWD_PAIR_HEADS = 1, /* AF_FWD_PAIR, default 1: with an even GQA group the two query tiles of a CTA are two
                                   heads of one kv head; 0: two consecutive row blocks of one head */
     AF_OPT_FWD_KEYS_BF16 = 2,  /* AF_FWD_KEYS_BF16, default 0: key tiles rotated in packed bf16 arithmetic (faster,

@@ -297,6 +297,61 @@ af_status resolve_strides(const af_strides* in, int H, int S, int D, af_strides*
     return AF_OK;
 }
 
+// One query tile per CTA instead of two?  With two, the tiles share every K and V tile and hide each other's latencies, but a
+// grid that leaves SMs idle is better spread out.  Measured with two and one per CTA: 24.1 / 20.2 us (B = 1, 16 / 4 heads,
+// S = 1024: 128 CTAs of one tile), 20.6 / 18.4 us (24 / 8 heads, S = 777: 168), 25.0 / 26.3 us (32 / 8 heads, S = 1024: 256).
+bool one_query_tile(const FwdParams& p) {
+    const int o = opt(AF_OPT_FWD_QTILES);
+    if (o != 2) return o == 1;
+    return static_cast<double>(p.B) * p.Hq * ((p.S + BM - 1) / BM) <= 1.2 * sm_count();
+}
+
+// Tiles of one sequence under a dense mask: the most key tiles (or, the other way round, query tiles) that one tile meets, and
+// their sum over all tiles.
+void tile_counts(int S, int causal, int window, double* longest, double* sum) {
+    const int tiles = (S + 127) / 128;
+    const int reach = window < 0 ? tiles : (window + 127) / 128 + 1;   // tiles from the diagonal on, to one side
+    *longest = *sum = 0.0;
+    for (int j = 0; j < tiles; ++j) {
+        const int one = reach < tiles - j ? reach : tiles - j, other = causal ? 0 : (reach - 1 < j ? reach - 1 : j);
+        const double n = one + other;
+        *longest = n > *longest ? n : *longest;
+        *sum += n;
+    }
+}
+
+// Cluster size (1, 2, 4 or 8) with the smallest estimated time for `ctas` pieces of work of `longest` tiles at most and `sum`
+// tiles in all, which a cluster can share out: the longer of the longest CTA and the total work over the SMs.  In us:
+// pair (a tile pair), cta (set-up and epilogue of a CTA), join (merging a cluster's results) and extra (what every
+// further CTA of a cluster costs the SMs: its own set-up, waiting for the others, and SMs held free until a whole
+// cluster fits).
+int cluster_size(double ctas, double longest, double sum, double pair, double cta, double join, double extra) {
+    const double sms = sm_count() > 0 ? sm_count() : 148;
+    int best = 1;
+    double best_time = 0.0;
+    for (int n = 1; n <= 8; n *= 2) {
+        const double a = longest / n * pair + cta + (n > 1 ? join : 0.0);
+        const double b = (sum * pair + ctas * (cta + (n - 1) * extra)) / sms;
+        const double t = a > b ? a : b;
+        if (n == 1 || t < 0.95 * best_time) {
+            best = n;
+            best_time = t;
+        }
+    }
+    return best;
+}
+
+// CTAs that share out the key tiles of a query tile (dense masks, one query tile per CTA).  Measured with 1 / 2 / 4 CTAs:
+// 118.6 / 69.9 / 96.6 us (2 / 1 heads, S = 8192, D = 128), 47.1 / 32.9 / 50.6 us (4 heads, S = 4000, D = 64), 19.8 / 16.7 /
+// 19.2 us (8 / 2 heads, S = 1000), 20.2 / 26.6 / 35.5 us (16 / 4 heads, S = 1024), 14.6 / 27.1 / 27.2 us (6 / 2 heads,
+// S = 2000, window 300).
+int fwd_splits(const FwdParams& p, int D) {
+    double longest, sum;
+    tile_counts(p.S, p.causal, p.window, &longest, &sum);
+    const double units = static_cast<double>(p.B) * p.Hq;
+    return cluster_size(units * ((p.S + BM - 1) / BM), longest, sum * units, D == 128 ? 1.8 : 1.3, 2.0, 4.5, 13.0);
+}
+
 template <int D, int NQ, bool ROPE, int KS, int VS, bool TAB = false, bool GEN = false>
 af_status launch_fwd_variant(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt,
                              FwdParams p, cudaStream_t stream) {
@@ -312,6 +367,17 @@ af_status launch_fwd_variant(const CUtensorMap& tq, const CUtensorMap& tk, const
     p.n_row_blocks = (p.S + rows_per_cta - 1) / rows_per_cta;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
     // (hybrid arm: the kernel waits for the RoPE pass on K that precedes it only before its first key-tile load)
+    if constexpr (NQ == 1 && !TAB && !GEN) {
+        p.splits = fwd_splits(p, D);
+        if (p.splits > 1) {
+            auto shared = attn_fwd_kernel<D, NQ, ROPE, KS, VS, false, false, false, true>;
+            static std::atomic<unsigned long long> configured_shared{0};
+            if (allow_dynamic_smem(shared, L::BYTES, configured_shared) != AF_OK) return AF_ERR_CUDA;
+            grid.z = p.splits;
+            return launch_cluster(shared, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, p.splits, tq, tk, tv, to,
+                                  tt, p);
+        }
+    }
     return launch_kernel(kern, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
 }
 
@@ -338,9 +404,10 @@ template <int D>
 af_status launch_fwd_blocks(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt,
                             const FwdParams& p, cudaStream_t stream) {
     // (p.bs_rowpair is set only for an odd GQA group, when the caller supplied the lists of row-block pairs)
-    const bool two_tiles = (p.group % 2) == 0 || p.bs_rowpair;
+    const bool can_two = (p.group % 2) == 0 || p.bs_rowpair;
+    const bool two_tiles = can_two && (opt(AF_OPT_FWD_QTILES) != 2 || !one_query_tile(p));
     if (p.bias || p.relu) {   // Section 3.1 extras: built for CTAs of two query tiles only
-        if (!two_tiles) return AF_ERR_SPEC;
+        if (!can_two) return AF_ERR_SPEC;
         return p.R > 0 ? launch_fwd_blocks_variant<D, 2, true, true>(tq, tk, tv, to, tt, p, stream)
                        : launch_fwd_blocks_variant<D, 2, false, true>(tq, tk, tv, to, tt, p, stream);
     }
@@ -357,8 +424,7 @@ af_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
     if (p.bias || p.relu)   // Section 3.1 extras (additive_bias, relu_attention): their own instantiation
         return p.R > 0 ? launch_fwd_variant<D, 2, true, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream)
                        : launch_fwd_variant<D, 2, false, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream);
-    const int nq = opt(AF_OPT_FWD_QTILES);
-    if (nq == 1) {
+    if (one_query_tile(p) && !(p.R > 0 && p.keys_bf16 && opt(AF_OPT_FWD_QTILES) == 2)) {
         return p.R > 0 ? launch_fwd_variant<D, 1, true, 2, 2>(tq, tk, tv, to, tt, p, stream)
                        : launch_fwd_variant<D, 1, false, 2, 2>(tq, tk, tv, to, tt, p, stream);
     }
@@ -480,44 +546,21 @@ af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMa
 }
 
 // CTAs per key tile of the one-pass kernel: 1, 2, 4 or 8 (a cluster that shares out the key tile's query tiles and sums dK
-// and dV over distributed shared memory).  The number with the smallest estimated time, from a model with three
-// measured constants: a tile pair (2.9 us at D = 128, 2.3 us at D = 64), set-up and epilogue of a CTA (6 us) and what
-// every further CTA of a cluster costs the SMs (18 us: its own set-up, waiting for the others, and SMs held free until
-// a whole cluster fits).  The time is the longer of the longest CTA and the total work over the SMs.
+// and dV over distributed shared memory).
 // Measured, whole backward, 1 / 2 / 4 / 8 CTAs: 52 / 38 / 36 / 43 us (B = 2, 6 q / 2 kv heads, S = 777, window 300, D = 128),
 // 129 / 76 / 65 / 65 us (B = 2, 16 / 2 heads, S = 596), 124 / 188 / 232 / 288 us (B = 4, 16 heads, S = 1024).
 // The lengths of block lists are not known here.  They are taken to be those of a pattern with one global key block and
 // four query blocks for each other key block: 449 / 260 / 247 / 319 us (B = 2, 16 / 4 heads, S = 4096, D = 128, such a list).
 int onepass_splits(int D, int units, int S, int group, int causal, int window, bool blocks) {
-    const double pair = D == 128 ? 2.9 : 2.3, cta = 6.0, extra = 18.0, sms = sm_count() > 0 ? sm_count() : 148;
     const int tiles = (S + 127) / 128;
-    double longest = 0.0, sum = 0.0;   // query tiles that see a key tile: the most, and over all key tiles
+    double longest, sum;   // query tiles that see a key tile
     if (blocks) {
         longest = tiles;
         sum = tiles + 4.0 * (tiles - 1);
     } else {
-        const int reach = window < 0 ? tiles : (window + 127) / 128 + 1;   // query tiles from the diagonal on
-        for (int j = 0; j < tiles; ++j) {
-            const int below = reach < tiles - j ? reach : tiles - j, above = causal ? 0 : (reach - 1 < j ? reach - 1 : j);
-            const double n = below + above;
-            longest = n > longest ? n : longest;
-            sum += n;
-        }
+        tile_counts(S, causal, window, &longest, &sum);
     }
-    longest *= group;
-    sum *= static_cast<double>(group) * units;
-    int best = 1;
-    double best_time = 0.0;
-    for (int n = 1; n <= 8; n *= 2) {
-        const double a = longest / n * pair + cta;
-        const double b = (sum * pair + static_cast<double>(units) * tiles * (cta + (n - 1) * extra)) / sms;
-        const double t = a > b ? a : b;
-        if (n == 1 || t < 0.95 * best_time) {
-            best = n;
-            best_time = t;
-        }
-    }
-    return best;
+    return cluster_size(static_cast<double>(units) * tiles, longest * group, sum * group * units, D == 128 ? 2.9 : 2.3, 6.0, 0.0, 18.0);
 }
 
 // One-pass sequence (bwd_fused_kernel.cuh): the set-up pass (zeroed fp32 dQ' accumulator, delta, rotated K and Q in the
@@ -845,7 +888,9 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     p.bs_col_idx = bs_col_idx;
     p.bs_order = bs_order;
     p.bs_rowpair = 0;
-    if (blocks && (gqa_group % 2) == 1 && blocks->pair_ptr && blocks->pair_idx && opt(AF_OPT_BS_ROWPAIR)) {
+    p.splits = 1;
+    if (blocks && (gqa_group % 2) == 1 && blocks->pair_ptr && blocks->pair_idx && opt(AF_OPT_BS_ROWPAIR) &&
+        (bias || relu || opt(AF_OPT_FWD_QTILES) != 2 || !one_query_tile(p))) {
         // odd GQA group: no two heads share K and V, so a CTA takes two row blocks of one head instead
         p.bs_row_ptr = blocks->pair_ptr;
         p.bs_col_idx = blocks->pair_idx;

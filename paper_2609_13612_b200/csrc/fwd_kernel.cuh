@@ -46,6 +46,7 @@ struct FwdParams {
     // with A = [kb_hi, kb_lo, 0 ...] in every query row and B = [e, e, 0 ...] in key row e (kb = slope / c split
     // into two bf16 values, e exact in bf16) - and the softmax warps run their plain straight-line code.
     int alibi_mma;
+    int splits;            // SPLIT kernels: CTAs per cluster, the grid's z dimension
 #ifdef AF_TRACE
     long long* trace;
 #endif
@@ -98,6 +99,8 @@ struct FwdSmem {
 #ifdef AF_TRACE
 __device__ long long* g_trace = nullptr;
 #endif
+constexpr int kFwdMaxSplits = 8;    // CTAs that share a query tile's key tiles, at most
+constexpr int kFwdMinTiles = 2;     // key tiles per CTA below which a query tile is not shared out further
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: O is rescaled only when the row max grows by more
 
 constexpr int kPParts = 2;   // P is handed to the MMA issuer in two column halves (four parts, and an S tile produced as
@@ -304,7 +307,10 @@ __device__ __forceinline__ bool softmax_tile_general(uint32_t tS, uint32_t tO, i
 // tm_t (the bf16 copy of the cos/sin table); otherwise in fp32 arithmetic from the fp32 table rows.
 // GEN: the instantiation for the variants with an additive bias or the ReLU normaliser (softmax_tile_general); kept
 // apart so that the kernels of the other variants carry none of its registers.
-template <int D, int NQ, bool ROPE, int KS, int VS, bool BS = false, bool TAB = false, bool GEN = false>
+// SPLIT (dense, NQ = 1): the grid's z dimension is a cluster of p.splits CTAs that share out the key tiles of a query tile.  Each
+// ends with an unnormalised O, m and l of its own; they are merged (log-sum-exp, in rank order) through distributed
+// shared memory, every CTA taking a share of the rows.  For grids that leave SMs idle: see fwd_splits (attnfuse.cu).
+template <int D, int NQ, bool ROPE, int KS, int VS, bool BS = false, bool TAB = false, bool GEN = false, bool SPLIT = false>
 __global__ void __launch_bounds__(128 * (2 + NQ), 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
@@ -312,6 +318,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     using L = FwdSmem<D, NQ, KS, VS, ROPE && TAB>;
     constexpr int TILE = L::TILE;
     constexpr int NBOX = D / BOX_COLS;
+    constexpr int kPartStride = D + 4;   // SPLIT: floats per staged row
+    static_assert(!SPLIT || 128 * kPartStride * 4 <= L::OFF_BAR, "the staged rows must fit in the operand tiles");
     constexpr uint32_t TMEM_COLS = (NQ * (BN + D) <= 256) ? 256u : 512u;
     constexpr uint32_t IDESC_S = idesc_bf16_f32(BM, BN, 0, 0);
     constexpr uint32_t IDESC_O = idesc_bf16_f32(BM, D, 0, 1);
@@ -354,6 +362,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             jlo[q] = 1;
             jhi[q] = 0;  // empty
         }
+    }
+    int parts = 1, rank = 0;   // CTAs that share this query tile's key tiles (a power of two, at least kFwdMinTiles each), and which one this is
+    if constexpr (SPLIT) {
+        static_assert(NQ == 1 && !BS && !TAB && !GEN, "built for dense masks and one query tile per CTA");
+        rank = static_cast<int>(blockIdx.z);
+        const int lo = jlo[0], n_all = jhi[0] - lo + 1;
+        while (parts < p.splits && n_all >= 2 * parts * kFwdMinTiles) parts *= 2;
+        if (rank >= parts) return;
+        jlo[0] = jlo_c = lo + n_all * rank / parts;
+        jhi[0] = jhi_c = lo + n_all * (rank + 1) / parts - 1;
     }
     // Block-sparse: the loops below run over positions in the row block's list (jlo = 0, jhi = length - 1, the
     // same for both query tiles, which share the row block); tile_at() gives the key tile of a position.
@@ -738,7 +756,20 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // epilogue (Section 4.4: save L = m + ln l)
         if (ok && jhi[q] >= jlo[q]) ok = mbar_wait_warp(&bars[L::B_ODONE + q], 0, abort_flag, 11);
         AF_STAMP(2 + q, 63, 0);  // O complete
-        if (ok && jhi[q] >= jlo[q]) {
+        if (SPLIT && parts > 1 && ok) {
+            // this CTA's share, unnormalised, over the operand tiles (idle now): rows of D + 4 floats, acc[D], m, l
+            tc_fence_after_sync();
+            float* row_p = reinterpret_cast<float*>(smem) + row * kPartStride;
+#pragma unroll 1
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t v[32];
+                tmem_ld32(tO + c * 32, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 32; e += 4) *reinterpret_cast<uint4*>(row_p + c * 32 + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+            }
+            *reinterpret_cast<float2*>(row_p + D) = make_float2(m_run, l_run);
+        } else if (ok && jhi[q] >= jlo[q]) {
             tc_fence_after_sync();
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
             const size_t orow = (static_cast<size_t>(bh) * p.S + i) * D;
@@ -815,6 +846,51 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         }
     }
 
+    if (SPLIT && parts > 1) {
+        // (every thread of every working CTA takes both barriers, also after a wait that gave up)
+        __syncwarp();
+        cluster_sync();
+        // a group of D / 4 lanes per row, all warps on this CTA's share of the rows
+        constexpr int LANES = D / 4, NROW = 32 / LANES, NWARP = 4 * (2 + NQ);
+        const uint32_t base = smem_u32(smem);
+        const int gl = lane % LANES;
+        if (!*abort_flag)
+#pragma unroll 1
+            for (int r = 128 * rank / parts + warp * NROW + lane / LANES; r < 128 * (rank + 1) / parts && i0[0] + r < p.S; r += NWARP * NROW) {
+                float2 ml[kFwdMaxSplits];
+                float4 v[kFwdMaxSplits];
+                float M = -INFINITY, l = 0.f;
+#pragma unroll
+                for (int c = 0; c < kFwdMaxSplits; ++c) {
+                    if (c < parts) {
+                        ml[c] = ld_cluster2(base + (r * kPartStride + D) * 4, c);
+                        v[c] = ld_cluster4(base + (r * kPartStride + gl * 4) * 4, c);
+                        M = fmaxf(M, ml[c].x);
+                    }
+                }
+                float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float ref = M == -INFINITY ? 0.f : M;
+#pragma unroll
+                for (int c = 0; c < kFwdMaxSplits; ++c) {
+                    if (c < parts) {
+                        const float f = ex2(ml[c].x - ref);   // nothing kept in a share: m = -inf -> 0
+                        y.x = fmaf(v[c].x, f, y.x);
+                        y.y = fmaf(v[c].y, f, y.y);
+                        y.z = fmaf(v[c].z, f, y.z);
+                        y.w = fmaf(v[c].w, f, y.w);
+                        l = fmaf(ml[c].y, f, l);
+                    }
+                }
+                const float inv = l > 0.f ? 1.f / l : 0.f;
+                const size_t at = static_cast<size_t>(b * p.Hq + hq[0]) * p.S + i0[0] + r;
+                if (p.o_f32) *reinterpret_cast<float4*>(static_cast<float*>(p.o) + at * D + gl * 4) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+                else *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.o) + at * D + gl * 4) =
+                    make_uint2(pack_bf16x2(y.x * inv, y.y * inv), pack_bf16x2(y.z * inv, y.w * inv));
+                if (gl == 0 && p.lse) p.lse[at] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+            }
+        __syncwarp();
+        cluster_sync();   // nobody leaves while its shared memory is being read
+    }
     tc_fence_before_sync();
     __syncthreads();
     AF_STAMP(0, 63, 1);  // all roles done

@@ -339,6 +339,14 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t saddr, int rank) {
     return v;
 }
 
+__device__ __forceinline__ float2 ld_cluster2(uint32_t saddr, int rank) {
+    uint32_t a;
+    float2 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+
 // four fp32 values added to global memory (16-byte aligned)
 __device__ __forceinline__ void red_add4(float* at, float4 v) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
