@@ -336,6 +336,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_MISC + 4);
 
     const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5)), lane = threadIdx.x & 31;
+    if (warp == 0 && elect_one()) {
+        prefetch_tmap(&tm_q);
+        prefetch_tmap(&tm_k);
+        prefetch_tmap(&tm_v);
+        if (tab_tiles) prefetch_tmap(&tm_t);
+    }
     // blockIdx.x: a head, or with pair_heads (even GQA group) a pair of adjacent heads that share a kv head.
     // Pairing heads gives both query tiles the same key range, so the two softmax warpgroups stay in
     // step down to the last tile; without it the tiles are rows [256 rb, +128) and [256 rb + 128, +128).
@@ -417,16 +423,53 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int n_it = jhi_c - jlo_c + 1;
     AF_STAMP(0, 63, 0);  // kernel entry
 
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < L::N_BARS; ++i) {
+    // Set-up, with as little as possible in a row (a CTA's first scores wait for it, and short key loops cannot hide it): the
+    // lanes of warp 0 initialise a barrier each and the warp requests its first tiles at once, while warp 1 allocates
+    // tensor memory.  Programmatic dependent launch: what comes before grid_dep_wait overlaps with the end of the kernel
+    // before this one in the stream, whose results (and buffers) may be touched behind it.  The hybrid arm waits later,
+    // before its first key tile: its Q, table and outputs are settled before the RoPE pass that precedes it starts.
+    // Measured with the output written box by box and L stored while the last products run (see the epilogue): hybrid arm
+    // 166.9 -> 161.1 us (B = 4, 32 / 8 heads, S = 2048, D = 128), without rotation 122.1 -> 118.7 us (S = 4096), 177.0 -> 174.0 us
+    // (B = 4, 12 heads, S = 4096, D = 64).
+    const bool hybrid = ROPE && !p.rot_k;
+    int first_it = 0;   // key tiles requested here already
+    if (warp == 0) {
+        static_assert(L::N_BARS <= 32, "one barrier per lane");
+        if (lane < L::N_BARS) {
             uint32_t cnt = 1;
-            if ((i >= L::B_QROT && i < L::B_QROT + NQ) || (i >= L::B_KROT && i < L::B_KROT + KS) ||
-                (i >= L::B_PREADY && i < L::B_PREADY + 4 * NQ) || i == L::B_TEMPTY)
+            if ((lane >= L::B_QROT && lane < L::B_QROT + NQ) || (lane >= L::B_KROT && lane < L::B_KROT + KS) ||
+                (lane >= L::B_PREADY && lane < L::B_PREADY + 4 * NQ) || lane == L::B_TEMPTY)
                 cnt = 4;  // one elected arrive per warp of the producing warpgroup
-            mbar_init(&bars[i], cnt);
+            mbar_init(&bars[lane], cnt);
         }
-        *abort_flag = 0;
+        if (lane == 0) *abort_flag = 0;
         fence_mbar_init();
+        __syncwarp();
+        if (!hybrid) grid_dep_wait();
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            if (jhi[q] < jlo[q]) continue;
+            if (elect_one()) {
+                mbar_arrive_expect_tx(&bars[L::B_QFULL + q], TILE);
+#pragma unroll
+                for (int bx = 0; bx < NBOX; ++bx)
+                    tma_load_4d(sQ + q * TILE + bx * BOX_BYTES, &tm_q, &bars[L::B_QFULL + q], bx * BOX_COLS, i0[q], hq[q], b);
+            }
+        }
+        if (!hybrid && !tab_tiles && n_it > 0) {
+            first_it = 1;
+            const int j0 = tile_at(jlo_c) * BN;
+            if (elect_one()) {
+                mbar_arrive_expect_tx(&bars[L::B_KFULL], TILE);
+#pragma unroll
+                for (int bx = 0; bx < NBOX; ++bx)
+                    tma_load_4d(sK + bx * BOX_BYTES, &tm_k, &bars[L::B_KFULL], bx * BOX_COLS, j0, hk, b);
+                mbar_arrive_expect_tx(&bars[L::B_VFULL], TILE);
+#pragma unroll
+                for (int bx = 0; bx < NBOX; ++bx)
+                    tma_load_4d(sV + bx * BOX_BYTES, &tm_v, &bars[L::B_VFULL], bx * BOX_COLS, j0, hk, b);
+            }
+        }
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, TMEM_COLS);
@@ -436,11 +479,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = warp_uniform(*tmem_slot);
-    // Programmatic dependent launch: everything up to here overlaps with the end of the kernel before this one in the
-    // stream, whose results (and buffers) may be touched from here on.  The hybrid arm waits later, in the producer:
-    // its Q, table and outputs are settled before the RoPE pass that precedes it starts.
     grid_dep_launch();
-    if (!(ROPE && !p.rot_k)) grid_dep_wait();
+    if (!hybrid) grid_dep_wait();
 
     // Register budget: the softmax warpgroups hold a full row of 128 scores; the others need little, but the
     // MMA issuer must not spill (it is the most latency-sensitive thread of the CTA: at 64 registers it spilled
@@ -452,26 +492,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         {
-            if (elect_one()) {
-                prefetch_tmap(&tm_q);
-                prefetch_tmap(&tm_k);
-                prefetch_tmap(&tm_v);
-                if (tab_tiles) prefetch_tmap(&tm_t);
-            }
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                if (jhi[q] < jlo[q]) continue;
-                if (elect_one()) {
-                    mbar_arrive_expect_tx(&bars[L::B_QFULL + q], TILE);
-#pragma unroll
-                    for (int bx = 0; bx < NBOX; ++bx)
-                        tma_load_4d(sQ + q * TILE + bx * BOX_BYTES, &tm_q, &bars[L::B_QFULL + q], bx * BOX_COLS, i0[q], hq[q], b);
-                }
-            }
             // hybrid arm: the keys are written by the RoPE pass launched just before this grid, which may still be
             // running (programmatic dependent launch); everything above overlaps with its tail
-            if (ROPE && !p.rot_k) grid_dep_wait();
-            for (int it = 0; it < n_it; ++it) {
+            if (hybrid) grid_dep_wait();
+            for (int it = first_it; it < n_it; ++it) {
                 const int j0 = tile_at(jlo_c + it) * BN;
                 const int ks = it % KS, vs = it % VS;
                 if (!mbar_wait_warp(&bars[L::B_KEMPTY + ks], ((it / KS) & 1) ^ 1, abort_flag, 1)) break;
@@ -753,7 +777,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             AF_STAMP(2 + q, n, 2);
             ++n;
         }
-        // epilogue (Section 4.4: save L = m + ln l)
+        // epilogue (Section 4.4: save L = m + ln l, while the last products run)
+        if (ok && !(SPLIT && parts > 1) && jhi[q] >= jlo[q] && p.lse && i < p.S) {
+            // softmax: L = m + ln l; relu_attention: n_i, the number of kept pairs of the row (its normaliser)
+            if (GEN && p.relu) p.lse[static_cast<size_t>(bh) * p.S + i] = l_run;
+            else p.lse[static_cast<size_t>(bh) * p.S + i] = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
+        }
         if (ok && jhi[q] >= jlo[q]) ok = mbar_wait_warp(&bars[L::B_ODONE + q], 0, abort_flag, 11);
         AF_STAMP(2 + q, 63, 0);  // O complete
         if (SPLIT && parts > 1 && ok) {
@@ -778,29 +807,29 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 // reads any more once O is complete, in the layout of the input tiles - and let TMA write it out.
                 // (Row-per-thread global stores touch 32 rows per instruction and kept the load/store unit busy
                 // for ~4 k cycles per CTA.)  Rows past S are clipped by the tensor map.
+                // Box by box (64 columns), so that one is on its way out while the next is converted.
                 uint8_t* stg = sQ + q * TILE;
 #pragma unroll 1
-                for (int c = 0; c < D / 32; ++c) {
-                    uint32_t v[32];
-                    tmem_ld32(tO + c * 32, v);
+                for (int bx = 0; bx < NBOX; ++bx) {
+                    uint32_t v[64];
+                    tmem_ld32(tO + bx * 64, v);
+                    tmem_ld32(tO + bx * 64 + 32, v + 32);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int e = 0; e < 32; e += 8)
-                        *reinterpret_cast<uint4*>(stg + swz_chunk_offset(row, c * 4 + (e >> 3))) = make_uint4(
+                    for (int e = 0; e < 64; e += 8)
+                        *reinterpret_cast<uint4*>(stg + swz_chunk_offset(row, bx * 8 + (e >> 3))) = make_uint4(
                             pack_bf16x2(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv),
                             pack_bf16x2(__uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv),
                             pack_bf16x2(__uint_as_float(v[e + 4]) * inv, __uint_as_float(v[e + 5]) * inv),
                             pack_bf16x2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv));
-                }
-                fence_proxy_async_smem();
-                asm volatile("bar.sync %0, 128;" ::"r"(4 + q) : "memory");   // this warpgroup only
-                if (row == 0) {
-#pragma unroll
-                    for (int bx = 0; bx < NBOX; ++bx)
+                    fence_proxy_async_smem();
+                    asm volatile("bar.sync %0, 128;" ::"r"(4 + q) : "memory");   // this warpgroup only
+                    if (row == 0) {
                         tma_store_4d(&tm_o, stg + bx * BOX_BYTES, bx * BOX_COLS, i0[q], hq[q], b);
-                    tma_store_commit();
-                    tma_store_wait_read();   // the buffer must stay in place until it has been read
+                        tma_store_commit();
+                    }
                 }
+                if (row == 0) tma_store_wait_read();   // the buffer must stay in place until it has been read
             }
 #pragma unroll 1
             for (int c = 0; p.o_f32 && c < D / 32; ++c) {
@@ -825,11 +854,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                                 pack_bf16x2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv));
                     }
                 }
-            }
-            if (p.lse && i < p.S) {
-                // softmax: L = m + ln l; relu_attention: n_i, the number of kept pairs of the row (its normaliser)
-                if (GEN && p.relu) p.lse[static_cast<size_t>(bh) * p.S + i] = l_run;
-                else p.lse[static_cast<size_t>(bh) * p.S + i] = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
             }
         }
         if (BS && ok && jhi[q] < jlo[q] && i < p.S) {
