@@ -612,8 +612,8 @@ af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CU
     const unsigned tiles = static_cast<unsigned>((sh->S + 127) / 128);
     const int first_ctas = first ? 1 : 0;   // rows of the grid
     dim3 grid(sh->B * sh->Hkv, tiles + first_ctas, splits);
-    st = p.R > 0 ? launch_cluster(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, splits, tkp, tv, tqp, tdo, p, fp, first_ctas, splits)
-                 : launch_cluster(kern, grid, dim3(512, 1, 1), L::BYTES, stream, true, splits, tk, tv, tq, tdo, p, fp, first_ctas, splits);
+    st = p.R > 0 ? launch_cluster(kern, grid, dim3(kFusedThreads, 1, 1), L::BYTES, stream, true, splits, tkp, tv, tqp, tdo, p, fp, first_ctas, splits)
+                 : launch_cluster(kern, grid, dim3(kFusedThreads, 1, 1), L::BYTES, stream, true, splits, tk, tv, tq, tdo, p, fp, first_ctas, splits);
     if (st != AF_OK) return st;
     const long long fthreads = static_cast<long long>(sh->S) * (D / 8);
     const int nh = sh->B * sh->Hq;
@@ -1250,11 +1250,21 @@ af_status bwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     if ((st = resolve_strides(skv, shape->Hkv, shape->S, shape->D, &stkv)) != AF_OK) return st;
     resolve_strides(nullptr, shape->Hq, shape->S, shape->D, &stc);
     if ((st = check_arch()) != AF_OK) return st;
+    const size_t off_k = bwd_delta_bytes(shape), off_q = off_k + bwd_kcache_bytes(shape);
+    const size_t off_acc = off_q + bwd_qcache_bytes(shape);
+    // One-pass sequence: room for both caches and the fp32 dQ' accumulator, and not switched off.
+    // It measured faster than the two-kernel sequence wherever it applies: D = 64 1.2-1.4 times on every shape tried;
+    // D = 128 522 against 622 us at B = 4, 32 / 8 heads, S = 2048, 447 against 487 us at S = 4096, B = 1, 808 against 879 us
+    // at 16 / 4 heads, S = 8192, 428 against 479 us without a causal mask at 16 / 8 heads, S = 4096; over block lists
+    // 684 against 830 us (B = 4, 32 / 8 heads, S = 4096), 84 against 97 us (B = 2, 12 heads, S = 2000), 259 against 370 us
+    // (B = 2, 16 / 4 heads, S = 4096).
+    const bool onepass = !gen && workspace_bytes >= off_acc + bwd_dqacc_bytes(shape) && opt(AF_OPT_BWD_ONEPASS) >= 1;
+    const int qrows = onepass ? 64 : 128;   // rows per TMA box of the streamed operands: the one-pass kernel takes half tiles
     CUtensorMap tq, tk, tv, tdo;
-    if ((st = make_tmap(&tq, q, shape->B, shape->Hq, shape->S, shape->D, stq, 128)) != AF_OK) return st;
+    if ((st = make_tmap(&tq, q, shape->B, shape->Hq, shape->S, shape->D, stq, qrows)) != AF_OK) return st;
     if ((st = make_tmap(&tk, k, shape->B, shape->Hkv, shape->S, shape->D, stkv, 128)) != AF_OK) return st;
     if ((st = make_tmap(&tv, v, shape->B, shape->Hkv, shape->S, shape->D, stkv, 128)) != AF_OK) return st;
-    if ((st = make_tmap(&tdo, d_o, shape->B, shape->Hq, shape->S, shape->D, stc, 128)) != AF_OK) return st;
+    if ((st = make_tmap(&tdo, d_o, shape->B, shape->Hq, shape->S, shape->D, stc, qrows)) != AF_OK) return st;
     BwdParams p;
     p.B = shape->B; p.Hq = shape->Hq; p.Hkv = shape->Hkv; p.S = shape->S; p.group = gqa_group;
     p.R = rope->rotary_dim;
@@ -1275,15 +1285,6 @@ af_status bwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     float* delta = static_cast<float*>(workspace);
     // rotated-K and rotated-Q caches: used when there is a rotation and the workspace has room behind delta
     CUtensorMap tkp, tqp;
-    const size_t off_k = bwd_delta_bytes(shape), off_q = off_k + bwd_kcache_bytes(shape);
-    const size_t off_acc = off_q + bwd_qcache_bytes(shape);
-    // One-pass sequence: room for both caches and the fp32 dQ' accumulator, and not switched off.
-    // It measured faster than the two-kernel sequence wherever it applies: D = 64 1.2-1.4 times on every shape tried;
-    // D = 128 522 against 622 us at B = 4, 32 / 8 heads, S = 2048, 447 against 487 us at S = 4096, B = 1, 808 against 879 us
-    // at 16 / 4 heads, S = 8192, 428 against 479 us without a causal mask at 16 / 8 heads, S = 4096; over block lists
-    // 684 against 830 us (B = 4, 32 / 8 heads, S = 4096), 84 against 97 us (B = 2, 12 heads, S = 2000), 259 against 370 us
-    // (B = 2, 16 / 4 heads, S = 4096).
-    const bool onepass = !gen && workspace_bytes >= off_acc + bwd_dqacc_bytes(shape) && opt(AF_OPT_BWD_ONEPASS) >= 1;
     const bool have_k = p.R > 0 && workspace_bytes >= off_q;
     const bool have_q = have_k && workspace_bytes >= off_acc;
     void* kc = static_cast<uint8_t*>(workspace) + off_k;
@@ -1294,7 +1295,7 @@ af_status bwd_impl(const af_shape* shape, const void* q, const void* k, const vo
         if ((st = make_tmap(&tkp, kc, shape->B, shape->Hkv, shape->S, shape->D, stk, 128)) != AF_OK) return st;
     }
     if (have_q) {
-        if ((st = make_tmap(&tqp, qc, shape->B, shape->Hq, shape->S, shape->D, stc, 128)) != AF_OK) return st;
+        if ((st = make_tmap(&tqp, qc, shape->B, shape->Hq, shape->S, shape->D, stc, qrows)) != AF_OK) return st;
     }
     // Under a causal mask (dense, not over block lists) the first query rows of every head are computed in fp32 by a
     // small kernel of their own and dropped from the MMA kernels: see bwd_first_rows.cuh.

@@ -123,7 +123,7 @@ __device__ __forceinline__ void first_rows_unit(const FirstRowsParams& p, int un
         const int prow = nh * NR;          // panel rows in use: r = hh * NR + i
         // 1. queries (rotated) and upstream gradients of the panel
         {
-            constexpr int CH = PANEL * D / 8 / NT;   // 16-byte chunks per thread and array
+            constexpr int CH = (PANEL * D / 8 + NT - 1) / NT;   // 16-byte chunks per thread and array
             uint4 qw[CH], gw[CH];
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
@@ -132,7 +132,7 @@ __device__ __forceinline__ void first_rows_unit(const FirstRowsParams& p, int un
                 const int h = hk * p.group + h0 + hh;
                 qw[c] = make_uint4(0u, 0u, 0u, 0u);
                 gw[c] = qw[c];
-                if (hh < nh && i < rows) {
+                if (idx < PANEL * D && hh < nh && i < rows) {
                     qw[c] = __ldg(reinterpret_cast<const uint4*>(p.q + b * p.qb + h * p.qh + i * p.qs + d));
                     gw[c] = __ldg(reinterpret_cast<const uint4*>(p.d_o + ((static_cast<size_t>(b) * p.Hq + h) * p.S + i) * D + d));
                 }
@@ -140,6 +140,7 @@ __device__ __forceinline__ void first_rows_unit(const FirstRowsParams& p, int un
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
                 const int idx = (tid + c * NT) * 8;
+                if (idx >= PANEL * D) break;
                 const uint32_t qa[4] = {qw[c].x, qw[c].y, qw[c].z, qw[c].w}, ga[4] = {gw[c].x, gw[c].y, gw[c].z, gw[c].w};
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {

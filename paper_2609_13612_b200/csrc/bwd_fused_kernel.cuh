@@ -16,31 +16,30 @@
 // (bf16, 128-byte rows of 64 query positions per key, 128-byte swizzle), where the same bytes are the K-major A
 // operand of dK' += dS^T Q' and the MN-major B operand of dQ'^T = K'^T dS^T; once a gradient warpgroup has read
 // its half of dP^T out of T2 that half is free for the dQ'^T partial of the same 64 query rows.
-// What bounds it: shared-memory bandwidth.  Every product whose two operands come from shared memory reads
-// 128 bytes per clock while it runs, and the N = 64 halves re-read the stationary operand twice per tile:
-// 384 KB of operand reads per tile pair (against 256 KB in the dK/dV role of the two-kernel sequence) plus the
-// TMA writes and the dS^T stores, about 3.8 k cycles of shared-memory time per tile pair; a timeline shows the
-// gradient passes crawling (3.8 k cycles instead of 1.3 k) whenever the tensor pipe is busy.  Measured 6.5 k
-// cycles per tile pair against 3.7 k + 3.2 k for the two roles of the two-kernel sequence: ahead where the dQ
-// role's CTAs are short (few key tiles per query tile), behind on long rows.  (A variant with ONE dP^T buffer
-// handed back as soon as it is in registers and ONE dQ'^T buffer of its own measured slower still, 8.0 k.)
+// The streamed operands have one full and one empty barrier per half tile, Q' and dO apart: with whole stages that
+// both issuers hand back, S^T of the next tile sat 1-2 k cycles per tile pair on a load that could only be requested
+// after the last dK' product of the tile before (D = 128, where shared memory holds two stages).
+// What bounds it at D = 128 (5.6 k cycles per tile pair; the five products take 2.6 k): the gradient phases, which
+// take 1.5 k cycles each for 32 columns per thread because their shared-memory accesses queue behind the reductions to
+// global memory (512 per tile pair, 26 cycles each per sub-partition; without them the backward is 1.17 times faster,
+// with stores in their place 1.02 times).  Measured and not kept: whole-tile products with N = 128 and a read-out of
+// 128 columns at once (same time per tile pair).
 // D = 64: the same kernel; dQ'^T then has M = 64 rows, which tcgen05 keeps in the first 16 lanes of each 32-lane quarter of
 // TMEM (row d in lane 32 (d / 16) + d % 16), so half of the reducing lanes carry a row; and the accumulators leave 128
 // TMEM columns free, so the partials get two 64-column buffers of their own and T2 never waits for a read-out.
 // Shared-memory traffic per tile pair is half that of D = 128; the sequence measured 1.23-1.31 times faster than the
 // two-kernel one on every shape tried (0.691 -> 0.546 ms at B = 4, 12 heads, N = 4096).
-// Warp roles (512 threads): warp 0 TMA producer; warps 1, 2, 3 MMA issuers (T1 and dV; T2 and dK'; dQ'^T), one
-// per SM sub-partition; warps 4-7 read the dQ'^T partials out of TMEM and add them to global memory; warps 8-11
-// and 12-15 are the two gradient warpgroups, one per column half.  A gradient warpgroup works in two phases per
-// tile (P^T from S^T, then dS^T from dP^T) and announces each on a barrier of its own, so that S^T of the next
-// tile is issued while dS^T is still being formed and dP^T of the next tile while the next P^T is.  A timeline of
-// the D = 64 kernel (4.4 k cycles per tile pair): phase P 1.5-2.3 k cycles for 64 columns (the exponentials of
-// both warpgroups share one special-function unit per sub-partition: 1 k cycles per tile pair is its floor, and
-// a microbenchmark of the phase alone gives 0.76 k for one warp per sub-partition, 1.1 k for two), phase dS
-// 0.9-1.1 k, the rest waits on the products.  Measured and not kept: both warpgroups on the same half with the
-// phases interleaved by half (each phase pays the TMEM load and store latencies again: 5.2 k cycles per pair);
-// working out the next tile's mask and addresses between the two phases (the warpgroups fall into step and the
-// shared exponential unit stretches phase P: 4.9 k).
+// Warp roles (768 threads): warp 0 TMA producer; warps 1, 2, 3 MMA issuers (T1 and dV; T2 and dK'; dQ'^T), one
+// per SM sub-partition; warps 4-7 read the dQ'^T partials out of TMEM and add them to global memory; warps 8-23 are
+// four gradient warpgroups, two per column half with 32 columns each.  A gradient warpgroup works in two phases per
+// tile (P^T from S^T, then dS^T from dP^T), so that S^T of the next tile is issued while dS^T is still being formed and
+// dP^T of the next tile while the next P^T is.  A phase is mostly latency (TMEM load, exponentials, TMEM or shared
+// store): four warps per sub-partition hide it better than two with 64 columns each, and one warp per warpgroup polls
+// the barriers while the others wait at the named one (polling warps take issue slots and shared-memory accesses).
+// Four warpgroups, half stages and the one polling warp together, backward alone: 542 -> 506 us (B = 4, 32 / 8 heads,
+// S = 2048, D = 128), 466 -> 444 us (B = 1, S = 4096), 127 -> 117 us (B = 4, 16 heads, S = 1024), 650 -> 605 us (B = 2,
+// 16 heads, S = 8192, window 1024, ALiBi), 481 -> 463 us (B = 4, 12 heads, S = 4096, D = 64).  Measured and not kept: two
+// warpgroups on the same half with the phases interleaved by half (each phase pays the TMEM latencies again).
 #pragma once
 #include "bwd_first_rows.cuh"
 #include "bwd_kernel.cuh"
@@ -58,8 +57,9 @@ struct BwdFusedSmem {
     static constexpr int OFF_DS = OFF_B + NST * TILE;
     static constexpr int OFF_STATS = OFF_DS + 2 * DS_HALF;
     static constexpr int OFF_BAR = OFF_STATS + 2 * 2 * 128 * 4;
-    static constexpr int B_XFULL = 0, B_YFULL = 1, B_AFULL = 2, B_BFULL = B_AFULL + NST, B_EMPTY = B_BFULL + NST,
-                         B_SFULL = B_EMPTY + NST, B_DPFULL = B_SFULL + 2, B_PRDY = B_DPFULL + 2, B_PDS = B_PRDY + 2,
+    // (A = Q', B = dO: one full and one empty barrier per half stage, index 2 * stage + half)
+    static constexpr int B_XFULL = 0, B_YFULL = 1, B_AFULL = 2, B_BFULL = B_AFULL + 2 * NST, B_AEMPTY = B_BFULL + 2 * NST,
+                         B_BEMPTY = B_AEMPTY + 2 * NST, B_SFULL = B_BEMPTY + 2 * NST, B_DPFULL = B_SFULL + 2, B_PRDY = B_DPFULL + 2, B_PDS = B_PRDY + 2,
                          B_DQFULL = B_PDS + 2, B_DSFREE = B_DQFULL + 2, B_T2FREE = B_DSFREE + 2, B_DONE = B_T2FREE + 2,
                          N_BARS = B_DONE + 1;
     static constexpr int OFF_MISC = OFF_BAR + N_BARS * 8;
@@ -84,7 +84,9 @@ struct BwdFusedSmem {
 #define AF_FSTAMP(role, it, ph) do { } while (0)
 #endif
 
-constexpr int kFusedLightRegs = 64, kFusedReduceRegs = 96, kFusedGradRegs = 176;
+// Registers: 768 threads at 80 give the six warpgroups 480 per thread slot to share; 48 + 48 + 4 x 96.
+constexpr int kFusedThreads = 768, kFusedGradThreads = 512;
+constexpr int kFusedLightRegs = 48, kFusedReduceRegs = 48, kFusedGradRegs = 96;
 constexpr int kFusedMinTiles = 2;           // streamed tiles per CTA below which a key tile is not shared out further
 constexpr uint32_t kFusedSmemCode = 0x40;   // status code: dynamic shared memory too misaligned for the layout
 
@@ -156,7 +158,7 @@ __device__ __forceinline__ void grad_phase_ds32(const uint32_t* dp, int col0, co
 // BS: block-sparse attention (Section 4.3) - the streamed query tiles of a key block come from its list of active
 // blocks (p.bs_ptr / p.bs_idx by key block, p.bs_order the launch order) instead of a contiguous range.
 template <int D, bool BS = false, bool SPLIT = false>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kFusedThreads, 1)
 attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_y,
                       const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const BwdParams p,
                       const FirstRowsParams fr, int first_ctas, int splits) {
@@ -187,7 +189,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         grid_dep_wait();
         grid_dep_launch();
         static_assert(FirstRowsSmem<D>::BYTES <= L::NEEDED, "the panels of the first rows must fit");
-        first_rows_unit<D, 512, true>(fr, blockIdx.x, reinterpret_cast<float*>(smem));
+        first_rows_unit<D, kFusedThreads, true>(fr, blockIdx.x, reinterpret_cast<float*>(smem));
         return;
     }
     uint8_t *sX = smem + L::OFF_X, *sY = smem + L::OFF_Y, *sA = smem + L::OFF_A, *sB = smem + L::OFF_B;
@@ -242,10 +244,11 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     if (threadIdx.x == 0) {
         for (int i = 0; i < L::N_BARS; ++i) {
             uint32_t cnt = 1;
-            if (i == L::B_PDS || i == L::B_PDS + 1 || i == L::B_PRDY || i == L::B_PRDY + 1 || i == L::B_T2FREE || i == L::B_T2FREE + 1)
-                cnt = 4;   // per-warp arrives
+            if (i == L::B_PDS || i == L::B_PDS + 1 || i == L::B_PRDY || i == L::B_PRDY + 1)
+                cnt = 8;   // per-warp arrives of the two gradient warpgroups of the half
+            if (i == L::B_T2FREE || i == L::B_T2FREE + 1) cnt = 4;
             if (i == L::B_DSFREE || i == L::B_DSFREE + 1 || i == L::B_DONE ||
-                (i >= L::B_EMPTY && i < L::B_EMPTY + NST))
+                (i >= L::B_BEMPTY && i < L::B_BEMPTY + 2 * NST))
                 cnt = 2;   // one arrival from each of two MMA issuers
             mbar_init(&bars[i], cnt);
         }
@@ -261,14 +264,13 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     tc_fence_after_sync();
     const uint32_t tmem_base = warp_uniform(*tmem_slot);
 #ifdef AF_TRACE
-    long long* const trc = (blockIdx.x == 0 && blockIdx.y == 0) ? g_trace : nullptr;
+    long long* const trc = (blockIdx.x == 0 && by == 0) ? g_trace : nullptr;
 #endif
     grid_dep_wait();     // delta, the RoPE passes and the zeroed accumulator precede this grid in the stream
     grid_dep_launch();
     if (warp == 0) AF_FSTAMP(5, 0, 0);
 
-    // register budgets per role (they sum to the 512 a scheduler's four warps share): the gradient warpgroups
-    // keep a half tile of probabilities next to a half tile of dP^T
+    // register budgets per role: the gradient warpgroups keep 32 columns of probabilities next to 32 of dP^T
     if (warp < 4) setmaxnreg_dec<kFusedLightRegs>();
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -286,16 +288,26 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         for (int n = 0; n < n_it; ++n) {
             const int st = n % NST, ah = cur.head, a0 = row0_of(cur);
             advance(cur);
-            if (!mbar_wait_warp(&bars[L::B_EMPTY + st], ((n / NST) & 1) ^ 1, abort_flag, 41)) break;
-            if (elect_one()) {
-                mbar_arrive_expect_tx(&bars[L::B_AFULL + st], TILE);
-                mbar_arrive_expect_tx(&bars[L::B_BFULL + st], TILE);
+            bool ok = true;
+#pragma unroll 1
+            for (int hf = 0; ok && hf < 2; ++hf) {
+                const int slot = 2 * st + hf;
+                ok = mbar_wait_warp(&bars[L::B_AEMPTY + slot], ((n / NST) & 1) ^ 1, abort_flag, 41);
+                if (ok && elect_one()) {
+                    mbar_arrive_expect_tx(&bars[L::B_AFULL + slot], TILE / 2);
 #pragma unroll
-                for (int bx = 0; bx < NBOX; ++bx) {
-                    tma_load_4d(sA + st * TILE + bx * BOX_BYTES, &tm_a, &bars[L::B_AFULL + st], bx * BOX_COLS, a0, ah, b);
-                    tma_load_4d(sB + st * TILE + bx * BOX_BYTES, &tm_b, &bars[L::B_BFULL + st], bx * BOX_COLS, a0, ah, b);
+                    for (int bx = 0; bx < NBOX; ++bx)
+                        tma_load_4d(sA + st * TILE + bx * BOX_BYTES + hf * (BOX_BYTES / 2), &tm_a, &bars[L::B_AFULL + slot], bx * BOX_COLS, a0 + hf * 64, ah, b);
+                }
+                if (ok) ok = mbar_wait_warp(&bars[L::B_BEMPTY + slot], ((n / NST) & 1) ^ 1, abort_flag, 57);
+                if (ok && elect_one()) {
+                    mbar_arrive_expect_tx(&bars[L::B_BFULL + slot], TILE / 2);
+#pragma unroll
+                    for (int bx = 0; bx < NBOX; ++bx)
+                        tma_load_4d(sB + st * TILE + bx * BOX_BYTES + hf * (BOX_BYTES / 2), &tm_b, &bars[L::B_BFULL + slot], bx * BOX_COLS, a0 + hf * 64, ah, b);
                 }
             }
+            if (!ok) break;
         }
     } else if (warp == 1 || warp == 2) {
         // ------------------------------------------------------------ MMA issuers 0 and 1
@@ -318,19 +330,20 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                     mma_ss_lo_rt(t_dst + hf * 64, s_lo + off, r_lo + off, dhi, IDESC_TH, kk > 0 ? 1u : 0u);
                 }
                 mma_commit(&bars[(who == 0 ? L::B_SFULL : L::B_DPFULL) + hf]);
+                if (who == 1) mma_commit(&bars[L::B_BEMPTY + 2 * st + hf]);
             };
-            auto wait_stream = [&](int n) {
-                const int st = n % NST;
-                bool r = mbar_wait_warp(&bars[L::B_AFULL + st], (n / NST) & 1, abort_flag, 43);
-                if (r) r = mbar_wait_warp(&bars[L::B_BFULL + st], (n / NST) & 1, abort_flag, 44);
+            // a half tile of Q' (which = B_AFULL) or of dO (B_BFULL) has arrived
+            auto wait_half = [&](int which, int n, int hf) {
+                const bool r = mbar_wait_warp(&bars[which + 2 * (n % NST) + hf], (n / NST) & 1, abort_flag, 43);
                 tc_fence_after_sync();
                 return r;
             };
-            if (ok && n_it > 0) ok = wait_stream(0);
-            if (ok && n_it > 0) {
-                issue_T(0, 0);
-                issue_T(0, 1);
-            }
+            const int t_stream = who == 0 ? L::B_AFULL : L::B_BFULL, acc_stream = who == 0 ? L::B_BFULL : L::B_AFULL;
+            if (n_it > 0)
+                for (int hf = 0; ok && hf < 2; ++hf) {
+                    ok = wait_half(t_stream, 0, hf);
+                    if (ok) issue_T(0, hf);
+                }
             for (int n = 0; ok && n < n_it; ++n) {
                 const int st = n % NST;
                 // MN-major B operand of the accumulator MMAs: 16 streamed rows (2 KB) per K step
@@ -340,7 +353,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                 for (int hf = 0; hf < 2; ++hf) {
                     AF_FSTAMP(who, n, hf * 4);
                     // issuer 0 goes on when P^T of the half is in TMEM, issuer 1 when dS^T is in shared memory
-                    ok = mbar_wait_warp(&bars[(who == 0 ? L::B_PRDY : L::B_PDS) + hf], n & 1, abort_flag, 45);
+                    ok = wait_half(acc_stream, n, hf);
+                    if (ok) ok = mbar_wait_warp(&bars[(who == 0 ? L::B_PRDY : L::B_PDS) + hf], n & 1, abort_flag, 45);
                     if (!ok) break;
                     AF_FSTAMP(who, n, hf * 4 + 1);
                     tc_fence_after_sync();
@@ -349,7 +363,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 #pragma unroll
                         for (int k4 = 0; k4 < 4; ++k4) {
                             const int kk = hf * 4 + k4;
-                            mma_ts_lo(acc_dst, t_dst + hf * 64 + k4 * 8, m_lo + kk * 128, dhi, IDESC_ACC, (n > 0 || kk > 0) ? 1u : 0u);
+                            // (a warpgroup's probabilities sit at the start of its own 32 score columns)
+                            mma_ts_lo(acc_dst, t_dst + hf * 64 + (k4 >> 1) * 32 + (k4 & 1) * 8, m_lo + kk * 128, dhi, IDESC_ACC, (n > 0 || kk > 0) ? 1u : 0u);
                         }
                     } else {
                         // A = dS^T half (K-major: 128 key rows of 128 bytes, 32 bytes per K step)
@@ -361,9 +376,9 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                         }
                         mma_commit(&bars[L::B_DSFREE + hf]);
                     }
-                    if (hf == 1) elect_commit(&bars[L::B_EMPTY + st]);
+                    elect_commit(&bars[(who == 0 ? L::B_BEMPTY : L::B_AEMPTY) + 2 * st + hf]);
                     if (next) {
-                        if (hf == 0) ok = wait_stream(n + 1);
+                        ok = wait_half(t_stream, n + 1, hf);
                         // T2's half is free once the dQ'^T partial of the same rows has been read out of it
                         if (ok && who == 1 && !kOwnDq) ok = mbar_wait_warp(&bars[L::B_T2FREE + hf], n & 1, abort_flag, 46);
                         if (!ok) break;
@@ -428,25 +443,29 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                 if (!ok) break;
                 if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 1);
                 tc_fence_after_sync();
-                uint32_t v[64];
-                tmem_ld32(tsrc + hf * 64, v);
-                tmem_ld32(tsrc + hf * 64 + 32, v + 32);
-                tmem_wait_ld();
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bars[L::B_T2FREE + hf]);
-                if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 2);
-                const int q0 = a0 + hf * 64;
+                const int q0 = a0 + hf * 64, nq = min(64, p.S - q0);
                 float* dst = p.dq_acc + ((static_cast<size_t>(b) * p.Hq + ah) * p.S + q0) * D + d;
-                const int nq = min(64, p.S - q0);
-                if (nq == 64) {
 #pragma unroll
-                    for (int q = 0; q < 64; ++q)
-                        if (has_row) asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + q * D), "f"(__uint_as_float(v[q])) : "memory");
-                } else {
+                for (int c = 0; c < 2; ++c) {   // 32 query rows at a time
+                    uint32_t v[32];
+                    tmem_ld32(tsrc + hf * 64 + c * 32, v);
+                    tmem_wait_ld();
+                    if (c == 1) {
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&bars[L::B_T2FREE + hf]);
+                        if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 2);
+                    }
+                    if (nq == 64) {
 #pragma unroll
-                    for (int q = 0; q < 64; ++q)
-                        if (has_row && q < nq) asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + q * D), "f"(__uint_as_float(v[q])) : "memory");
+                        for (int q = 0; q < 32; ++q)
+                            if (has_row) asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + (c * 32 + q) * D), "f"(__uint_as_float(v[q])) : "memory");
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 32; ++q)
+                            if (has_row && c * 32 + q < nq)
+                                asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + (c * 32 + q) * D), "f"(__uint_as_float(v[q])) : "memory");
+                    }
                 }
                 if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 3);
             }
@@ -455,11 +474,14 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         // ------------------------------------------------------------ gradient warpgroups (one TMEM lane = key row per thread)
         setmaxnreg_inc<kFusedGradRegs>();
         const int gtid = threadIdx.x - 256;
-        const int hf = gtid >> 7;                    // column half (64 streamed rows) owned by this warpgroup
+        const int wg = gtid >> 7;                    // 0..3: owns 32 of the 128 streamed rows (columns of T1 and T2)
+        const int hf = wg >> 1, col0 = wg * 32;      // the half they belong to, the first of them
         const int tid = gtid & 127;
         const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
         const uint32_t tb = tmem_base + lane_addr;
         const int xrow = x0 + tid;                   // key row j
+        const int wg_bar = wg < 2 ? 1 + wg : 2 + wg;   // this warpgroup's named barrier (3 is the one of all four)
+        const bool polls = (warp & 3) == 0;   // one warp of the warpgroup polls the barriers, the others wait at the named one
         const bool alibi = p.slopes != nullptr;
         constexpr float kLog2e = 1.4426950408889634f;
         const uint32_t ds_row_addr = smem_u32(sDS + hf * L::DS_HALF) + static_cast<uint32_t>(tid) * 128;
@@ -476,8 +498,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             const int ah = cur.head, a0 = row0_of(cur);
             advance(cur);
             nx_a0 = a0;
-            if (tid < 64) {
-                const int qi = a0 + hf * 64 + tid;
+            if (tid < 32) {
+                const int qi = a0 + col0 + tid;
                 const size_t r = (static_cast<size_t>(b) * p.Hq + ah) * p.S + min(qi, p.S - 1);
                 nx_in = qi < p.S;
                 nx_l = p.lse[r];
@@ -486,8 +508,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             if (alibi) nx_slope = p.slopes[ah];
         };
         auto store_stats = [&](int n) {
-            if (tid < 64) {
-                float* dst = sStats + (n & 1) * 256 + hf * 64 + tid;
+            if (tid < 32) {
+                float* dst = sStats + (n & 1) * 256 + col0 + tid;
                 dst[0] = nx_in ? -nx_l * kLog2e : -INFINITY;   // kept negated
                 dst[128] = nx_in ? -nx_d : 0.f;
             }
@@ -508,65 +530,53 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             if (need_mask) kept_queries_of_key(ms, xrow, a0, mlo, mn);
             const float sb = -my_slope2;
             const float bias_base = sb * static_cast<float>(a0 - xrow);
-            // the previous tile's dS^T half must have been consumed by both MMAs that read it
-            if ((warp & 3) == 0) AF_FSTAMP(2 + hf, n, 0);
-            ok = bar_all(ok && mbar_wait(&bars[L::B_SFULL + hf], n & 1, abort_flag, 51), 1 + hf, 128);
+            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 0);
+            ok = bar_all(ok && (!polls || mbar_wait(&bars[L::B_SFULL + hf], n & 1, abort_flag, 51)), wg_bar, 128);
             if (!ok) break;
-            if ((warp & 3) == 0) AF_FSTAMP(2 + hf, n, 1);
+            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 1);
             tc_fence_after_sync();
-            // both 32-column chunks are requested up front; the second one lands while the first is worked on
-            uint32_t pe_keep[64];
-            tmem_ld32(tb + T1 + hf * 64, pe_keep);
+            uint32_t pe_keep[32];
+            tmem_ld32(tb + T1 + col0, pe_keep);
             tmem_wait_ld();
-            tmem_ld32(tb + T1 + hf * 64 + 32, pe_keep + 32);
-#pragma unroll
-            for (int qt = 0; qt < 2; ++qt) {
-                const int col0 = hf * 64 + qt * 32;
-                const uint32_t out_col = hf * 64 + qt * 16;
-                const float cbias = fmaf(sb, static_cast<float>(col0), bias_base);
-                if (qt == 1) tmem_wait_ld();
-                if (alibi) {
-                    if (need_mask) grad_phase_p32<true, true>(tb + T1, col0, out_col, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep + qt * 32);
-                    else grad_phase_p32<false, true>(tb + T1, col0, out_col, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep + qt * 32);
-                } else {
-                    if (need_mask) grad_phase_p32<true, false>(tb + T1, col0, out_col, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep + qt * 32);
-                    else grad_phase_p32<false, false>(tb + T1, col0, out_col, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep + qt * 32);
-                }
+            const float cbias = fmaf(sb, static_cast<float>(col0), bias_base);
+            if (alibi) {
+                if (need_mask) grad_phase_p32<true, true>(tb + T1, col0, col0, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep);
+                else grad_phase_p32<false, true>(tb + T1, col0, col0, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep);
+            } else {
+                if (need_mask) grad_phase_p32<true, false>(tb + T1, col0, col0, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep);
+                else grad_phase_p32<false, false>(tb + T1, col0, col0, p.scale_log2, cbias, sb, sL2, mlo, mn, pe_keep);
             }
             tmem_wait_st();
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[L::B_PRDY + hf]);
-            if ((warp & 3) == 0) AF_FSTAMP(2 + hf, n, 2);
+            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 2);
             // the previous tile's dS^T half must have been consumed by both MMAs that read it
-            ok = mbar_wait(&bars[L::B_DSFREE + hf], (n & 1) ^ 1, abort_flag, 50);
+            if (polls) ok = mbar_wait(&bars[L::B_DSFREE + hf], (n & 1) ^ 1, abort_flag, 50);
             // (the vote keeps the warpgroup together: a warp that gave up must not leave the others at the barrier above)
-            ok = bar_all(ok && mbar_wait(&bars[L::B_DPFULL + hf], n & 1, abort_flag, 53), 1 + hf, 128);
+            ok = bar_all(ok && (!polls || mbar_wait(&bars[L::B_DPFULL + hf], n & 1, abort_flag, 53)), wg_bar, 128);
             if (!ok) break;
-            if ((warp & 3) == 0) AF_FSTAMP(2 + hf, n, 3);
+            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 3);
             tc_fence_after_sync();
-            uint32_t dp[64];
-            tmem_ld32(tb + T2 + hf * 64, dp);
+            uint32_t dp[32];
+            tmem_ld32(tb + T2 + col0, dp);
             tmem_wait_ld();
-            tmem_ld32(tb + T2 + hf * 64 + 32, dp + 32);
-            grad_phase_ds32(dp, hf * 64, sDl, pe_keep, ds_row_addr, tid & 7, 0);
-            tmem_wait_ld();
-            grad_phase_ds32(dp + 32, hf * 64 + 32, sDl, pe_keep + 32, ds_row_addr, tid & 7, 4);
+            grad_phase_ds32(dp, col0, sDl, pe_keep, ds_row_addr, tid & 7, (wg & 1) * 4);
             fence_proxy_async_smem();   // dS^T in shared memory is read by the tensor core's asynchronous proxy
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[L::B_PDS + hf]);
-            if ((warp & 3) == 0) AF_FSTAMP(2 + hf, n, 4);
+            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 4);
             if (n + 1 < n_it) store_stats(n + 1);   // (published by the named barrier at the top of the next iteration)
         }
-        // (every thread of both warpgroups takes this barrier, also after a wait that gave up in one of them:
-        // a warpgroup that left its loop early must not leave the other alone at it)
-        ok = wg_all(ok && (n_it <= 0 || mbar_wait(&bars[L::B_DONE], 0, abort_flag, 52)));
+        // (every thread of the four warpgroups takes this barrier, also after a wait that gave up in one of them:
+        // a warpgroup that left its loop early must not leave the others alone at it)
+        ok = wg_all<kFusedGradThreads>(ok && (n_it <= 0 || mbar_wait(&bars[L::B_DONE], 0, abort_flag, 52)));
         if (ok && n_it <= 0) {
             // no query tile sees this key tile: its gradient rows are zero
             const size_t row0 = (static_cast<size_t>(b) * p.Hkv + xh) * p.S + x0;
             const int rows = min(128, p.S - x0);
-            for (int idx = gtid; idx < rows * (D / 4); idx += 256) {
+            for (int idx = gtid; idx < rows * (D / 4); idx += kFusedGradThreads) {
                 const size_t off = (row0 + idx / (D / 4)) * D + (idx % (D / 4)) * 4;
                 for (int w2 = 0; w2 < 2; ++w2) {
                     void* out = w2 == 0 ? p.out1 : p.out2;
@@ -577,21 +587,21 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         }
         if (SPLIT && ok && parts > 1) {
             // (the staging buffers cover the stationary tile and dS^T, which the last dQ'^T products read)
-            ok = wg_all(mbar_wait(&bars[L::B_DQFULL], (n_it - 1) & 1, abort_flag, 55) &&
+            ok = wg_all<kFusedGradThreads>(mbar_wait(&bars[L::B_DQFULL], (n_it - 1) & 1, abort_flag, 55) &&
                         mbar_wait(&bars[L::B_DQFULL + 1], (n_it - 1) & 1, abort_flag, 56));
         }
         if (SPLIT && ok && parts > 1) {
             tc_fence_after_sync();
-            stage_acc<D>(tb + ACC1, stg0, gtid, 1.f);
-            stage_acc<D>(tb + ACC2, stg1, gtid, p.scale);
+            stage_acc<D, kFusedGradThreads>(tb + ACC1, stg0, gtid, 1.f);
+            stage_acc<D, kFusedGradThreads>(tb + ACC2, stg1, gtid, p.scale);
         }
         if (ok && n_it > 0 && (!SPLIT || parts == 1)) {
             tc_fence_after_sync();
             float* stg = reinterpret_cast<float*>(sA);
             const size_t out_row0 = (static_cast<size_t>(b) * p.Hkv + xh) * p.S + x0;
             const int add_rows = first_ctas ? fr.rows : 0;
-            store_acc_rotated<D>(tb + ACC1, stg, gtid, 1.f, 0, p.table, x0, p.S, p.out1, out_row0, p.out_f32, add_rows);
-            store_acc_rotated<D>(tb + ACC2, stg, gtid, p.scale, p.R, p.table, x0, p.S, p.out2, out_row0, p.out_f32, add_rows);
+            store_acc_rotated<D, kFusedGradThreads>(tb + ACC1, stg, gtid, 1.f, 0, p.table, x0, p.S, p.out1, out_row0, p.out_f32, add_rows);
+            store_acc_rotated<D, kFusedGradThreads>(tb + ACC2, stg, gtid, p.scale, p.R, p.table, x0, p.S, p.out2, out_row0, p.out_f32, add_rows);
         }
     }
 
@@ -602,8 +612,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         if (warp >= 8 && !*abort_flag) {
             const int gtid = threadIdx.x - 256, add_rows = first_ctas ? fr.rows : 0;
             const size_t out_row0 = (static_cast<size_t>(b) * p.Hkv + xh) * p.S + x0;
-            store_shared_rows<D>(stg0, rank, parts, gtid, 0, p.table, x0, p.S, p.out1, out_row0, p.out_f32, add_rows);
-            store_shared_rows<D>(stg1, rank, parts, gtid, p.R, p.table, x0, p.S, p.out2, out_row0, p.out_f32, add_rows);
+            store_shared_rows<D, kFusedGradThreads>(stg0, rank, parts, gtid, 0, p.table, x0, p.S, p.out1, out_row0, p.out_f32, add_rows);
+            store_shared_rows<D, kFusedGradThreads>(stg1, rank, parts, gtid, p.R, p.table, x0, p.S, p.out2, out_row0, p.out_f32, add_rows);
         }
         __syncwarp();
         cluster_sync();   // nobody leaves while its shared memory is being read

@@ -162,8 +162,9 @@ struct BwdSmem {
     static_assert(128 * STG_STRIDE * 4 <= 2 * NST * TILE, "staging buffer must fit in the stream stages");
 };
 
-// Named barriers of the gradient warpgroups: id 3 joins both (256 threads), ids 1 and 2 one each.
-__device__ __forceinline__ void wg_sync() { asm volatile("bar.sync 3, 256;" ::: "memory"); }
+// Named barriers of the gradient warpgroups: id 3 joins all of them (NT threads), ids 1, 2 (and 4, 5) one each.
+template <int NT = 256>
+__device__ __forceinline__ void wg_sync() { asm volatile("bar.sync 3, %0;" ::"n"(NT) : "memory"); }
 // Barrier that also ANDs a flag, so that a wait that gave up in one thread ends the loop in all of
 // them (nobody is left alone at a barrier).  id/count: 3/256 for both warpgroups, 1+hf/128 for one.
 __device__ __forceinline__ bool bar_all(bool v, int id, int count) {
@@ -175,16 +176,36 @@ __device__ __forceinline__ bool bar_all(bool v, int id, int count) {
         : "memory");
     return r != 0;
 }
-__device__ __forceinline__ bool wg_all(bool v) { return bar_all(v, 3, 256); }
+template <int NT = 256>
+__device__ __forceinline__ bool wg_all(bool v) { return bar_all(v, 3, NT); }
 
-// Epilogue helper: the 256 threads of the two gradient warpgroups move a [128 x D] fp32 accumulator
-// from TMEM (thread gtid reads lane gtid % 128, column half gtid / 128) through shared memory to
-// global memory, scaling it and, when R > 0, applying the transpose rotation for positions row0..
+// Thread gtid of NT moves lane gtid % 128, columns [D / (NT / 128)] of its warpgroup, of an accumulator to the staging rows.
+template <int D, int NT = 256>
+__device__ __forceinline__ void stage_acc(uint32_t t_acc, float* stg, int gtid, float mul) {
+    constexpr int STRIDE = BwdSmem<D>::STG_STRIDE, COLS = D / (NT / 128), STEP = COLS < 32 ? COLS : 32;
+    const int lane_row = gtid & 127, part = gtid >> 7;
+#pragma unroll 1
+    for (int cc = 0; cc < COLS / STEP; ++cc) {
+        const int col = part * COLS + cc * STEP;
+        uint32_t v[STEP];
+        if constexpr (STEP == 32) tmem_ld32(t_acc + col, v);
+        else tmem_ld16(t_acc + col, v);
+        tmem_wait_ld();
+        float4* dst = reinterpret_cast<float4*>(stg + lane_row * STRIDE + col);
+#pragma unroll
+        for (int e = 0; e < STEP; e += 4)
+            dst[e >> 2] = make_float4(__uint_as_float(v[e]) * mul, __uint_as_float(v[e + 1]) * mul,
+                                      __uint_as_float(v[e + 2]) * mul, __uint_as_float(v[e + 3]) * mul);
+    }
+}
+
+// Epilogue helper: the NT threads of the gradient warpgroups move a [128 x D] fp32 accumulator from TMEM through
+// shared memory to global memory, scaling it and, when R > 0, applying the transpose rotation for positions row0..
 // (gradients w.r.t. rotated rows are rotated back).  Global writes are coalesced along D.  (Writing each
 // thread's TMEM row straight to global memory - no staging, no barriers, cos/sin read per row - measured
 // slower: a warp's store then touches 32 rows, and the store rate is what bounds this epilogue.)
 // Rows below add_rows (fp32 output only) are added to what is there instead of stored.
-template <int D>
+template <int D, int NT = 256>
 __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, int gtid, float mul, int R,
                                                   const float2* table, int row0, int S, void* out, size_t out_row0,
                                                   int out_f32, int add_rows = 0) {
@@ -195,7 +216,7 @@ __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, in
     // frequencies' cos/sin come from the table once (first row, and the next one to get the step angle as
     // a difference of angles) and then walk by the angle-addition recurrence: no table read in the loop.
     constexpr int TPR = D / 4;        // threads per row
-    constexpr int RPP = 256 / TPR;    // rows per pass (8 for D = 128, 16 for D = 64)
+    constexpr int RPP = NT / TPR;     // rows per pass
     const int d = (gtid % TPR) * 4, rsub = gtid / TPR;
     const int half = R >> 1;
     const bool rot = d < R;           // R is a multiple of 8: the four columns are on one side of R and of R / 2
@@ -216,20 +237,8 @@ __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, in
             if (upper) sst[u] = -sst[u];                  // the sign rides along with sn
         }
     }
-    const int lane_row = gtid & 127, chalf = gtid >> 7;
-#pragma unroll 1
-    for (int cc = 0; cc < D / 64; ++cc) {
-        const int col = chalf * (D / 2) + cc * 32;
-        uint32_t v[32];
-        tmem_ld32(t_acc + col, v);
-        tmem_wait_ld();
-        float4* dst = reinterpret_cast<float4*>(stg + lane_row * STRIDE + col);
-#pragma unroll
-        for (int e = 0; e < 32; e += 4)
-            dst[e >> 2] = make_float4(__uint_as_float(v[e]) * mul, __uint_as_float(v[e + 1]) * mul,
-                                      __uint_as_float(v[e + 2]) * mul, __uint_as_float(v[e + 3]) * mul);
-    }
-    wg_sync();
+    stage_acc<D, NT>(t_acc, stg, gtid, mul);
+    wg_sync<NT>();
 #pragma unroll 2
     for (int r = rsub; r < 128; r += RPP) {
         if (row0 + r < S) {
@@ -261,33 +270,16 @@ __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, in
             }
         }
     }
-    wg_sync();
+    wg_sync<NT>();
 }
 
 // The same epilogue for a key tile whose query tiles were shared out among the CTAs of a cluster: every CTA stages its partial
 // accumulator (stage_acc), and after a cluster barrier CTA `rank` of `n` sums rows [128 rank / n, 128 (rank + 1) / n) over
 // the cluster, in rank order (reproducible), and stores them (store_shared_rows).
-template <int D>
-__device__ __forceinline__ void stage_acc(uint32_t t_acc, float* stg, int gtid, float mul) {
-    constexpr int STRIDE = BwdSmem<D>::STG_STRIDE;
-    const int lane_row = gtid & 127, chalf = gtid >> 7;
-#pragma unroll 1
-    for (int cc = 0; cc < D / 64; ++cc) {
-        const int col = chalf * (D / 2) + cc * 32;
-        uint32_t v[32];
-        tmem_ld32(t_acc + col, v);
-        tmem_wait_ld();
-        float4* dst = reinterpret_cast<float4*>(stg + lane_row * STRIDE + col);
-#pragma unroll
-        for (int e = 0; e < 32; e += 4)
-            dst[e >> 2] = make_float4(__uint_as_float(v[e]) * mul, __uint_as_float(v[e + 1]) * mul,
-                                      __uint_as_float(v[e + 2]) * mul, __uint_as_float(v[e + 3]) * mul);
-    }
-}
-template <int D>
+template <int D, int NT>
 __device__ __forceinline__ void store_shared_rows(const float* stg, int rank, int n, int gtid, int R, const float2* table, int row0,
                                                   int S, void* out, size_t out_row0, int out_f32, int add_rows) {
-    constexpr int STRIDE = BwdSmem<D>::STG_STRIDE, TPR = D / 4, RPP = 256 / TPR;
+    constexpr int STRIDE = BwdSmem<D>::STG_STRIDE, TPR = D / 4, RPP = NT / TPR;
     const int d = (gtid % TPR) * 4, half = R >> 1;
     const bool rot = d < R, upper = d >= half;
     const int partner = upper ? d - half : d + half;
