@@ -954,10 +954,16 @@ af_status attnfuse_fwd_fp8(const af_shape* shape, const void* q8, const void* k8
         return AF_ERR_SPEC;
     af_status st = check_arch();
     if (st != AF_OK) return st;
-    CUtensorMap tq, tk, tv;
+    CUtensorMap tq, tk, tv, to;
     if ((st = make_tmap_u8(&tq, q8, shape->B, shape->Hq, shape->S, shape->D)) != AF_OK) return st;
     if ((st = make_tmap_u8(&tk, k8, shape->B, shape->Hkv, shape->S, shape->D)) != AF_OK) return st;
     if ((st = make_tmap_u8(&tv, vt8, shape->B, shape->Hkv, shape->D, shape->S)) != AF_OK) return st;
+    to = tq;   // (fp32 output is stored directly)
+    if (o_dtype == AF_BF16) {
+        af_strides sto;
+        resolve_strides(nullptr, shape->Hq, shape->S, shape->D, &sto);
+        if ((st = make_tmap(&to, o, shape->B, shape->Hq, shape->S, shape->D, sto, BM)) != AF_OK) return st;
+    }
     Fp8Params p;
     p.B = shape->B; p.Hq = shape->Hq; p.Hkv = shape->Hkv; p.S = shape->S; p.group = gqa_group;
     p.causal = mask->causal ? 1 : 0;
@@ -972,7 +978,7 @@ af_status attnfuse_fwd_fp8(const af_shape* shape, const void* q8, const void* k8
     if (allow_dynamic_smem(attn_fwd_fp8_kernel, Fp8Smem::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
     return launch_kernel(attn_fwd_fp8_kernel, grid, dim3(512, 1, 1), Fp8Smem::BYTES, static_cast<cudaStream_t>(cuda_stream), true, tq,
-                         tk, tv, p);
+                         tk, tv, to, p);
 }
 
 size_t attnfuse_fwd_hybrid_workspace_bytes(const af_shape* shape) {

@@ -26,7 +26,8 @@ struct Fp8Params {
 struct Fp8Smem {
     static constexpr int TILE = 128 * 128;        // 128 rows of 128 one-byte elements: one TMA box
     static constexpr int NQ = 2, KS = 2, VS = 2;
-    static constexpr int OFF_Q = 0, OFF_K = OFF_Q + NQ * TILE, OFF_V = OFF_K + KS * TILE, OFF_BAR = OFF_V + VS * TILE;
+    static constexpr int OFF_Q = 0, OFF_K = OFF_Q + NQ * TILE, OFF_V = OFF_K + KS * TILE, OFF_O = OFF_V + VS * TILE;
+    static constexpr int OFF_BAR = OFF_O + NQ * 2 * TILE;   // bf16 output tiles: two boxes of 64 columns each
     static constexpr int B_QFULL = 0, B_KFULL = B_QFULL + NQ, B_KEMPTY = B_KFULL + KS, B_VFULL = B_KEMPTY + KS,
                          B_VEMPTY = B_VFULL + VS, B_SFULL = B_VEMPTY + VS, B_PREADY = B_SFULL + NQ, B_ODONE = B_PREADY + 2 * NQ,
                          N_BARS = B_ODONE + NQ;
@@ -152,7 +153,7 @@ __device__ __forceinline__ bool softmax_tile_fp8(uint32_t tS, uint32_t tO, int n
 
 __global__ void __launch_bounds__(512, 1)
 attn_fwd_fp8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                    const __grid_constant__ CUtensorMap tm_vt, const Fp8Params p) {
+                    const __grid_constant__ CUtensorMap tm_vt, const __grid_constant__ CUtensorMap tm_o, const Fp8Params p) {
     using L = Fp8Smem;
     constexpr int D = 128, NQ = L::NQ, KS = L::KS, VS = L::VS, TILE = L::TILE;
     constexpr uint32_t TMEM_COLS = 512;
@@ -191,11 +192,34 @@ attn_fwd_fp8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     auto active = [&](int q, int j) { return j >= jlo[q] && j <= jhi[q]; };
     const int n_it = jhi_c - jlo_c + 1;
 
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < L::N_BARS; ++i)
-            mbar_init(&bars[i], (i >= L::B_PREADY && i < L::B_PREADY + 2 * NQ) ? 4 : 1);   // P: one arrive per warp
-        *abort_flag = 0;
+    // Set-up with little in a row, as in the bf16 kernel: a barrier per lane of warp 0, which then requests the first tiles
+    // while warp 1 allocates tensor memory; what comes before grid_dep_wait overlaps with the kernel before this one.
+    // With the bf16 output through TMA (see the epilogue): 117.4 -> 111.4 us (32 / 8 heads, S = 4096), 61.5 -> 56.9 us (the
+    // same with a window of 512), 1542 -> 1483 us (S = 16384), 32.3 -> 31.8 us (B = 2, 12 heads, S = 2000).
+    if (warp == 0) {
+        static_assert(L::N_BARS <= 32, "one barrier per lane");
+        if (lane < L::N_BARS)
+            mbar_init(&bars[lane], (lane >= L::B_PREADY && lane < L::B_PREADY + 2 * NQ) ? 4 : 1);   // P: one arrive per warp
+        if (lane == 0) *abort_flag = 0;
         fence_mbar_init();
+        __syncwarp();
+        grid_dep_wait();
+        if (lane == 0) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                if (jhi[q] < jlo[q]) continue;
+                mbar_arrive_expect_tx(&bars[L::B_QFULL + q], TILE);
+                tma_load_4d(sQ + q * TILE, &tm_q, &bars[L::B_QFULL + q], 0, i0[q], hq[q], b);
+            }
+            if (n_it > 0) {
+                const int j0 = jlo_c * BN;
+                mbar_arrive_expect_tx(&bars[L::B_KFULL], TILE);
+                tma_load_4d(sK, &tm_k, &bars[L::B_KFULL], 0, j0, hk, b);
+                mbar_arrive_expect_tx(&bars[L::B_VFULL], TILE);
+                tma_load_4d(sV, &tm_vt, &bars[L::B_VFULL], j0, 0, hk, b);   // V^T: keys innermost
+            }
+        }
+        __syncwarp();
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, TMEM_COLS);
@@ -205,23 +229,14 @@ attn_fwd_fp8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
-    grid_dep_launch();   // programmatic dependent launch: the set-up above overlaps with the end of the previous kernel
+    grid_dep_launch();
     grid_dep_wait();
 
     if (warp < 8) setmaxnreg_dec<80>();
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            prefetch_tmap(&tm_q);
-            prefetch_tmap(&tm_k);
-            prefetch_tmap(&tm_vt);
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                if (jhi[q] < jlo[q]) continue;
-                mbar_arrive_expect_tx(&bars[L::B_QFULL + q], TILE);
-                tma_load_4d(sQ + q * TILE, &tm_q, &bars[L::B_QFULL + q], 0, i0[q], hq[q], b);
-            }
-            for (int it = 0; it < n_it; ++it) {
+            for (int it = 1; it < n_it; ++it) {   // (the first tiles were requested above)
                 const int j0 = (jlo_c + it) * BN;
                 const int ks = it % KS, vs = it % VS;
                 if (!mbar_wait(&bars[L::B_KEMPTY + ks], ((it / KS) & 1) ^ 1, abort_flag, 61)) break;
@@ -331,35 +346,54 @@ attn_fwd_fp8_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             ++n;
         }
         if (ok && jhi[q] >= jlo[q]) ok = mbar_wait_warp(&bars[L::B_ODONE + q], 0, abort_flag, 68);
+        // (the vote keeps the warpgroup together at the barriers of the epilogue)
+        ok = bar_all(ok, 4 + q, 128);
         if (ok && jhi[q] >= jlo[q]) {
             tc_fence_after_sync();
             const float inv = l_run > 0.f ? p.out_scale / l_run : 0.f;
-            const size_t orow = (static_cast<size_t>(bh) * p.S + i) * D;
+            if (p.lse && i < p.S)
+                p.lse[static_cast<size_t>(bh) * p.S + i] = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
+            if (!p.o_f32) {
+                // bf16: through shared memory and TMA, box by box (row-per-thread stores touch 32 rows per instruction);
+                // rows past S are clipped by the tensor map
+                uint8_t* stg = smem + L::OFF_O + q * 2 * TILE;
 #pragma unroll 1
-            for (int c = 0; c < D / 32; ++c) {
-                uint32_t v[32];
-                tmem_ld32(tO + c * 32, v);
-                tmem_wait_ld();
-                if (i < p.S) {
-                    if (p.o_f32) {
+                for (int bx = 0; bx < 2; ++bx) {
+                    uint32_t v[64];
+                    tmem_ld32(tO + bx * 64, v);
+                    tmem_ld32(tO + bx * 64 + 32, v + 32);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 64; e += 8)
+                        *reinterpret_cast<uint4*>(stg + swz_chunk_offset(row, bx * 8 + (e >> 3))) = make_uint4(
+                            pack_bf16x2(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv),
+                            pack_bf16x2(__uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv),
+                            pack_bf16x2(__uint_as_float(v[e + 4]) * inv, __uint_as_float(v[e + 5]) * inv),
+                            pack_bf16x2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv));
+                    fence_proxy_async_smem();
+                    asm volatile("bar.sync %0, 128;" ::"r"(4 + q) : "memory");   // this warpgroup only
+                    if (row == 0) {
+                        tma_store_4d(&tm_o, stg + bx * BOX_BYTES, bx * BOX_COLS, i0[q], hq[q], b);
+                        tma_store_commit();
+                    }
+                }
+                if (row == 0) tma_store_wait_read();   // the buffer must stay in place until it has been read
+            } else {
+                const size_t orow = (static_cast<size_t>(bh) * p.S + i) * D;
+#pragma unroll 1
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t v[32];
+                    tmem_ld32(tO + c * 32, v);
+                    tmem_wait_ld();
+                    if (i < p.S) {
                         float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.o) + orow + c * 32);
 #pragma unroll
                         for (int e = 0; e < 32; e += 4)
                             dst[e >> 2] = make_float4(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv,
                                                       __uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv);
-                    } else {
-                        uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.o) + orow + c * 32);
-#pragma unroll
-                        for (int e = 0; e < 32; e += 8)
-                            dst[e >> 3] = make_uint4(pack_bf16x2(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv),
-                                                     pack_bf16x2(__uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv),
-                                                     pack_bf16x2(__uint_as_float(v[e + 4]) * inv, __uint_as_float(v[e + 5]) * inv),
-                                                     pack_bf16x2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv));
                     }
                 }
             }
-            if (p.lse && i < p.S)
-                p.lse[static_cast<size_t>(bh) * p.S + i] = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
         }
     }
 
