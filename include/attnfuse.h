@@ -14,7 +14,7 @@
  *    reported by return code; nothing throws or aborts.
  *  - Device-side waits are bounded.  A wait that runs out makes the kernel return early and
  *    records a code that attnfuse_device_status() reports; outputs of that launch are undefined.
- *  - Forward and backward are run-to-run deterministic (no atomics in the data path).
+ *  - Run-to-run deterministic, except the one-pass backward's dQ, whose fp32 partial sums are reduced in no fixed order.
  */
 #ifndef ATTNFUSE_H_
 #define ATTNFUSE_H_
