@@ -89,7 +89,7 @@ __device__ __forceinline__ void first_rows_unit(const FirstRowsParams& p, int un
     if (p.R > 0) {
         const int n4 = rows * (p.R >> 1) / 2;   // float4 = two {cos, sin} pairs; R / 2 is a multiple of 8
         for (int idx = tid; idx < n4; idx += NT)
-            reinterpret_cast<float4*>(cs)[idx] = __ldg(reinterpret_cast<const float4*>(p.table) + idx);
+            reinterpret_cast<float4*>(cs)[idx] = ld_global(reinterpret_cast<const float4*>(p.table) + idx);
     }
     // keys and values of the first rows (8 bf16 per load); gradients start at zero
     static_assert(NR * D / 8 <= NT, "at most one 16-byte chunk of K and of V per thread");
@@ -97,8 +97,8 @@ __device__ __forceinline__ void first_rows_unit(const FirstRowsParams& p, int un
         const int j = tid / (D / 8), d = (tid % (D / 8)) * 8;
         uint4 kw = make_uint4(0u, 0u, 0u, 0u), vw = kw;
         if (j < rows) {
-            kw = __ldg(reinterpret_cast<const uint4*>(kbase + j * p.ks + d));
-            vw = __ldg(reinterpret_cast<const uint4*>(vbase + j * p.ks + d));
+            kw = ld_global(reinterpret_cast<const uint4*>(kbase + j * p.ks + d));
+            vw = ld_global(reinterpret_cast<const uint4*>(vbase + j * p.ks + d));
         }
         const uint32_t ka[4] = {kw.x, kw.y, kw.z, kw.w}, va[4] = {vw.x, vw.y, vw.z, vw.w};
 #pragma unroll
@@ -133,8 +133,8 @@ __device__ __forceinline__ void first_rows_unit(const FirstRowsParams& p, int un
                 qw[c] = make_uint4(0u, 0u, 0u, 0u);
                 gw[c] = qw[c];
                 if (idx < PANEL * D && hh < nh && i < rows) {
-                    qw[c] = __ldg(reinterpret_cast<const uint4*>(p.q + b * p.qb + h * p.qh + i * p.qs + d));
-                    gw[c] = __ldg(reinterpret_cast<const uint4*>(p.d_o + ((static_cast<size_t>(b) * p.Hq + h) * p.S + i) * D + d));
+                    qw[c] = ld_global(reinterpret_cast<const uint4*>(p.q + b * p.qb + h * p.qh + i * p.qs + d));
+                    gw[c] = ld_global(reinterpret_cast<const uint4*>(p.d_o + ((static_cast<size_t>(b) * p.Hq + h) * p.S + i) * D + d));
                 }
             }
 #pragma unroll

@@ -206,14 +206,14 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     const int b = blockIdx.x / p.Hkv, xh = blockIdx.x - b * p.Hkv;
     // heaviest key tiles first under a causal mask; with block lists the caller's order
     const int by = static_cast<int>(blockIdx.y) - first_ctas;
-    const int x0 = ((BS && p.bs_order) ? __ldg(p.bs_order + by) : by) * 128;
+    const int x0 = ((BS && p.bs_order) ? ld_global(p.bs_order + by) : by) * 128;
     int lo, hi;
     qtile_range(ms, x0, lo, hi);
     int bs_base = 0;
     if constexpr (BS) {   // positions in the key block's list instead of a tile range
-        bs_base = __ldg(p.bs_ptr + x0 / 128);
+        bs_base = ld_global(p.bs_ptr + x0 / 128);
         lo = 0;
-        hi = __ldg(p.bs_ptr + x0 / 128 + 1) - bs_base - 1;
+        hi = ld_global(p.bs_ptr + x0 / 128 + 1) - bs_base - 1;
     }
     const int per_head = hi - lo + 1;
     const int n_all = per_head > 0 ? per_head * p.group : 0;
@@ -239,7 +239,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             ++c.head;
         }
     };
-    auto row0_of = [&](const Cursor& c) { return (BS ? __ldg(p.bs_idx + bs_base + lo + c.pos) : lo + c.pos) * 128; };
+    auto row0_of = [&](const Cursor& c) { return (BS ? ld_global(p.bs_idx + bs_base + lo + c.pos) : lo + c.pos) * 128; };
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < L::N_BARS; ++i) {
@@ -649,13 +649,13 @@ __global__ void __launch_bounds__(256) bwd_dq_finish_kernel(const float* __restr
     for (int u = 0; u < kFinishHeads; ++u)
         if (h0 + u < NH) {
             const float* row = acc + (static_cast<size_t>(h0 + u) * S + s) * D;
-            a[u] = __ldcs(reinterpret_cast<const float4*>(row + d0));
-            b[u] = __ldcs(reinterpret_cast<const float4*>(row + d1));
+            a[u] = ld_global_cs(reinterpret_cast<const float4*>(row + d0));
+            b[u] = ld_global_cs(reinterpret_cast<const float4*>(row + d1));
         }
     float4 cs = make_float4(scale, scale, scale, scale), sn = make_float4(0.f, 0.f, 0.f, 0.f);
     if (rot) {
-        const float4 t01 = __ldg(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0));
-        const float4 t23 = __ldg(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0 + 2));
+        const float4 t01 = ld_global(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0));
+        const float4 t23 = ld_global(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0 + 2));
         cs = make_float4(t01.x * scale, t01.z * scale, t23.x * scale, t23.z * scale);
         sn = make_float4(t01.y * scale, t01.w * scale, t23.y * scale, t23.w * scale);
     }

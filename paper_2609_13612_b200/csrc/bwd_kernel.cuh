@@ -108,8 +108,8 @@ __global__ void __launch_bounds__(256) bwd_prologue_kernel(const BwdProloguePara
             const long long idx = idx0 + u * 256;
             a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
             if (idx / TPR < p.rows) {
-                a[u] = __ldg(p.o + idx);
-                b[u] = __ldg(p.d_o + idx);
+                a[u] = ld_global(p.o + idx);
+                b[u] = ld_global(p.d_o + idx);
             }
         }
 #pragma unroll
@@ -228,8 +228,8 @@ __device__ __forceinline__ void store_acc_rotated(uint32_t t_acc, float* stg, in
         const int r0 = min(row0 + rsub, S - 1), r1 = min(row0 + rsub + RPP, S - 1);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const float2 t0 = __ldg(table + static_cast<size_t>(r0) * half + fi + u);
-            const float2 t1 = __ldg(table + static_cast<size_t>(r1) * half + fi + u);
+            const float2 t0 = ld_global(table + static_cast<size_t>(r0) * half + fi + u);
+            const float2 t1 = ld_global(table + static_cast<size_t>(r1) * half + fi + u);
             c[u] = t0.x;
             sn[u] = upper ? -t0.y : t0.y;                 // transpose rotation: y c + other s below R/2, y c - other s above
             cst[u] = fmaf(t1.x, t0.x, t1.y * t0.y);       // cos(a1 - a0)
@@ -290,8 +290,8 @@ __device__ __forceinline__ void store_shared_rows(const float* stg, int rank, in
         float4 t01 = y, t23 = y;
         if (rot) {
             const float4* t = reinterpret_cast<const float4*>(table + static_cast<size_t>(row0 + r) * half + (upper ? d - half : d));
-            t01 = __ldg(t);
-            t23 = __ldg(t + 1);
+            t01 = ld_global(t);
+            t23 = ld_global(t + 1);
         }
         for (int c = 0; c < n; ++c) {
             const float4 v = ld_cluster4(base + (r * STRIDE + d) * 4, c);
@@ -386,7 +386,7 @@ __device__ __forceinline__ void grad_pass32_general(uint32_t t1, uint32_t t2, in
     tmem_ld32(t2 + col0, dp);
     float bv[32];
 #pragma unroll
-    for (int c = 0; c < 32; ++c) bv[c] = (bias && c < cols_ok) ? __ldg(bias + c * col_stride) : 0.f;
+    for (int c = 0; c < 32; ++c) bv[c] = (bias && c < cols_ok) ? ld_global(bias + c * col_stride) : 0.f;
     tmem_wait_ld();
 #pragma unroll
     for (int c = 0; c < 32; c += 2) {
@@ -466,16 +466,16 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     const int xh_count = DKV ? p.Hkv : p.Hq;
     const int b = blockIdx.x / xh_count, xh = blockIdx.x - b * xh_count;
     // heaviest tiles first: under a causal mask early key tiles and late query tiles see the most work
-    const int x0 = ((BS && p.bs_order) ? __ldg(p.bs_order + blockIdx.y)
+    const int x0 = ((BS && p.bs_order) ? ld_global(p.bs_order + blockIdx.y)
                                        : (DKV ? static_cast<int>(blockIdx.y) : static_cast<int>(gridDim.y - 1 - blockIdx.y))) * 128;
     int lo, hi;  // streamed tile range
     if (DKV) qtile_range(ms, x0, lo, hi);
     else tile_range(ms, x0, lo, hi);
     int bs_base = 0;
     if constexpr (BS) {   // block-sparse: positions in the stationary block's list instead of a tile range
-        bs_base = __ldg(p.bs_ptr + x0 / 128);
+        bs_base = ld_global(p.bs_ptr + x0 / 128);
         lo = 0;
-        hi = __ldg(p.bs_ptr + x0 / 128 + 1) - bs_base - 1;
+        hi = ld_global(p.bs_ptr + x0 / 128 + 1) - bs_base - 1;
     }
     const int per_head = hi - lo + 1;
     const int n_it = DKV ? per_head * p.group : per_head;
@@ -483,7 +483,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     auto stream_head = [&](int n) { return DKV ? xh * p.group + n / per_head : xh / p.group; };
     auto stream_row0 = [&](int n) {
         const int pos = lo + (DKV ? n % per_head : n);
-        return (BS ? __ldg(p.bs_idx + bs_base + pos) : pos) * 128;
+        return (BS ? ld_global(p.bs_idx + bs_base + pos) : pos) * 128;
     };
     // The producer and the gradient warpgroups walk the same sequence with a cursor instead: a division and a modulo
     // per tile are some 350 cycles of dependent integer arithmetic each, on the warpgroups' loop-carried chain.
@@ -497,7 +497,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             ++c.head;
         }
     };
-    auto row0_of = [&](const Cursor& c) { return (BS ? __ldg(p.bs_idx + bs_base + lo + c.pos) : lo + c.pos) * 128; };
+    auto row0_of = [&](const Cursor& c) { return (BS ? ld_global(p.bs_idx + bs_base + lo + c.pos) : lo + c.pos) * 128; };
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < L::N_BARS; ++i) {

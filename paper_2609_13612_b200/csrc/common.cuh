@@ -118,7 +118,7 @@ __device__ __forceinline__ void rotate_tile_smem(uint8_t* tile, int row0, int S,
         int r = idx / CP, cp = idx - r * CP;
         int prow = min(row0 + r, S - 1);
         const float4* tb = reinterpret_cast<const float4*>(table + static_cast<size_t>(prow) * half + cp * 8);
-        float4 t0 = __ldg(tb), t1 = __ldg(tb + 1), t2 = __ldg(tb + 2), t3 = __ldg(tb + 3);
+        float4 t0 = ld_global(tb), t1 = ld_global(tb + 1), t2 = ld_global(tb + 2), t3 = ld_global(tb + 3);
         uint4* pl = reinterpret_cast<uint4*>(tile + swz_chunk_offset(r, cp));
         uint4* ph = reinterpret_cast<uint4*>(tile + swz_chunk_offset(r, cp + CP));
         uint4 lo = *pl, hi = *ph;
@@ -157,7 +157,7 @@ __device__ __forceinline__ void rotate_load_step(const float2* table, int S, int
     const float4* tb = reinterpret_cast<const float4*>(table + static_cast<size_t>(S) * (R >> 1) + cp * 8);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const float4 t = __ldg(tb + u);   // {cos0, sin0, cos1, sin1}
+        const float4 t = ld_global(tb + u);   // {cos0, sin0, cos1, sin1}
         step.c[u] = make_float2(t.x, t.z);
         step.s[u] = make_float2(t.y, t.w);
         step.ns[u] = make_float2(-t.y, -t.w);
@@ -172,7 +172,7 @@ __device__ __forceinline__ void rotate_prefetch(RotState<CP>& st, const float2* 
     const float4* tb = reinterpret_cast<const float4*>(table + static_cast<size_t>(prow) * (R >> 1) + cp * 8);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const float4 t = __ldg(tb + u);
+        const float4 t = ld_global(tb + u);
         st.c[u] = make_float2(t.x, t.z);
         st.s[u] = make_float2(t.y, t.w);
     }
@@ -294,7 +294,7 @@ __device__ __forceinline__ void rotate_tile_share(uint8_t* tile, const float2* t
         const float4* tb = reinterpret_cast<const float4*>(table + static_cast<size_t>(prow) * (R >> 1) + cp * 8);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const float4 t = __ldg(tb + u);
+            const float4 t = ld_global(tb + u);
             st.c[u] = make_float2(t.x, t.z);
             st.s[u] = make_float2(t.y, t.w);
         }

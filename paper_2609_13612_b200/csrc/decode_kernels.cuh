@@ -144,8 +144,10 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         prefetch_tmap(&tm_v);
     }
     __syncthreads();
-    grid_dep_launch();   // programmatic dependent launch: the set-up above overlaps with the end of the previous kernel
+    // Programmatic dependent launch: the set-up above overlaps with the end of the previous kernel.  The wait comes before the
+    // signal, so that whatever is launched behind this kernel also finds the kernels before it complete.
     grid_dep_wait();
+    grid_dep_launch();
 
     uint8_t* wbase = smem + warp * L::WARP_BYTES;
     uint64_t* wbar = bars + warp * kDecStages;
@@ -176,8 +178,8 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         const uint32_t* qr = reinterpret_cast<const uint32_t*>(p.q + (static_cast<size_t>(b) * p.Hq + h) * D) + (lane & 3);
 #pragma unroll
         for (int ks = 0; ks < KSTEPS; ++ks) {
-            qb[nt][ks][0] = __ldg(qr + ks * 8);
-            qb[nt][ks][1] = __ldg(qr + ks * 8 + 4);
+            qb[nt][ks][0] = ld_global(qr + ks * 8);
+            qb[nt][ks][1] = ld_global(qr + ks * 8 + 4);
         }
     }
     // this lane's result columns: heads 8 nt + 2 (lane % 4) + {0, 1}
@@ -390,15 +392,15 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         auto load_batch = [&](int s0) {   // (short straight code: every instruction of this part is fetched cold)
 #pragma unroll
             for (int r = 0; r < ROUNDS; ++r)
-                ml[r] = (r * LANES + gl < kDecBatch && s0 + r * LANES + gl < n) ? __ldcg(pm + s0 + r * LANES + gl) : make_float2(-INFINITY, 0.f);
+                ml[r] = (r * LANES + gl < kDecBatch && s0 + r * LANES + gl < n) ? ld_global_cg(pm + s0 + r * LANES + gl) : make_float2(-INFINITY, 0.f);
 #pragma unroll
-            for (int u = 0; u < kDecBatch; ++u) v[u] = __ldcg(po + static_cast<size_t>(min(s0 + u, n - 1)) * D4);
+            for (int u = 0; u < kDecBatch; ++u) v[u] = ld_global_cg(po + static_cast<size_t>(min(s0 + u, n - 1)) * D4);
         };
         load_batch(0);
         float M = ml[0].x;
 #pragma unroll
         for (int r = 1; r < ROUNDS; ++r) M = fmaxf(M, ml[r].x);
-        for (int s = kDecBatch + gl; s < n; s += LANES) M = fmaxf(M, __ldcg(pm + s).x);
+        for (int s = kDecBatch + gl; s < n; s += LANES) M = fmaxf(M, ld_global_cg(pm + s).x);
 #pragma unroll
         for (int off = LANES / 2; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
         const float ref = M == -INFINITY ? 0.f : M;

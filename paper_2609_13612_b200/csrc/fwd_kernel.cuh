@@ -229,12 +229,12 @@ __device__ __forceinline__ bool softmax_tile_general(uint32_t tS, uint32_t tO, i
         float bv[4] = {0.f, 0.f, 0.f, 0.f};
         if (bias_row) {
             if (vec && e4 + 4 <= cols_ok) {
-                const float4 b4 = __ldg(reinterpret_cast<const float4*>(bias_row + e4));
+                const float4 b4 = ld_global(reinterpret_cast<const float4*>(bias_row + e4));
                 bv[0] = b4.x; bv[1] = b4.y; bv[2] = b4.z; bv[3] = b4.w;
             } else {
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    if (e4 + u < cols_ok) bv[u] = __ldg(bias_row + e4 + u);
+                    if (e4 + u < cols_ok) bv[u] = ld_global(bias_row + e4 + u);
             }
         }
 #pragma unroll
@@ -351,8 +351,36 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
     for (int q = 0; q < NQ; ++q) hq[q] = p.pair_heads ? 2 * u + q : u;
     const int hk = hq[0] / p.group;
+    auto init_barriers = [&] {   // warp 0
+        static_assert(L::N_BARS <= 32, "one barrier per lane");
+        if (lane < L::N_BARS) {
+            uint32_t cnt = 1;
+            if ((lane >= L::B_QROT && lane < L::B_QROT + NQ) || (lane >= L::B_KROT && lane < L::B_KROT + KS) ||
+                (lane >= L::B_PREADY && lane < L::B_PREADY + 4 * NQ) || lane == L::B_TEMPTY)
+                cnt = 4;  // one elected arrive per warp of the producing warpgroup
+            mbar_init(&bars[lane], cnt);
+        }
+        if (lane == 0) *abort_flag = 0;
+        fence_mbar_init();
+        __syncwarp();
+    };
+    auto alloc_tmem = [&] {
+        if (warp == 1) {
+            tmem_alloc(tmem_slot, TMEM_COLS);
+            tmem_relinquish();
+        }
+    };
+    // The lists are the caller's device memory: the kernel before this one may still be writing them.  (Their three dependent
+    // reads are the longest part of the set-up, so the rest of it goes in front of the wait.)
+    if constexpr (BS) {
+        if (warp == 0) init_barriers();
+        alloc_tmem();
+        grid_dep_wait();
+    }
+    const int* const row_ptr = BS ? settled(p.bs_row_ptr) : nullptr;
+    const int* const col_idx = BS ? settled(p.bs_col_idx) : nullptr;
     // heaviest row blocks first: the last ones under a causal mask; with block lists the caller's order
-    const int rb = (BS && p.bs_order) ? __ldg(p.bs_order + blockIdx.y) : p.n_row_blocks - 1 - static_cast<int>(blockIdx.y);
+    const int rb = (BS && p.bs_order) ? ld_global(p.bs_order + blockIdx.y) : p.n_row_blocks - 1 - static_cast<int>(blockIdx.y);
     const MaskSpec ms{p.S, p.causal, p.window};
 
     int i0[NQ], jlo[NQ], jhi[NQ];
@@ -381,16 +409,15 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     // Block-sparse: the loops below run over positions in the row block's list (jlo = 0, jhi = length - 1, the
     // same for both query tiles, which share the row block); tile_at() gives the key tile of a position.
-    if constexpr (BS) grid_dep_wait();   // the lists are read here
     int bs_base = 0;
     int last_act[NQ];   // row-pair mode: last list position that is active for query tile q (-1: none)
 #pragma unroll
     for (int q = 0; q < NQ; ++q) last_act[q] = -1;
     const bool rowpair = BS && NQ == 2 && p.bs_rowpair;
     if constexpr (BS) {
-        bs_base = __ldg(p.bs_row_ptr + rb);
+        bs_base = ld_settled(row_ptr + rb);
         const int first_row = rowpair ? rb * NQ * BM : rb * BM;
-        const int len = (first_row < p.S) ? __ldg(p.bs_row_ptr + rb + 1) - bs_base : 0;
+        const int len = (first_row < p.S) ? ld_settled(row_ptr + rb + 1) - bs_base : 0;
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
             jlo[q] = 0;
@@ -400,7 +427,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         jhi_c = len - 1;
         if (rowpair) {
             for (int pos = 0; pos < len; ++pos) {
-                const int ent = __ldg(p.bs_col_idx + bs_base + pos);
+                const int ent = ld_settled(col_idx + bs_base + pos);
 #pragma unroll
                 for (int q = 0; q < NQ; ++q)
                     if ((ent >> (28 + q)) & 1) last_act[q] = pos;
@@ -413,10 +440,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 }
         }
     }
-    auto tile_at = [&](int pos) { return BS ? (__ldg(p.bs_col_idx + bs_base + pos) & 0x0fffffff) : pos; };
+    auto tile_at = [&](int pos) { return BS ? (ld_settled(col_idx + bs_base + pos) & 0x0fffffff) : pos; };
     // is list position / key tile j part of query tile q's work?
     auto active = [&](int q, int j) {
-        if (rowpair) return jhi[q] >= jlo[q] && ((__ldg(p.bs_col_idx + bs_base + j) >> (28 + q)) & 1) != 0;
+        if (rowpair) return jhi[q] >= jlo[q] && ((ld_settled(col_idx + bs_base + j) >> (28 + q)) & 1) != 0;
         return j >= jlo[q] && j <= jhi[q];
     };
     auto is_last = [&](int q, int j) { return rowpair ? j == last_act[q] : j == jhi[q]; };
@@ -434,17 +461,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const bool hybrid = ROPE && !p.rot_k;
     int first_it = 0;   // key tiles requested here already
     if (warp == 0) {
-        static_assert(L::N_BARS <= 32, "one barrier per lane");
-        if (lane < L::N_BARS) {
-            uint32_t cnt = 1;
-            if ((lane >= L::B_QROT && lane < L::B_QROT + NQ) || (lane >= L::B_KROT && lane < L::B_KROT + KS) ||
-                (lane >= L::B_PREADY && lane < L::B_PREADY + 4 * NQ) || lane == L::B_TEMPTY)
-                cnt = 4;  // one elected arrive per warp of the producing warpgroup
-            mbar_init(&bars[lane], cnt);
-        }
-        if (lane == 0) *abort_flag = 0;
-        fence_mbar_init();
-        __syncwarp();
+        if constexpr (!BS) init_barriers();
         if (!hybrid) grid_dep_wait();
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
@@ -471,10 +488,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             }
         }
     }
-    if (warp == 1) {
-        tmem_alloc(tmem_slot, TMEM_COLS);
-        tmem_relinquish();
-    }
+    if constexpr (!BS) alloc_tmem();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();

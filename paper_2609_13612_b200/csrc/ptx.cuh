@@ -159,6 +159,43 @@ __device__ __forceinline__ void prefetch_tmap(const void* tmap) {
 // dependent grid that was launched with that attribute start before this grid has finished.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Loads from global memory that stay behind grid_dep_wait.  __ldg (and a const __restrict__ pointer) promises that nothing writes
+// the data while the kernel runs, which gives the compiler leave to move the load to the front of the kernel, before
+// the wait; and that is where it was seen to move the lists of the block-sparse forward.  Everything that the kernels
+// before this one in the stream may have written is therefore read with these: volatile, in the order written.
+template <typename T>
+__device__ __forceinline__ T ld_words(const uint32_t* w) {
+    T v;
+    memcpy(&v, w, sizeof(T));
+    return v;
+}
+#define AF_LD_GLOBAL(name, op)                                                                                                    \
+    template <typename T>                                                                                                         \
+    __device__ __forceinline__ T name(const T* at) {                                                                              \
+        static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "one load");                                           \
+        uint32_t w[sizeof(T) / 4];                                                                                                \
+        if constexpr (sizeof(T) == 4) asm volatile("ld.global" op ".b32 %0, [%1];" : "=r"(w[0]) : "l"(at));                       \
+        else if constexpr (sizeof(T) == 8) asm volatile("ld.global" op ".v2.b32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(at)); \
+        else asm volatile("ld.global" op ".v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(at)); \
+        return ld_words<T>(w);                                                                                                    \
+    }
+AF_LD_GLOBAL(ld_global, "")
+AF_LD_GLOBAL(ld_global_cs, ".cs")   // read once
+AF_LD_GLOBAL(ld_global_cg, ".cg")   // L2 only: written by other CTAs of this grid
+#undef AF_LD_GLOBAL
+// For data that a loop reads again and again (block lists): `settled` ties a pointer to this point of the program, and
+// ld_settled of such a pointer may be moved and shared by the compiler, but not to before it.  (Block-sparse forward with
+// its lists read by volatile loads: 395 -> 402 us at B = 4, 12 heads, S = 4096, D = 64, all blocks active.)
+template <typename T>
+__device__ __forceinline__ const T* settled(const T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
+__device__ __forceinline__ int ld_settled(const int* at) {
+    int v;
+    asm("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(at));
+    return v;
+}
 
 // ---------------------------------------------------------------- TMEM allocation (one warp, converged)
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_result, uint32_t ncols) {

@@ -46,7 +46,7 @@ __device__ __forceinline__ void rope_apply_heads(long long idx, int h0, const ui
     };
     if (c < CP) {
         const float4* tb = reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * (R >> 1) + c * 8);
-        float4 t0 = __ldg(tb), t1 = __ldg(tb + 1), t2 = __ldg(tb + 2), t3 = __ldg(tb + 3);
+        float4 t0 = ld_global(tb), t1 = ld_global(tb + 1), t2 = ld_global(tb + 2), t3 = ld_global(tb + 3);
         t0.y *= sgn; t0.w *= sgn; t1.y *= sgn; t1.w *= sgn;
         t2.y *= sgn; t2.w *= sgn; t3.y *= sgn; t3.w *= sgn;
         uint4 lo[HPT], hi[HPT];
@@ -54,8 +54,8 @@ __device__ __forceinline__ void rope_apply_heads(long long idx, int h0, const ui
         for (int u = 0; u < HPT; ++u) {
             if (h0 + u < NH) {
                 const size_t base = in_base(h0 + u);
-                lo[u] = __ldcs(x + base + c);
-                hi[u] = __ldcs(x + base + c + CP);
+                lo[u] = ld_global_cs(x + base + c);
+                hi[u] = ld_global_cs(x + base + c + CP);
             }
         }
 #pragma unroll
@@ -76,7 +76,7 @@ __device__ __forceinline__ void rope_apply_heads(long long idx, int h0, const ui
         for (int u = 0; u < HPT; ++u) {
             if (h0 + u < NH) {
                 const size_t base = (static_cast<size_t>(h0 + u) * S + s) * row_chunks;
-                y[base + cc] = __ldcs(x + in_base(h0 + u) + cc);
+                y[base + cc] = ld_global_cs(x + in_base(h0 + u) + cc);
             }
         }
     }
