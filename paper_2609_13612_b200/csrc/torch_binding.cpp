@@ -148,14 +148,17 @@ at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& l
 }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// Runs a C entry point without the interpreter lock (a launch may block while the device's queue is full).
-template <typename F>
-void call(F&& f) {
+// Runs a C entry point without the interpreter lock (a launch may block while the device's queue is full).  The arguments are
+// plain values, evaluated by the caller while it holds the lock: data_ptr() of a tensor without storage throws.
+template <typename... P, typename... A>
+void call(af_status (*entry_point)(P...), A... args) {
     int code;
     {
-        PyThreadState* save = PyEval_SaveThread();
-        code = static_cast<int>(f());
-        PyEval_RestoreThread(save);
+        struct Released {
+            PyThreadState* state = PyEval_SaveThread();
+            ~Released() { PyEval_RestoreThread(state); }
+        } released;
+        code = static_cast<int>(entry_point(args...));
     }
     if (code != 0) raise_status(code, api.strerror_(static_cast<af_status>(code)));
 }
@@ -230,10 +233,8 @@ PyObject* fwd(PyObject* const* a, Py_ssize_t n) {
     Out o(a[7], true, x.q.sizes(), dtype(a[9]), x.q);
     Out l(a[8], truth(a[10]), {x.sh.B, x.sh.Hq, x.sh.S}, at::kFloat, x.q);
     require(o.t.is_contiguous() && (o.t.scalar_type() == at::kBFloat16 || o.t.scalar_type() == at::kFloat), "out: contiguous, bf16 or fp32");
-    call([&] {
-        return api.fwd(&x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale,
-                       o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), stream());
-    });
+    call(api.fwd, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale,
+         o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), stream());
     return pair(o, l);
 }
 
@@ -250,11 +251,8 @@ PyObject* fwd_hybrid(PyObject* const* a, Py_ssize_t n) {
     require(o.t.is_contiguous() && (o.t.scalar_type() == at::kBFloat16 || o.t.scalar_type() == at::kFloat), "out: contiguous, bf16 or fp32");
     const at::Tensor* given = tensor(a[11]);
     const at::Tensor ws = given ? *given : empty({static_cast<int64_t>(api.fwd_hybrid_workspace_bytes(&x.sh))}, at::kByte, x.q);
-    call([&] {
-        return api.fwd_hybrid(&x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group,
-                              scale, o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), ws.data_ptr(),
-                              ws.nbytes(), stream());
-    });
+    call(api.fwd_hybrid, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group,
+         scale, o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), ws.data_ptr(), ws.nbytes(), stream());
     return pair(o, l);
 }
 
@@ -269,10 +267,8 @@ PyObject* fwd_blocks(PyObject* const* a, Py_ssize_t n) {
     const af_blocks bl = blocks_of(a[7], x.sh.S);
     Out o(a[8], true, x.q.sizes(), dtype(a[10]), x.q);
     Out l(a[9], true, {x.sh.B, x.sh.Hq, x.sh.S}, at::kFloat, x.q);
-    call([&] {
-        return api.fwd_blocks(&x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group,
-                              scale, &bl, o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), stream());
-    });
+    call(api.fwd_blocks, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group,
+         scale, &bl, o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), stream());
     return pair(o, l);
 }
 
@@ -290,10 +286,8 @@ PyObject* fwd_fp8(PyObject* const* a, Py_ssize_t n) {
     Out o(Py_None, true, q.sizes(), dtype(a[8]), q);
     Out l(Py_None, true, {B, Hq, S}, at::kFloat, q);
     const af_shape sh = {static_cast<int>(B), static_cast<int>(Hq), static_cast<int>(Hkv), static_cast<int>(S), static_cast<int>(D)};
-    call([&] {
-        return api.fwd_fp8(&sh, q.data_ptr(), k.data_ptr(), v.data_ptr(), &m, Hkv > 0 ? static_cast<int>(Hq / Hkv) : 0, scale, s_q, s_k,
-                           s_v, o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), stream());
-    });
+    call(api.fwd_fp8, &sh, q.data_ptr(), k.data_ptr(), v.data_ptr(), &m, Hkv > 0 ? static_cast<int>(Hq / Hkv) : 0, scale, s_q,
+         s_k, s_v, o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), stream());
     return pair(o, l);
 }
 
@@ -314,17 +308,13 @@ PyObject* bwd(PyObject* const* a, Py_ssize_t n) {
     Out dq(Py_None, true, x.q.sizes(), tq, x.q), dk(Py_None, true, x.k.sizes(), tkv, x.q), dv(Py_None, true, x.k.sizes(), tkv, x.q);
     if (a[13] != Py_None) {
         const af_blocks bl = blocks_of(a[13], x.sh.S);
-        call([&] {
-            return api.bwd_blocks(&x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), o.data_ptr(), static_cast<const float*>(lse.data_ptr()),
-                                  d_o.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale, &bl, dq.data(), out_code(tq),
-                                  dk.data(), dv.data(), out_code(tkv), ws.data_ptr(), ws.numel(), stream());
-        });
+        call(api.bwd_blocks, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), o.data_ptr(),
+             static_cast<const float*>(lse.data_ptr()), d_o.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale, &bl,
+             dq.data(), out_code(tq), dk.data(), dv.data(), out_code(tkv), ws.data_ptr(), ws.numel(), stream());
     } else {
-        call([&] {
-            return api.bwd(&x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), o.data_ptr(), static_cast<const float*>(lse.data_ptr()),
-                           d_o.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale, dq.data(), out_code(tq), dk.data(),
-                           dv.data(), out_code(tkv), ws.data_ptr(), ws.numel(), stream());
-        });
+        call(api.bwd, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), o.data_ptr(),
+             static_cast<const float*>(lse.data_ptr()), d_o.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale,
+             dq.data(), out_code(tq), dk.data(), dv.data(), out_code(tkv), ws.data_ptr(), ws.numel(), stream());
     }
     PyObject* g[3] = {dq.result(), dk.result(), dv.result()};
     PyObject* t = g[0] && g[1] && g[2] ? PyTuple_Pack(3, g[0], g[1], g[2]) : nullptr;
@@ -359,10 +349,8 @@ PyObject* decode(PyObject* const* a, Py_ssize_t n) {
         ws = empty({static_cast<int64_t>(api.decode_workspace_bytes(&sh, n_splits))}, at::kByte, q);
         ws.zero_();
     }
-    call([&] {
-        return api.decode(&sh, q.data_ptr(), k.data_ptr(), v.data_ptr(), &skv, &m, sh.Hkv > 0 ? sh.Hq / sh.Hkv : 0, scale, o.data(),
-                          static_cast<float*>(l.data()), n_splits, ws.data_ptr(), ws.nbytes(), stream());
-    });
+    call(api.decode, &sh, q.data_ptr(), k.data_ptr(), v.data_ptr(), &skv, &m, sh.Hkv > 0 ? sh.Hq / sh.Hkv : 0, scale, o.data(),
+         static_cast<float*>(l.data()), n_splits, ws.data_ptr(), ws.nbytes(), stream());
     return pair(o, l);
 }
 

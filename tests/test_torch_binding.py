@@ -23,6 +23,23 @@ def test_tensors_off_the_device_are_refused(call):
     assert e.value.code == -2
 
 
+def test_tensors_without_storage_raise():
+    """data_ptr() of a fake tensor throws: the exception has to reach the caller (and leave the interpreter lock held)."""
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    with FakeTensorMode():
+        q = torch.empty(1, 2, 128, 128, dtype=torch.bfloat16, device="cuda")
+        lse, codes = torch.empty(1, 2, 128, device="cuda"), torch.empty(1, 2, 128, 128, dtype=torch.uint8, device="cuda")
+        x = dict(out=torch.empty_like(q), lse=lse)
+        calls = [lambda: af.fwd(q, q, q, ROPE, None, MASK, 0.1, **x),
+                 lambda: af.fwd_hybrid(q, q, q, ROPE, None, MASK, 0.1, workspace=codes, **x),
+                 lambda: af.fwd_fp8(codes, codes, codes, MASK, 0.1),
+                 lambda: af.bwd(q, q, q, q, lse, q, ROPE, None, MASK, 0.1, workspace=codes),
+                 lambda: af.decode(q[:, :, 0].contiguous(), q, q, MASK, 0.1, out=q[:, :, 0], lse=lse[:, :, 0], workspace=codes)]
+        for call in calls:
+            with pytest.raises(RuntimeError):
+                call()
+
+
 @pytest.mark.parametrize("bad", [None, 3.0, "q"])
 def test_arguments_of_another_kind_are_refused(bad):
     with pytest.raises(TypeError):
