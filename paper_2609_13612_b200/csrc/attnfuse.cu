@@ -301,8 +301,6 @@ af_status resolve_strides(const af_strides* in, int H, int S, int D, af_strides*
 // grid that leaves SMs idle is better spread out.  Measured with two and one per CTA: 24.1 / 20.2 us (B = 1, 16 / 4 heads,
 // S = 1024: 128 CTAs of one tile), 20.6 / 18.4 us (24 / 8 heads, S = 777: 168), 25.0 / 26.3 us (32 / 8 heads, S = 1024: 256).
 bool one_query_tile(const FwdParams& p) {
-    const int o = opt(AF_OPT_FWD_QTILES);
-    if (o != 2) return o == 1;
     return static_cast<double>(p.B) * p.Hq * ((p.S + BM - 1) / BM) <= 1.2 * sm_count();
 }
 
@@ -362,7 +360,8 @@ af_status launch_fwd_variant(const CUtensorMap& tq, const CUtensorMap& tk, const
     // an even GQA group lets the two query tiles of a CTA be two heads of one kv head (same key range)
     p.pair_heads = (NQ == 2 && (p.group % 2) == 0 && opt(AF_OPT_FWD_PAIR_HEADS)) ? 1 : 0;
     // (measured: +5 % at config 3 with the rotation warps at work, -1 % without them; option value 2 takes it there too)
-    p.alibi_mma = (L::HAS_AX && !GEN && p.slopes && (opt(AF_OPT_FWD_ALIBI_MMA) >= 2 || (ROPE && opt(AF_OPT_FWD_ALIBI_MMA) == 1))) ? 1 : 0;
+    const int alibi_mma = opt(AF_OPT_FWD_ALIBI_MMA);
+    p.alibi_mma = (L::HAS_AX && !GEN && p.slopes && (alibi_mma >= 2 || (ROPE && alibi_mma == 1))) ? 1 : 0;
     const int rows_per_cta = p.pair_heads ? BM : BM * NQ;
     p.n_row_blocks = (p.S + rows_per_cta - 1) / rows_per_cta;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
@@ -394,7 +393,8 @@ af_status launch_fwd_blocks_variant(const CUtensorMap& tq, const CUtensorMap& tk
     // blocks 2 rb and 2 rb + 1 of one head
     p.pair_heads = (NQ == 2 && !p.bs_rowpair) ? 1 : 0;
     // (measured: +5 % at config 3 with the rotation warps at work, -1 % without them; option value 2 takes it there too)
-    p.alibi_mma = (L::HAS_AX && !GEN && p.slopes && (opt(AF_OPT_FWD_ALIBI_MMA) >= 2 || (ROPE && opt(AF_OPT_FWD_ALIBI_MMA) == 1))) ? 1 : 0;
+    const int alibi_mma = opt(AF_OPT_FWD_ALIBI_MMA);
+    p.alibi_mma = (L::HAS_AX && !GEN && p.slopes && (alibi_mma >= 2 || (ROPE && alibi_mma == 1))) ? 1 : 0;
     p.n_row_blocks = (p.S + BM - 1) / BM;
     if (p.bs_rowpair) p.n_row_blocks = (p.n_row_blocks + 1) / 2;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
@@ -402,12 +402,9 @@ af_status launch_fwd_blocks_variant(const CUtensorMap& tq, const CUtensorMap& tk
 }
 template <int D>
 af_status launch_fwd_blocks(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt,
-                            const FwdParams& p, cudaStream_t stream) {
-    // (p.bs_rowpair is set only for an odd GQA group, when the caller supplied the lists of row-block pairs)
-    const bool can_two = (p.group % 2) == 0 || p.bs_rowpair;
-    const bool two_tiles = can_two && (opt(AF_OPT_FWD_QTILES) != 2 || !one_query_tile(p));
+                            const FwdParams& p, bool two_tiles, cudaStream_t stream) {
     if (p.bias || p.relu) {   // Section 3.1 extras: built for CTAs of two query tiles only
-        if (!can_two) return AF_ERR_SPEC;
+        if (!two_tiles) return AF_ERR_SPEC;
         return p.R > 0 ? launch_fwd_blocks_variant<D, 2, true, true>(tq, tk, tv, to, tt, p, stream)
                        : launch_fwd_blocks_variant<D, 2, false, true>(tq, tk, tv, to, tt, p, stream);
     }
@@ -420,11 +417,11 @@ af_status launch_fwd_blocks(const CUtensorMap& tq, const CUtensorMap& tk, const 
 
 template <int D>
 af_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt, const FwdParams& p,
-                     cudaStream_t stream) {
+                     bool two_tiles, cudaStream_t stream) {
     if (p.bias || p.relu)   // Section 3.1 extras (additive_bias, relu_attention): their own instantiation
         return p.R > 0 ? launch_fwd_variant<D, 2, true, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream)
                        : launch_fwd_variant<D, 2, false, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream);
-    if (one_query_tile(p) && !(p.R > 0 && p.keys_bf16 && opt(AF_OPT_FWD_QTILES) == 2)) {
+    if (!two_tiles) {
         return p.R > 0 ? launch_fwd_variant<D, 1, true, 2, 2>(tq, tk, tv, to, tt, p, stream)
                        : launch_fwd_variant<D, 1, false, 2, 2>(tq, tk, tv, to, tt, p, stream);
     }
@@ -889,13 +886,23 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     p.bs_order = bs_order;
     p.bs_rowpair = 0;
     p.splits = 1;
-    if (blocks && (gqa_group % 2) == 1 && blocks->pair_ptr && blocks->pair_idx && opt(AF_OPT_BS_ROWPAIR) &&
-        (bias || relu || opt(AF_OPT_FWD_QTILES) != 2 || !one_query_tile(p))) {
-        // odd GQA group: no two heads share K and V, so a CTA takes two row blocks of one head instead
-        p.bs_row_ptr = blocks->pair_ptr;
-        p.bs_col_idx = blocks->pair_idx;
-        p.bs_order = blocks->pair_order;
-        p.bs_rowpair = 1;
+    // One or two query tiles per CTA, decided here once for the whole call (another thread may set the option meanwhile): the
+    // lists below and the kernel have to agree.
+    const int qtiles = opt(AF_OPT_FWD_QTILES);
+    const bool spread = qtiles == 2 && !bias && !relu && one_query_tile(p);
+    bool two_tiles;
+    if (bs_row_ptr) {
+        two_tiles = (gqa_group % 2) == 0 && !spread;
+        if (blocks && (gqa_group % 2) == 1 && blocks->pair_ptr && blocks->pair_idx && opt(AF_OPT_BS_ROWPAIR) && !spread) {
+            // odd GQA group: no two heads share K and V, so a CTA takes two row blocks of one head instead
+            p.bs_row_ptr = blocks->pair_ptr;
+            p.bs_col_idx = blocks->pair_idx;
+            p.bs_order = blocks->pair_order;
+            p.bs_rowpair = 1;
+            two_tiles = true;
+        }
+    } else {
+        two_tiles = qtiles != 1 && (!spread || (Rr > 0 && keys_bf16));   // (packed-bf16 keys: built for two)
     }
     p.rot_k = k_prerotated ? 0 : 1;
     p.keys_bf16 = keys_bf16 ? 1 : 0;
@@ -909,8 +916,10 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
 #endif
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     if (bs_row_ptr)
-        return shape->D == 128 ? launch_fwd_blocks<128>(tq, tk, tv, to, tt, p, stream) : launch_fwd_blocks<64>(tq, tk, tv, to, tt, p, stream);
-    return shape->D == 128 ? launch_fwd<128>(tq, tk, tv, to, tt, p, stream) : launch_fwd<64>(tq, tk, tv, to, tt, p, stream);
+        return shape->D == 128 ? launch_fwd_blocks<128>(tq, tk, tv, to, tt, p, two_tiles, stream)
+                               : launch_fwd_blocks<64>(tq, tk, tv, to, tt, p, two_tiles, stream);
+    return shape->D == 128 ? launch_fwd<128>(tq, tk, tv, to, tt, p, two_tiles, stream)
+                           : launch_fwd<64>(tq, tk, tv, to, tt, p, two_tiles, stream);
 }
 }  // namespace
 

@@ -165,3 +165,37 @@ def test_bigbird_n4096_forward_and_backward():
     a[0, :] = True
     a[:, 0] = True      # one global block row and column; band of three: (3 * 32 - 2 + 62) / 1024 = 15 %
     run_bwd(w, a)
+
+
+def test_the_query_tiles_option_may_change_while_calls_run():
+    """Lists and kernel are chosen by one reading of the option: every call takes the one or the other way in whole."""
+    import threading
+    q, k, v = (pu.to_dev(synth.draw(W("bs_toggle", 2, 3, 3, 1100, 64, theta=1e4, seed_id=440), n)) for n in "qkv")
+    rope, mask = af.RopeSpec(theta=1e4, rotary_dim=64), af.MaskSpec(causal=False)
+    table = af.rope_table(rope, 1100)
+    bm = af.BlockMask(bigbird_blocks(9, seed=8))
+    call = lambda **kw: af.fwd_blocks(q, k, v, rope, table, mask, 0.125, bm, **kw)
+    want = []
+    for o in (2, 3):
+        with af.option(af.OPT_FWD_QTILES, o):
+            want.append(call()[0])
+    stop = threading.Event()
+
+    def toggle():
+        while not stop.is_set():
+            for o in (2, 3):
+                af.set_option(af.OPT_FWD_QTILES, o)
+    old = af.get_option(af.OPT_FWD_QTILES)
+    t = threading.Thread(target=toggle)
+    t.start()
+    try:
+        outs = []
+        for _ in range(300):
+            out = torch.full_like(want[0], float("nan"))
+            outs.append(call(out=out)[0])
+        torch.cuda.synchronize()
+    finally:
+        stop.set()
+        t.join()
+        af.set_option(af.OPT_FWD_QTILES, old)
+    assert all(torch.equal(o, want[0]) or torch.equal(o, want[1]) for o in outs)
