@@ -300,8 +300,9 @@ af_status resolve_strides(const af_strides* in, int H, int S, int D, af_strides*
 // One query tile per CTA instead of two?  With two, the tiles share every K and V tile and hide each other's latencies, but a
 // grid that leaves SMs idle is better spread out.  Measured with two and one per CTA: 24.1 / 20.2 us (B = 1, 16 / 4 heads,
 // S = 1024: 128 CTAs of one tile), 20.6 / 18.4 us (24 / 8 heads, S = 777: 168), 25.0 / 26.3 us (32 / 8 heads, S = 1024: 256).
+// (The grid of the whole problem counts, also for a launch of a part of it: attnfuse_fwd_host promises the bits of attnfuse_fwd.)
 bool one_query_tile(const FwdParams& p) {
-    return static_cast<double>(p.B) * p.Hq * ((p.S + BM - 1) / BM) <= 1.2 * sm_count();
+    return static_cast<double>(p.heads) * ((p.S + BM - 1) / BM) <= 1.2 * sm_count();
 }
 
 // Tiles of one sequence under a dense mask: the most key tiles (or, the other way round, query tiles) that one tile meets, and
@@ -346,7 +347,7 @@ int cluster_size(double ctas, double longest, double sum, double pair, double ct
 int fwd_splits(const FwdParams& p, int D) {
     double longest, sum;
     tile_counts(p.S, p.causal, p.window, &longest, &sum);
-    const double units = static_cast<double>(p.B) * p.Hq;
+    const double units = static_cast<double>(p.heads);
     return cluster_size(units * ((p.S + BM - 1) / BM), longest, sum * units, D == 128 ? 1.8 : 1.3, 2.0, 4.5, 13.0);
 }
 
@@ -833,7 +834,7 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
                    int gqa_group, float softmax_scale, const int* bs_row_ptr, const int* bs_col_idx,
                    const int* bs_order, void* o, af_dtype o_dtype, float* lse, bool k_prerotated, void* cuda_stream,
                    const af_blocks* blocks = nullptr, const float* bias = nullptr, int bias_B = 1, int bias_H = 1,
-                   int relu = 0) {
+                   int relu = 0, long long all_heads = 0) {   // all_heads: of the whole problem, where this call is a part of one
     af_status st = check_common(shape, rope, rope_table, mask, gqa_group);
     if (st != AF_OK) return st;
     if (!q || !k || !v || !o) return AF_ERR_NULL;
@@ -886,6 +887,7 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     p.bs_order = bs_order;
     p.bs_rowpair = 0;
     p.splits = 1;
+    p.heads = all_heads > 0 ? all_heads : static_cast<long long>(shape->B) * shape->Hq;
     // One or two query tiles per CTA, decided here once for the whole call (another thread may set the option meanwhile): the
     // lists below and the kernel have to agree.
     const int qtiles = opt(AF_OPT_FWD_QTILES);
@@ -1131,9 +1133,10 @@ af_status attnfuse_fwd_host(const af_shape* shape, const void* q_host, const voi
             skv.b = static_cast<int64_t>(shape->Hkv) * shape->S * shape->D;
             // the output of a chunk is contiguous [bn, heads, S, D] only if the chunk covers whole batch elements or
             // a single one; both hold here (bn = 1 when nh < Hkv)
-            st = attnfuse_fwd(&cs, dq + q_off, dk + k_off, dv + k_off, &sq, &skv, rope, rope_table, &cm, gqa_group,
-                              softmax_scale, dob + q_off, AF_BF16, lse_host ? reinterpret_cast<float*>(dl + l_off) : nullptr,
-                              pipe->compute);
+            st = fwd_impl(&cs, dq + q_off, dk + k_off, dv + k_off, &sq, &skv, rope, rope_table, &cm, gqa_group, softmax_scale,
+                          nullptr, nullptr, nullptr, dob + q_off, AF_BF16,
+                          lse_host ? reinterpret_cast<float*>(dl + l_off) : nullptr, false, pipe->compute, nullptr, nullptr, 1, 1,
+                          0, static_cast<long long>(shape->B) * shape->Hq);
             if (st != AF_OK) return st;
             if (cudaEventRecord(e_k, pipe->compute) != cudaSuccess || cudaStreamWaitEvent(pipe->d2h, e_k, 0) != cudaSuccess)
                 return AF_ERR_CUDA;

@@ -47,6 +47,7 @@ struct FwdParams {
     // into two bf16 values, e exact in bf16) - and the softmax warps run their plain straight-line code.
     int alibi_mma;
     int splits;            // SPLIT kernels: CTAs per cluster, the grid's z dimension
+    long long heads;       // host side: heads (B * Hq) of the whole problem, of which this launch may be a part
 #ifdef AF_TRACE
     long long* trace;
 #endif

@@ -174,6 +174,28 @@ def test_forward_from_host_buffers(w):
     assert torch.equal(o_dev.cpu(), ho) and torch.equal(l_dev.cpu(), hl)
 
 
+@pytest.mark.parametrize("w", [
+    W("host_bits_gqa", 1, 32, 8, 1000, 128, theta=5e5, seed_id=145),               # a chunk alone would leave SMs idle
+    W("host_bits_alibi", 1, 16, 8, 1500, 128, theta=1e4, alibi=True, seed_id=146),
+    W("host_bits_noncausal", 2, 16, 8, 700, 64, theta=1e4, causal=False, seed_id=147),
+    W("host_bits_small", 1, 4, 4, 1000, 128, theta=1e4, seed_id=148),              # shared key tiles, in whole and in part
+], ids=lambda w: w.name)
+def test_forward_from_host_buffers_has_the_bits_of_the_device_call(w):
+    """The grid of a chunk is laid out as that of the whole problem."""
+    from paper_2609_13612_b200 import binding
+    dev = {k: pu.to_dev(v) for k, v in synth.draw_all(w).items()}
+    rope, mask = pu.specs(w)
+    table = af.rope_table(rope, w.S)
+    o, lse = af.fwd(dev["q"], dev["k"], dev["v"], rope, table, mask, w.scale)
+    host = {k: dev[k].cpu().pin_memory() for k in "qkv"}
+    ho, hl = torch.empty_like(host["q"]).pin_memory(), torch.empty(w.B, w.Hq, w.S).pin_memory()
+    staging = torch.empty(binding.fwd_host_staging_bytes(w.B, w.Hq, w.Hkv, w.S, w.D), dtype=torch.uint8, device="cuda")
+    af.fwd_host(host["q"], host["k"], host["v"], rope, table, mask, w.scale, ho, hl, staging)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    assert torch.equal(ho, o.cpu()) and torch.equal(hl, lse.cpu())
+
+
 def test_forward_fp32_output():
     run_case(W("fp32_out", 1, 4, 2, 300, 128, theta=1e4, seed_id=120), out_dtype=torch.float32)
 
