@@ -80,9 +80,10 @@ typedef enum {
     AF_OPT_BS_ROWPAIR = 3,     /* AF_BS_ROWPAIR, default 1: block-sparse forward with an odd GQA group gives a CTA two
                                   row blocks of one head when the caller supplied pair lists */
     AF_OPT_BWD_ONEPASS = 4,    /* AF_BWD_ONEPASS, default 1: where the one-pass sequence of attnfuse_bwd applies (workspace
-                                  of attnfuse_bwd_onepass_workspace_bytes) it is taken, since it measured faster
-                                  everywhere (2, kept from when it did not: the same); 0: never - always the two-kernel sequence, whose dQ is
-                                  bit-reproducible */
+                                  of attnfuse_bwd_onepass_workspace_bytes) it is taken where it gains most: always at
+                                  D = 64, at D = 128 when rows are short (at most 12 kept key tiles per query tile on
+                                  average, and not over block lists); 2: whenever it applies (also faster there); 0: never - always the
+                                  two-kernel sequence, whose dQ is bit-reproducible */
     AF_OPT_FWD_ALIBI_MMA = 5,  /* AF_FWD_ALIBI_MMA, default 1: the forward kernel adds the ALiBi term slope (j - i) with one
                                   more K step of the score product (the slope split into two bf16 values, the key column
                                   exact in bf16) instead of one fused multiply-add per score in the softmax warps - in the kernels that rotate

@@ -1270,13 +1270,19 @@ af_status bwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     if ((st = check_arch()) != AF_OK) return st;
     const size_t off_k = bwd_delta_bytes(shape), off_q = off_k + bwd_kcache_bytes(shape);
     const size_t off_acc = off_q + bwd_qcache_bytes(shape);
-    // One-pass sequence: room for both caches and the fp32 dQ' accumulator, and not switched off.
-    // It measured faster than the two-kernel sequence wherever it applies: D = 64 1.2-1.4 times on every shape tried;
-    // D = 128 522 against 622 us at B = 4, 32 / 8 heads, S = 2048, 447 against 487 us at S = 4096, B = 1, 808 against 879 us
-    // at 16 / 4 heads, S = 8192, 428 against 479 us without a causal mask at 16 / 8 heads, S = 4096; over block lists
-    // 684 against 830 us (B = 4, 32 / 8 heads, S = 4096), 84 against 97 us (B = 2, 12 heads, S = 2000), 259 against 370 us
-    // (B = 2, 16 / 4 heads, S = 4096).
-    const bool onepass = !gen && workspace_bytes >= off_acc + bwd_dqacc_bytes(shape) && opt(AF_OPT_BWD_ONEPASS) >= 1;
+    // One-pass sequence: room for both caches and the fp32 dQ' accumulator, and not switched off.  It measured faster than the
+    // two-kernel sequence wherever it applies, but the order of its additions to dQ is not fixed.  So it is the default
+    // where it gains most - at D = 64 (1.2-1.4 times on every shape tried) and on short rows at D = 128 (at most 12 kept
+    // key tiles per query tile on average: 522 against 622 us at B = 4, 32 / 8 heads, S = 2048) - and taken on request only
+    // (AF_OPT_BWD_ONEPASS = 2) on long rows (447 against 487 us at S = 4096, B = 1, 32 / 8 heads; 808 against 879 us at
+    // 16 / 4 heads, S = 8192) and over block lists (684 against 830 us at B = 4, 32 / 8 heads, S = 4096) of D = 128, where dQ has
+    // always come out bit-reproducible by default.
+    const int mode = opt(AF_OPT_BWD_ONEPASS);
+    const double n_tiles = (shape->S + 127) / 128;
+    double avg_tiles = mask->causal ? 0.5 * (n_tiles + 1) : n_tiles;
+    if (mask->window >= 0) avg_tiles = fmin(avg_tiles, (mask->causal ? 1.0 : 2.0) * mask->window / 128.0 + 1.5);
+    const bool onepass = !gen && workspace_bytes >= off_acc + bwd_dqacc_bytes(shape) &&
+                         (mode >= 2 || (mode == 1 && (shape->D == 64 || (!blocks && avg_tiles <= 12.0))));
     const int qrows = onepass ? 64 : 128;   // rows per TMA box of the streamed operands: the one-pass kernel takes half tiles
     CUtensorMap tq, tk, tv, tdo;
     if ((st = make_tmap(&tq, q, shape->B, shape->Hq, shape->S, shape->D, stq, qrows)) != AF_OK) return st;

@@ -234,3 +234,20 @@ def test_both_backward_sequences_on_long_rows_sampled_units(mode):
     torch.cuda.synchronize()
     assert af.device_status()[0] == 0
     _check_units(w, ((0, 1),), t, o, lse, grads, "long rows")
+
+
+@pytest.mark.parametrize("S,blocks", [(4096, False), (1024, True)], ids=["long_rows", "block_lists"])
+def test_gradients_are_reproducible_by_default_at_d128_on_long_rows_and_over_block_lists(S, blocks):
+    """The library by itself takes the two-kernel sequence there, with room for either: no sum in an open order."""
+    w = W("repeat_dq", 1, 8, 2, S, 128, theta=5e5, backward=True, seed_id=234)
+    dev = {k: pu.to_dev(v) for k, v in synth.draw_all(w).items()}
+    rope, mask = pu.specs(w)
+    table = af.rope_table(rope, S)
+    bm = af.BlockMask(np.tril(np.ones((S // 128, S // 128), bool))) if blocks else None
+    o, lse = pu.gpu_fwd(w, dev)
+    runs = [af.bwd(dev["q"], dev["k"], dev["v"], o, lse, dev["do"], rope, table, mask, w.scale, dq_dtype=torch.float32, blocks=bm)
+            for _ in range(6)]
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    for other in runs[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(runs[0], other))
