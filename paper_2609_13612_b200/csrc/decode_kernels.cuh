@@ -394,7 +394,8 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
             for (int r = 0; r < ROUNDS; ++r)
                 ml[r] = (r * LANES + gl < kDecBatch && s0 + r * LANES + gl < n) ? ld_global_cg(pm + s0 + r * LANES + gl) : make_float2(-INFINITY, 0.f);
 #pragma unroll
-            for (int u = 0; u < kDecBatch; ++u) v[u] = ld_global_cg(po + static_cast<size_t>(min(s0 + u, n - 1)) * D4);
+            for (int u = 0; u < kDecBatch; ++u)   // (no row beyond the last: zero, since its weight of zero does not cancel an infinity)
+                v[u] = s0 + u < n ? ld_global_cg(po + static_cast<size_t>(s0 + u) * D4) : make_float4(0.f, 0.f, 0.f, 0.f);
         };
         load_batch(0);
         float M = ml[0].x;

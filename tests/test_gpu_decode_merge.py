@@ -23,3 +23,22 @@ def test_decode_merges(group, Hkv, N, splits, D):
     want_o, want_l = oracle_decode(q, k, v, D ** -0.5)
     pu.assert_close("decode O", pu.to_np(o), want_o)
     assert np.abs(pu.to_np(lse) - want_l).max() <= pu.LSE_TOL
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("splits", [1, 3, 19, 20, 21, 24])
+def test_infinities_of_the_cache_stay_infinities(splits, D):
+    """An infinity in V makes its head dim infinite (its weight is positive), whichever split holds it; the others stay
+    finite."""
+    N = 3000
+    q, k, v = draw(1, 6, 2, N, D, 930)
+    qd, kd, vd = pu.to_dev(q), pu.to_dev(k), pu.to_dev(v)
+    vd[:, :, N - 2, 5] = float("inf")     # last split
+    vd[:, :, 3, 9] = -float("inf")        # first
+    vd[:, :, N // 2, 17] = float("inf")
+    o, lse = af.decode(qd, kd, vd, af.MaskSpec(), 1.0 / 64, n_splits=splits)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0 and torch.isfinite(lse).all()
+    for d in range(D):
+        want = {5: float("inf"), 17: float("inf"), 9: -float("inf")}.get(d)
+        assert torch.isfinite(o[..., d]).all() if want is None else (o[..., d] == want).all(), d
