@@ -98,10 +98,22 @@ const at::Tensor& need(PyObject* o) {
 }
 void* ptr(const at::Tensor* t) { return t ? t->data_ptr() : nullptr; }
 
+// float(o): a number, a one-element tensor, a text
 double number(PyObject* o) {
-    const double r = PyFloat_AsDouble(o);
-    if (r == -1.0 && PyErr_Occurred()) throw Raised();
+    PyObject* f = PyNumber_Float(o);
+    if (!f) throw Raised();
+    const double r = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
     return r;
+}
+// int(o), its low 32 bits: also of a float or a text
+int integer(PyObject* o) {
+    PyObject* l = PyNumber_Long(o);
+    if (!l) throw Raised();
+    const unsigned long r = PyLong_AsUnsignedLongMask(l);
+    Py_DECREF(l);
+    if (r == static_cast<unsigned long>(-1) && PyErr_Occurred()) throw Raised();
+    return static_cast<int>(r);
 }
 at::ScalarType dtype(PyObject* o) {
     if (!THPDtype_Check(o)) raise(PyExc_TypeError, "expected a torch.dtype");
@@ -121,7 +133,7 @@ af_rope rope_of(PyObject* spec) {
 af_mask mask_of(PyObject* spec) {
     af_mask m;
     m.causal = Attr(spec, names.causal).as_bool() ? 1 : 0;
-    m.window = static_cast<int>(Attr(spec, names.window).as_int());
+    m.window = integer(Attr(spec, names.window).v);
     const Attr slopes(spec, names.alibi_slopes);
     const at::Tensor* sl = tensor(slopes.v);
     require(!sl || (sl->scalar_type() == at::kFloat && sl->is_contiguous()), "alibi_slopes: fp32, contiguous");
@@ -272,12 +284,18 @@ PyObject* fwd_blocks(PyObject* const* a, Py_ssize_t n) {
     return pair(o, l);
 }
 
+// 8-bit codes, contiguous; elements of another size are taken as that many codes each
+at::Tensor codes(PyObject* o) {
+    const at::Tensor& t = need(o);
+    at::Tensor c = t.element_size() == 1 ? t : t.view(at::kByte);
+    require(c.is_contiguous() && c.dim() == 4, "q8, k8, vt8: contiguous 4-D tensors of 8-bit codes");
+    return c;
+}
+
 // fwd_fp8(q8, k8, vt8, mask, scale, scale_q, scale_k, scale_v, out_dtype)
 PyObject* fwd_fp8(PyObject* const* a, Py_ssize_t n) {
     check_args(n, 9);
-    const at::Tensor &q = need(a[0]), &k = need(a[1]), &v = need(a[2]);
-    for (const at::Tensor* t : {&q, &k, &v})
-        require(t->element_size() == 1 && t->is_contiguous() && t->dim() == 4, "q8, k8, vt8: contiguous 4-D tensors of 8-bit codes");
+    const at::Tensor q = codes(a[0]), k = codes(a[1]), v = codes(a[2]);
     const int64_t B = q.size(0), Hq = q.size(1), S = q.size(2), D = q.size(3), Hkv = k.size(1);
     require(k.sizes() == at::IntArrayRef({B, Hkv, S, D}) && v.sizes() == at::IntArrayRef({B, Hkv, D, S}), "k8: [B, Hkv, S, D], vt8: [B, Hkv, D, S]");
     const af_mask m = mask_of(a[3]);

@@ -1,4 +1,6 @@
-"""Argument checks of the native side of the Python binding (no GPU needed: nothing here reaches a launch)."""
+"""Arguments of the native side of the Python binding: what it refuses (no GPU needed: nothing there reaches a launch) and what
+it accepts."""
+import numpy as np
 import pytest
 import torch
 
@@ -44,3 +46,19 @@ def test_tensors_without_storage_raise():
 def test_arguments_of_another_kind_are_refused(bad):
     with pytest.raises(TypeError):
         af.fwd(bad, CPU, CPU, ROPE, None, MASK, 0.1)
+
+
+@pytest.mark.gpu
+def test_numbers_and_codes_of_other_types_are_accepted():
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, k, v = (torch.randn(1, 2, 400, 64, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    want = af.fwd(q, k, v, ROPE, None, af.MaskSpec(window=300), 0.125)
+    for window, scale in ((300.0, 0.125), ("300", "0.125"), (torch.tensor(300), torch.tensor(0.125)), (np.float32(300), np.float64(0.125))):
+        got = af.fwd(q, k, v, ROPE, None, af.MaskSpec(window=window), scale)
+        assert all(torch.equal(x, y) for x, y in zip(got, want))
+    codes = [torch.randn(*s, generator=g, device="cuda").to(torch.float8_e4m3fn) for s in ((1, 2, 400, 128), (1, 2, 400, 128), (1, 2, 128, 400))]
+    want = af.fwd_fp8(*codes, MASK, 0.1)
+    for dt in (torch.uint8, torch.int8, torch.int16, torch.int32, torch.bfloat16):
+        got = af.fwd_fp8(*(c.view(dt) for c in codes), MASK, "0.1", scale_q=1)
+        assert all(torch.equal(x, y) for x, y in zip(got, want)), dt
+    assert af.device_status()[0] == 0
