@@ -298,11 +298,33 @@ af_status resolve_strides(const af_strides* in, int H, int S, int D, af_strides*
 }
 
 // One query tile per CTA instead of two?  With two, the tiles share every K and V tile and hide each other's latencies, but a
-// grid that leaves SMs idle is better spread out.  Measured with two and one per CTA: 24.1 / 20.2 us (B = 1, 16 / 4 heads,
-// S = 1024: 128 CTAs of one tile), 20.6 / 18.4 us (24 / 8 heads, S = 777: 168), 25.0 / 26.3 us (32 / 8 heads, S = 1024: 256).
+// grid that leaves SMs idle is better spread out: 24.1 / 20.2 us with two and one per CTA (B = 1, 16 / 4 heads, S = 1024:
+// 128 tiles), 25.0 / 26.3 us (32 / 8 heads, S = 1024: 256 tiles).
+// Up to one tile per SM the answer is yes.  A little beyond, some SMs get two CTAs one after the other, which is fine where those
+// are the short ones of a causal mask (20.6 / 18.4 us, 24 / 8 heads, S = 777: 168 tiles) and costs half as much again where
+// all are alike (26.2 / 38.0 us, 20 / 4 heads, S = 1024, no causal mask: 160; 21.9 / 27.1 us, one head, S = 20480, window
+// 300).  There the longest chain decides, in us: a CTA with n key tiles takes c1 + n t1 with one query tile and c2 + n t2 with
+// two (fitted to 118 measured grids of 100 to 177 tiles; it picks the faster way in all of them).  The lengths of block
+// lists are not known here.
 // (The grid of the whole problem counts, also for a launch of a part of it: attnfuse_fwd_host promises the bits of attnfuse_fwd.)
-bool one_query_tile(const FwdParams& p) {
-    return static_cast<double>(p.heads) * ((p.S + BM - 1) / BM) <= 1.2 * sm_count();
+bool one_query_tile(const FwdParams& p, int D) {
+    const int sms = sm_count(), rows = (p.S + BM - 1) / BM;
+    const double tiles = static_cast<double>(p.heads) * rows;
+    if (tiles <= sms) return true;
+    if (tiles > 1.2 * sms || p.bs_row_ptr) return false;
+    auto length = [&](int row) {   // key tiles of a row block
+        const int hi = p.causal ? row : (p.window >= 0 ? (row * BM + BM - 1 + p.window) / BN : rows - 1);
+        const int lo = p.window >= 0 && row * BM > p.window ? (row * BM - p.window) / BN : 0;
+        return (hi < rows - 1 ? hi : rows - 1) - lo + 1;
+    };
+    int longest = 0;
+    for (int r = 0; r < rows; ++r) longest = length(r) > longest ? length(r) : longest;
+    const double t1 = D == 128 ? 1.75 : 1.47, c1 = D == 128 ? 4.9 : 4.0, t2 = D == 128 ? 2.23 : 1.88, c2 = D == 128 ? 8.4 : 7.0;
+    // launched last row blocks first: the last tile of the first wave, and the one that follows it on its SM
+    const int heads = static_cast<int>(p.heads);
+    const double pair = 2 * c1 + t1 * (length(rows - 1 - (sms - 1) / heads) + length(rows - 1 - sms / heads));
+    const double one = c1 + t1 * longest;
+    return (one > pair ? one : pair) < c2 + t2 * longest;
 }
 
 // Tiles of one sequence under a dense mask: the most key tiles (or, the other way round, query tiles) that one tile meets, and
@@ -891,7 +913,7 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     // One or two query tiles per CTA, decided here once for the whole call (another thread may set the option meanwhile): the
     // lists below and the kernel have to agree.
     const int qtiles = opt(AF_OPT_FWD_QTILES);
-    const bool spread = qtiles == 2 && !bias && !relu && one_query_tile(p);
+    const bool spread = qtiles == 2 && !bias && !relu && one_query_tile(p, shape->D);
     bool two_tiles;
     if (bs_row_ptr) {
         two_tiles = (gqa_group % 2) == 0 && !spread;

@@ -43,3 +43,28 @@ def test_shared_key_tiles(w, out_dtype):
 def test_forward_small_two_query_tiles_per_cta(w):
     with af.option(af.OPT_FWD_QTILES, 3):
         run_case(w)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,S,causal,window,same_as", [
+    (1, 20, 4, 1024, True, -1, 1),     # 160 tiles: the CTAs that follow others on an SM are the short ones
+    (1, 20, 4, 1024, False, -1, 3),    # all alike: two waves of one tile would be slower than one of two
+    (1, 2, 2, 10752, True, 300, 3),
+    (1, 160, 8, 128, True, -1, 3),
+    (1, 18, 6, 1024, False, -1, 1),    # 144 tiles: one wave either way
+])
+def test_query_tiles_per_cta_on_grids_a_little_larger_than_the_device(B, Hq, Hkv, S, causal, window, same_as):
+    """The choice shows in the bits: with ALiBi the kernels for one and for two query tiles add the term in different places."""
+    g = torch.Generator(device="cuda").manual_seed(808)
+    q, k, v = (torch.randn(B, h, S, 128, generator=g, device="cuda").to(torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    slopes = torch.tensor([2.0 ** (-8.0 * (h + 1) / Hq) for h in range(Hq)], device="cuda")
+    rope, mask = af.RopeSpec(theta=1e4, rotary_dim=128), af.MaskSpec(causal=causal, window=window, alibi_slopes=slopes)
+    table = af.rope_table(rope, S)
+    got = {}
+    for option in (1, 2, 3):
+        with af.option(af.OPT_FWD_QTILES, option):
+            got[option] = af.fwd(q, k, v, rope, table, mask, 128 ** -0.5)[1]
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:   # the line lies at the number of SMs
+        assert not torch.equal(got[1], got[3])
+        assert torch.equal(got[2], got[same_as])
