@@ -716,8 +716,14 @@ template <int D, int NT>
 af_status launch_decode(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t stream) {
     static std::atomic<unsigned long long> configured{0};
     if (allow_dynamic_smem(decode_split_kernel<D, NT>, DecodeSmem<D>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
+    // A dependent launch saves about 1 us.  Behind a grid that streams for long it costs more: its CTAs wait on the SMs that come
+    // free first, and the next grid then streams more slowly from where they sit (641 against 604 us with a plain launch at
+    // B = 16, 8 kv heads, 65536 keys, D = 128: 33.6 MB per CTA; 166 / 159 us at 8.4 MB; 54.6 / 54.6 us at 2.6 MB; with 1 MB
+    // and less it is 1 to 8 % faster).
+    const double kept = p.window >= 0 && p.window < p.N ? p.window + 1 : p.N;
+    const bool dependent = kept / p.n_splits * D * 4 <= 4e6;
     return launch_kernel(decode_split_kernel<D, NT>, dim3(p.n_splits, p.B * p.Hkv, 1), dim3(kDecWarps * 32, 1, 1),
-                         DecodeSmem<D>::BYTES, stream, true, tk, tv, p);
+                         DecodeSmem<D>::BYTES, stream, dependent, tk, tv, p);
 }
 
 size_t bwd_delta_bytes(const af_shape* sh) {

@@ -42,3 +42,14 @@ def test_infinities_of_the_cache_stay_infinities(splits, D):
     for d in range(D):
         want = {5: float("inf"), 17: float("inf"), 9: -float("inf")}.get(d)
         assert torch.isfinite(o[..., d]).all() if want is None else (o[..., d] == want).all(), d
+
+
+@pytest.mark.parametrize("D,N", [(128, 7812), (128, 7813), (64, 15626)])   # 4 MB of keys and values per CTA: dependent or plain launch
+def test_long_splits(D, N):
+    q, k, v = draw(1, 2, 1, N, D, 940)
+    o, lse = af.decode(pu.to_dev(q), pu.to_dev(k), pu.to_dev(v), af.MaskSpec(), D ** -0.5, n_splits=1)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    want_o, want_l = oracle_decode(q, k, v, D ** -0.5)
+    pu.assert_close("decode O", pu.to_np(o), want_o)
+    assert np.abs(pu.to_np(lse) - want_l).max() <= pu.LSE_TOL
