@@ -59,7 +59,7 @@ typedef struct { float theta; int rotary_dim; int pos_offset; } af_rope;
  * the scaled score. */
 typedef struct { int causal; int window; const float* alibi_slopes; } af_mask;
 
-int         attnfuse_version(void);   /* 100 x major + minor: 110 adds the variant, one-pass backward and fp8 entries */
+int         attnfuse_version(void);   /* 100 x major + minor: 110 adds the variant, one-pass backward and fp8 entries, 111 the list lengths of af_blocks */
 const char* attnfuse_strerror(af_status st);
 
 /* ---- tuning options ---------------------------------------------------------------------------------
@@ -186,6 +186,11 @@ typedef struct {
     const int* pair_ptr;
     const int* pair_idx;
     const int* pair_order;
+    /* Optional (0 = not known): the longest list by key block and the number of listed blocks, which the caller knows when
+     * it builds the lists.  With them the one-pass backward shares out long lists over several CTAs where that is
+     * faster; without them (or with values that no lists of nb blocks can have) a key block is one CTA's work. */
+    int col_longest;
+    int listed;
 } af_blocks;
 
 /* attnfuse_fwd over the listed blocks. */

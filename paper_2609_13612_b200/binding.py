@@ -37,7 +37,7 @@ class _Blocks(ctypes.Structure):
     _fields_ = [("block", ctypes.c_int), ("row_ptr", ctypes.c_void_p), ("col_idx", ctypes.c_void_p),
                 ("col_ptr", ctypes.c_void_p), ("row_idx", ctypes.c_void_p), ("row_order", ctypes.c_void_p),
                 ("col_order", ctypes.c_void_p), ("pair_ptr", ctypes.c_void_p), ("pair_idx", ctypes.c_void_p),
-                ("pair_order", ctypes.c_void_p)]
+                ("pair_order", ctypes.c_void_p), ("col_longest", ctypes.c_int), ("listed", ctypes.c_int)]
 
 
 class _Variant(ctypes.Structure):
@@ -375,6 +375,7 @@ def fwd_hybrid(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: Rop
 class BlockMask:
     """Active 128 x 128 blocks of a block-sparse mask (Section 4.3) as device index lists: CSR by query row
     block and CSC by key block.  Built once from a boolean [nb, nb] matrix (nb = ceil(S / 128))."""
+    col_longest, listed = 0, 0   # not known (an object restored from before they were kept)
 
     def __init__(self, active, device="cuda"):
         a = torch.as_tensor(active).to(torch.bool).cpu()
@@ -388,6 +389,7 @@ class BlockMask:
         counts_t = at.sum(1).to(torch.int32)
         self.col_ptr = torch.cat([torch.zeros(1, dtype=torch.int32), counts_t.cumsum(0).to(torch.int32)]).to(device)
         self.row_idx = at.nonzero()[:, 1].to(torch.int32).contiguous().to(device)
+        self.col_longest, self.listed = int(counts_t.max()) if self.nb else 0, int(counts_t.sum())
         # launch orders: longest lists first
         self.row_order = torch.argsort(counts, descending=True, stable=True).to(torch.int32).to(device)
         self.col_order = torch.argsort(counts_t, descending=True, stable=True).to(torch.int32).to(device)
@@ -411,7 +413,7 @@ class BlockMask:
     def struct(self):
         return _Blocks(128, self.row_ptr.data_ptr(), self.col_idx.data_ptr(), self.col_ptr.data_ptr(),
                        self.row_idx.data_ptr(), self.row_order.data_ptr(), self.col_order.data_ptr(),
-                       self.pair_ptr.data_ptr(), self.pair_idx.data_ptr(), self.pair_order.data_ptr())
+                       self.pair_ptr.data_ptr(), self.pair_idx.data_ptr(), self.pair_order.data_ptr(), self.col_longest, self.listed)
 
 
 def fwd_blocks(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: RopeSpec, table: Optional[torch.Tensor],

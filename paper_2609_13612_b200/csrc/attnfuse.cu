@@ -569,14 +569,16 @@ af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMa
 // and dV over distributed shared memory).
 // Measured, whole backward, 1 / 2 / 4 / 8 CTAs: 52 / 38 / 36 / 43 us (B = 2, 6 q / 2 kv heads, S = 777, window 300, D = 128),
 // 129 / 76 / 65 / 65 us (B = 2, 16 / 2 heads, S = 596), 124 / 188 / 232 / 288 us (B = 4, 16 heads, S = 1024).
-// The lengths of block lists are not known here.  They are taken to be those of a pattern with one global key block and
-// four query blocks for each other key block: 449 / 260 / 247 / 319 us (B = 2, 16 / 4 heads, S = 4096, D = 128, such a list).
-int onepass_splits(int D, int units, int S, int group, int causal, int window, bool blocks) {
+// Over block lists the caller's figures stand for the counts: with them the estimate is within 1.25 times of the fastest of
+// the four on 164 measured cases (7 patterns, D = 64 and 128), and never slower than one CTA.  A wrong figure costs more (256
+// key tiles with a diagonal and its neighbours, D = 64: 35 us with 1 CTA, 59 us with 2), so without figures it is 1.
+int onepass_splits(int D, int units, int S, int group, int causal, int window, const af_blocks* blocks) {
     const int tiles = (S + 127) / 128;
     double longest, sum;   // query tiles that see a key tile
     if (blocks) {
-        longest = tiles;
-        sum = tiles + 4.0 * (tiles - 1);
+        longest = blocks->col_longest;
+        sum = blocks->listed;
+        if (longest < 1 || longest > tiles || sum < longest || sum > longest * tiles) return 1;
     } else {
         tile_counts(S, causal, window, &longest, &sum);
     }
@@ -624,7 +626,7 @@ af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CU
     p.bs_ptr = a.blocks ? a.blocks->col_ptr : nullptr;
     p.bs_idx = a.blocks ? a.blocks->row_idx : nullptr;
     p.bs_order = a.blocks ? a.blocks->col_order : nullptr;
-    const int splits = onepass_splits(D, sh->B * sh->Hkv, sh->S, p.group, p.causal, p.window, a.blocks != nullptr);
+    const int splits = onepass_splits(D, sh->B * sh->Hkv, sh->S, p.group, p.causal, p.window, a.blocks);
     auto kern = a.blocks ? (splits > 1 ? attn_bwd_fused_kernel<D, true, true> : attn_bwd_fused_kernel<D, true, false>)
                          : (splits > 1 ? attn_bwd_fused_kernel<D, false, true> : attn_bwd_fused_kernel<D, false, false>);
     static std::atomic<unsigned long long> configured[4];
@@ -743,7 +745,7 @@ size_t bwd_dqacc_bytes(const af_shape* sh) {
 
 extern "C" {
 
-int attnfuse_version(void) { return 110; }
+int attnfuse_version(void) { return 111; }
 
 const char* attnfuse_strerror(af_status st) {
     switch (st) {

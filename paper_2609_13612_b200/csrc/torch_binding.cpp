@@ -37,7 +37,7 @@ PyObject* error_class = nullptr;
 // attribute names, interned once
 struct Names {
     PyObject *theta, *rotary_dim, *pos_offset, *causal, *window, *alibi_slopes, *nb, *row_ptr, *col_idx, *col_ptr, *row_idx,
-        *row_order, *col_order, *pair_ptr, *pair_idx, *pair_order;
+        *row_order, *col_order, *pair_ptr, *pair_idx, *pair_order, *col_longest, *listed;
 } names;
 
 struct Raised {};   // a Python exception is set
@@ -148,7 +148,8 @@ af_blocks blocks_of(PyObject* mask, int64_t S) {
     require(Attr(mask, names.nb).as_int() == (S + 127) / 128, "block mask of another sequence length");
     return {128, index_list(mask, names.row_ptr), index_list(mask, names.col_idx), index_list(mask, names.col_ptr),
             index_list(mask, names.row_idx), index_list(mask, names.row_order), index_list(mask, names.col_order),
-            index_list(mask, names.pair_ptr), index_list(mask, names.pair_idx), index_list(mask, names.pair_order)};
+            index_list(mask, names.pair_ptr), index_list(mask, names.pair_idx), index_list(mask, names.pair_order),
+            integer(Attr(mask, names.col_longest).v), integer(Attr(mask, names.listed).v)};
 }
 
 af_strides strides_of(const at::Tensor& t) {
@@ -434,6 +435,7 @@ PyMODINIT_FUNC PyInit__torch_binding(void) {
     auto intern = [](const char* s) { return PyUnicode_InternFromString(s); };
     names = {intern("theta"),   intern("rotary_dim"), intern("pos_offset"), intern("causal"),    intern("window"),   intern("alibi_slopes"),
              intern("nb"),      intern("row_ptr"),    intern("col_idx"),    intern("col_ptr"),   intern("row_idx"),  intern("row_order"),
-             intern("col_order"), intern("pair_ptr"), intern("pair_idx"),   intern("pair_order")};
+             intern("col_order"), intern("pair_ptr"), intern("pair_idx"),   intern("pair_order"), intern("col_longest"),
+             intern("listed")};
     return PyModule_Create(&module);
 }

@@ -199,3 +199,23 @@ def test_the_query_tiles_option_may_change_while_calls_run():
         t.join()
         af.set_option(af.OPT_FWD_QTILES, old)
     assert all(torch.equal(o, want[0]) or torch.equal(o, want[1]) for o in outs)
+
+
+@pytest.mark.parametrize("known", [True, False], ids=["lengths", "no_lengths"])
+@pytest.mark.parametrize("pattern", ["band", "global"])
+def test_one_pass_backward_with_and_without_the_list_lengths(pattern, known):
+    """The lengths only say how many CTAs share a key block's list (2 and 4 for these two), and without them it is one."""
+    w = W("bsb_lengths", 1, 8, 2, 2048, 64, theta=1e4, causal=False, backward=True, seed_id=441)
+    a = bigbird_blocks(16, window=1, n_global=1 if pattern == "global" else 0, n_random=0, seed=9)
+    t, dev, o, lse, bm = run_fwd(w, a)
+    assert bm.col_longest == (16 if pattern == "global" else 3) and bm.listed == a.sum()
+    if not known:
+        del bm.col_longest, bm.listed
+    rope, mask = pu.specs(w)
+    table = af.rope_table(rope, w.S)
+    got = af.bwd(dev["q"], dev["k"], dev["v"], o, lse, dev["do"], rope, table, mask, w.scale, blocks=bm)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    want = oracle.bwd(t["q"], t["k"], t["v"], t["do"], theta=w.theta, rotary_dim=w.R, causal=False, scale=w.scale, blocks=a, block_size=128)
+    for name, x, ref in zip(("dQ", "dK", "dV"), got, want):
+        pu.assert_close("%s %s" % (w.name, name), pu.to_np(x), ref)
