@@ -548,6 +548,13 @@ af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CU
                              int dq_f32, void* dk, void* dv, int dkv_f32, float* delta, const FirstRowsParams& fp,
                              const OnePassArgs& a, cudaStream_t stream);
 
+// The one-pass kernel runs the first query rows in a further row of its own grid when dK and dV are fp32 (and the grid has room
+// for one more).
+constexpr unsigned kMaxGridY = 65535;
+bool first_rows_in_grid(const FirstRowsParams& fp, int dkv_f32) {
+    return fp.rows > 0 && dkv_f32 && static_cast<unsigned>((fp.S + 127) / 128) < kMaxGridY;
+}
+
 template <int D>
 af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                      const CUtensorMap& tdo, const CUtensorMap* tkp, const CUtensorMap* tqp, const void* k,
@@ -560,8 +567,7 @@ af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMa
                                          dk, dv, dkv_f32, delta, fp, *onepass, stream)
                  : launch_bwd_mma<D>(sh, tq, tk, tv, tdo, tkp, tqp, k, stkv, kcache, o, d_o, p, dq, dq_f32, dk, dv,
                                      dkv_f32, delta, blocks, stream);
-    // (the one-pass kernel runs them in its own grid when dK and dV are fp32)
-    if (st != AF_OK || fp.rows == 0 || (onepass && dkv_f32)) return st;
+    if (st != AF_OK || fp.rows == 0 || (onepass && first_rows_in_grid(fp, dkv_f32))) return st;
     return launch_first_rows<D>(fp, stream);
 }
 
@@ -592,7 +598,6 @@ struct OnePassArgs {
     af_strides stq;
     void* qcache;
     float* dq_acc;
-    size_t dq_acc_bytes;
     const af_blocks* blocks;   // block-sparse lists or nullptr
 };
 template <int D>
@@ -602,7 +607,7 @@ af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CU
                              int dq_f32, void* dk, void* dv, int dkv_f32, float* delta, const FirstRowsParams& fp,
                              const OnePassArgs& a, cudaStream_t stream) {
     using L = BwdFusedSmem<D>;
-    const bool first = fp.rows > 0 && dkv_f32;   // the first query rows in the one-pass kernel's own grid
+    const bool first = first_rows_in_grid(fp, dkv_f32);
     BwdPrologueParams pp = {};
     pp.R = p.R;
     pp.table = p.table;
@@ -639,8 +644,8 @@ af_status launch_bwd_onepass(const af_shape* sh, const CUtensorMap& tq, const CU
     if (st != AF_OK) return st;
     const long long fthreads = static_cast<long long>(sh->S) * (D / 8);
     const int nh = sh->B * sh->Hq;
-    const unsigned fy = static_cast<unsigned>((nh + kFinishHeads - 1) / kFinishHeads);
-    if (fy > 65535) return AF_ERR_SHAPE;
+    unsigned fy = static_cast<unsigned>((nh + kFinishHeads - 1) / kFinishHeads);
+    if (fy > kMaxGridY) fy = kMaxGridY;   // (the kernel goes on from there)
     return launch_kernel(bwd_dq_finish_kernel<D>, dim3(static_cast<unsigned>((fthreads + 255) / 256), fy, 1), dim3(256, 1, 1), 0,
                          stream, true, static_cast<const float*>(a.dq_acc), dq, dq_f32, p.table, nh, sh->S, p.R, p.scale, first ? fp.rows : 0);
 }
@@ -1368,7 +1373,6 @@ af_status bwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     OnePassArgs op = {};
     op.q = q; op.stq = stq; op.qcache = qc;
     op.dq_acc = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + off_acc);
-    op.dq_acc_bytes = bwd_dqacc_bytes(shape);
     op.blocks = blocks;
     p.dq_acc = nullptr;
     return shape->D == 128

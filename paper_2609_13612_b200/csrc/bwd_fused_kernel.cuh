@@ -641,42 +641,44 @@ __global__ void __launch_bounds__(256) bwd_dq_finish_kernel(const float* __restr
     const long long idx = blockIdx.x * 256ll + threadIdx.x;
     const int s = static_cast<int>(idx / SPR), c = static_cast<int>(idx % SPR);
     if (s >= S || s < skip_rows) return;
-    const int half = R >> 1, rslots = R >> 3, h0 = blockIdx.y * kFinishHeads;
+    const int half = R >> 1, rslots = R >> 3;
     const bool rot = c < rslots;
     const int d0 = rot ? 4 * c : R + 8 * (c - rslots), d1 = rot ? d0 + half : d0 + 4;
-    float4 a[kFinishHeads], b[kFinishHeads];
+    for (int h0 = blockIdx.y * kFinishHeads; h0 < NH; h0 += gridDim.y * kFinishHeads) {   // (more than 4 x 65535 heads: again)
+        float4 a[kFinishHeads], b[kFinishHeads];
 #pragma unroll
-    for (int u = 0; u < kFinishHeads; ++u)
-        if (h0 + u < NH) {
-            const float* row = acc + (static_cast<size_t>(h0 + u) * S + s) * D;
-            a[u] = ld_global_cs(reinterpret_cast<const float4*>(row + d0));
-            b[u] = ld_global_cs(reinterpret_cast<const float4*>(row + d1));
-        }
-    float4 cs = make_float4(scale, scale, scale, scale), sn = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (rot) {
-        const float4 t01 = ld_global(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0));
-        const float4 t23 = ld_global(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0 + 2));
-        cs = make_float4(t01.x * scale, t01.z * scale, t23.x * scale, t23.z * scale);
-        sn = make_float4(t01.y * scale, t01.w * scale, t23.y * scale, t23.w * scale);
-    }
-#pragma unroll
-    for (int u = 0; u < kFinishHeads; ++u)
-        if (h0 + u < NH) {
-            // transpose rotation: a c + b s below R / 2, b c - a s above
-            const float4 y0 = make_float4(fmaf(a[u].x, cs.x, b[u].x * sn.x), fmaf(a[u].y, cs.y, b[u].y * sn.y),
-                                          fmaf(a[u].z, cs.z, b[u].z * sn.z), fmaf(a[u].w, cs.w, b[u].w * sn.w));
-            const float4 y1 = make_float4(fmaf(b[u].x, cs.x, -a[u].x * sn.x), fmaf(b[u].y, cs.y, -a[u].y * sn.y),
-                                          fmaf(b[u].z, cs.z, -a[u].z * sn.z), fmaf(b[u].w, cs.w, -a[u].w * sn.w));
-            const size_t row = (static_cast<size_t>(h0 + u) * S + s) * D;
-            if (out_f32) {
-                *reinterpret_cast<float4*>(static_cast<float*>(out) + row + d0) = y0;
-                *reinterpret_cast<float4*>(static_cast<float*>(out) + row + d1) = y1;
-            } else {
-                __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + row;
-                *reinterpret_cast<uint2*>(o + d0) = make_uint2(pack_bf16x2(y0.x, y0.y), pack_bf16x2(y0.z, y0.w));
-                *reinterpret_cast<uint2*>(o + d1) = make_uint2(pack_bf16x2(y1.x, y1.y), pack_bf16x2(y1.z, y1.w));
+        for (int u = 0; u < kFinishHeads; ++u)
+            if (h0 + u < NH) {
+                const float* row = acc + (static_cast<size_t>(h0 + u) * S + s) * D;
+                a[u] = ld_global_cs(reinterpret_cast<const float4*>(row + d0));
+                b[u] = ld_global_cs(reinterpret_cast<const float4*>(row + d1));
             }
+        float4 cs = make_float4(scale, scale, scale, scale), sn = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (rot) {
+            const float4 t01 = ld_global(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0));
+            const float4 t23 = ld_global(reinterpret_cast<const float4*>(table + static_cast<size_t>(s) * half + d0 + 2));
+            cs = make_float4(t01.x * scale, t01.z * scale, t23.x * scale, t23.z * scale);
+            sn = make_float4(t01.y * scale, t01.w * scale, t23.y * scale, t23.w * scale);
         }
+#pragma unroll
+        for (int u = 0; u < kFinishHeads; ++u)
+            if (h0 + u < NH) {
+                // transpose rotation: a c + b s below R / 2, b c - a s above
+                const float4 y0 = make_float4(fmaf(a[u].x, cs.x, b[u].x * sn.x), fmaf(a[u].y, cs.y, b[u].y * sn.y),
+                                              fmaf(a[u].z, cs.z, b[u].z * sn.z), fmaf(a[u].w, cs.w, b[u].w * sn.w));
+                const float4 y1 = make_float4(fmaf(b[u].x, cs.x, -a[u].x * sn.x), fmaf(b[u].y, cs.y, -a[u].y * sn.y),
+                                              fmaf(b[u].z, cs.z, -a[u].z * sn.z), fmaf(b[u].w, cs.w, -a[u].w * sn.w));
+                const size_t row = (static_cast<size_t>(h0 + u) * S + s) * D;
+                if (out_f32) {
+                    *reinterpret_cast<float4*>(static_cast<float*>(out) + row + d0) = y0;
+                    *reinterpret_cast<float4*>(static_cast<float*>(out) + row + d1) = y1;
+                } else {
+                    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + row;
+                    *reinterpret_cast<uint2*>(o + d0) = make_uint2(pack_bf16x2(y0.x, y0.y), pack_bf16x2(y0.z, y0.w));
+                    *reinterpret_cast<uint2*>(o + d1) = make_uint2(pack_bf16x2(y1.x, y1.y), pack_bf16x2(y1.z, y1.w));
+                }
+            }
+    }
 }
 
 }  // namespace af

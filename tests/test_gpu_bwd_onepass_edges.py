@@ -47,3 +47,44 @@ def test_key_tiles_shared_out_over_a_cluster(B, Hkv, group, S, D, causal, window
         pu.assert_close_scaled("%s %s" % (w.name, name), pu.to_np(g), ref)
     # the sums over the cluster run in rank order
     assert torch.equal(got[1], again[1]) and torch.equal(got[2], again[2])
+
+
+def test_more_heads_than_a_grid_dimension_takes_in_groups():
+    """The last pass of dQ takes the heads in groups of four along y (at most 65535)."""
+    B, H, S, D = 4, 65540, 8, 64
+    g = torch.Generator(device="cuda").manual_seed(811)
+    q, k, v, do = (torch.randn(B, H, S, D, generator=g, device="cuda").to(torch.bfloat16) for _ in range(4))
+    rope, mask = af.RopeSpec(), af.MaskSpec()
+    o, lse = af.fwd(q, k, v, rope, None, mask, 0.125)
+    got = af.bwd(q, k, v, o, lse, do, rope, None, mask, 0.125)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    for b in range(B):
+        qf, kf, vf = (t[b].float().requires_grad_() for t in (q, k, v))
+        s = (qf @ kf.transpose(1, 2) * 0.125).masked_fill(torch.ones(S, S, device="cuda").triu(1).bool(), float("-inf"))
+        (torch.softmax(s, -1) @ vf).backward(do[b].float())
+        for x, ref in zip(got, (qf.grad, kf.grad, vf.grad)):
+            # (a bf16 dQ is off by half an ulp, 2^-9 of its value)
+            assert ((x[b].float() - ref).abs() <= 2e-2 + pu.BF16_ULP * ref.abs()).all()
+
+
+def test_as_many_key_tiles_as_a_grid_dimension_takes():
+    """65535 key tiles: no row of the grid is left for the first query rows.  With a window the rows of a slice of the sequence
+    are those of the whole, away from its ends."""
+    S, D, W_, M = 65535 * 128, 64, 100, 1024
+    g = torch.Generator(device="cuda").manual_seed(812)
+    q, k, v, do = (torch.randn(1, 1, S, D, generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(4))
+    rope, mask = af.RopeSpec(), af.MaskSpec(window=W_)
+
+    def run(a, b):
+        x = [t[:, :, a:b].contiguous() for t in (q, k, v, do)]
+        o, lse = af.fwd(x[0], x[1], x[2], rope, None, mask, 0.125)
+        return (o,) + af.bwd(x[0], x[1], x[2], o, lse, x[3], rope, None, mask, 0.125)
+    whole = run(0, S)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    for a in (0, S // 2 // 128 * 128, S - M):
+        lo, hi = (0 if a == 0 else 2 * W_), (M if a + M == S else M - 2 * W_)
+        for x, y in zip(whole, run(a, a + M)):
+            x, y = x[:, :, a + lo:a + hi].float(), y[:, :, lo:hi].float()
+            assert torch.isfinite(x).all() and ((x - y).abs() <= 2e-2 + pu.BF16_ULP * y.abs()).all()
