@@ -385,8 +385,17 @@ __device__ __forceinline__ void grad_pass32_general(uint32_t t1, uint32_t t2, in
     tmem_ld32(t1 + col0, s);
     tmem_ld32(t2 + col0, dp);
     float bv[32];
+    // (dQ: the columns are adjacent; one decision for the warp, where lanes past the end of the sequence have no row)
+    if (!DKV && __all_sync(0xffffffffu, !bias || (cols_ok >= 32 && (reinterpret_cast<uintptr_t>(bias) & 15u) == 0))) {
 #pragma unroll
-    for (int c = 0; c < 32; ++c) bv[c] = (bias && c < cols_ok) ? ld_global(bias + c * col_stride) : 0.f;
+        for (int c = 0; c < 32; c += 4) {
+            const float4 b4 = bias ? ld_global(reinterpret_cast<const float4*>(bias + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            bv[c] = b4.x; bv[c + 1] = b4.y; bv[c + 2] = b4.z; bv[c + 3] = b4.w;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) bv[c] = (bias && c < cols_ok) ? ld_global(bias + c * col_stride) : 0.f;
+    }
     tmem_wait_ld();
 #pragma unroll
     for (int c = 0; c < 32; c += 2) {
@@ -465,6 +474,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     // stationary tile: DKV -> key tile of kv head (b, hk); DQ -> query tile of head (b, h)
     const int xh_count = DKV ? p.Hkv : p.Hq;
     const int b = blockIdx.x / xh_count, xh = blockIdx.x - b * xh_count;
+    // (the lists may be read in front of the wait: the set-up pass, which precedes this kernel, has waited for their writers)
+    const int* const bs_ptr = BS ? settled(p.bs_ptr) : nullptr;
+    const int* const bs_idx = BS ? settled(p.bs_idx) : nullptr;
     // heaviest tiles first: under a causal mask early key tiles and late query tiles see the most work
     const int x0 = ((BS && p.bs_order) ? ld_global(p.bs_order + blockIdx.y)
                                        : (DKV ? static_cast<int>(blockIdx.y) : static_cast<int>(gridDim.y - 1 - blockIdx.y))) * 128;
@@ -473,9 +485,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     else tile_range(ms, x0, lo, hi);
     int bs_base = 0;
     if constexpr (BS) {   // block-sparse: positions in the stationary block's list instead of a tile range
-        bs_base = ld_global(p.bs_ptr + x0 / 128);
+        bs_base = ld_settled(bs_ptr + x0 / 128);
         lo = 0;
-        hi = ld_global(p.bs_ptr + x0 / 128 + 1) - bs_base - 1;
+        hi = ld_settled(bs_ptr + x0 / 128 + 1) - bs_base - 1;
     }
     const int per_head = hi - lo + 1;
     const int n_it = DKV ? per_head * p.group : per_head;
@@ -483,7 +495,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     auto stream_head = [&](int n) { return DKV ? xh * p.group + n / per_head : xh / p.group; };
     auto stream_row0 = [&](int n) {
         const int pos = lo + (DKV ? n % per_head : n);
-        return (BS ? ld_global(p.bs_idx + bs_base + pos) : pos) * 128;
+        return (BS ? ld_settled(bs_idx + bs_base + pos) : pos) * 128;
     };
     // The producer and the gradient warpgroups walk the same sequence with a cursor instead: a division and a modulo
     // per tile are some 350 cycles of dependent integer arithmetic each, on the warpgroups' loop-carried chain.
@@ -497,7 +509,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             ++c.head;
         }
     };
-    auto row0_of = [&](const Cursor& c) { return (BS ? ld_global(p.bs_idx + bs_base + lo + c.pos) : lo + c.pos) * 128; };
+    auto row0_of = [&](const Cursor& c) { return (BS ? ld_settled(bs_idx + bs_base + lo + c.pos) : lo + c.pos) * 128; };
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < L::N_BARS; ++i) {
@@ -526,6 +538,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     grid_dep_launch();
     AF_BSTAMP(5, 0, 0);
 
+    // (bias / relu, dK and dV) The general pass holds 32 scores, 32 dP, 32 biases and two rows of results at once, too much for
+    // 128 registers: 80 + 40 + 2 x 192 of the 512 take 110 instead of 117 us at 8 / 4 heads, S = 1000, D = 128 (dQ: slower).
+    constexpr bool kMoreRegs = GEN && DKV;
+    if constexpr (kMoreRegs) {
+        if (warp < 4) setmaxnreg_dec<80>();
+    }
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (elect_one()) {
@@ -655,6 +673,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
         }
     } else if (warp >= 4 && warp < 8) {
         // ------------------------------------------------------------ rotation warpgroup: X once, every A tile
+        if constexpr (kMoreRegs) setmaxnreg_dec<40>();
         if (ROT_A) {
             const int t = threadIdx.x - 128;
             auto run = [&](auto cp_tag) {
@@ -690,6 +709,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
         }
     } else if (warp >= 8) {
         // ------------------------------------------------------------ gradient warpgroups (one TMEM lane per thread)
+        if constexpr (kMoreRegs) setmaxnreg_inc<192>();
         const int gtid = threadIdx.x - 256;          // 0..255 over both warpgroups
         const int hf = gtid >> 7;                    // column half owned by this warpgroup
         const int tid = gtid & 127;                  // == TMEM lane
