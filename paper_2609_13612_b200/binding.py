@@ -164,10 +164,15 @@ def _load_native():
     global _native
     L = lib()
     if _native is None:
+        from .build import BINDING, abi_tag
         try:
             from . import _torch_binding
         except ImportError as e:
-            raise AttnFuseError(-1, "_torch_binding.so is not built (%s); run `python -m paper_2609_13612_b200.build`" % e)
+            raise AttnFuseError(-1, "_torch_binding.so %s (%s); run `python -m paper_2609_13612_b200.build`" % (
+                "does not load" if os.path.exists(BINDING) else "is not built", e))
+        if _torch_binding.ABI_TAG != abi_tag():
+            raise AttnFuseError(-1, "_torch_binding.so was %s, this is %s; run `python -m paper_2609_13612_b200.build`" % (
+                _torch_binding.ABI_TAG, abi_tag()[len("built for "):]))
         _bind(_torch_binding, L)
         _native = _torch_binding   # (last: another thread may call through it as soon as it is set)
     return _native

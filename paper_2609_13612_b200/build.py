@@ -4,6 +4,7 @@ from __future__ import annotations
 import glob
 import os
 import subprocess
+import sys
 import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -27,10 +28,23 @@ def is_stale() -> bool:
     return any(os.path.getmtime(s) > t for s in _sources())
 
 
+def abi_tag() -> str:
+    """What the native binding depends on: it is built for one Python and one torch."""
+    import torch
+    return "built for Python %d.%d, torch %s" % (sys.version_info[0], sys.version_info[1], torch.__version__)
+
+
+def binding_is_stale() -> bool:
+    deps = [BINDING_SRC, os.path.join(os.path.dirname(PKG), "include", "attnfuse.h")]
+    if not os.path.exists(BINDING) or any(os.path.getmtime(d) > os.path.getmtime(BINDING) for d in deps):
+        return True
+    with open(BINDING, "rb") as f:
+        return abi_tag().encode() + b"\0" not in f.read()
+
+
 def build_binding(force: bool = False) -> str:
     """The native side of the Python binding: a CPython module over torch's C++ headers, host code only."""
-    deps = [BINDING_SRC, os.path.join(os.path.dirname(PKG), "include", "attnfuse.h")]
-    if not force and os.path.exists(BINDING) and all(os.path.getmtime(d) <= os.path.getmtime(BINDING) for d in deps):
+    if not force and not binding_is_stale():
         return BINDING
     import torch
     root = os.path.dirname(os.path.abspath(torch.__file__))
@@ -39,7 +53,7 @@ def build_binding(force: bool = False) -> str:
            sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
     tmp = BINDING + ".tmp.%d" % os.getpid()
     subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++20", "-shared", "-fPIC", "-fvisibility=hidden",
-                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] +
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), '-DAF_ABI_TAG="%s"' % abi_tag()] +
                           ["-isystem" + d for d in inc] + ["-o", tmp, BINDING_SRC, "-L" + os.path.join(root, "lib"),
                            "-Wl,-rpath," + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
     os.replace(tmp, BINDING)

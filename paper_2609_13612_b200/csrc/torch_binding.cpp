@@ -437,5 +437,7 @@ PyMODINIT_FUNC PyInit__torch_binding(void) {
              intern("nb"),      intern("row_ptr"),    intern("col_idx"),    intern("col_ptr"),   intern("row_idx"),  intern("row_order"),
              intern("col_order"), intern("pair_ptr"), intern("pair_idx"),   intern("pair_order"), intern("col_longest"),
              intern("listed")};
-    return PyModule_Create(&module);
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "ABI_TAG", AF_ABI_TAG) < 0) Py_CLEAR(m);
+    return m;
 }

@@ -62,3 +62,13 @@ def test_numbers_and_codes_of_other_types_are_accepted():
         got = af.fwd_fp8(*(c.view(dt) for c in codes), MASK, "0.1", scale_q=1)
         assert all(torch.equal(x, y) for x, y in zip(got, want)), dt
     assert af.device_status()[0] == 0
+
+
+def test_a_binding_built_for_another_torch_is_stale(monkeypatch):
+    from paper_2609_13612_b200 import binding, build
+    assert not build.binding_is_stale() and binding._load_native().ABI_TAG == build.abi_tag()
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert build.binding_is_stale()
+    monkeypatch.setattr(binding, "_native", None)
+    with pytest.raises(af.AttnFuseError, match="torch 0.0.1"):
+        binding._load_native()
