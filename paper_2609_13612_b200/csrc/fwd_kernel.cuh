@@ -813,7 +813,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int e = 0; e < 32; e += 4) *reinterpret_cast<uint4*>(row_p + c * 32 + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
             }
             *reinterpret_cast<float2*>(row_p + D) = make_float2(m_run, l_run);
-        } else if (ok && jhi[q] >= jlo[q]) {
+        } else if (!(SPLIT && parts > 1) && jhi[q] >= jlo[q]) {
             tc_fence_after_sync();
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
             const size_t orow = (static_cast<size_t>(bh) * p.S + i) * D;
@@ -823,50 +823,43 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 // (Row-per-thread global stores touch 32 rows per instruction and kept the load/store unit busy
                 // for ~4 k cycles per CTA.)  Rows past S are clipped by the tensor map.
                 // Box by box (64 columns), so that one is on its way out while the next is converted.
+                // (A warp whose wait gave up takes the barriers all the same: the others must not be left alone there.)
                 uint8_t* stg = sQ + q * TILE;
 #pragma unroll 1
                 for (int bx = 0; bx < NBOX; ++bx) {
-                    uint32_t v[64];
-                    tmem_ld32(tO + bx * 64, v);
-                    tmem_ld32(tO + bx * 64 + 32, v + 32);
-                    tmem_wait_ld();
+                    if (ok) {
+                        uint32_t v[64];
+                        tmem_ld32(tO + bx * 64, v);
+                        tmem_ld32(tO + bx * 64 + 32, v + 32);
+                        tmem_wait_ld();
 #pragma unroll
-                    for (int e = 0; e < 64; e += 8)
-                        *reinterpret_cast<uint4*>(stg + swz_chunk_offset(row, bx * 8 + (e >> 3))) = make_uint4(
-                            pack_bf16x2(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv),
-                            pack_bf16x2(__uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv),
-                            pack_bf16x2(__uint_as_float(v[e + 4]) * inv, __uint_as_float(v[e + 5]) * inv),
-                            pack_bf16x2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv));
-                    fence_proxy_async_smem();
+                        for (int e = 0; e < 64; e += 8)
+                            *reinterpret_cast<uint4*>(stg + swz_chunk_offset(row, bx * 8 + (e >> 3))) = make_uint4(
+                                pack_bf16x2(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv),
+                                pack_bf16x2(__uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv),
+                                pack_bf16x2(__uint_as_float(v[e + 4]) * inv, __uint_as_float(v[e + 5]) * inv),
+                                pack_bf16x2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv));
+                        fence_proxy_async_smem();
+                    }
                     asm volatile("bar.sync %0, 128;" ::"r"(4 + q) : "memory");   // this warpgroup only
-                    if (row == 0) {
+                    if (ok && row == 0) {
                         tma_store_4d(&tm_o, stg + bx * BOX_BYTES, bx * BOX_COLS, i0[q], hq[q], b);
                         tma_store_commit();
                     }
                 }
-                if (row == 0) tma_store_wait_read();   // the buffer must stay in place until it has been read
-            }
+                if (ok && row == 0) tma_store_wait_read();   // the buffer must stay in place until it has been read
+            } else if (ok) {
 #pragma unroll 1
-            for (int c = 0; p.o_f32 && c < D / 32; ++c) {
-                uint32_t v[32];
-                tmem_ld32(tO + c * 32, v);
-                tmem_wait_ld();
-                if (i < p.S) {
-                    if (p.o_f32) {
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t v[32];
+                    tmem_ld32(tO + c * 32, v);
+                    tmem_wait_ld();
+                    if (i < p.S) {
                         float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.o) + orow + c * 32);
 #pragma unroll
                         for (int e = 0; e < 32; e += 4)
                             dst[e >> 2] = make_float4(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv,
                                                       __uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv);
-                    } else {
-                        uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.o) + orow + c * 32);
-#pragma unroll
-                        for (int e = 0; e < 32; e += 8)
-                            dst[e >> 3] = make_uint4(
-                                pack_bf16x2(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv),
-                                pack_bf16x2(__uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv),
-                                pack_bf16x2(__uint_as_float(v[e + 4]) * inv, __uint_as_float(v[e + 5]) * inv),
-                                pack_bf16x2(__uint_as_float(v[e + 6]) * inv, __uint_as_float(v[e + 7]) * inv));
                     }
                 }
             }
