@@ -65,11 +65,21 @@ def test_block_sparse_forward(w, pattern):
     run_fwd(w, pattern((w.S + 127) // 128))
 
 
-def test_block_sparse_row_blocks_without_active_blocks_give_zero_rows():
+@pytest.mark.parametrize("w,pattern", FWD_CASES, ids=lambda x: x.name if hasattr(x, "name") else "")
+def test_block_sparse_forward_two_query_tiles_per_cta(w, pattern):
+    """Grids as small as these take one query tile per CTA by themselves; larger ones the kernels for two (pairs of heads,
+    pairs of row blocks)."""
+    with af.option(af.OPT_FWD_QTILES, 3):
+        run_fwd(w, pattern((w.S + 127) // 128))
+
+
+@pytest.mark.parametrize("qtiles", [2, 3])
+def test_block_sparse_row_blocks_without_active_blocks_give_zero_rows(qtiles):
     w = W("bs_empty_rows", 1, 4, 2, 512, 128, theta=1e4, causal=False, seed_id=410)
     a = np.zeros((4, 4), dtype=bool)
     a[0, 1] = a[2, 0] = a[2, 3] = True          # row blocks 1 and 3 have nothing
-    t, dev, o, lse, _ = run_fwd(w, a)
+    with af.option(af.OPT_FWD_QTILES, qtiles):
+        t, dev, o, lse, _ = run_fwd(w, a)
     assert torch.all(o[:, :, 128:256] == 0) and torch.all(torch.isneginf(lse[:, :, 128:256]))
 
 
@@ -81,15 +91,22 @@ def test_block_sparse_row_pairs_of_one_head():
     a = np.tril(bigbird_blocks(nb, seed=7, causal=True))
     a[3, :] = False           # row block 3 (second of pair 1) has nothing
     a[6, :] = a[7, :] = False   # pair 3 has nothing
-    t, dev, o, lse, _ = run_fwd(w, a)
+    with af.option(af.OPT_FWD_QTILES, 3):   # (by itself a grid of 54 tiles takes one row block per CTA)
+        t, dev, o, lse, _ = run_fwd(w, a)
     for r in (3, 6, 7):
         assert torch.all(o[:, :, 128 * r:128 * (r + 1)] == 0) and torch.all(torch.isneginf(lse[:, :, 128 * r:128 * (r + 1)]))
 
 
+def test_block_sparse_row_pairs_by_default_on_a_large_grid():
+    """Odd group, D = 64, 252 tiles: more than one per SM, so pairs of row blocks without being asked."""
+    w = W("bs_rowpair_default", 3, 7, 7, 1500, 64, theta=1e4, causal=False, seed_id=413)
+    run_fwd(w, bigbird_blocks(12, seed=18))
+
+
 @pytest.mark.parametrize("w,pattern", [FWD_CASES[4], FWD_CASES[5]], ids=lambda x: x.name if hasattr(x, "name") else "")
 def test_block_sparse_forward_one_row_block_per_cta(w, pattern):
-    """The same odd-group cases without the pair lists (one query tile per CTA)."""
-    with af.option(af.OPT_BS_ROWPAIR, 0):
+    """The odd-group cases where two query tiles per CTA are asked for but the pair lists may not be used."""
+    with af.option(af.OPT_BS_ROWPAIR, 0), af.option(af.OPT_FWD_QTILES, 3):
         run_fwd(w, pattern((w.S + 127) // 128))
 
 

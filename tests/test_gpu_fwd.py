@@ -80,15 +80,17 @@ def test_forward_alibi_in_the_softmax_warps(w):
     """ALiBi has two implementations in the forward kernel: by default one more K step of the score product adds
     slope (j - i) (run by every other ALiBi case of this suite); with the option off the softmax warps add it,
     one fused multiply-add per score.  Both are held to the oracle."""
-    with af.option(af.OPT_FWD_ALIBI_MMA, 0):
-        run_case(w)
+    for qtiles in (2, 3):   # one query tile per CTA (grids as small as these) and two
+        with af.option(af.OPT_FWD_ALIBI_MMA, 0), af.option(af.OPT_FWD_QTILES, qtiles):
+            run_case(w)
 
 
 @pytest.mark.parametrize("w", ALIBI_CASES, ids=lambda w: w.name)
 def test_forward_alibi_by_the_tensor_core(w):
     assert af.get_option(af.OPT_FWD_ALIBI_MMA) == 1   # the default: in the kernels that rotate on chip
-    with af.option(af.OPT_FWD_ALIBI_MMA, 2):          # here: also without RoPE
-        run_case(w)
+    for qtiles in (2, 3):
+        with af.option(af.OPT_FWD_ALIBI_MMA, 2), af.option(af.OPT_FWD_QTILES, qtiles):   # here: also without RoPE
+            run_case(w)
 
 
 @pytest.mark.parametrize("w", SMALL[3:8], ids=lambda w: w.name)
@@ -101,7 +103,7 @@ def test_forward_small_one_query_tile_per_cta(w):
 def test_forward_small_row_block_pairs(w):
     """Even GQA groups with head pairing switched off: the two query tiles of a work item are consecutive row
     blocks of one head, with different key ranges."""
-    with af.option(af.OPT_FWD_PAIR_HEADS, 0):
+    with af.option(af.OPT_FWD_PAIR_HEADS, 0), af.option(af.OPT_FWD_QTILES, 3):
         run_case(w)
 
 
