@@ -14,7 +14,11 @@
  *    reported by return code; nothing throws or aborts.
  *  - Device-side waits are bounded.  A wait that runs out makes the kernel return early and
  *    records a code that attnfuse_device_status() reports; outputs of that launch are undefined.
- *  - Run-to-run deterministic, except the one-pass backward's dQ, whose fp32 partial sums are reduced in no fixed order.
+ *  - Run-to-run deterministic, except the one-pass backward's dQ, whose fp32 partial sums are reduced in no fixed order
+ *    (see AF_OPT_BWD_ONEPASS for where that sequence is the default).  The last bits of a result may depend on the other heads
+ *    and batch elements of the call: the number of heads decides how a grid is laid out, i.e. which sums are split.
+ *  - Every kernel that starts as a programmatic dependent of the kernel before it in the stream waits for that kernel to
+ *    complete before it reads or writes memory of the caller's that the kernel may be using.
  */
 #ifndef ATTNFUSE_H_
 #define ATTNFUSE_H_
@@ -294,7 +298,8 @@ af_status attnfuse_fwd_host(const af_shape* shape, const void* q_host, const voi
  * rows need 16-byte alignment and strides that are multiples of 8 elements); lse (nullable): [B,Hq] fp32.
  * gqa_group <= 16; D in {64, 128}.  n_splits <= 0: attnfuse_decode_splits(shape), the largest count that keeps the
  * grid of n_splits x B x Hkv CTAs within one CTA per SM of the current device (one wave) with at least 128 keys
- * per split, and one split for up to 640 keys.  Larger requests are clamped to that many per kept (not windowed
+ * per split, but of more than 20 no more than pay for their merge (a bound that grows with the square root of D x S: 74 for one
+ * kv head, 20000 keys, D = 128), and one split for up to 640 keys.  Larger requests are clamped to that many per kept (not windowed
  * away) keys and to 256 splits.
  * workspace: attnfuse_decode_workspace_bytes(shape, n_splits) device bytes: a ticket counter per (batch, kv head)
  * at its head, then the partials.  Both phases run in ONE launch: the CTA that finishes last for a kv head merges

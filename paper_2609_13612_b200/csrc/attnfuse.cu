@@ -575,8 +575,8 @@ af_status launch_bwd(const af_shape* sh, const CUtensorMap& tq, const CUtensorMa
 // and dV over distributed shared memory).
 // Measured, whole backward, 1 / 2 / 4 / 8 CTAs: 52 / 38 / 36 / 43 us (B = 2, 6 q / 2 kv heads, S = 777, window 300, D = 128),
 // 129 / 76 / 65 / 65 us (B = 2, 16 / 2 heads, S = 596), 124 / 188 / 232 / 288 us (B = 4, 16 heads, S = 1024).
-// Over block lists the caller's figures stand for the counts: with them the estimate is within 1.25 times of the fastest of
-// the four on 164 measured cases (7 patterns, D = 64 and 128), and never slower than one CTA.  A wrong figure costs more (256
+// Over block lists the caller's figures stand for the counts: with them the estimate is within 1.4 times of the fastest of
+// the four on 164 measured cases (7 patterns, D = 64 and 128), and at most 5 % slower than one CTA.  A wrong figure costs more (256
 // key tiles with a diagonal and its neighbours, D = 64: 35 us with 1 CTA, 59 us with 2), so without figures it is 1.
 int onepass_splits(int D, int units, int S, int group, int causal, int window, const af_blocks* blocks) {
     const int tiles = (S + 127) / 128;

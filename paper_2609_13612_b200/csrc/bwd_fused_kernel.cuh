@@ -19,7 +19,7 @@
 // The streamed operands have one full and one empty barrier per half tile, Q' and dO apart: with whole stages that
 // both issuers hand back, S^T of the next tile sat 1-2 k cycles per tile pair on a load that could only be requested
 // after the last dK' product of the tile before (D = 128, where shared memory holds two stages).
-// What bounds it at D = 128 (5.6 k cycles per tile pair; the five products take 2.6 k): the gradient phases, which
+// What bounds it at D = 128 (5.0-5.2 k cycles per tile pair; the five products take 2.6 k): the gradient phases, which
 // take 1.5 k cycles each for 32 columns per thread because their shared-memory accesses queue behind the reductions to
 // global memory (512 per tile pair, 26 cycles each per sub-partition; without them the backward is 1.17 times faster,
 // with stores in their place 1.02 times).  Measured and not kept: whole-tile products with N = 128 and a read-out of
