@@ -373,10 +373,10 @@ int fwd_splits(const FwdParams& p, int D) {
     return cluster_size(units * ((p.S + BM - 1) / BM), longest, sum * units, D == 128 ? 1.8 : 1.3, 2.0, 4.5, 13.0);
 }
 
-template <int D, int NQ, bool ROPE, int KS, int VS, bool TAB = false, bool GEN = false>
+template <int D, int NQ, int ROPE, int KS, int VS, bool TAB = false, bool GEN = false>
 af_status launch_fwd_variant(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt,
                              FwdParams p, cudaStream_t stream) {
-    using L = FwdSmem<D, NQ, KS, VS, ROPE && TAB>;
+    using L = FwdSmem<D, NQ, KS, VS, ROPE == kRotAll && TAB>;
     auto kern = attn_fwd_kernel<D, NQ, ROPE, KS, VS, false, TAB, GEN>;
     static std::atomic<unsigned long long> configured{0};
     if (allow_dynamic_smem(kern, L::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
@@ -396,16 +396,16 @@ af_status launch_fwd_variant(const CUtensorMap& tq, const CUtensorMap& tk, const
             static std::atomic<unsigned long long> configured_shared{0};
             if (allow_dynamic_smem(shared, L::BYTES, configured_shared) != AF_OK) return AF_ERR_CUDA;
             grid.z = p.splits;
-            return launch_cluster(shared, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, p.splits, tq, tk, tv, to,
+            return launch_cluster(shared, grid, dim3(fwd_threads(NQ, ROPE), 1, 1), L::BYTES, stream, true, p.splits, tq, tk, tv, to,
                                   tt, p);
         }
     }
-    return launch_kernel(kern, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
+    return launch_kernel(kern, grid, dim3(fwd_threads(NQ, ROPE), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
 }
 
 // Block-sparse variant (Section 4.3): the grid is (heads or head pairs, 128-row blocks); every CTA walks the
 // list of active key blocks of its row block.  An even GQA group pairs two heads per CTA, otherwise one head.
-template <int D, int NQ, bool ROPE, bool GEN = false>
+template <int D, int NQ, int ROPE, bool GEN = false>
 af_status launch_fwd_blocks_variant(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                     const CUtensorMap& to, const CUtensorMap& tt, FwdParams p, cudaStream_t stream) {
     using L = FwdSmem<D, NQ, 2, 2>;
@@ -421,36 +421,36 @@ af_status launch_fwd_blocks_variant(const CUtensorMap& tq, const CUtensorMap& tk
     p.n_row_blocks = (p.S + BM - 1) / BM;
     if (p.bs_rowpair) p.n_row_blocks = (p.n_row_blocks + 1) / 2;
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
-    return launch_kernel(kern, grid, dim3(128 * (2 + NQ), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
+    return launch_kernel(kern, grid, dim3(fwd_threads(NQ, ROPE), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
 }
 template <int D>
 af_status launch_fwd_blocks(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt,
                             const FwdParams& p, bool two_tiles, cudaStream_t stream) {
     if (p.bias || p.relu) {   // Section 3.1 extras: built for CTAs of two query tiles only
         if (!two_tiles) return AF_ERR_SPEC;
-        return p.R > 0 ? launch_fwd_blocks_variant<D, 2, true, true>(tq, tk, tv, to, tt, p, stream)
-                       : launch_fwd_blocks_variant<D, 2, false, true>(tq, tk, tv, to, tt, p, stream);
+        return p.R > 0 ? launch_fwd_blocks_variant<D, 2, kRotAll, true>(tq, tk, tv, to, tt, p, stream)
+                       : launch_fwd_blocks_variant<D, 2, kRotNone, true>(tq, tk, tv, to, tt, p, stream);
     }
     if (two_tiles)
-        return p.R > 0 ? launch_fwd_blocks_variant<D, 2, true>(tq, tk, tv, to, tt, p, stream)
-                       : launch_fwd_blocks_variant<D, 2, false>(tq, tk, tv, to, tt, p, stream);
-    return p.R > 0 ? launch_fwd_blocks_variant<D, 1, true>(tq, tk, tv, to, tt, p, stream)
-                   : launch_fwd_blocks_variant<D, 1, false>(tq, tk, tv, to, tt, p, stream);
+        return p.R > 0 ? launch_fwd_blocks_variant<D, 2, kRotAll>(tq, tk, tv, to, tt, p, stream)
+                       : launch_fwd_blocks_variant<D, 2, kRotNone>(tq, tk, tv, to, tt, p, stream);
+    return p.R > 0 ? launch_fwd_blocks_variant<D, 1, kRotAll>(tq, tk, tv, to, tt, p, stream)
+                   : launch_fwd_blocks_variant<D, 1, kRotNone>(tq, tk, tv, to, tt, p, stream);
 }
 
 template <int D>
 af_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, const CUtensorMap& tt, const FwdParams& p,
                      bool two_tiles, cudaStream_t stream) {
     if (p.bias || p.relu)   // Section 3.1 extras (additive_bias, relu_attention): their own instantiation
-        return p.R > 0 ? launch_fwd_variant<D, 2, true, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream)
-                       : launch_fwd_variant<D, 2, false, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream);
-    if (!two_tiles) {
-        return p.R > 0 ? launch_fwd_variant<D, 1, true, 2, 2>(tq, tk, tv, to, tt, p, stream)
-                       : launch_fwd_variant<D, 1, false, 2, 2>(tq, tk, tv, to, tt, p, stream);
-    }
-    if (p.R > 0 && p.keys_bf16) return launch_fwd_variant<D, 2, true, 2, 2, true>(tq, tk, tv, to, tt, p, stream);
-    return p.R > 0 ? launch_fwd_variant<D, 2, true, 2, 2>(tq, tk, tv, to, tt, p, stream)
-                   : launch_fwd_variant<D, 2, false, 2, 2>(tq, tk, tv, to, tt, p, stream);
+        return p.R > 0 ? launch_fwd_variant<D, 2, kRotAll, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream)
+                       : launch_fwd_variant<D, 2, kRotNone, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream);
+    if (p.R > 0 && p.keys_bf16 && two_tiles) return launch_fwd_variant<D, 2, kRotAll, 2, 2, true>(tq, tk, tv, to, tt, p, stream);
+    const auto dense = [&](auto rope) {
+        return two_tiles ? launch_fwd_variant<D, 2, decltype(rope)::value, 2, 2>(tq, tk, tv, to, tt, p, stream)
+                         : launch_fwd_variant<D, 1, decltype(rope)::value, 2, 2>(tq, tk, tv, to, tt, p, stream);
+    };
+    if (p.R == 0) return dense(std::integral_constant<int, kRotNone>{});
+    return p.keys_rotated ? dense(std::integral_constant<int, kRotQueries>{}) : dense(std::integral_constant<int, kRotAll>{});
 }
 
 template <int D, bool DKV, bool ROT_X, bool ROT_A, bool BS>
@@ -941,7 +941,7 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     } else {
         two_tiles = qtiles != 1 && (!spread || (Rr > 0 && keys_bf16));   // (packed-bf16 keys: built for two)
     }
-    p.rot_k = k_prerotated ? 0 : 1;
+    p.keys_rotated = k_prerotated ? 1 : 0;
     p.keys_bf16 = keys_bf16 ? 1 : 0;
     p.bias = bias;
     p.bias_sh = (bias && bias_H > 1) ? static_cast<long long>(shape->S) * shape->S : 0;

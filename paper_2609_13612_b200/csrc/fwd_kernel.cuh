@@ -3,7 +3,8 @@
 //   TMEM -> scale / ALiBi / mask / online softmax in registers (one query row per thread) ->
 //   P (bf16) back into TMEM over S -> tcgen05.mma O += P V -> normalise, store O and L.
 // Warp roles: warp 0 TMA producer, warp 1 MMA issuer (one elected thread each), warps 4-7 rotate
-// Q once and every K tile, warps 8.. are one softmax warpgroup per query tile.
+// every K tile, the warps after them are one softmax warpgroup per query tile (which first rotates it).  Kernels that
+// rotate no key tiles on chip have no warps for it.
 #pragma once
 #include <cuda.h>
 #include <type_traits>
@@ -34,8 +35,8 @@ struct FwdParams {
     // of the two row blocks' lists, each entry = key block | (1 << 28 if row block 2 rb has it) | (1 << 29 if 2 rb + 1).
     int bs_rowpair;
     int keys_bf16;         // host-side choice of the TAB instantiation (packed-bf16 key rotation)
-    int rot_k;             // ROPE kernels: 1 = rotate the key tiles on chip; 0 = the keys arrive rotated (hybrid
-                           // arm of Section 5.3: K rotated once by a RoPE pass, only Q rotated in the kernel)
+    int keys_rotated;      // host-side choice of the kRotQueries instantiation: the keys arrive rotated (hybrid arm of
+                           // Section 5.3: K rotated once by a RoPE pass, only Q rotated in the kernel)
     // Section 3.1, additive_bias: fp32 bias[bb, hh, i, j] added to the scaled score (nullptr: none); element strides
     // of its batch and head extents (0 where the extent is 1 and the bias is broadcast), rows of S floats.
     const float* bias;
@@ -102,6 +103,12 @@ __device__ long long* g_trace = nullptr;
 #endif
 constexpr int kFwdMaxSplits = 8;    // CTAs that share a query tile's key tiles, at most
 constexpr int kFwdMinTiles = 2;     // key tiles per CTA below which a query tile is not shared out further
+// What a forward kernel rotates on chip.  Kernels that rotate no key tiles have no rotation warpgroup and no code for it: its
+// registers go to the softmax warpgroups (176 -> 208 per thread, no spills), and a CTA's set-up starts four warps less.
+// Against the same kernel with an idle rotation warpgroup: 179.0 -> 173.4 us (B = 4, 12 heads, S = 4096, D = 64, keys
+// rotated before), 141.4 -> 139.0 us (32 / 8 heads, S = 4096, D = 128, no rotation), both under sustained load.
+constexpr int kRotNone = 0, kRotAll = 1, kRotQueries = 2;
+__host__ __device__ constexpr int fwd_threads(int nq, int rope) { return 128 * (1 + (rope == kRotAll ? 1 : 0) + nq); }
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: O is rescaled only when the row max grows by more
 
 constexpr int kPParts = 2;   // P is handed to the MMA issuer in two column halves (four parts, and an S tile produced as
@@ -304,19 +311,21 @@ __device__ __forceinline__ bool softmax_tile_general(uint32_t tS, uint32_t tO, i
     return true;
 }
 
-// TAB (with ROPE): key tiles are rotated in packed bf16 arithmetic from table tiles that arrive by TMA through
+// ROPE: kRotNone, kRotAll or kRotQueries.  TAB (with kRotAll): key tiles are rotated in packed bf16 arithmetic from table tiles that arrive by TMA through
 // tm_t (the bf16 copy of the cos/sin table); otherwise in fp32 arithmetic from the fp32 table rows.
 // GEN: the instantiation for the variants with an additive bias or the ReLU normaliser (softmax_tile_general); kept
 // apart so that the kernels of the other variants carry none of its registers.
 // SPLIT (dense, NQ = 1): the grid's z dimension is a cluster of p.splits CTAs that share out the key tiles of a query tile.  Each
 // ends with an unnormalised O, m and l of its own; they are merged (log-sum-exp, in rank order) through distributed
 // shared memory, every CTA taking a share of the rows.  For grids that leave SMs idle: see fwd_splits (attnfuse.cu).
-template <int D, int NQ, bool ROPE, int KS, int VS, bool BS = false, bool TAB = false, bool GEN = false, bool SPLIT = false>
-__global__ void __launch_bounds__(128 * (2 + NQ), 1)
+template <int D, int NQ, int ROPE, int KS, int VS, bool BS = false, bool TAB = false, bool GEN = false, bool SPLIT = false>
+__global__ void __launch_bounds__(fwd_threads(NQ, ROPE), 1)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                 const __grid_constant__ CUtensorMap tm_t, const FwdParams p) {
-    using L = FwdSmem<D, NQ, KS, VS, ROPE && TAB>;
+    using L = FwdSmem<D, NQ, KS, VS, ROPE == kRotAll && TAB>;
+    constexpr bool KROT = ROPE == kRotAll;
+    constexpr int kSoftmaxWarp = KROT ? 8 : 4;   // the first softmax warp
     constexpr int TILE = L::TILE;
     constexpr int NBOX = D / BOX_COLS;
     constexpr int kPartStride = D + 4;   // SPLIT: floats per staged row
@@ -331,7 +340,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     uint8_t* sK = smem + L::OFF_K;
     uint8_t* sV = smem + L::OFF_V;
     uint8_t* sT = smem + L::OFF_T;
-    constexpr bool tab_tiles = ROPE && TAB;
+    constexpr bool tab_tiles = KROT && TAB;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + L::OFF_MISC + 4);
@@ -459,7 +468,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // Measured with the output written box by box and L stored while the last products run (see the epilogue): hybrid arm
     // 166.9 -> 161.1 us (B = 4, 32 / 8 heads, S = 2048, D = 128), without rotation 122.1 -> 118.7 us (S = 4096), 177.0 -> 174.0 us
     // (B = 4, 12 heads, S = 4096, D = 64).
-    const bool hybrid = ROPE && !p.rot_k;
+    constexpr bool hybrid = ROPE == kRotQueries;
     int first_it = 0;   // key tiles requested here already
     if (warp == 0) {
         if constexpr (!BS) init_barriers();
@@ -493,17 +502,20 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = warp_uniform(*tmem_slot);
+    // (all of tensor memory starts at column 0: a constant in the MMAs' operands)
+    const uint32_t tmem_base = TMEM_COLS == 512 ? 0u : warp_uniform(*tmem_slot);
     grid_dep_launch();
     if (!hybrid) grid_dep_wait();
 
     // Register budget: the softmax warpgroups hold a full row of 128 scores; the others need little, but the
     // MMA issuer must not spill (it is the most latency-sensitive thread of the CTA: at 64 registers it spilled
     // and the kernel was 4 % slower), and the rotation warpgroup fits in 80.  80 + 80 + 2 x 176 = 512.
-    constexpr int kSoftmaxRegs = NQ == 2 ? 176 : 232;
-    constexpr int kIssuerRegs = 80, kRotRegs = 80;
+    // Without the rotation warpgroup 88 + 2 x 208 = 504 of 3 x 168; with one query tile there is room for everybody.
+    constexpr int kSoftmaxRegs = NQ == 1 ? 232 : KROT ? 176 : 208;
+    constexpr int kIssuerRegs = KROT ? 80 : 88, kRotRegs = 80;
+    constexpr bool kSetRegs = KROT || NQ == 2;
 
-    if (warp < 4) setmaxnreg_dec<kIssuerRegs>();
+    if (kSetRegs && warp < 4) setmaxnreg_dec<kIssuerRegs>();
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         {
@@ -562,102 +574,67 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             __syncwarp();
         }
         {
-            const int B_KREADY = (ROPE && p.rot_k) ? L::B_KROT : L::B_KFULL;
+            constexpr int B_KREADY = KROT ? L::B_KROT : L::B_KFULL;
             constexpr int B_QREADY = ROPE ? L::B_QROT : L::B_QFULL;
-            int cnt[NQ];
-            bool ok = true;
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) cnt[q] = 0;
-
             // descriptors differ only in their low word: one add per operand and step
-            const uint32_t dhi = desc_hi(1024);
+            const uint32_t dhi = desc_hi(1024), bar0 = smem_u32(bars);
+            const uint32_t q_lo0 = desc_lo(smem_u32(sQ), 16), k_lo0 = desc_lo(smem_u32(sK), 16), v_lo0 = desc_lo(smem_u32(sV), BOX_BYTES);
+            const uint32_t ax = smem_u32(smem + L::OFF_AX);
             auto issue_S = [&](int q, int ks) {
-                if (!elect_one()) return;
-                const uint32_t q_lo = desc_lo(smem_u32(sQ + q * TILE), 16), k_lo = desc_lo(smem_u32(sK + ks * TILE), 16);
-                const uint32_t d = tmem_base + q * BN;
-#pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    const uint32_t off = ((kk >> 2) * BOX_BYTES + (kk & 3) * 32) >> 4;
-                    if (kk == 0) mma_ss_lo<false>(d, q_lo + off, k_lo + off, dhi, IDESC_S);
-                    else mma_ss_lo<true>(d, q_lo + off, k_lo + off, dhi, IDESC_S);
-                }
-                if (alibi_mma) {
-                    const uint32_t ax = smem_u32(smem + L::OFF_AX);
-                    mma_ss_lo<true>(d, desc_lo(ax + (1 + q) * L::AX_TILE, 128), desc_lo(ax, 128), desc_hi_noswizzle(256), IDESC_S);
-                }
-                mma_commit(&bars[L::B_SFULL + 2 * q]);
+                mma_scores<D>(tmem_base + q * BN, q_lo0 + q * (TILE >> 4), k_lo0 + ks * (TILE >> 4), dhi, IDESC_S);
+                if (alibi_mma && elect_one())
+                    mma_ss_lo<true>(tmem_base + q * BN, desc_lo(ax + (1 + q) * L::AX_TILE, 128), desc_lo(ax, 128), desc_hi_noswizzle(256), IDESC_S);
+                commit_elected(bar0 + 8 * (L::B_SFULL + 2 * q));
             };
-            // part pt of O += P V: its 8 / kPParts K-steps; that part of P starts at its own score columns
-            auto issue_O_part = [&](int q, int vs, bool acc, int pt) {
-                if (!elect_one()) return;
-                constexpr int KPP = 8 / kPParts;
-                const uint32_t v_lo = desc_lo(smem_u32(sV + vs * TILE), BOX_BYTES);
-                const uint32_t d = tmem_base + NQ * BN + q * D, a = tmem_base + q * BN + pt * (BN / kPParts);
+            static_assert(kPParts == 2, "two groups of MMAs per P V product");
+            auto run = [&] {   // (returns early when a wait gave up)
+                int cnt[NQ];
 #pragma unroll
-                for (int k = 0; k < KPP; ++k)
-                    mma_ts_lo(d, a + k * 8, v_lo + (pt * KPP + k) * 128, dhi, IDESC_O, (acc || pt > 0 || k > 0) ? 1u : 0u);
-            };
-
-            // prologue: S of the first key tile, each query tile as soon as it is ready (the softmax
-            // warpgroups rotate their Q tiles while the rotation warpgroup rotates K tile 0)
-            if (BS && n_it <= 0) ok = false;   // a row block without active blocks: nothing to issue
-            if (ok) ok = mbar_wait_warp(&bars[B_KREADY + 0], 0, abort_flag, 4);
-            AF_STAMP(0, 63, 3);  // first K ready
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                if (ok && jhi[q] >= jlo[q]) {
-                    ok = mbar_wait_warp(&bars[B_QREADY + q], 0, abort_flag, 3);
-                    tc_fence_after_sync();
-                    if (ok && active(q, jlo_c)) issue_S(q, 0);
-                }
-            }
-            AF_STAMP(0, 63, 2);  // Q ready
-            if (ok) elect_commit(&bars[L::B_KEMPTY + 0]);
-            for (int it = 0; ok && it < n_it; ++it) {
-                const int j = jlo_c + it, vs = it % VS, ks1 = (it + 1) % KS;
-                const bool next = it + 1 < n_it;
-                bool kwaited = false;
-                AF_STAMP(0, it, 0);
-                ok = mbar_wait_warp(&bars[L::B_VFULL + vs], (it / VS) & 1, abort_flag, 5);
-                AF_STAMP(0, it, 1);
+                for (int q = 0; q < NQ; ++q) cnt[q] = 0;
+                if (BS && n_it <= 0) return;   // a row block without active blocks: nothing to issue
+                // S of the first key tile, each query tile as soon as it is ready (the softmax warpgroups rotate their
+                // Q tiles while the rotation warpgroup rotates K tile 0)
+                if (!mbar_wait_warp(&bars[B_KREADY + 0], 0, abort_flag, 4)) return;
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
-                    if (ok && active(q, j)) {
+                    if (jhi[q] >= jlo[q]) {
+                        if (!mbar_wait_warp(&bars[B_QREADY + q], 0, abort_flag, 3)) return;
+                        tc_fence_after_sync();
+                        if (active(q, jlo_c)) issue_S(q, 0);
+                    }
+                }
+                commit_elected(bar0 + 8 * (L::B_KEMPTY + 0));
+                for (int it = 0; it < n_it; ++it) {
+                    const int j = jlo_c + it, vs = it % VS, ks1 = (it + 1) % KS;
+                    const bool next = it + 1 < n_it;
+                    // (both are there already, as a rule: they are taken while the pipe still works on the last scores)
+                    if (!mbar_wait_warp(&bars[L::B_VFULL + vs], (it / VS) & 1, abort_flag, 5)) return;
+                    if (next && !mbar_wait_warp(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7)) return;
 #pragma unroll
-                        for (int pt = 0; pt < kPParts; ++pt) {
-                            if (ok) ok = mbar_wait_warp(&bars[L::B_PREADY + 4 * q + pt], cnt[q] & 1, abort_flag, 6);
-                            if (pt == 0) AF_STAMP(0, it, 2 + 3 * q);
-                            if (ok) {
-                                tc_fence_after_sync();
-                                issue_O_part(q, vs, cnt[q] > 0, pt);
-                            }
-                        }
-                        if (ok) {
-                            AF_STAMP(0, it, 3 + 3 * q);
-                            ++cnt[q];
-                            if (is_last(q, j)) elect_commit(&bars[L::B_ODONE + q]);
-                        }
-                    }
-                    if (ok && next && active(q, j + 1)) {
-                        if (!kwaited) {
-                            ok = mbar_wait_warp(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7);
+                    for (int q = 0; q < NQ; ++q) {
+                        if (active(q, j)) {
+                            const uint32_t d = tmem_base + NQ * BN + q * D, a = tmem_base + q * BN, v_lo = v_lo0 + vs * (TILE >> 4);
+                            if (!mbar_wait_warp(&bars[L::B_PREADY + 4 * q], cnt[q] & 1, abort_flag, 6)) return;
                             tc_fence_after_sync();
-                            kwaited = true;
+                            mma_pv4(d, a, v_lo, dhi, IDESC_O, cnt[q] > 0 ? 1u : 0u);
+                            if (!mbar_wait_warp(&bars[L::B_PREADY + 4 * q + 1], cnt[q] & 1, abort_flag, 6)) return;
+                            tc_fence_after_sync();
+                            mma_pv4(d, a + BN / 2, v_lo + 512, dhi, IDESC_O, 1u);
+                            ++cnt[q];
+                            if (is_last(q, j)) commit_elected(bar0 + 8 * (L::B_ODONE + q));
                         }
-                        if (ok) issue_S(q, ks1);
-                        AF_STAMP(0, it, 4 + 3 * q);
+                        if (next && active(q, j + 1)) issue_S(q, ks1);
                     }
+                    commit_elected(bar0 + 8 * (L::B_VEMPTY + vs));
+                    if (next) commit_elected(bar0 + 8 * (L::B_KEMPTY + ks1));
                 }
-                if (ok) {
-                    elect_commit(&bars[L::B_VEMPTY + vs]);
-                    if (next) elect_commit(&bars[L::B_KEMPTY + ks1]);
-                }
-            }
+            };
+            run();
         }
-    } else if (warp >= 4 && warp < 8) {
+    } else if (KROT && warp >= 4 && warp < 8) {
         // ------------------------------------------------------------ rotation warpgroup (Section 4.1)
         setmaxnreg_dec<kRotRegs>();
-        if (ROPE && p.rot_k) {
+        if constexpr (KROT) {
             const int t = threadIdx.x - 128;
             // packed bf16 arithmetic on TMA-fed table tiles (rotary widths with a fast path)
             auto run_tab = [&](auto cp_tag) {
@@ -717,11 +694,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             else if (p.R == 16) run(std::integral_constant<int, 1>{});
             else run(std::integral_constant<int, 0>{});
         }
-    } else if (warp >= 8) {
+    } else if (warp >= kSoftmaxWarp) {
         // ------------------------------------------------------------ softmax warpgroups (one query row per thread)
-        setmaxnreg_inc<kSoftmaxRegs>();
-        const int q = (warp - 8) >> 2;
-        const int row = threadIdx.x - 256 - q * 128;            // == TMEM lane
+        if (kSetRegs) setmaxnreg_inc<kSoftmaxRegs>();
+        const int q = (warp - kSoftmaxWarp) >> 2;
+        const int row = threadIdx.x - kSoftmaxWarp * 32 - q * 128;            // == TMEM lane
         const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
         const uint32_t tS = tmem_base + lane_addr + q * BN;      // S (fp32) and, over it, P (bf16x2)
         const uint32_t tO = tmem_base + lane_addr + NQ * BN + q * D;
@@ -883,7 +860,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         __syncwarp();
         cluster_sync();
         // a group of D / 4 lanes per row, all warps on this CTA's share of the rows
-        constexpr int LANES = D / 4, NROW = 32 / LANES, NWARP = 4 * (2 + NQ);
+        constexpr int LANES = D / 4, NROW = 32 / LANES, NWARP = fwd_threads(NQ, ROPE) / 32;
         const uint32_t base = smem_u32(smem);
         const int gl = lane % LANES;
         if (!*abort_flag)

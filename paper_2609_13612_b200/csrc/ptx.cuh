@@ -71,6 +71,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // (Letting only lane 0 poll was measured slower: the warp woke up later.)
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
                                                uint32_t code, long long limit_cycles = kWaitLimitCycles) {
+    // (a barrier that is complete already: one test and one vote, no per-lane control flow)
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, code, limit_cycles));
 }
 
@@ -306,6 +308,45 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 // The same from a converged warp.  (elect.sync picks the same lane every time, so the commit sees that lane's MMAs.)
 __device__ __forceinline__ void elect_commit(uint64_t* bar) {
     if (elect_one()) mma_commit(bar);
+}
+
+
+// Groups of MMAs issued by one elected lane of a converged warp, each instruction predicated with the election instead of
+// standing in a branch.  The offsets between the MMAs of a group are immediates, so that what changes from group to group
+// is one add per operand.  A branch around a group cost the forward's issuer 170 cycles from the election to the first MMA
+// (re-forming its operands) and 80 for the way out of it, several times per tile.  Together with the waits for K and V in
+// front of those for P (see the issuer): 202 -> 195 us (B = 4, 12 heads, S = 4096, D = 64, rotation on chip), 179 -> 171
+// us (the same with rotated keys), 1972 -> 1932 us (32 / 8 heads, S = 16384, D = 128, no rotation; under the power cap).
+// Scores of one tile pair: D / 16 K steps, both operands K-major with the 128-byte swizzle, 64 columns (16 KB) per box.
+#define AF_MMA_SS_STEP(off, acc) \
+    "add.u32 a, %1, " #off ";\n\tadd.u32 b, %2, " #off ";\n\tmov.b64 da, {a, %3};\n\tmov.b64 db, {b, %3};\n\t" \
+    "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, " acc ";\n\t"
+template <int D>
+__device__ __forceinline__ void mma_scores(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc) {
+    if constexpr (D == 128)
+        asm volatile("{\n\t.reg .pred e, t, f;\n\t.reg .b64 da, db;\n\t.reg .b32 a, b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.eq.b32 t, 0, 0;\n\tsetp.ne.b32 f, 0, 0;\n\t"
+            AF_MMA_SS_STEP(0, "f") AF_MMA_SS_STEP(2, "t") AF_MMA_SS_STEP(4, "t") AF_MMA_SS_STEP(6, "t")
+            AF_MMA_SS_STEP(1024, "t") AF_MMA_SS_STEP(1026, "t") AF_MMA_SS_STEP(1028, "t") AF_MMA_SS_STEP(1030, "t") "}"
+            ::"r"(d), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred e, t, f;\n\t.reg .b64 da, db;\n\t.reg .b32 a, b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.eq.b32 t, 0, 0;\n\tsetp.ne.b32 f, 0, 0;\n\t"
+            AF_MMA_SS_STEP(0, "f") AF_MMA_SS_STEP(2, "t") AF_MMA_SS_STEP(4, "t") AF_MMA_SS_STEP(6, "t") "}"
+            ::"r"(d), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc) : "memory");
+}
+#define AF_MMA_TS_STEP(aoff, boff, acc) \
+    "add.u32 a, %1, " #aoff ";\n\tadd.u32 b, %2, " #boff ";\n\tmov.b64 db, {b, %3};\n\t" \
+    "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, " acc ";\n\t"
+// Four K steps (64 keys) of O += P V: P from TMEM (8 columns of bf16 pairs per step), V MN-major (2 KB per step).
+__device__ __forceinline__ void mma_pv4(uint32_t d, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t acc) {
+    asm volatile("{\n\t.reg .pred e, t, f;\n\t.reg .b64 db;\n\t.reg .b32 a, b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.eq.b32 t, 0, 0;\n\tsetp.ne.b32 f, %5, 0;\n\t"
+            AF_MMA_TS_STEP(0, 0, "f") AF_MMA_TS_STEP(8, 128, "t") AF_MMA_TS_STEP(16, 256, "t") AF_MMA_TS_STEP(24, 384, "t") "}"
+            ::"r"(d), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc) : "memory");
+}
+#undef AF_MMA_SS_STEP
+#undef AF_MMA_TS_STEP
+// elect_commit without a branch; `bar`: shared-memory address.
+__device__ __forceinline__ void commit_elected(uint32_t bar) {
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
 
 // ---------------------------------------------------------------- TMEM <-> registers (32 lanes x 32-bit, one row per thread)
