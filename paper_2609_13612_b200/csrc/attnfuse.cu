@@ -11,6 +11,7 @@
 
 #include "../../include/attnfuse.h"
 #include "fwd_kernel.cuh"
+#include "fwd64_kernel.cuh"
 #include "bwd_kernel.cuh"
 #include "bwd_first_rows.cuh"
 #include "bwd_fused_kernel.cuh"
@@ -403,6 +404,61 @@ af_status launch_fwd_variant(const CUtensorMap& tq, const CUtensorMap& tk, const
     return launch_kernel(kern, grid, dim3(fwd_threads(NQ, ROPE), 1, 1), L::BYTES, stream, true, tq, tk, tv, to, tt, p);
 }
 
+// Heads per CTA of the kernel with four query tiles (D = 64, dense masks; fwd64_kernel.cuh): heads of one kv head on the same rows as far as the group allows (they end together), else row
+// blocks of one head.
+int heads_of_four(int group) { return !opt(AF_OPT_FWD_PAIR_HEADS) ? 1 : (group % 4) == 0 ? 4 : (group % 2) == 0 ? 2 : 1; }
+
+// Work of a dense forward grid whose CTAs take `rows` consecutive row blocks of `heads` heads each, in key tiles: of the longest CTA and
+// in all, and the number of CTAs.
+struct FwdGrid {
+    double longest, sum, ctas;
+};
+FwdGrid fwd_grid(const FwdParams& p, int rows, int heads) {
+    FwdGrid g = {0.0, 0.0, 0.0};
+    const int blocks = (p.S + BM - 1) / BM;
+    for (int r = 0; r < blocks; r += rows) {
+        const int last = r + rows < blocks ? r + rows - 1 : blocks - 1;
+        const int hi = p.causal ? last : (p.window >= 0 ? (last * BM + BM - 1 + p.window) / BN : blocks - 1);
+        const int lo = p.window >= 0 && r * BM > p.window ? (r * BM - p.window) / BN : 0;
+        const double n = (hi < blocks - 1 ? hi : blocks - 1) - lo + 1;
+        g.longest = n > g.longest ? n : g.longest;
+        g.sum += n;
+        g.ctas += 1.0;
+    }
+    const double units = static_cast<double>(p.heads) / heads;
+    g.sum *= units;
+    g.ctas *= units;
+    return g;
+}
+// Four query tiles per CTA or two (D = 64)?  Four are faster per tile, 2.85 against 2 x 1.6 us per key tile, but make fewer and longer
+// CTAs.  The longer of the longest CTA and the work over the SMs decides, or, where all CTAs are about as long, the number of
+// waves (203 / 246 us at 16 / 4 heads, S = 5000, no causal mask: 160 CTAs of four); measured, two / four: 200 / 185 us (B = 4, 12
+// heads, S = 4096: 384 CTAs of four), 44.7 / 37.1 us (B = 8, S = 1024: 192), 98 / 104 us (B = 2, S = 4096: 192, with longer
+// ones), 38.8 / 56.7 us (32 / 8 heads, S = 2048: 128).
+bool four_query_tiles(const FwdParams& p) {
+    const int pair = (p.group % 2) == 0 && opt(AF_OPT_FWD_PAIR_HEADS) ? 2 : 1, quad = heads_of_four(p.group);
+    const double sms = sm_count();
+    auto time = [&](const FwdGrid& g, double cta, double tile) {
+        const double chain = cta + tile * g.longest, all = (cta * g.ctas + tile * g.sum) / sms;
+        if (g.sum > 0.75 * g.longest * g.ctas) return chain * ceil(g.ctas / sms);
+        return chain > all ? chain : all;
+    };
+    return time(fwd_grid(p, 4 / quad, quad), 8.0, 2.85) < 0.98 * time(fwd_grid(p, 2 / pair, pair), 7.0, 1.6);
+}
+
+// Four query tiles per CTA (D = 64, dense masks; fwd64_kernel.cuh).
+template <int ROPE>
+af_status launch_fwd64(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, FwdParams p,
+                       cudaStream_t stream) {
+    auto kern = attn_fwd64_kernel<ROPE>;
+    static std::atomic<unsigned long long> configured{0};
+    if (allow_dynamic_smem(kern, Fwd64Smem::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
+    const int heads = p.four_tiles;
+    const int rows_per_cta = BM * Fwd64Smem::NQ / heads;
+    p.n_row_blocks = (p.S + rows_per_cta - 1) / rows_per_cta;
+    return launch_kernel(kern, dim3(p.B * p.Hq / heads, p.n_row_blocks, 1), dim3(fwd64_threads(ROPE), 1, 1), Fwd64Smem::BYTES, stream, true,
+                         tq, tk, tv, to, p, heads);
+}
 // Block-sparse variant (Section 4.3): the grid is (heads or head pairs, 128-row blocks); every CTA walks the
 // list of active key blocks of its row block.  An even GQA group pairs two heads per CTA, otherwise one head.
 template <int D, int NQ, int ROPE, bool GEN = false>
@@ -446,6 +502,8 @@ af_status launch_fwd(const CUtensorMap& tq, const CUtensorMap& tk, const CUtenso
                        : launch_fwd_variant<D, 2, kRotNone, 2, 2, false, true>(tq, tk, tv, to, tt, p, stream);
     if (p.R > 0 && p.keys_bf16 && two_tiles) return launch_fwd_variant<D, 2, kRotAll, 2, 2, true>(tq, tk, tv, to, tt, p, stream);
     const auto dense = [&](auto rope) {
+        if constexpr (D == 64)
+            if (two_tiles && p.four_tiles) return launch_fwd64<decltype(rope)::value>(tq, tk, tv, to, p, stream);
         return two_tiles ? launch_fwd_variant<D, 2, decltype(rope)::value, 2, 2>(tq, tk, tv, to, tt, p, stream)
                          : launch_fwd_variant<D, 1, decltype(rope)::value, 2, 2>(tq, tk, tv, to, tt, p, stream);
     };
@@ -946,6 +1004,7 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
         two_tiles = qtiles != 1 && (!spread || (Rr > 0 && keys_bf16));   // (packed-bf16 keys: built for two)
     }
     p.keys_rotated = k_prerotated ? 1 : 0;
+    p.four_tiles = shape->D == 64 && qtiles == 2 && two_tiles && !bs_row_ptr && !bias && !relu && !keys_bf16 && four_query_tiles(p) ? heads_of_four(gqa_group) : 0;
     p.keys_bf16 = keys_bf16 ? 1 : 0;
     p.bias = bias;
     p.bias_sh = (bias && bias_H > 1) ? static_cast<long long>(shape->S) * shape->S : 0;

@@ -141,6 +141,10 @@ __device__ __forceinline__ void rotate_tile_smem(uint8_t* tile, int row0, int S,
 // run of consecutive tiles needs no table read at all; callers re-read the table every
 // kRotResync tiles to keep the accumulated rounding of the recurrence far below bf16 resolution.
 constexpr int kRotResync = 16;
+// The forward's key tiles re-read it every kKeyRun tiles, so that a pass over the keys ahead of the kernel can give the same
+// bits without walking far (rope_key_tiles_kernel: with 16 tiles the walk cost that pass 10 us at 32 / 8 heads, S = 4096,
+// D = 128, with 4 it takes 4; on chip 163 us either way).
+constexpr int kKeyRun = 4;
 // The arithmetic uses the packed fp32 instructions of sm_100 (two lanes per instruction): a bf16x2
 // word holds two adjacent columns, i.e. two frequencies, so cos and sin are kept as float2 pairs.
 template <int CP>

@@ -48,6 +48,7 @@ struct FwdParams {
     // into two bf16 values, e exact in bf16) - and the softmax warps run their plain straight-line code.
     int alibi_mma;
     int splits;            // SPLIT kernels: CTAs per cluster, the grid's z dimension
+    int four_tiles;        // host-side choice of the kernel with four query tiles per CTA (fwd64_kernel.cuh): its heads per CTA
     long long heads;       // host side: heads (B * Hq) of the whole problem, of which this launch may be a part
 #ifdef AF_TRACE
     long long* trace;
@@ -669,7 +670,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int it = 0; ok && it < n_it; ++it) {
                     const int ks = it % KS;
                     // (listed tiles need not be consecutive: the cos/sin state is read for every tile)
-                    if (CP > 0 && (BS || (it % kRotResync) == 0))
+                    if (CP > 0 && (BS || (it % kKeyRun) == 0))
                         rotate_prefetch(st, p.table, tile_at(jlo_c + it) * BN, p.S, p.R, t);
                     AF_STAMP(1, it, 0);
                     ok = mbar_wait_warp(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);

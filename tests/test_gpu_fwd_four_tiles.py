@@ -1,0 +1,70 @@
+"""Forward with four query tiles per CTA (D = 64, dense masks, grids that fill the device): 64-key steps, groups that put four, two or
+one head into a CTA, row blocks without rows, ragged lengths at the edges of steps and tiles, windows that start in the second half of
+a key tile, both output types."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_13612_b200 as af
+from paper_2609_13612_b200 import synth
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+W = synth.Workload
+
+
+@pytest.mark.parametrize("w", [
+    W("one_tile_each", 40, 8, 2, 65, 64, theta=1e4, seed_id=901),
+    W("second_step_full", 40, 8, 8, 128, 64, theta=1e4, seed_id=902),
+    W("rows_beyond_a_step", 32, 8, 4, 129, 64, theta=1e4, seed_id=903),
+    W("two_heads_two_blocks", 16, 12, 2, 257, 64, theta=1e4, rotary_dim=32, seed_id=904),
+    W("one_head_four_blocks", 16, 9, 3, 511, 64, theta=1e4, seed_id=905),
+    W("fifth_block", 16, 6, 6, 577, 64, theta=1e4, rotary_dim=16, seed_id=906),
+    W("window_in_second_half", 12, 8, 8, 700, 64, theta=1e4, window=70, seed_id=907),
+    W("window_alibi", 12, 8, 4, 640, 64, theta=1e4, window=200, alibi=True, seed_id=908),
+    W("window_zero", 24, 8, 8, 300, 64, theta=1e4, window=0, seed_id=909),
+    W("noncausal", 12, 8, 1, 450, 64, theta=1e4, causal=False, seed_id=910),
+    W("noncausal_window", 12, 9, 9, 500, 64, theta=1e4, causal=False, window=130, seed_id=911),
+    W("no_rotation", 12, 16, 4, 520, 64, rotary_dim=0, seed_id=912),
+    W("rotary_48", 12, 12, 12, 400, 64, theta=1e4, rotary_dim=48, seed_id=913),
+], ids=lambda w: w.name)
+@pytest.mark.parametrize("out_dtype", [torch.bfloat16, torch.float32], ids=["bf16", "fp32"])
+def test_against_the_oracle_and_the_kernel_for_two(w, out_dtype):
+    t = synth.draw_all(w)
+    dev = {k: pu.to_dev(v) for k, v in t.items()}
+    rope, mask = pu.specs(w)
+    table = af.rope_table(rope, w.S)
+    want_o, want_l = oracle.run_workload(w, t)
+    # non-causal windows and ALiBi give few-key rows, whose outputs carry the roundings undivided: the generated examples' bound
+    for call in (af.fwd, af.fwd_hybrid):
+        o = torch.full((w.B, w.Hq, w.S, w.D), float("nan"), dtype=out_dtype, device="cuda")
+        lse = torch.full((w.B, w.Hq, w.S), float("nan"), dtype=torch.float32, device="cuda")
+        call(dev["q"], dev["k"], dev["v"], rope, table, mask, w.scale, out=o, lse=lse)
+        torch.cuda.synchronize()
+        assert af.device_status()[0] == 0
+        pu.assert_close_scaled(w.name, pu.to_np(o), want_o)
+        assert np.abs(pu.to_np(lse) - want_l).max() <= pu.LSE_TOL
+    with af.option(af.OPT_FWD_QTILES, 3):
+        o2, _ = af.fwd(dev["q"], dev["k"], dev["v"], rope, table, mask, w.scale, out_dtype=out_dtype)
+    torch.cuda.synchronize()
+    pu.assert_close_scaled(w.name + " two", pu.to_np(o2), want_o)
+
+
+def test_infinite_and_nan_scores_as_in_the_kernel_for_two():
+    """A key row of -inf takes part with weight zero (NaN where the products are), a NaN key row spoils the rows that see it."""
+    g = torch.Generator(device="cuda").manual_seed(914)
+    q, k, v = (torch.randn(16, h, 300, 64, generator=g, device="cuda").to(torch.bfloat16) for h in (8, 8, 8))
+    q = q.abs()
+    k[:, :, 7] = float("-inf")
+    k[:, 1, 200] = float("nan")
+    got = {}
+    for option in (2, 3):
+        with af.option(af.OPT_FWD_QTILES, option):
+            got[option] = af.fwd(q, k, v, af.RopeSpec(rotary_dim=0), None, af.MaskSpec(), 0.125)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    for a, b in zip(got[2], got[3]):
+        assert torch.equal(torch.isnan(a), torch.isnan(b)) and torch.equal(torch.isinf(a), torch.isinf(b))
+        ok = torch.isfinite(b)
+        assert (a[ok].float() - b[ok].float()).abs().max().item() <= 2.0 ** -6   # one bf16 ulp at |x| < 4, and P's rounding
