@@ -148,6 +148,20 @@ af_status attnfuse_fwd(const af_shape* shape, const void* q, const void* k, cons
                        int gqa_group, float softmax_scale,
                        void* o, af_dtype o_dtype, float* lse, void* cuda_stream);
 
+/* ---- forward with scratch memory --------------------------------------------------------------------
+ * attnfuse_fwd, with the bits of attnfuse_fwd, for callers that can lend it device memory: where it is faster
+ * a first launch writes the rotated keys into `scratch` with the arithmetic of the on-chip
+ * rotation, and the forward kernel then rotates only its query tiles.
+ * attnfuse_fwd_scratch_bytes: how much it would use, 0 where it would use none.  scratch (device, 16-byte aligned)
+ * may be NULL or too small: the keys are then rotated on chip.  Its content afterwards is unspecified. */
+size_t    attnfuse_fwd_scratch_bytes(const af_shape* shape, const af_rope* rope, const af_mask* mask, int gqa_group);
+af_status attnfuse_fwd_scratch(const af_shape* shape, const void* q, const void* k, const void* v,
+                               const af_strides* sq, const af_strides* skv,
+                               const af_rope* rope, const void* rope_table, const af_mask* mask,
+                               int gqa_group, float softmax_scale,
+                               void* o, af_dtype o_dtype, float* lse,
+                               void* scratch, size_t scratch_bytes, void* cuda_stream);
+
 /* ---- hybrid arm of Section 5.3: rotate K once, fuse only the Q rotation -------------------------------
  * Same result as attnfuse_fwd (up to the bf16 rounding of a few rotated elements).  A RoPE pass writes
  * K' = RoPE(K) into the workspace (contiguous [B,Hkv,S,D] bf16), then the forward kernel runs with the

@@ -105,6 +105,11 @@ def lib() -> ctypes.CDLL:
         L.attnfuse_fwd.restype = i
         L.attnfuse_fwd.argtypes = [P(_Shape), vp, vp, vp, P(_Strides), P(_Strides), P(_Rope), vp, P(_Mask), i, f,
                                    vp, i, vp, vp]
+        L.attnfuse_fwd_scratch_bytes.restype = sz
+        L.attnfuse_fwd_scratch_bytes.argtypes = [P(_Shape), P(_Rope), P(_Mask), i]
+        L.attnfuse_fwd_scratch.restype = i
+        L.attnfuse_fwd_scratch.argtypes = [P(_Shape), vp, vp, vp, P(_Strides), P(_Strides), P(_Rope), vp, P(_Mask), i, f,
+                                           vp, i, vp, vp, sz, vp]
         L.attnfuse_fwd_fp8.restype = i
         L.attnfuse_fwd_fp8.argtypes = [P(_Shape), vp, vp, vp, P(_Mask), i, f, f, f, f, vp, i, vp, vp]
         L.attnfuse_fwd_variant.restype = i
@@ -155,7 +160,7 @@ _native = None
 def _bind(native, L) -> None:
     """Hand the native module the entry points of the loaded library."""
     native.bind({n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in (
-        "attnfuse_strerror", "attnfuse_fwd", "attnfuse_fwd_hybrid", "attnfuse_fwd_hybrid_workspace_bytes", "attnfuse_fwd_blocks",
+        "attnfuse_strerror", "attnfuse_fwd", "attnfuse_fwd_scratch", "attnfuse_fwd_scratch_bytes", "attnfuse_fwd_hybrid", "attnfuse_fwd_hybrid_workspace_bytes", "attnfuse_fwd_blocks",
         "attnfuse_fwd_fp8", "attnfuse_bwd", "attnfuse_bwd_blocks", "attnfuse_bwd_onepass_workspace_bytes", "attnfuse_decode",
         "attnfuse_decode_splits", "attnfuse_decode_workspace_bytes")}, AttnFuseError)
 
@@ -288,7 +293,9 @@ def rope(x: torch.Tensor, rope_spec: RopeSpec, table: Optional[torch.Tensor], in
 def fwd(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, rope_spec: RopeSpec, table: Optional[torch.Tensor],
         mask: MaskSpec, softmax_scale: float, out: Optional[torch.Tensor] = None,
         lse: Optional[torch.Tensor] = None, out_dtype: torch.dtype = torch.bfloat16, want_lse: bool = True):
-    """Fused forward.  q [B,Hq,S,D], k/v [B,Hkv,S,D] bf16 (last dim contiguous).  Returns (o, lse)."""
+    """Fused forward.  q [B,Hq,S,D], k/v [B,Hkv,S,D] bf16 (last dim contiguous).  Returns (o, lse).
+    Where it is faster, and memory for it is to be had, the keys are rotated once, ahead of the kernel, into scratch memory from
+    torch's allocator (attnfuse_fwd_scratch); the result has the same bits either way."""
     return (_native or _load_native()).fwd(q, k, v, rope_spec, table, mask, softmax_scale, out, lse, out_dtype, want_lse)
 
 

@@ -555,6 +555,23 @@ af_status launch_rope(const void* x_in, const af_strides& st, void* x_out, int B
                          static_cast<long long>(st.b), static_cast<long long>(st.h), static_cast<long long>(st.s));
 }
 
+// K' for the forward kernel, with the bits of its on-chip rotation (rope_key_tiles_kernel; rotary widths without the angle-addition
+// walk read the table for every row on chip, too, as the RoPE pass does).  x_out: contiguous.
+af_status launch_rope_keys(const void* k, const af_strides& st, void* out, int B, int H, int S, int D, int R, const void* rope_table,
+                           cudaStream_t stream) {
+    auto launch = [&](auto kern) {
+        const dim3 grid((S + BN - 1) / BN, static_cast<unsigned>(B) * H, 1);
+        return launch_kernel(kern, grid, dim3(128, 1, 1), 0, stream, true, static_cast<const uint4*>(k), static_cast<uint4*>(out),
+                             static_cast<const float2*>(rope_table), H, S, D, static_cast<long long>(st.b),
+                             static_cast<long long>(st.h), static_cast<long long>(st.s));
+    };
+    if (R == 128) return launch(rope_key_tiles_kernel<8>);
+    if (R == 64) return launch(rope_key_tiles_kernel<4>);
+    if (R == 32) return launch(rope_key_tiles_kernel<2>);
+    if (R == 16) return launch(rope_key_tiles_kernel<1>);
+    return launch_rope(k, st, out, B, H, S, D, R, rope_table, 0, stream);
+}
+
 // The set-up pass of a backward sequence (bwd_prologue_kernel): delta always, the rest as the parameters say.
 template <int D>
 af_status launch_prologue(const af_shape* sh, const void* o, const void* d_o, float* delta, BwdPrologueParams p, cudaStream_t stream) {
@@ -925,13 +942,41 @@ af_status attnfuse_rope(const af_shape* shape, int n_heads, const void* x_in, vo
 }  // extern "C"
 
 namespace {
+// Is it faster to rotate the keys once, ahead of the forward kernel, than every key tile in every CTA that walks it?
+// On chip a key tile costs the CTAs that walk it 0.3 us each, on the longest CTA and on the SMs alike; ahead of the kernel a launch
+// (2 us) and two passes over the keys.  Measured, on chip / ahead, under sustained load: 163 / 146 us (32 / 8 heads, S = 4096,
+// D = 128), 327 / 278 us (the same without a causal mask, B = 4, S = 2048), 78 / 65 us (8 / 8 heads, S = 4096), 104 / 103 us (B = 8,
+// 8 / 8 heads, S = 2048), 72 / 74 us (B = 16, S = 1024), 12.7 / 14.2 us (B = 4, 32 / 8 heads, S = 256).
+bool keys_once(const af_shape* sh, const af_rope* rope, const af_mask* mask) {
+    if (rope->rotary_dim == 0 || keys_rotate_in_bf16(rope->rotary_dim)) return false;
+    // The bits of the on-chip rotation depend on where a CTA's run of tiles starts: at key 0 without a window, in CTAs that are
+    // not a share of a cluster.
+    if (mask->window >= 0 && mask->window < sh->S - 1) return false;
+    // (With slopes the two kernels' row constants are contracted differently: the last bit of a few outputs.)
+    if (mask->alibi_slopes) return false;
+    if (static_cast<long long>(sh->B) * sh->Hkv > 65535) return false;   // a grid dimension
+    FwdParams p = {};
+    p.S = sh->S; p.causal = mask->causal ? 1 : 0; p.window = -1;
+    p.group = sh->Hq / sh->Hkv;
+    p.heads = static_cast<long long>(sh->B) * sh->Hq;
+    const int qtiles = opt(AF_OPT_FWD_QTILES);
+    if (qtiles == 1 || (qtiles == 2 && one_query_tile(p, sh->D))) return false;
+    const bool four = sh->D == 64 && qtiles == 2 && four_query_tiles(p);
+    const int heads = four ? heads_of_four(p.group) : (p.group % 2) == 0 && opt(AF_OPT_FWD_PAIR_HEADS) ? 2 : 1;
+    const FwdGrid g = fwd_grid(p, (four ? 4 : 2) / heads, heads);
+    const double visits = g.sum / (sm_count() > 0 ? sm_count() : 148);
+    const double saved = 0.3 * (visits > g.longest ? visits : g.longest);
+    return saved > 2.0 + 0.2e-6 * attnfuse_fwd_hybrid_workspace_bytes(sh);
+}
+
 // Forward, dense (bs_row_ptr == nullptr) or over CSR lists of active 128 x 128 blocks.
 af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const void* v, const af_strides* sq,
                    const af_strides* skv, const af_rope* rope, const void* rope_table, const af_mask* mask,
                    int gqa_group, float softmax_scale, const int* bs_row_ptr, const int* bs_col_idx,
                    const int* bs_order, void* o, af_dtype o_dtype, float* lse, bool k_prerotated, void* cuda_stream,
                    const af_blocks* blocks = nullptr, const float* bias = nullptr, int bias_B = 1, int bias_H = 1,
-                   int relu = 0, long long all_heads = 0) {   // all_heads: of the whole problem, where this call is a part of one
+                   int relu = 0, long long all_heads = 0,     // all_heads: of the whole problem, where this call is a part of one
+                   void* keys_out = nullptr) {                // rotate the keys into this buffer first, and on chip only the queries
     af_status st = check_common(shape, rope, rope_table, mask, gqa_group);
     if (st != AF_OK) return st;
     if (!q || !k || !v || !o) return AF_ERR_NULL;
@@ -948,6 +993,13 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     if ((st = resolve_strides(skv, shape->Hkv, shape->S, shape->D, &stkv)) != AF_OK) return st;
     if ((st = check_arch()) != AF_OK) return st;
 
+    if (keys_out) {
+        if ((st = launch_rope_keys(k, stkv, keys_out, shape->B, shape->Hkv, shape->S, shape->D, rope->rotary_dim, rope_table,
+                                   static_cast<cudaStream_t>(cuda_stream))) != AF_OK)
+            return st;
+        k = keys_out;
+        k_prerotated = true;
+    }
     CUtensorMap tq, tk, tv, to;
     if ((st = make_tmap(&tq, q, shape->B, shape->Hq, shape->S, shape->D, stq, BM)) != AF_OK) return st;
     af_strides stk = stkv;
@@ -1088,6 +1140,24 @@ af_status attnfuse_fwd_fp8(const af_shape* shape, const void* q8, const void* k8
     dim3 grid(p.pair_heads ? p.B * p.Hq / 2 : p.B * p.Hq, p.n_row_blocks, 1);
     return launch_kernel(attn_fwd_fp8_kernel, grid, dim3(512, 1, 1), Fp8Smem::BYTES, static_cast<cudaStream_t>(cuda_stream), true, tq,
                          tk, tv, to, p);
+}
+
+size_t attnfuse_fwd_scratch_bytes(const af_shape* shape, const af_rope* rope, const af_mask* mask, int gqa_group) {
+    if (check_common(shape, rope, reinterpret_cast<const void*>(16), mask, gqa_group) != AF_OK) return 0;   // (any table)
+    return keys_once(shape, rope, mask) ? attnfuse_fwd_hybrid_workspace_bytes(shape) : 0;
+}
+
+af_status attnfuse_fwd_scratch(const af_shape* shape, const void* q, const void* k, const void* v, const af_strides* sq,
+                               const af_strides* skv, const af_rope* rope, const void* rope_table, const af_mask* mask,
+                               int gqa_group, float softmax_scale, void* o, af_dtype o_dtype, float* lse, void* scratch,
+                               size_t scratch_bytes, void* cuda_stream) {
+    af_status st = check_common(shape, rope, rope_table, mask, gqa_group);
+    if (st != AF_OK) return st;
+    if (!scratch || !keys_once(shape, rope, mask) || scratch_bytes < attnfuse_fwd_hybrid_workspace_bytes(shape))
+        return attnfuse_fwd(shape, q, k, v, sq, skv, rope, rope_table, mask, gqa_group, softmax_scale, o, o_dtype, lse, cuda_stream);
+    if (!aligned16(scratch)) return AF_ERR_ALIGN;
+    return fwd_impl(shape, q, k, v, sq, skv, rope, rope_table, mask, gqa_group, softmax_scale, nullptr, nullptr, nullptr, o,
+                    o_dtype, lse, false, cuda_stream, nullptr, nullptr, 1, 1, 0, 0, scratch);
 }
 
 size_t attnfuse_fwd_hybrid_workspace_bytes(const af_shape* shape) {

@@ -95,4 +95,65 @@ rope_apply_kernel(const uint4* x, uint4* y, const float2* __restrict__ table, in
                           R, sgn, xb, xh, xs);
 }
 
+// K' = RoPE(K) for the forward kernel, with the bits that its on-chip rotation of a key tile gives (rotate_tile_fast on tiles
+// that start at key 0): the cos/sin state of a thread's rows is read from the table at the first tile of a run of kKeyRun
+// and walked from there by the same angle-addition steps.  A block takes one key tile of one head; its 128 threads own
+// the same chunk pairs and rows as the rotation warpgroup.  The walk to the block's own tile (at most 24 steps of two
+// dependent multiply-adds) runs while the loads of the tile's rows are in flight.  R = 16 CP; columns past R are copied.
+template <int CP>
+__global__ void __launch_bounds__(128)
+rope_key_tiles_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, const float2* __restrict__ table, int H, int S, int D,
+                      long long xb, long long xh, long long xs) {
+    grid_dep_wait();
+    grid_dep_launch();   // (the forward kernel may be scheduled; it waits for this grid before its first key tile)
+    constexpr int RP = 128 / CP;
+    const int t = threadIdx.x, rg = t / CP, cp = t % CP;
+    const int tile = blockIdx.x, row0 = tile * BN;
+    const int h = blockIdx.y % H;
+    const size_t in0 = static_cast<size_t>((blockIdx.y / H * xb + h * xh) >> 3), step_in = static_cast<size_t>(xs >> 3);
+    const int chunks = D >> 3;
+    const size_t out0 = static_cast<size_t>(blockIdx.y) * S * chunks;
+    uint4 lo[CP], hi[CP];
+#pragma unroll
+    for (int k = 0; k < CP; ++k) {
+        const int r = row0 + rg + RP * k;
+        if (r < S) {
+            lo[k] = ld_global_cs(x + in0 + r * step_in + cp);
+            hi[k] = ld_global_cs(x + in0 + r * step_in + cp + CP);
+        }
+    }
+    RotStep step;
+    RotState<CP> st;
+    rotate_load_step<CP>(table, S, 16 * CP, t, step);
+    rotate_prefetch(st, table, tile / kKeyRun * kKeyRun * BN, S, 16 * CP, t);
+    auto advance = [&] {
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const float2 nc = __ffma2_rn(st.s[w], step.ns[w], __fmul2_rn(st.c[w], step.c[w]));
+            const float2 nsn = __ffma2_rn(st.c[w], step.s[w], __fmul2_rn(st.s[w], step.c[w]));
+            st.c[w] = nc;
+            st.s[w] = nsn;
+        }
+    };
+    for (int n = (tile % kKeyRun) * CP; n > 0; --n) advance();
+#pragma unroll
+    for (int k = 0; k < CP; ++k) {
+        const int r = row0 + rg + RP * k;
+        rotate_word2(lo[k].x, hi[k].x, st.c[0], st.s[0]);
+        rotate_word2(lo[k].y, hi[k].y, st.c[1], st.s[1]);
+        rotate_word2(lo[k].z, hi[k].z, st.c[2], st.s[2]);
+        rotate_word2(lo[k].w, hi[k].w, st.c[3], st.s[3]);
+        advance();
+        if (r < S) {
+            y[out0 + static_cast<size_t>(r) * chunks + cp] = lo[k];
+            y[out0 + static_cast<size_t>(r) * chunks + cp + CP] = hi[k];
+        }
+    }
+    const int rest = chunks - 2 * CP;
+    for (int i = t; i < 128 * rest; i += 128) {
+        const int r = row0 + i / rest, c = 2 * CP + i % rest;
+        if (r < S) y[out0 + static_cast<size_t>(r) * chunks + c] = ld_global_cs(x + in0 + r * step_in + c);
+    }
+}
+
 }  // namespace af

@@ -8,6 +8,7 @@
 #include <Python.h>
 
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDAGraphsC10Utils.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
@@ -21,6 +22,8 @@ namespace {
 struct Api {
     decltype(&attnfuse_strerror) strerror_;
     decltype(&attnfuse_fwd) fwd;
+    decltype(&attnfuse_fwd_scratch) fwd_scratch;
+    decltype(&attnfuse_fwd_scratch_bytes) fwd_scratch_bytes;
     decltype(&attnfuse_fwd_hybrid) fwd_hybrid;
     decltype(&attnfuse_fwd_hybrid_workspace_bytes) fwd_hybrid_workspace_bytes;
     decltype(&attnfuse_fwd_blocks) fwd_blocks;
@@ -246,8 +249,22 @@ PyObject* fwd(PyObject* const* a, Py_ssize_t n) {
     Out o(a[7], true, x.q.sizes(), dtype(a[9]), x.q);
     Out l(a[8], truth(a[10]), {x.sh.B, x.sh.Hq, x.sh.S}, at::kFloat, x.q);
     require(o.t.is_contiguous() && (o.t.scalar_type() == at::kBFloat16 || o.t.scalar_type() == at::kFloat), "out: contiguous, bf16 or fp32");
-    call(api.fwd, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale,
-         o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), stream());
+    // (scratch from torch's allocator, which orders its reuse on the current stream)
+    at::Tensor scratch;
+    if (const size_t bytes = api.fwd_scratch_bytes(&x.sh, &r, &m, x.group)) {
+        // a call with outputs of the caller's own allocates nothing while its stream is being captured: a capture that torch does
+        // not know of would be broken by it
+        if (!(o.given && (l.given || !l.any)) || c10::cuda::currentStreamCaptureStatusMayInitCtx() == c10::cuda::CaptureStatus::None) {
+            try {
+                scratch = empty({static_cast<int64_t>(bytes)}, at::kByte, x.q);
+            } catch (const c10::OutOfMemoryError&) {   // the keys are rotated on chip then
+            }
+        }
+    }
+    const bool lent = scratch.defined();
+    call(api.fwd_scratch, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale,
+         o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), lent ? scratch.data_ptr() : nullptr,
+         lent ? scratch.nbytes() : size_t{0}, stream());
     return pair(o, l);
 }
 
@@ -401,6 +418,8 @@ PyObject* bind(PyObject*, PyObject* args) {
     };
     get("attnfuse_strerror", api.strerror_);
     get("attnfuse_fwd", api.fwd);
+    get("attnfuse_fwd_scratch", api.fwd_scratch);
+    get("attnfuse_fwd_scratch_bytes", api.fwd_scratch_bytes);
     get("attnfuse_fwd_hybrid", api.fwd_hybrid);
     get("attnfuse_fwd_hybrid_workspace_bytes", api.fwd_hybrid_workspace_bytes);
     get("attnfuse_fwd_blocks", api.fwd_blocks);
