@@ -164,6 +164,21 @@ at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& l
 }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// Memory that a call works faster with but does not need: from torch's allocator, on the device and for the stream of the launch (its
+// reuse is then ordered).  An undefined tensor where there is none.
+// `allocates`: the call allocates its outputs anyway.  One with outputs of the caller's own allocates nothing while its stream is being
+// captured (a capture that torch does not know of would be broken by it), and no capture of another stream, by this thread or
+// another, may be broken by a cudaMalloc here: the thread's capture mode is relaxed meanwhile.
+at::Tensor scratch_if_any(size_t bytes, bool allocates) {
+    if (!allocates && c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None) return {};
+    const c10::cuda::CUDAStreamCaptureModeGuard relaxed(cudaStreamCaptureModeRelaxed);
+    try {
+        return at::detail::empty_cuda({static_cast<int64_t>(bytes)}, at::kByte, c10::Device(c10::kCUDA, c10::cuda::current_device()), std::nullopt);
+    } catch (const c10::OutOfMemoryError&) {
+        return {};
+    }
+}
+
 // Runs a C entry point without the interpreter lock (a launch may block while the device's queue is full).  The arguments are
 // plain values, evaluated by the caller while it holds the lock: data_ptr() of a tensor without storage throws.
 template <typename... P, typename... A>
@@ -249,18 +264,8 @@ PyObject* fwd(PyObject* const* a, Py_ssize_t n) {
     Out o(a[7], true, x.q.sizes(), dtype(a[9]), x.q);
     Out l(a[8], truth(a[10]), {x.sh.B, x.sh.Hq, x.sh.S}, at::kFloat, x.q);
     require(o.t.is_contiguous() && (o.t.scalar_type() == at::kBFloat16 || o.t.scalar_type() == at::kFloat), "out: contiguous, bf16 or fp32");
-    // (scratch from torch's allocator, which orders its reuse on the current stream)
-    at::Tensor scratch;
-    if (const size_t bytes = api.fwd_scratch_bytes(&x.sh, &r, &m, x.group)) {
-        // a call with outputs of the caller's own allocates nothing while its stream is being captured: a capture that torch does
-        // not know of would be broken by it
-        if (!(o.given && (l.given || !l.any)) || c10::cuda::currentStreamCaptureStatusMayInitCtx() == c10::cuda::CaptureStatus::None) {
-            try {
-                scratch = empty({static_cast<int64_t>(bytes)}, at::kByte, x.q);
-            } catch (const c10::OutOfMemoryError&) {   // the keys are rotated on chip then
-            }
-        }
-    }
+    const size_t bytes = api.fwd_scratch_bytes(&x.sh, &r, &m, x.group);
+    const at::Tensor scratch = bytes ? scratch_if_any(bytes, !(o.given && (l.given || !l.any))) : at::Tensor();
     const bool lent = scratch.defined();
     call(api.fwd_scratch, &x.sh, x.q.data_ptr(), x.k.data_ptr(), x.v.data_ptr(), &x.sq, &x.skv, &r, ptr(table), &m, x.group, scale,
          o.data(), out_code(o.t.scalar_type()), static_cast<float*>(l.data()), lent ? scratch.data_ptr() : nullptr,
