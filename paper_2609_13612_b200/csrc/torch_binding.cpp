@@ -165,18 +165,19 @@ at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& l
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
 // Memory that a call works faster with but does not need: from torch's allocator, on the device and for the stream of the launch (its
-// reuse is then ordered).  An undefined tensor where there is none.
+// reuse is then ordered).  An undefined tensor where there is none to be had, for whatever reason: the call must not fail over it.
 // `allocates`: the call allocates its outputs anyway.  One with outputs of the caller's own allocates nothing while its stream is being
 // captured (a capture that torch does not know of would be broken by it), and no capture of another stream, by this thread or
 // another, may be broken by a cudaMalloc here: the thread's capture mode is relaxed meanwhile.
 at::Tensor scratch_if_any(size_t bytes, bool allocates) {
-    if (!allocates && c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None) return {};
-    const c10::cuda::CUDAStreamCaptureModeGuard relaxed(cudaStreamCaptureModeRelaxed);
     try {
-        return at::detail::empty_cuda({static_cast<int64_t>(bytes)}, at::kByte, c10::Device(c10::kCUDA, c10::cuda::current_device()), std::nullopt);
-    } catch (const c10::OutOfMemoryError&) {
-        return {};
+        if (!allocates && c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None) return {};
+        const c10::cuda::CUDAStreamCaptureModeGuard relaxed(cudaStreamCaptureModeRelaxed);
+        at::Tensor t = at::detail::empty_cuda({static_cast<int64_t>(bytes)}, at::kByte, c10::Device(c10::kCUDA, c10::cuda::current_device()), std::nullopt);
+        if ((reinterpret_cast<uintptr_t>(t.data_ptr()) & 15) == 0) return t;
+    } catch (const std::exception&) {   // (any allocator's: torch's own raises several, one plugged in by the user its own)
     }
+    return {};
 }
 
 // Runs a C entry point without the interpreter lock (a launch may block while the device's queue is full).  The arguments are

@@ -1,4 +1,9 @@
-"""Where the binding's forward gets its scratch memory: a call that can do without must not break somebody's capture."""
+"""Where the binding's forward gets its scratch memory: a call that can do without must not break somebody's capture or fail with
+the allocator."""
+import os
+import subprocess
+import sys
+import textwrap
 import threading
 
 import pytest
@@ -8,6 +13,7 @@ import paper_2609_13612_b200 as af
 
 pytestmark = pytest.mark.gpu
 SHAPE = (1, 16, 4, 3000, 128)
+SCRATCH = 4 * 3000 * 128 * 2
 
 
 def problem(seed):
@@ -47,3 +53,59 @@ def test_another_threads_capture_survives_a_first_call():
     assert not failed and x.eq(2.0).all()
     assert torch.equal(out, want[0]) and torch.equal(lse, want[1])
     assert af.device_status()[0] == 0
+
+
+ALLOCATOR = r"""
+#include <cuda_runtime.h>
+#include <stdexcept>
+#include <sys/types.h>
+extern "C" {
+ssize_t watched = -1;   // a size that this allocator has trouble with
+int mode = 0, hits = 0;
+void* take(ssize_t size, int, cudaStream_t) {
+    void* p = nullptr;
+    if (size == watched) {
+        ++hits;
+        if (mode == 0) throw std::runtime_error("no memory of this size");
+        if (cudaMalloc(&p, size + 256) != cudaSuccess) return nullptr;
+        return static_cast<char*>(p) + 8;
+    }
+    return cudaMalloc(&p, size) == cudaSuccess ? p : nullptr;
+}
+void give(void* p, ssize_t size, int, cudaStream_t) {
+    cudaDeviceSynchronize();
+    cudaFree(size == watched && mode == 1 ? static_cast<char*>(p) - 8 : p);
+}
+}
+"""
+
+
+def test_an_allocator_that_fails_in_its_own_way(tmp_path):
+    """Memory that a call can do without: neither another exception than torch's nor a misaligned block may fail it."""
+    src, so = tmp_path / "allocator.cpp", tmp_path / "allocator.so"
+    src.write_text(ALLOCATOR)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-I" + cuda + "/include", "-o", str(so), str(src), "-L" + cuda + "/lib64", "-lcudart"], check=True)
+    code = textwrap.dedent("""
+        import ctypes, sys, torch
+        sys.path[:0] = [%r, %r]
+        lib = ctypes.CDLL(%r)
+        torch.cuda.memory.change_current_allocator(torch.cuda.memory.CUDAPluggableAllocator(%r, "take", "give"))
+        import paper_2609_13612_b200 as af
+        import test_gpu_fwd_scratch_memory as t
+        args = t.problem(933)
+        out, lse = torch.zeros_like(args[0]), torch.zeros(t.SHAPE[0], t.SHAPE[1], t.SHAPE[3], device="cuda")
+        want = af.fwd_variant(*args)   # on chip, the same bits
+        for mode in (0, 1):
+            out.zero_()
+            ctypes.c_int.in_dll(lib, "mode").value = mode
+            ctypes.c_ssize_t.in_dll(lib, "watched").value = t.SCRATCH
+            af.fwd(*args, out=out, lse=lse)
+            torch.cuda.synchronize()
+            ctypes.c_ssize_t.in_dll(lib, "watched").value = -1
+            assert torch.equal(out, want[0]) and torch.equal(lse, want[1]), mode
+        assert ctypes.c_int.in_dll(lib, "hits").value == 2 and af.device_status()[0] == 0
+        print("allocator ok")
+    """) % (os.path.dirname(os.path.dirname(os.path.abspath(__file__))), os.path.dirname(os.path.abspath(__file__)), str(so), str(so))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "allocator ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
