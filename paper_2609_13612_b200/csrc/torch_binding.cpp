@@ -8,6 +8,7 @@
 #include <Python.h>
 
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGraphsC10Utils.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
@@ -164,17 +165,28 @@ at::Tensor empty(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& l
 }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// Does the memory belong to the private pool that torch makes for a graph?  (A user's own pools have a zero there.)
+bool in_graph_pool(const void* p) {
+    const size_t a = reinterpret_cast<size_t>(p);
+    for (const auto& s : c10::cuda::CUDACachingAllocator::snapshot({0, 0}, false).segments)
+        if (s.address <= a && a - s.address < s.total_size) return s.owner_private_pool_id.first != 0;
+    return false;
+}
+
 // Memory that a call works faster with but does not need: from torch's allocator, on the device and for the stream of the launch (its
 // reuse is then ordered).  An undefined tensor where there is none to be had, for whatever reason: the call must not fail over it.
 // `allocates`: the call allocates its outputs anyway.  One with outputs of the caller's own allocates nothing while its stream is being
 // captured (a capture that torch does not know of would be broken by it), and no capture of another stream, by this thread or
 // another, may be broken by a cudaMalloc here: the thread's capture mode is relaxed meanwhile.
+// A captured launch writes the memory at every replay, long after this call has given it back: only the pool of torch's own graph,
+// which nobody outside the graph is served from, is lent to one.
 at::Tensor scratch_if_any(size_t bytes, bool allocates) {
     try {
-        if (!allocates && c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None) return {};
+        const bool captured = c10::cuda::currentStreamCaptureStatusMayInitCtx() != c10::cuda::CaptureStatus::None;
+        if (captured && !allocates) return {};
         const c10::cuda::CUDAStreamCaptureModeGuard relaxed(cudaStreamCaptureModeRelaxed);
         at::Tensor t = at::detail::empty_cuda({static_cast<int64_t>(bytes)}, at::kByte, c10::Device(c10::kCUDA, c10::cuda::current_device()), std::nullopt);
-        if ((reinterpret_cast<uintptr_t>(t.data_ptr()) & 15) == 0) return t;
+        if ((reinterpret_cast<uintptr_t>(t.data_ptr()) & 15) == 0 && (!captured || in_graph_pool(t.data_ptr()))) return t;
     } catch (const std::exception&) {   // (any allocator's: torch's own raises several, one plugged in by the user its own)
     }
     return {};

@@ -1,5 +1,6 @@
-"""Where the binding's forward gets its scratch memory: a call that can do without must not break somebody's capture or fail with
-the allocator."""
+"""Where the binding's forward gets its scratch memory: a call that can do without must not break somebody's capture, fail with the
+allocator, or leave memory to others that a captured graph still writes."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -109,3 +110,47 @@ def test_an_allocator_that_fails_in_its_own_way(tmp_path):
     """) % (os.path.dirname(os.path.dirname(os.path.abspath(__file__))), os.path.dirname(os.path.abspath(__file__)), str(so), str(so))
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "allocator ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+def test_a_capture_that_torch_does_not_know_of():
+    """Outputs allocated by the call, memory from torch's ordinary pool: what the call returns to the pool goes to others, and a
+    replay must not write there."""
+    rt = ctypes.CDLL("libcudart.so.12")
+    args = problem(932)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        want = af.fwd(*args)
+        warm = af.fwd(*args)
+        s.synchronize()
+        del warm   # (its memory and the scratch memory are in the stream's pool now)
+        handle, graph, exe = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p(), ctypes.c_void_p()
+        assert rt.cudaStreamBeginCapture(handle, 1) == 0   # thread-local mode
+        got = af.fwd(*args)
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) == 0
+        others = [torch.full((SCRATCH,), 7, dtype=torch.uint8, device="cuda") for _ in range(8)]
+        for x in got:
+            x.zero_()
+        assert rt.cudaGraphInstantiate(ctypes.byref(exe), graph, ctypes.c_ulonglong(0)) == 0
+        assert rt.cudaGraphLaunch(exe, handle) == 0
+        s.synchronize()
+    assert rt.cudaGraphExecDestroy(exe) == 0 and rt.cudaGraphDestroy(graph) == 0
+    assert all(x.eq(7).all() for x in others)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert af.device_status()[0] == 0
+
+
+def test_a_graph_of_torchs_own_is_still_lent_memory():
+    """The same bits, and the graph holds the launch that rotates the keys, too."""
+    args = problem(934)
+    want = af.fwd(*args)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        got = af.fwd(*args)
+    nodes = ctypes.c_size_t()
+    assert ctypes.CDLL("libcudart.so.12").cudaGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(nodes)) == 0
+    assert nodes.value == 2
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert af.device_status()[0] == 0
