@@ -795,7 +795,7 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
 }
 
 template <int D, int NT>
-af_status launch_decode(const CUtensorMap& tk, const CUtensorMap& tv, DecodeParams p, cudaStream_t stream) {
+af_status launch_decode(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeParams& p, cudaStream_t stream) {
     static std::atomic<unsigned long long> configured{0};
     if (allow_dynamic_smem(decode_split_kernel<D, NT>, DecodeSmem<D>::BYTES, configured) != AF_OK) return AF_ERR_CUDA;
     // A dependent launch saves about 1 us.  Behind a grid that streams for long it costs more: its CTAs wait on the SMs that come
@@ -804,10 +804,6 @@ af_status launch_decode(const CUtensorMap& tk, const CUtensorMap& tv, DecodePara
     // and less it is 1 to 8 % faster).
     const double kept = p.window >= 0 && p.window < p.N ? p.window + 1 : p.N;
     const bool dependent = kept / p.n_splits * D * 4 <= 4e6;
-    // (7.14 -> 6.79 us at 32 / 8 heads, 4096 keys, 27.6 -> 26.2 us at 64 / 8 heads, 32768 keys, 15.1 -> 14.2 us at B = 4, 4096
-    // keys, caches rotating over 400 MB; one CTA per kv head has no merge to hide behind: 5.18 -> 5.25 us at 512 keys;
-    // D = 64 loses, 7.8 -> 8.1 us at 8 / 8 heads, 8192 keys)
-    p.prefetch = dependent && D == 128 && p.n_splits > 1 ? 1 : 0;
     return launch_kernel(decode_split_kernel<D, NT>, dim3(p.n_splits, p.B * p.Hkv, 1), dim3(kDecWarps * 32, 1, 1),
                          DecodeSmem<D>::BYTES, stream, dependent, tk, tv, p);
 }

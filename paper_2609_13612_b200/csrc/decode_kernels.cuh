@@ -39,7 +39,6 @@ struct DecodeParams {
     unsigned int* tickets;
     __nv_bfloat16* o;           // [B, Hq, D]
     float* lse;                 // [B, Hq] or nullptr
-    int prefetch;               // bring the first tiles into L2 before the kernel before this one has ended
 };
 
 constexpr int kCombineMaxSplits = 256;
@@ -143,16 +142,6 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     if (lane == 0) {
         prefetch_tmap(&tm_k);
         prefetch_tmap(&tm_v);
-        // The tiles that fill this warp's stages, into L2 already: HBM is idle while the kernel before this one ends (a decode
-        // call spends its last microseconds on merging), and a line brought into L2 early stays coherent with what that
-        // kernel may still write.  The loads themselves wait for it.
-        if (p.prefetch)
-            for (int i = 0; i < min(nt_tiles, kDecStages); ++i)
-#pragma unroll
-                for (int bx = 0; bx < NBOX; ++bx) {
-                    tma_prefetch_4d(&tm_k, bx * 64, k_lo + kDecTile * (warp + kDecWarps * i), hk, b);
-                    tma_prefetch_4d(&tm_v, bx * 64, k_lo + kDecTile * (warp + kDecWarps * i), hk, b);
-                }
     }
     __syncthreads();
     // Programmatic dependent launch: the set-up above overlaps with the end of the previous kernel.  The wait comes before the

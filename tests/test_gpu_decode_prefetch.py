@@ -1,5 +1,4 @@
-"""Decoding asks for its first tiles in L2 before the kernel in front of it has ended: a cache that this kernel is still writing must be
-read as written."""
+"""A decode launch starts while the kernel in front of it ends: a cache that this kernel is still writing must be read as written."""
 import pytest
 import torch
 
