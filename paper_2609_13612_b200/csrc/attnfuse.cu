@@ -939,10 +939,13 @@ af_status attnfuse_rope(const af_shape* shape, int n_heads, const void* x_in, vo
 
 namespace {
 // Is it faster to rotate the keys once, ahead of the forward kernel, than every key tile in every CTA that walks it?
-// On chip a key tile costs the CTAs that walk it 0.3 us each, on the longest CTA and on the SMs alike; ahead of the kernel a launch
-// (2 us) and two passes over the keys.  Measured, on chip / ahead, under sustained load: 163 / 146 us (32 / 8 heads, S = 4096,
-// D = 128), 327 / 278 us (the same without a causal mask, B = 4, S = 2048), 78 / 65 us (8 / 8 heads, S = 4096), 104 / 103 us (B = 8,
-// 8 / 8 heads, S = 2048), 72 / 74 us (B = 16, S = 1024), 12.7 / 14.2 us (B = 4, 32 / 8 heads, S = 256).
+// On chip a key tile costs the CTAs that walk it 0.3 us each, on the longest CTA and on the SMs alike, if all its columns are rotated:
+// in proportion less for a part of them, and 1.6 times that where the table is read for every row (widths without the
+// angle-addition walk).  Ahead of the kernel it costs a launch (2.5 us) and two passes over the keys.
+// Measured on 115 grids, on chip / ahead: all columns 163 / 146 us (32 / 8 heads, S = 4096, D = 128), 103 / 94 us (B = 8, 4 / 4 heads,
+// S = 2963), 72 / 74 us (B = 16, 8 / 8 heads, S = 1024); half of them 26.3 / 31.3 us (B = 3, 12 / 4 heads, S = 1035), 74.0 / 74.8 us (B = 8,
+// 8 / 4 heads, S = 1701), 110.9 / 107.3 us (B = 2, 64 / 8 heads, S = 1475); 32 of 128 31.2 / 38.4 us (24 / 12 heads, S = 1430); 16 of
+// 128 24.0 / 34.0 us (32 / 8 heads, S = 1105); 96 of 128 67.4 / 53.9 us (B = 8, 8 / 2 heads, S = 1284).
 bool keys_once(const af_shape* sh, const af_rope* rope, const af_mask* mask) {
     if (rope->rotary_dim == 0 || keys_rotate_in_bf16(rope->rotary_dim)) return false;
     // The bits of the on-chip rotation depend on where a CTA's run of tiles starts: at key 0 without a window, in CTAs that are
@@ -961,8 +964,9 @@ bool keys_once(const af_shape* sh, const af_rope* rope, const af_mask* mask) {
     const int heads = four ? heads_of_four(p.group) : (p.group % 2) == 0 && opt(AF_OPT_FWD_PAIR_HEADS) ? 2 : 1;
     const FwdGrid g = fwd_grid(p, (four ? 4 : 2) / heads, heads);
     const double visits = g.sum / (sm_count() > 0 ? sm_count() : 148);
-    const double saved = 0.3 * (visits > g.longest ? visits : g.longest);
-    return saved > 2.0 + 0.2e-6 * attnfuse_fwd_hybrid_workspace_bytes(sh);
+    const int R = rope->rotary_dim;
+    const double tile = 0.3 * ((R & (R - 1)) == 0 ? 1.0 : 1.6) * R / sh->D;
+    return tile * (visits > g.longest ? visits : g.longest) > 2.5 + 0.2e-6 * attnfuse_fwd_hybrid_workspace_bytes(sh);
 }
 
 // Forward, dense (bs_row_ptr == nullptr) or over CSR lists of active 128 x 128 blocks.
