@@ -292,14 +292,14 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 #pragma unroll 1
             for (int hf = 0; ok && hf < 2; ++hf) {
                 const int slot = 2 * st + hf;
-                ok = mbar_wait_warp(&bars[L::B_AEMPTY + slot], ((n / NST) & 1) ^ 1, abort_flag, 41);
+                ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_AEMPTY + slot], ((n / NST) & 1) ^ 1, abort_flag, 41);
                 if (ok && elect_one()) {
                     mbar_arrive_expect_tx(&bars[L::B_AFULL + slot], TILE / 2);
 #pragma unroll
                     for (int bx = 0; bx < NBOX; ++bx)
                         tma_load_4d(sA + st * TILE + bx * BOX_BYTES + hf * (BOX_BYTES / 2), &tm_a, &bars[L::B_AFULL + slot], bx * BOX_COLS, a0 + hf * 64, ah, b);
                 }
-                if (ok) ok = mbar_wait_warp(&bars[L::B_BEMPTY + slot], ((n / NST) & 1) ^ 1, abort_flag, 57);
+                if (ok) ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_BEMPTY + slot], ((n / NST) & 1) ^ 1, abort_flag, 57);
                 if (ok && elect_one()) {
                     mbar_arrive_expect_tx(&bars[L::B_BFULL + slot], TILE / 2);
 #pragma unroll
@@ -315,7 +315,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         //   issuer 1: T2 = V dO^T   and dK' += dS^T Q'   (A from shared memory)
         {
             const int who = warp - 1;
-            bool ok = mbar_wait_warp(&bars[who == 0 ? L::B_XFULL : L::B_YFULL], 0, abort_flag, 42);
+            bool ok = mbar_wait_warp_quick<D == 64>(&bars[who == 0 ? L::B_XFULL : L::B_YFULL], 0, abort_flag, 42);
             const uint32_t dhi = desc_hi(1024);
             const uint32_t s_lo = desc_lo(smem_u32(who == 0 ? sX : sY), 16);
             const uint32_t t_dst = tmem_base + (who == 0 ? T1 : T2);
@@ -334,7 +334,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             };
             // a half tile of Q' (which = B_AFULL) or of dO (B_BFULL) has arrived
             auto wait_half = [&](int which, int n, int hf) {
-                const bool r = mbar_wait_warp(&bars[which + 2 * (n % NST) + hf], (n / NST) & 1, abort_flag, 43);
+                const bool r = mbar_wait_warp_quick<D == 64>(&bars[which + 2 * (n % NST) + hf], (n / NST) & 1, abort_flag, 43);
                 tc_fence_after_sync();
                 return r;
             };
@@ -354,7 +354,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                     AF_FSTAMP(who, n, hf * 4);
                     // issuer 0 goes on when P^T of the half is in TMEM, issuer 1 when dS^T is in shared memory
                     ok = wait_half(acc_stream, n, hf);
-                    if (ok) ok = mbar_wait_warp(&bars[(who == 0 ? L::B_PRDY : L::B_PDS) + hf], n & 1, abort_flag, 45);
+                    if (ok) ok = mbar_wait_warp_quick<D == 64>(&bars[(who == 0 ? L::B_PRDY : L::B_PDS) + hf], n & 1, abort_flag, 45);
                     if (!ok) break;
                     AF_FSTAMP(who, n, hf * 4 + 1);
                     tc_fence_after_sync();
@@ -380,7 +380,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                     if (next) {
                         ok = wait_half(t_stream, n + 1, hf);
                         // T2's half is free once the dQ'^T partial of the same rows has been read out of it
-                        if (ok && who == 1 && !kOwnDq) ok = mbar_wait_warp(&bars[L::B_T2FREE + hf], n & 1, abort_flag, 46);
+                        if (ok && who == 1 && !kOwnDq) ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_T2FREE + hf], n & 1, abort_flag, 46);
                         if (!ok) break;
                         tc_fence_after_sync();
                         AF_FSTAMP(who, n, hf * 4 + 2);
@@ -395,17 +395,17 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     } else if (warp == 3) {
         // ------------------------------------------------------------ MMA issuer 2: dQ'^T half = K'^T dS^T half -> T2 half
         {
-            bool ok = mbar_wait_warp(&bars[L::B_XFULL], 0, abort_flag, 47);
+            bool ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_XFULL], 0, abort_flag, 47);
             const uint32_t dhi = desc_hi(1024);
             const uint32_t a_lo = desc_lo(smem_u32(sX), BOX_BYTES);   // MN-major: 16 key rows (2 KB) per K step
             for (int n = 0; ok && n < n_it; ++n) {
 #pragma unroll 1   // (rolled: half the issuer's loop code; the instruction path is the tightest resource of this kernel)
                 for (int hf = 0; hf < 2; ++hf) {
                     AF_FSTAMP(6, n, hf * 4);
-                    ok = mbar_wait_warp(&bars[L::B_PDS + hf], n & 1, abort_flag, 48);
+                    ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_PDS + hf], n & 1, abort_flag, 48);
                     AF_FSTAMP(6, n, hf * 4 + 1);
                     // (own buffers: the previous tile's partial of this half must have been read out)
-                    if (ok && kOwnDq && n > 0) ok = mbar_wait_warp(&bars[L::B_T2FREE + hf], (n - 1) & 1, abort_flag, 54);
+                    if (ok && kOwnDq && n > 0) ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_T2FREE + hf], (n - 1) & 1, abort_flag, 54);
                     if (!ok) break;
                     AF_FSTAMP(6, n, hf * 4 + 2);
                     tc_fence_after_sync();
@@ -439,7 +439,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 #pragma unroll 1
             for (int hf = 0; hf < 2; ++hf) {
                 if (warp == 4) AF_FSTAMP(4, n, hf * 4);
-                ok = mbar_wait_warp(&bars[L::B_DQFULL + hf], n & 1, abort_flag, 49);
+                ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_DQFULL + hf], n & 1, abort_flag, 49);
                 if (!ok) break;
                 if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 1);
                 tc_fence_after_sync();

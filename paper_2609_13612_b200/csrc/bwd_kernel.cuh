@@ -560,7 +560,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
         for (int n = 0; n < n_it; ++n) {
             const int st = n % NST, ah = cur.head, a0 = row0_of(cur);
             advance(cur);
-            if (!mbar_wait_warp(&bars[L::B_EMPTY + st], ((n / NST) & 1) ^ 1, abort_flag, 21)) break;
+            if (!mbar_wait_warp_quick(&bars[L::B_EMPTY + st], ((n / NST) & 1) ^ 1, abort_flag, 21)) break;
             if (elect_one()) {
                 mbar_arrive_expect_tx(&bars[L::B_AFULL + st], TILE);
                 mbar_arrive_expect_tx(&bars[L::B_BFULL + st], TILE);
@@ -584,7 +584,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             const int who = warp - 1;
             bool ok = true;
             if (who == 0) {
-                ok = mbar_wait_warp(&bars[B_XREADY], 0, abort_flag, 22);
+                ok = mbar_wait_warp_quick(&bars[B_XREADY], 0, abort_flag, 22);
                 if (ok && ROT_X && p.store_x && elect_one()) {
                     // publish the rotated stationary tile (rows past S are clipped by the tensor map)
 #pragma unroll
@@ -592,7 +592,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     tma_store_commit();
                 }
             } else {
-                ok = mbar_wait_warp(&bars[L::B_YFULL], 0, abort_flag, 23);
+                ok = mbar_wait_warp_quick(&bars[L::B_YFULL], 0, abort_flag, 23);
             }
             const uint32_t xa = smem_u32(sX), ya = smem_u32(sY);
             constexpr uint32_t IDESC_TH = idesc_bf16_f32(128, 64, 0, 0);   // half tile: 64 streamed rows
@@ -614,9 +614,9 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             };
             auto wait_stream = [&](int n) {
                 const int st = n % NST;
-                bool r = mbar_wait_warp(&bars[(who == 0 ? B_AREADY : L::B_BFULL) + st], (n / NST) & 1, abort_flag, 24);
+                bool r = mbar_wait_warp_quick(&bars[(who == 0 ? B_AREADY : L::B_BFULL) + st], (n / NST) & 1, abort_flag, 24);
                 // the accumulator MMAs of issuer 1 (DKV) read A as well, those of issuer 0 (DKV) read Bc
-                if (r && DKV) r = mbar_wait_warp(&bars[(who == 0 ? L::B_BFULL : B_AREADY) + st], (n / NST) & 1, abort_flag, 25);
+                if (r && DKV) r = mbar_wait_warp_quick(&bars[(who == 0 ? L::B_BFULL : B_AREADY) + st], (n / NST) & 1, abort_flag, 25);
                 tc_fence_after_sync();
                 return r;
             };
@@ -639,7 +639,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     // this half: 4 K = 16 steps over its 64 streamed rows; the bf16 operands sit at the start of
                     // the half's own columns of T1 (issuer 0) or T2 (issuer 1)
                     AF_BSTAMP(who, n, 3 * hf);
-                    ok = mbar_wait_warp(&bars[L::B_PDS + hf], n & 1, abort_flag, 26);
+                    ok = mbar_wait_warp_quick(&bars[L::B_PDS + hf], n & 1, abort_flag, 26);
                     AF_BSTAMP(who, n, 3 * hf + 1);
                     if (!ok) break;
                     tc_fence_after_sync();
@@ -691,7 +691,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     // (listed tiles need not be consecutive: then the cos/sin state is read for every tile)
                     if (CP > 0 && (BS || (run_pos % kRotResync) == 0)) rotate_prefetch(st, p.table, a0, p.S, p.R, t);
                     AF_BSTAMP(4, n, 0);
-                    if (!mbar_wait_warp(&bars[L::B_AFULL + sg], (n / NST) & 1, abort_flag, 28)) return;
+                    if (!mbar_wait_warp_quick(&bars[L::B_AFULL + sg], (n / NST) & 1, abort_flag, 28)) return;
                     AF_BSTAMP(4, n, 1);
                     if (CP > 0) rotate_tile_fast(sA + sg * TILE, st, step, t);
                     else rotate_tile_smem(sA + sg * TILE, a0, p.S, p.R, p.table, t, 128);

@@ -126,13 +126,13 @@ constexpr int kPParts = 2;   // P is handed to the MMA issuer in two column halv
 //    first four K-steps of O += P V run while the second half of the exponentials is computed.
 // P halves sit at the start of their own 64 score columns (bf16 pairs: 32 columns each).
 // Returns false if a bounded wait gave up.
-template <int D, bool MASKED, bool ALIBI>
+template <int D, bool MASKED, bool ALIBI, bool QUICK>
 __device__ __forceinline__ bool softmax_tile_halves(uint32_t tS, uint32_t tO, int n, float scale_log2, float kb,
                                                     float bias0, int mlo, uint32_t mn, uint64_t* s_full, uint64_t* p_ready,
                                                     uint32_t parity, volatile uint32_t* abort_flag, int lane, float& m_run,
                                                     float& l_run) {
     uint32_t v[BN];
-    if (!mbar_wait_warp(&s_full[0], parity, abort_flag, 10)) return false;
+    if (!mbar_wait_warp_quick<QUICK>(&s_full[0], parity, abort_flag, 10)) return false;
     tc_fence_after_sync();
     tmem_ld32(tS, v);
     tmem_ld32(tS + 32, v + 32);
@@ -326,6 +326,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const __grid_constant__ CUtensorMap tm_t, const FwdParams p) {
     using L = FwdSmem<D, NQ, KS, VS, ROPE == kRotAll && TAB>;
     constexpr bool KROT = ROPE == kRotAll;
+    constexpr bool kQuick = NQ > 1;   // form of the waits (mbar_wait_warp_quick)
     constexpr int kSoftmaxWarp = KROT ? 8 : 4;   // the first softmax warp
     constexpr int TILE = L::TILE;
     constexpr int NBOX = D / BOX_COLS;
@@ -526,7 +527,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             for (int it = first_it; it < n_it; ++it) {
                 const int j0 = tile_at(jlo_c + it) * BN;
                 const int ks = it % KS, vs = it % VS;
-                if (!mbar_wait_warp(&bars[L::B_KEMPTY + ks], ((it / KS) & 1) ^ 1, abort_flag, 1)) break;
+                if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_KEMPTY + ks], ((it / KS) & 1) ^ 1, abort_flag, 1)) break;
                 if (elect_one()) {
                     mbar_arrive_expect_tx(&bars[L::B_KFULL + ks], TILE);
 #pragma unroll
@@ -535,13 +536,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 }
                 if (tab_tiles) {
                     // the single table stage is free once the previous tile has been rotated
-                    if (!mbar_wait_warp(&bars[L::B_TEMPTY], (it & 1) ^ 1, abort_flag, 12)) break;
+                    if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_TEMPTY], (it & 1) ^ 1, abort_flag, 12)) break;
                     if (elect_one()) {
                         mbar_arrive_expect_tx(&bars[L::B_TFULL], 256u * p.R);
                         tma_load_2d(sT, &tm_t, &bars[L::B_TFULL], 0, j0);
                     }
                 }
-                if (!mbar_wait_warp(&bars[L::B_VEMPTY + vs], ((it / VS) & 1) ^ 1, abort_flag, 2)) break;
+                if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_VEMPTY + vs], ((it / VS) & 1) ^ 1, abort_flag, 2)) break;
                 if (elect_one()) {
                     mbar_arrive_expect_tx(&bars[L::B_VFULL + vs], TILE);
 #pragma unroll
@@ -595,11 +596,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (BS && n_it <= 0) return;   // a row block without active blocks: nothing to issue
                 // S of the first key tile, each query tile as soon as it is ready (the softmax warpgroups rotate their
                 // Q tiles while the rotation warpgroup rotates K tile 0)
-                if (!mbar_wait_warp(&bars[B_KREADY + 0], 0, abort_flag, 4)) return;
+                if (!mbar_wait_warp_quick<kQuick>(&bars[B_KREADY + 0], 0, abort_flag, 4)) return;
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
                     if (jhi[q] >= jlo[q]) {
-                        if (!mbar_wait_warp(&bars[B_QREADY + q], 0, abort_flag, 3)) return;
+                        if (!mbar_wait_warp_quick<kQuick>(&bars[B_QREADY + q], 0, abort_flag, 3)) return;
                         tc_fence_after_sync();
                         if (active(q, jlo_c)) issue_S(q, 0);
                     }
@@ -609,16 +610,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     const int j = jlo_c + it, vs = it % VS, ks1 = (it + 1) % KS;
                     const bool next = it + 1 < n_it;
                     // (both are there already, as a rule: they are taken while the pipe still works on the last scores)
-                    if (!mbar_wait_warp(&bars[L::B_VFULL + vs], (it / VS) & 1, abort_flag, 5)) return;
-                    if (next && !mbar_wait_warp(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7)) return;
+                    if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_VFULL + vs], (it / VS) & 1, abort_flag, 5)) return;
+                    if (next && !mbar_wait_warp_quick<kQuick>(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7)) return;
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
                         if (active(q, j)) {
                             const uint32_t d = tmem_base + NQ * BN + q * D, a = tmem_base + q * BN, v_lo = v_lo0 + vs * (TILE >> 4);
-                            if (!mbar_wait_warp(&bars[L::B_PREADY + 4 * q], cnt[q] & 1, abort_flag, 6)) return;
+                            if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_PREADY + 4 * q], cnt[q] & 1, abort_flag, 6)) return;
                             tc_fence_after_sync();
                             mma_pv4(d, a, v_lo, dhi, IDESC_O, cnt[q] > 0 ? 1u : 0u);
-                            if (!mbar_wait_warp(&bars[L::B_PREADY + 4 * q + 1], cnt[q] & 1, abort_flag, 6)) return;
+                            if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_PREADY + 4 * q + 1], cnt[q] & 1, abort_flag, 6)) return;
                             tc_fence_after_sync();
                             mma_pv4(d, a + BN / 2, v_lo + 512, dhi, IDESC_O, 1u);
                             ++cnt[q];
@@ -644,8 +645,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int it = 0; ok && it < n_it; ++it) {
                     const int ks = it % KS;
                     AF_STAMP(1, it, 0);
-                    ok = mbar_wait_warp(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);
-                    if (ok) ok = mbar_wait_warp(&bars[L::B_TFULL], it & 1, abort_flag, 13);
+                    ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);
+                    if (ok) ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_TFULL], it & 1, abort_flag, 13);
                     AF_STAMP(1, it, 1);
                     if (!ok) break;
                     rotate_tile_tab<CP>(sK + ks * TILE, sT, t);
@@ -673,7 +674,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     if (CP > 0 && (BS || (it % kKeyRun) == 0))
                         rotate_prefetch(st, p.table, tile_at(jlo_c + it) * BN, p.S, p.R, t);
                     AF_STAMP(1, it, 0);
-                    ok = mbar_wait_warp(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);
+                    ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);
                     AF_STAMP(1, it, 1);
                     if (!ok) break;
                     if (CP > 0) rotate_tile_fast(sK + ks * TILE, st, step, t);
@@ -725,7 +726,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     rotate_load_step<CPT>(p.table, p.S, p.R, row, step);
                     rotate_prefetch(st, p.table, i0[q], p.S, p.R, row);
                 }
-                ok = mbar_wait_warp(&bars[L::B_QFULL + q], 0, abort_flag, 8);
+                ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_QFULL + q], 0, abort_flag, 8);
                 if (!ok) return;
                 if (CP > 0) rotate_tile_fast(sQ + q * TILE, st, step, row);
                 else rotate_tile_smem(sQ + q * TILE, i0[q], p.S, p.R, p.table, row, 128);
@@ -761,11 +762,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (p.relu) ok = softmax_tile_general<D, true>(tS, tO, n, p.scale_log2, slope2, j0 - i, mlo, mn, brow, cols_ok, vec, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
                 else ok = softmax_tile_general<D, false>(tS, tO, n, p.scale_log2, slope2, j0 - i, mlo, mn, brow, cols_ok, vec, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
             } else if (alibi) {
-                if (need_mask) ok = softmax_tile_halves<D, true, true>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
-                else ok = softmax_tile_halves<D, false, true>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
+                if (need_mask) ok = softmax_tile_halves<D, true, true, kQuick>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
+                else ok = softmax_tile_halves<D, false, true, kQuick>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
             } else {
-                if (need_mask) ok = softmax_tile_halves<D, true, false>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
-                else ok = softmax_tile_halves<D, false, false>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
+                if (need_mask) ok = softmax_tile_halves<D, true, false, kQuick>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
+                else ok = softmax_tile_halves<D, false, false, kQuick>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
             }
             AF_STAMP(2 + q, n, 2);
             ++n;
@@ -776,7 +777,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (GEN && p.relu) p.lse[static_cast<size_t>(bh) * p.S + i] = l_run;
             else p.lse[static_cast<size_t>(bh) * p.S + i] = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
         }
-        if (ok && jhi[q] >= jlo[q]) ok = mbar_wait_warp(&bars[L::B_ODONE + q], 0, abort_flag, 11);
+        if (ok && jhi[q] >= jlo[q]) ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_ODONE + q], 0, abort_flag, 11);
         AF_STAMP(2 + q, 63, 0);  // O complete
         if (SPLIT && parts > 1 && ok) {
             // this CTA's share, unnormalised, over the operand tiles (idle now): rows of D + 4 floats, acc[D], m, l

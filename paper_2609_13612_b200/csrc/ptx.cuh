@@ -71,9 +71,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // (Letting only lane 0 poll was measured slower: the warp woke up later.)
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
                                                uint32_t code, long long limit_cycles = kWaitLimitCycles) {
-    // (a barrier that is complete already: one test and one vote, no per-lane control flow)
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, code, limit_cycles));
+}
+// The same with one test and one vote in front: a barrier that is complete already costs no per-lane control flow, every other
+// one a little more, and every wait some code.  Pays in kernels of several tiles whose chains hide each other's waits
+// (one-pass backward at D = 64 702 -> 687 us, B = 16, 8 heads, S = 2213), costs where one chain is all there is: 13.9 -> 14.5 us
+// (forward, one query tile, B = 2, 6 / 2 heads, S = 777, window and slopes), 35.2 -> 35.5 us (backward at D = 128 of the same call),
+// 390.7 -> 392.1 us (8-bit operands, 8 heads, S = 16384).
+template <bool QUICK = true>
+__device__ __forceinline__ bool mbar_wait_warp_quick(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t code) {
+    if (QUICK && __all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return mbar_wait_warp(bar, parity, abort_flag, code);
 }
 
 // Self-test of the time-out path: one CTA, one barrier that nothing ever arrives on.  Warp 1 waits on it with
