@@ -609,9 +609,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int it = 0; it < n_it; ++it) {
                     const int j = jlo_c + it, vs = it % VS, ks1 = (it + 1) % KS;
                     const bool next = it + 1 < n_it;
-                    // (both are there already, as a rule: they are taken while the pipe still works on the last scores)
+                    // The next K is there already, as a rule.  It is taken while the pipe still works on the last scores, but with two
+                    // query tiles at D = 64, whose scores are short, between the halves of the first P V: 103.0 / 97.1 us in front / between
+                    // (B = 3, 2 / 1 heads, S = 7552, no rotation), 43.2 / 41.4 us (B = 2, 4 heads, S = 3000); D = 128 the other way round, 104.0 /
+                    // 105.1 us (8 / 2 heads, S = 7552) and 116.4 / 117.4 us (32 / 8 heads, S = 4096).
+                    constexpr bool kBetween = D == 64 && NQ == 2;
+                    bool k_waits = next;
+                    const auto k_ready = [&] {
+                        if (k_waits && !mbar_wait_warp_quick<kQuick>(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7)) return false;
+                        k_waits = false;
+                        return true;
+                    };
                     if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_VFULL + vs], (it / VS) & 1, abort_flag, 5)) return;
-                    if (next && !mbar_wait_warp_quick<kQuick>(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7)) return;
+                    if (!kBetween && !k_ready()) return;
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
                         if (active(q, j)) {
@@ -619,13 +629,17 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                             if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_PREADY + 4 * q], cnt[q] & 1, abort_flag, 6)) return;
                             tc_fence_after_sync();
                             mma_pv4(d, a, v_lo, dhi, IDESC_O, cnt[q] > 0 ? 1u : 0u);
+                            if (kBetween && !k_ready()) return;
                             if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_PREADY + 4 * q + 1], cnt[q] & 1, abort_flag, 6)) return;
                             tc_fence_after_sync();
                             mma_pv4(d, a + BN / 2, v_lo + 512, dhi, IDESC_O, 1u);
                             ++cnt[q];
                             if (is_last(q, j)) commit_elected(bar0 + 8 * (L::B_ODONE + q));
                         }
-                        if (next && active(q, j + 1)) issue_S(q, ks1);
+                        if (next && active(q, j + 1)) {
+                            if (kBetween && !k_ready()) return;
+                            issue_S(q, ks1);
+                        }
                     }
                     commit_elected(bar0 + 8 * (L::B_VEMPTY + vs));
                     if (next) commit_elected(bar0 + 8 * (L::B_KEMPTY + ks1));
