@@ -638,6 +638,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         }
                         if (next && active(q, j + 1)) {
                             if (kBetween && !k_ready()) return;
+                            if (!active(q, j)) tc_fence_after_sync();   // (else the wait for P has one behind it)
                             issue_S(q, ks1);
                         }
                     }
