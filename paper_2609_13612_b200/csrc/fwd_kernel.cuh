@@ -624,7 +624,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     if (!kBetween && !k_ready()) return;
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
-                        if (active(q, j)) {
+                        const bool now = active(q, j);
+                        if (now) {
                             const uint32_t d = tmem_base + NQ * BN + q * D, a = tmem_base + q * BN, v_lo = v_lo0 + vs * (TILE >> 4);
                             if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_PREADY + 4 * q], cnt[q] & 1, abort_flag, 6)) return;
                             tc_fence_after_sync();
@@ -638,7 +639,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         }
                         if (next && active(q, j + 1)) {
                             if (kBetween && !k_ready()) return;
-                            if (!active(q, j)) tc_fence_after_sync();   // (else the wait for P has one behind it)
+                            if (!now) tc_fence_after_sync();   // (else the wait for P has one behind it)
                             issue_S(q, ks1);
                         }
                     }
