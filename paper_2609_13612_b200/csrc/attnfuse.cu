@@ -1056,7 +1056,9 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
         two_tiles = qtiles != 1 && (!spread || (Rr > 0 && keys_bf16));   // (packed-bf16 keys: built for two)
     }
     p.keys_rotated = k_prerotated ? 1 : 0;
-    p.four_tiles = shape->D == 64 && qtiles == 2 && two_tiles && !bs_row_ptr && !bias && !relu && !keys_bf16 && four_query_tiles(p) ? heads_of_four(gqa_group) : 0;
+    // (the kernel with four query tiles adds the ALiBi term in its softmax warps: not for a caller who asked for the other way)
+    const bool four_can = two_tiles && !bs_row_ptr && !bias && !relu && !keys_bf16 && !(p.slopes && opt(AF_OPT_FWD_ALIBI_MMA) >= 2);
+    p.four_tiles = shape->D == 64 && qtiles == 2 && four_can && four_query_tiles(p) ? heads_of_four(gqa_group) : 0;
     p.keys_bf16 = keys_bf16 ? 1 : 0;
     p.bias = bias;
     p.bias_sh = (bias && bias_H > 1) ? static_cast<long long>(shape->S) * shape->S : 0;

@@ -68,3 +68,20 @@ def test_infinite_and_nan_scores_as_in_the_kernel_for_two():
         assert torch.equal(torch.isnan(a), torch.isnan(b)) and torch.equal(torch.isinf(a), torch.isinf(b))
         ok = torch.isfinite(b)
         assert (a[ok].float() - b[ok].float()).abs().max().item() <= 2.0 ** -6   # one bf16 ulp at |x| < 4, and P's rounding
+
+
+def test_alibi_by_the_tensor_core_where_it_was_asked_for():
+    """AF_OPT_FWD_ALIBI_MMA = 2 is for every forward kernel that can: with slopes it keeps away from the kernel for four, which cannot."""
+    g = torch.Generator(device="cuda").manual_seed(915)
+    q, k, v = (torch.randn(16, h, 600, 64, generator=g, device="cuda").to(torch.bfloat16) for h in (16, 4, 4))
+    slopes = torch.tensor([2.0 ** -(h / 2 + 1) for h in range(16)], dtype=torch.float32, device="cuda")
+    args = (q, k, v, af.RopeSpec(rotary_dim=0), None, af.MaskSpec(alibi_slopes=slopes), 0.125)
+    with af.option(af.OPT_FWD_ALIBI_MMA, 2):
+        got = af.fwd(*args)
+        with af.option(af.OPT_FWD_QTILES, 3):
+            want = af.fwd(*args)
+    plain = af.fwd(*args)
+    torch.cuda.synchronize()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert not torch.equal(plain[0], want[0])   # (by itself this call takes four: other last bits)
+    assert af.device_status()[0] == 0
