@@ -37,7 +37,7 @@ __device__ __forceinline__ bool softmax_block64(uint32_t tS, uint32_t tO, bool f
                                                 uint32_t mn, uint64_t* s_full, uint64_t* p_ready, uint32_t parity,
                                                 volatile uint32_t* abort_flag, int lane, float& m_run, float& l_run) {
     uint32_t v[64];
-    if (!mbar_wait_warp_quick(s_full, parity, abort_flag, 60)) return false;
+    if (!mbar_wait_warp_quick(s_full, parity, abort_flag, 80)) return false;
     tc_fence_after_sync();
     tmem_ld32(tS, v);
     tmem_ld32(tS + 32, v + 32);
@@ -198,12 +198,12 @@ attn_fwd64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         const uint32_t tS = tmem_base + q * 64, tO = tmem_base + 256 + q * 64;
         auto load = [&](int it) {   // key tile `it` into its stages, which the issuers have handed back
             const int st = it % KS, par = ((it / KS) & 1) ^ 1, j0 = (j_first + it) * 128;
-            if (!mbar_wait_warp_quick(&bars[L::B_KEMPTY + st], par, abort_flag, 61)) return false;
+            if (!mbar_wait_warp_quick(&bars[L::B_KEMPTY + st], par, abort_flag, 81)) return false;
             if (elect_one()) {
                 mbar_arrive_expect_tx(&bars[L::B_KFULL + st], TILE);
                 tma_load_4d(sK + st * TILE, &tm_k, &bars[L::B_KFULL + st], 0, j0, hk, b);
             }
-            if (!mbar_wait_warp_quick(&bars[L::B_VEMPTY + st], par, abort_flag, 62)) return false;
+            if (!mbar_wait_warp_quick(&bars[L::B_VEMPTY + st], par, abort_flag, 82)) return false;
             if (elect_one()) {
                 mbar_arrive_expect_tx(&bars[L::B_VFULL + st], TILE);
                 tma_load_4d(sV + st * TILE, &tm_v, &bars[L::B_VFULL + st], 0, j0, hk, b);
@@ -220,23 +220,23 @@ attn_fwd64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 mma_scores<D>(tS, q_lo, k_lo + (n & 1) * 512, dhi, IDESC_S);
                 commit_elected(bar0 + 8 * (L::B_SFULL + q));
             };
-            if (hi >= lo && !mbar_wait_warp_quick(&bars[B_QREADY + q], 0, abort_flag, 64)) return;
-            if (!mbar_wait_warp_quick(&bars[B_KREADY], 0, abort_flag, 63)) return;
+            if (hi >= lo && !mbar_wait_warp_quick(&bars[B_QREADY + q], 0, abort_flag, 84)) return;
+            if (!mbar_wait_warp_quick(&bars[B_KREADY], 0, abort_flag, 83)) return;
             if (lo == n_first && hi >= lo) issue_S(n_first, k_lo0);
             if ((n_first & 1) || n_first == n_last) commit_elected(bar0 + 8 * L::B_KEMPTY);
             int st = 0;   // stage of block n's key tile, and the parity of its full barriers
             uint32_t par = 0;
-            if (!mbar_wait_warp_quick(&bars[L::B_VFULL], 0, abort_flag, 65)) return;
+            if (!mbar_wait_warp_quick(&bars[L::B_VFULL], 0, abort_flag, 85)) return;
             for (int n = n_first; n <= n_last; ++n) {
                 const bool next = n < n_last, last_half = (n & 1) || !next;
                 int st1 = st;
                 uint32_t par1 = par;
                 if (n & 1) {
                     if (++st1 == KS) st1 = 0, par1 ^= 1;
-                    if (next && !mbar_wait_warp_quick(&bars[B_KREADY + st1], par1, abort_flag, 66)) return;
+                    if (next && !mbar_wait_warp_quick(&bars[B_KREADY + st1], par1, abort_flag, 86)) return;
                 }
                 if (n >= lo && n <= hi) {
-                    if (!mbar_wait_warp_quick(&bars[L::B_PREADY + q], (n - lo) & 1, abort_flag, 67)) return;
+                    if (!mbar_wait_warp_quick(&bars[L::B_PREADY + q], (n - lo) & 1, abort_flag, 87)) return;
                     tc_fence_after_sync();
                     mma_pv4(tO, tS, v_lo0 + st * (TILE >> 4) + (n & 1) * 512, dhi, IDESC_O, n > lo ? 1u : 0u);
                 }
@@ -248,7 +248,7 @@ attn_fwd64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     const int it = (n >> 1) - j_first;
                     // (the stage of the tile before this one)
                     if (warp == 0 && it > 0 && it + KS - 1 < n_tiles && !load(it + KS - 1)) return;
-                    if (next && !mbar_wait_warp_quick(&bars[L::B_VFULL + st1], par1, abort_flag, 65)) return;
+                    if (next && !mbar_wait_warp_quick(&bars[L::B_VFULL + st1], par1, abort_flag, 85)) return;
                 }
                 st = st1;
                 par = par1;
@@ -268,7 +268,7 @@ attn_fwd64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 for (int it = 0; ok && it < n_tiles; ++it) {
                     const int ks = it % KS;
                     if (CP > 0 && (it % kKeyRun) == 0) rotate_prefetch(st, p.table, (j_first + it) * 128, p.S, p.R, t);
-                    ok = mbar_wait_warp_quick(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 68);
+                    ok = mbar_wait_warp_quick(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 88);
                     if (!ok) break;
                     if (CP > 0) rotate_tile_fast(sK + ks * TILE, st, step, t);
                     else rotate_tile_smem(sK + ks * TILE, (j_first + it) * 128, p.S, p.R, p.table, t, 128);
@@ -305,7 +305,7 @@ attn_fwd64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     rotate_load_step<CPT>(p.table, p.S, p.R, row, step);
                     rotate_prefetch(st, p.table, my_i0, p.S, p.R, row);
                 }
-                ok = mbar_wait_warp_quick(&bars[L::B_QFULL + q], 0, abort_flag, 69);
+                ok = mbar_wait_warp_quick(&bars[L::B_QFULL + q], 0, abort_flag, 89);
                 if (!ok) return;
                 if (CP > 0) rotate_tile_fast(tile, st, step, row);
                 else rotate_tile_smem(tile, my_i0, p.S, p.R, p.table, row, 128);
@@ -345,7 +345,7 @@ attn_fwd64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         const int bh = b * p.Hq + my_h;
         if (ok && my_hi >= my_lo && p.lse && i < p.S)
             p.lse[static_cast<size_t>(bh) * p.S + i] = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
-        if (ok && my_hi >= my_lo) ok = mbar_wait_warp_quick(&bars[L::B_ODONE + q], 0, abort_flag, 70);
+        if (ok && my_hi >= my_lo) ok = mbar_wait_warp_quick(&bars[L::B_ODONE + q], 0, abort_flag, 90);
         if (my_hi >= my_lo) {
             tc_fence_after_sync();
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
