@@ -63,7 +63,8 @@ typedef struct { float theta; int rotary_dim; int pos_offset; } af_rope;
  * the scaled score. */
 typedef struct { int causal; int window; const float* alibi_slopes; } af_mask;
 
-int         attnfuse_version(void);   /* 100 x major + minor: 110 adds the variant, one-pass backward and fp8 entries, 111 the list lengths of af_blocks */
+int         attnfuse_version(void);   /* 100 x major + minor: 110 adds the variant, one-pass backward and fp8 entries, 111 the list lengths of af_blocks,
+                                         112 attnfuse_fwd_scratch and value 4 of AF_OPT_FWD_QTILES */
 const char* attnfuse_strerror(af_status st);
 
 /* ---- tuning options ---------------------------------------------------------------------------------
@@ -76,9 +77,12 @@ const char* attnfuse_strerror(af_status st);
  * attnfuse_get_option returns -1 for one. */
 typedef enum {
     AF_OPT_FWD_QTILES = 0,     /* AF_FWD_NQ, default 2: query tiles per CTA of the forward kernel: 2 = two, or one where two
-                                  would leave SMs idle; 1 = one; 3 = always two */
+                                  would leave SMs idle, or four (D = 64, dense masks) where they fill the device;
+                                  1 = one; 3 = always two; 4 = four wherever they are built, else two.  Four tiles
+                                  take the keys in steps of 64: last bits differ from those of one or two */
     AF_OPT_FWD_PAIR_HEADS = 1, /* AF_FWD_PAIR, default 1: with an even GQA group the two query tiles of a CTA are two
-                                  heads of one kv head; 0: two consecutive row blocks of one head */
+                                  heads of one kv head (four tiles: four or two heads, as the group allows);
+                                  0: consecutive row blocks of one head */
     AF_OPT_FWD_KEYS_BF16 = 2,  /* AF_FWD_KEYS_BF16, default 0: key tiles rotated in packed bf16 arithmetic (faster,
                                   about 1.4 times the rounding error on rotated keys; forward only) */
     AF_OPT_BS_ROWPAIR = 3,     /* AF_BS_ROWPAIR, default 1: block-sparse forward with an odd GQA group gives a CTA two
@@ -92,7 +96,8 @@ typedef enum {
                                   more K step of the score product (the slope split into two bf16 values, the key column
                                   exact in bf16) instead of one fused multiply-add per score in the softmax warps - in the kernels that rotate
                                   on chip, where it measured faster; 2: in every forward kernel; 0: never.  Not used by the additive_bias / relu_attention variants nor together with
-                                  AF_OPT_FWD_KEYS_BF16 (no shared memory left for the two small operand tiles) */
+                                  AF_OPT_FWD_KEYS_BF16 (no shared memory left for the two small operand tiles), nor by
+                                  the kernel with four query tiles, which 2 therefore keeps calls with slopes away from */
     AF_OPT_COUNT_ = 6
 } af_option;
 af_status attnfuse_set_option(af_option option, int value);

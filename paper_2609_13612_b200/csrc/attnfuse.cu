@@ -446,6 +446,8 @@ bool four_query_tiles(const FwdParams& p) {
     return time(fwd_grid(p, 4 / quad, quad), 8.0, 2.85) < 0.98 * time(fwd_grid(p, 2 / pair, pair), 7.0, 1.6);
 }
 
+bool takes_four(const FwdParams& p, int D, int qtiles) { return D == 64 && (qtiles == 4 || (qtiles == 2 && four_query_tiles(p))); }
+
 // Four query tiles per CTA (D = 64, dense masks; fwd64_kernel.cuh).
 template <int ROPE>
 af_status launch_fwd64(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to, FwdParams p,
@@ -825,7 +827,7 @@ size_t bwd_dqacc_bytes(const af_shape* sh) {
 
 extern "C" {
 
-int attnfuse_version(void) { return 111; }
+int attnfuse_version(void) { return 112; }
 
 const char* attnfuse_strerror(af_status st) {
     switch (st) {
@@ -960,7 +962,7 @@ bool keys_once(const af_shape* sh, const af_rope* rope, const af_mask* mask) {
     p.heads = static_cast<long long>(sh->B) * sh->Hq;
     const int qtiles = opt(AF_OPT_FWD_QTILES);
     if (qtiles == 1 || (qtiles == 2 && one_query_tile(p, sh->D))) return false;
-    const bool four = sh->D == 64 && qtiles == 2 && four_query_tiles(p);
+    const bool four = takes_four(p, sh->D, qtiles);
     const int heads = four ? heads_of_four(p.group) : (p.group % 2) == 0 && opt(AF_OPT_FWD_PAIR_HEADS) ? 2 : 1;
     const FwdGrid g = fwd_grid(p, (four ? 4 : 2) / heads, heads);
     const double visits = g.sum / (sm_count() > 0 ? sm_count() : 148);
@@ -1058,7 +1060,7 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     p.keys_rotated = k_prerotated ? 1 : 0;
     // (the kernel with four query tiles adds the ALiBi term in its softmax warps: not for a caller who asked for the other way)
     const bool four_can = two_tiles && !bs_row_ptr && !bias && !relu && !keys_bf16 && !(p.slopes && opt(AF_OPT_FWD_ALIBI_MMA) >= 2);
-    p.four_tiles = shape->D == 64 && qtiles == 2 && four_can && four_query_tiles(p) ? heads_of_four(gqa_group) : 0;
+    p.four_tiles = four_can && takes_four(p, shape->D, qtiles) ? heads_of_four(gqa_group) : 0;
     p.keys_bf16 = keys_bf16 ? 1 : 0;
     p.bias = bias;
     p.bias_sh = (bias && bias_H > 1) ? static_cast<long long>(shape->S) * shape->S : 0;

@@ -28,6 +28,11 @@ W = synth.Workload
     W("noncausal_window", 12, 9, 9, 500, 64, theta=1e4, causal=False, window=130, seed_id=911),
     W("no_rotation", 12, 16, 4, 520, 64, rotary_dim=0, seed_id=912),
     W("rotary_48", 12, 12, 12, 400, 64, theta=1e4, rotary_dim=48, seed_id=913),
+    # (128 k - window) / 64 is odd where window mod 128 is 1 ... 64: a CTA's first step is the second half of a key tile
+    W("odd_first_step", 6, 8, 2, 700, 64, theta=1e4, window=40, rotary_dim=32, seed_id=916),
+    W("odd_first_step_rows", 4, 6, 6, 1300, 64, theta=1e4, window=130, rotary_dim=16, seed_id=917),
+    W("odd_first_step_noncausal", 3, 9, 3, 1100, 64, theta=1e4, causal=False, window=150, seed_id=918),
+    W("odd_first_step_alibi", 3, 4, 2, 900, 64, theta=1e4, window=300, alibi=True, seed_id=919),
 ], ids=lambda w: w.name)
 @pytest.mark.parametrize("out_dtype", [torch.bfloat16, torch.float32], ids=["bf16", "fp32"])
 def test_against_the_oracle_and_the_kernel_for_two(w, out_dtype):
@@ -40,7 +45,8 @@ def test_against_the_oracle_and_the_kernel_for_two(w, out_dtype):
     for call in (af.fwd, af.fwd_hybrid):
         o = torch.full((w.B, w.Hq, w.S, w.D), float("nan"), dtype=out_dtype, device="cuda")
         lse = torch.full((w.B, w.Hq, w.S), float("nan"), dtype=torch.float32, device="cuda")
-        call(dev["q"], dev["k"], dev["v"], rope, table, mask, w.scale, out=o, lse=lse)
+        with af.option(af.OPT_FWD_QTILES, 4):
+            call(dev["q"], dev["k"], dev["v"], rope, table, mask, w.scale, out=o, lse=lse)
         torch.cuda.synchronize()
         assert af.device_status()[0] == 0
         pu.assert_close_scaled(w.name, pu.to_np(o), want_o)
@@ -49,6 +55,25 @@ def test_against_the_oracle_and_the_kernel_for_two(w, out_dtype):
         o2, _ = af.fwd(dev["q"], dev["k"], dev["v"], rope, table, mask, w.scale, out_dtype=out_dtype)
     torch.cuda.synchronize()
     pu.assert_close_scaled(w.name + " two", pu.to_np(o2), want_o)
+    if w.S >= 128 and w.window != 0:   # (steps of 64 keys: other last bits, where rows have more than a step)
+        assert not torch.equal(o, o2)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,S,window,four", [
+    (16, 16, 4, 600, -1, True), (4, 12, 12, 4096, -1, True), (8, 12, 12, 1024, -1, True), (16, 8, 4, 900, 70, True),
+    (1, 16, 4, 2048, -1, False), (2, 12, 12, 4096, -1, False), (16, 6, 6, 577, -1, False),
+])
+def test_which_calls_take_four(B, Hq, Hkv, S, window, four):
+    g = torch.Generator(device="cuda").manual_seed(920)
+    q, k, v = (torch.randn(B, h, S, 64, generator=g, device="cuda").to(torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    got = {}
+    for option in (2, 3, 4):
+        with af.option(af.OPT_FWD_QTILES, option):
+            got[option] = af.fwd(q, k, v, af.RopeSpec(rotary_dim=0), None, af.MaskSpec(window=window), 0.125, out_dtype=torch.float32)[0]
+    torch.cuda.synchronize()
+    assert not torch.equal(got[3], got[4])
+    assert torch.equal(got[2], got[4 if four else 3])
+    assert af.device_status()[0] == 0
 
 
 def test_infinite_and_nan_scores_as_in_the_kernel_for_two():
@@ -59,12 +84,12 @@ def test_infinite_and_nan_scores_as_in_the_kernel_for_two():
     k[:, :, 7] = float("-inf")
     k[:, 1, 200] = float("nan")
     got = {}
-    for option in (2, 3):
+    for option in (4, 3):
         with af.option(af.OPT_FWD_QTILES, option):
             got[option] = af.fwd(q, k, v, af.RopeSpec(rotary_dim=0), None, af.MaskSpec(), 0.125)
     torch.cuda.synchronize()
     assert af.device_status()[0] == 0
-    for a, b in zip(got[2], got[3]):
+    for a, b in zip(got[4], got[3]):
         assert torch.equal(torch.isnan(a), torch.isnan(b)) and torch.equal(torch.isinf(a), torch.isinf(b))
         ok = torch.isfinite(b)
         assert (a[ok].float() - b[ok].float()).abs().max().item() <= 2.0 ** -6   # one bf16 ulp at |x| < 4, and P's rounding

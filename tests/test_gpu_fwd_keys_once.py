@@ -21,7 +21,7 @@ def scratch_bytes(B, Hq, Hkv, S, D, R, causal=True, window=-1, slopes=None):
     (1, 40, 8, 5000, 128, 32, True),
     (2, 16, 4, 5200, 128, 16, False),
     (1, 32, 8, 2049, 128, 96, True),     # no angle-addition walk: the table is read for every row
-    (4, 12, 12, 2300, 64, 64, True),     # four query tiles per CTA
+    (4, 12, 12, 2300, 64, 64, True),
     (4, 12, 4, 1700, 64, 32, False),
 ])
 def test_same_bits_as_on_chip(B, Hq, Hkv, S, D, R, causal):
@@ -38,6 +38,51 @@ def test_same_bits_as_on_chip(B, Hq, Hkv, S, D, R, causal):
     torch.cuda.synchronize()
     assert af.device_status()[0] == 0
     assert torch.equal(o, want_o) and torch.equal(lse, want_l) and torch.equal(kv, before)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,S,R,causal", [(4, 16, 4, 2300, 64, True), (8, 16, 4, 2300, 32, True), (8, 16, 4, 4600, 16, True),
+                                                 (4, 16, 4, 2300, 48, True), (4, 9, 9, 1900, 64, False), (4, 12, 6, 2111, 64, True)])
+def test_same_bits_with_four_query_tiles(B, Hq, Hkv, S, R, causal):
+    g = torch.Generator(device="cuda").manual_seed(923)
+    q, k, v = (torch.randn(B, h, S, 64, generator=g, device="cuda").to(torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    rope, mask = af.RopeSpec(theta=1e4, rotary_dim=R), af.MaskSpec(causal=causal)
+    args = (q, k, v, rope, af.rope_table(rope, S), mask, 0.125)
+    with af.option(af.OPT_FWD_QTILES, 4):
+        assert scratch_bytes(B, Hq, Hkv, S, 64, R, causal) == B * Hkv * S * 64 * 2
+        got, want = af.fwd(*args), af.fwd_variant(*args)
+    with af.option(af.OPT_FWD_QTILES, 3):
+        two = af.fwd(*args)
+    torch.cuda.synchronize()
+    assert af.device_status()[0] == 0
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert not torch.equal(got[0], two[0])
+
+
+def test_scratch_that_is_missing_short_or_misaligned():
+    B, Hq, Hkv, S, D = 1, 16, 4, 3000, 128
+    g = torch.Generator(device="cuda").manual_seed(924)
+    q, k, v = (torch.randn(B, h, S, D, generator=g, device="cuda").to(torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    rope = af.RopeSpec(theta=1e4, rotary_dim=D)
+    table = af.rope_table(rope, S)
+    want = af.fwd_variant(q, k, v, rope, table, af.MaskSpec(), 0.09)
+    n = scratch_bytes(B, Hq, Hkv, S, D, D)
+    assert n > 0
+    scratch = torch.empty(n + 16, dtype=torch.uint8, device="cuda")
+    sh, r, m = b._Shape(B, Hq, Hkv, S, D), b._Rope(1e4, D, 0), b._Mask(1, -1, None)
+    for at, size, status in ((None, 0, 0), (scratch.data_ptr(), n - 1, 0), (scratch.data_ptr(), n, 0), (scratch.data_ptr() + 8, n, 4)):
+        scratch.fill_(7)
+        o, lse = torch.full_like(q, 3.0), torch.full((B, Hq, S), 3.0, device="cuda")
+        assert af.lib().attnfuse_fwd_scratch(ctypes.byref(sh), q.data_ptr(), k.data_ptr(), v.data_ptr(), None, None, ctypes.byref(r),
+                                             table.data_ptr(), ctypes.byref(m), Hq // Hkv, 0.09, o.data_ptr(), 0, lse.data_ptr(), at, size,
+                                             torch.cuda.current_stream().cuda_stream) == status
+        torch.cuda.synchronize()
+        if status:
+            assert o.eq(3.0).all() and lse.eq(3.0).all()
+        else:
+            assert torch.equal(o, want[0]) and torch.equal(lse, want[1])
+        used = not scratch[:n].eq(7).all()
+        assert used == (size == n and status == 0) and scratch[n:].eq(7).all()
+    assert af.device_status()[0] == 0
 
 
 def test_where_no_scratch_is_used():
