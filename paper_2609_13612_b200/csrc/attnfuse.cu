@@ -430,22 +430,61 @@ FwdGrid fwd_grid(const FwdParams& p, int rows, int heads) {
     g.ctas *= units;
     return g;
 }
-// Four query tiles per CTA or two (D = 64)?  Four are faster per tile, 2.85 against 2 x 1.6 us per key tile, but make fewer and longer
-// CTAs.  The longer of the longest CTA and the work over the SMs decides, or, where all CTAs are about as long, the number of
-// waves (203 / 246 us at 16 / 4 heads, S = 5000, no causal mask: 160 CTAs of four); measured, two / four: 200 / 185 us (B = 4, 12
-// heads, S = 4096: 384 CTAs of four), 44.7 / 37.1 us (B = 8, S = 1024: 192), 98 / 104 us (B = 2, S = 4096: 192, with longer
-// ones), 38.8 / 56.7 us (32 / 8 heads, S = 2048: 128).
+// Estimated time of a dense forward grid whose CTAs take `rows` consecutive row blocks of `heads` heads each: every CTA goes to the SM that
+// is free first, in launch order.  In us: cta (set-up and epilogue of a CTA) and tile (a key tile, if all its query tiles see it).
+double grid_time(const FwdParams& p, int rows, int heads, double cta, double tile) {
+    struct Group {   // SMs that are free at the same time
+        double at;
+        long long sms;
+    };
+    constexpr int kMax = 256;
+    Group q[kMax + 1];   // by time; at most one group per SM, and one more while one is split
+    const int sms = sm_count() > 0 ? (sm_count() < kMax ? sm_count() : kMax) : 148;
+    int n = 1;
+    q[0] = {0.0, sms};
+    double end = 0.0;
+    const int blocks = (p.S + BM - 1) / BM;
+    for (int r = (blocks - 1) / rows * rows; r >= 0; r -= rows) {
+        double pairs = 0.0;   // query tiles times the key tiles that they see
+        for (int x = r; x < r + rows && x < blocks; ++x) {
+            const int hi = p.causal ? x : (p.window >= 0 ? (x * BM + BM - 1 + p.window) / BN : blocks - 1);
+            const int lo = p.window >= 0 && x * BM > p.window ? (x * BM - p.window) / BN : 0;
+            pairs += (hi < blocks - 1 ? hi : blocks - 1) - lo + 1;
+        }
+        const double len = cta + tile * pairs / rows;
+        for (long long left = p.heads / heads; left > 0;) {
+            const Group first = q[0];
+            const long long k = first.sms < left ? first.sms : left;
+            left -= k;
+            int from = 0;   // groups that stay: q[from, n)
+            if (k == first.sms) from = 1;
+            else q[0].sms -= k;
+            const double at = first.at + len;
+            int i = n;
+            while (i > from && q[i - 1].at > at) --i;
+            // one place to the left for what stays in front of the new group, if the first one is gone; else one to the right behind it
+            if (from) {
+                for (int j = 1; j < i; ++j) q[j - 1] = q[j];
+                q[i - 1] = {at, k};
+            } else {
+                for (int j = n; j > i; --j) q[j] = q[j - 1];
+                q[i] = {at, k};
+                ++n;
+            }
+            end = at > end ? at : end;
+        }
+    }
+    return end;
+}
+// Four query tiles per CTA or two (D = 64)?  Four are faster per tile, 3.1 against 2 x 1.6 us per key tile, but make fewer and longer
+// CTAs; what that means for the last wave decides, so the grids are played through (fitted to 150 measured ones: the choice costs
+// 0.2 % on average and 9 % at worst).  Measured, two / four: 200 / 185 us (B = 4, 12 heads, S = 4096), 44.7 / 37.1 us (B = 8, 12 heads,
+// S = 1024), 58.5 / 75.2 us (8 / 2 heads, S = 6128, window 2364), 63.3 / 100.9 us (B = 3, 4 heads, S = 3200, window 1586 to both sides),
+// 174.7 / 138.9 us (B = 4, 36 / 12 heads, S = 3270, window 136), 98 / 104 us (B = 2, 12 heads, S = 4096), 38.8 / 56.7 us (32 / 8 heads, S = 2048).
 bool four_query_tiles(const FwdParams& p) {
     const int pair = (p.group % 2) == 0 && opt(AF_OPT_FWD_PAIR_HEADS) ? 2 : 1, quad = heads_of_four(p.group);
-    const double sms = sm_count();
-    auto time = [&](const FwdGrid& g, double cta, double tile) {
-        const double chain = cta + tile * g.longest, all = (cta * g.ctas + tile * g.sum) / sms;
-        if (g.sum > 0.75 * g.longest * g.ctas) return chain * ceil(g.ctas / sms);
-        return chain > all ? chain : all;
-    };
-    return time(fwd_grid(p, 4 / quad, quad), 8.0, 2.85) < 0.98 * time(fwd_grid(p, 2 / pair, pair), 7.0, 1.6);
+    return grid_time(p, 4 / quad, quad, 7.0, 3.1) < grid_time(p, 2 / pair, pair, 7.0, 1.6);
 }
-
 bool takes_four(const FwdParams& p, int D, int qtiles) { return D == 64 && (qtiles == 4 || (qtiles == 2 && four_query_tiles(p))); }
 
 // Four query tiles per CTA (D = 64, dense masks; fwd64_kernel.cuh).

@@ -61,7 +61,9 @@ def test_against_the_oracle_and_the_kernel_for_two(w, out_dtype):
 
 @pytest.mark.parametrize("B,Hq,Hkv,S,window,four", [
     (16, 16, 4, 600, -1, True), (4, 12, 12, 4096, -1, True), (8, 12, 12, 1024, -1, True), (16, 8, 4, 900, 70, True),
-    (1, 16, 4, 2048, -1, False), (2, 12, 12, 4096, -1, False), (16, 6, 6, 577, -1, False),
+    (1, 16, 4, 2048, -1, False), (2, 12, 12, 4096, -1, False),
+    # grids whose last wave decides (two / four: 58 / 75, 175 / 139, 64 / 51 us)
+    (1, 8, 2, 6128, 2364, False), (4, 36, 12, 3270, 136, True), (8, 24, 8, 896, -1, True),
 ])
 def test_which_calls_take_four(B, Hq, Hkv, S, window, four):
     g = torch.Generator(device="cuda").manual_seed(920)
