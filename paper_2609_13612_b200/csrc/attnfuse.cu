@@ -431,8 +431,9 @@ FwdGrid fwd_grid(const FwdParams& p, int rows, int heads) {
     return g;
 }
 // Estimated time of a dense forward grid whose CTAs take `rows` consecutive row blocks of `heads` heads each: every CTA goes to the SM that
-// is free first, in launch order.  In us: cta (set-up and epilogue of a CTA) and tile (a key tile, if all its query tiles see it).
-double grid_time(const FwdParams& p, int rows, int heads, double cta, double tile) {
+// is free first, in launch order.  In us: cta (set-up and epilogue of a CTA), tile (a key tile, if all its query tiles see it) and least
+// (a key tile that only some of them see, at least).
+double grid_time(const FwdParams& p, int rows, int heads, double cta, double tile, double least) {
     struct Group {   // SMs that are free at the same time
         double at;
         long long sms;
@@ -446,12 +447,17 @@ double grid_time(const FwdParams& p, int rows, int heads, double cta, double til
     const int blocks = (p.S + BM - 1) / BM;
     for (int r = (blocks - 1) / rows * rows; r >= 0; r -= rows) {
         double pairs = 0.0;   // query tiles times the key tiles that they see
+        int last = -1, first_key = blocks;
         for (int x = r; x < r + rows && x < blocks; ++x) {
             const int hi = p.causal ? x : (p.window >= 0 ? (x * BM + BM - 1 + p.window) / BN : blocks - 1);
             const int lo = p.window >= 0 && x * BM > p.window ? (x * BM - p.window) / BN : 0;
-            pairs += (hi < blocks - 1 ? hi : blocks - 1) - lo + 1;
+            const int end_key = hi < blocks - 1 ? hi : blocks - 1;
+            pairs += end_key - lo + 1;
+            last = end_key > last ? end_key : last;
+            first_key = lo < first_key ? lo : first_key;
         }
-        const double len = cta + tile * pairs / rows;
+        const double all = tile * pairs / rows, chain = least * (last - first_key + 1);
+        const double len = cta + (all > chain ? all : chain);
         for (long long left = p.heads / heads; left > 0;) {
             const Group first = q[0];
             const long long k = first.sms < left ? first.sms : left;
@@ -477,13 +483,13 @@ double grid_time(const FwdParams& p, int rows, int heads, double cta, double til
     return end;
 }
 // Four query tiles per CTA or two (D = 64)?  Four are faster per tile, 3.1 against 2 x 1.6 us per key tile, but make fewer and longer
-// CTAs; what that means for the last wave decides, so the grids are played through (fitted to 150 measured ones: the choice costs
+// CTAs; what that means for the last wave decides, so the grids are played through (fitted to 300 measured ones: the choice costs
 // 0.2 % on average and 9 % at worst).  Measured, two / four: 200 / 185 us (B = 4, 12 heads, S = 4096), 44.7 / 37.1 us (B = 8, 12 heads,
 // S = 1024), 58.5 / 75.2 us (8 / 2 heads, S = 6128, window 2364), 63.3 / 100.9 us (B = 3, 4 heads, S = 3200, window 1586 to both sides),
 // 174.7 / 138.9 us (B = 4, 36 / 12 heads, S = 3270, window 136), 98 / 104 us (B = 2, 12 heads, S = 4096), 38.8 / 56.7 us (32 / 8 heads, S = 2048).
 bool four_query_tiles(const FwdParams& p) {
     const int pair = (p.group % 2) == 0 && opt(AF_OPT_FWD_PAIR_HEADS) ? 2 : 1, quad = heads_of_four(p.group);
-    return grid_time(p, 4 / quad, quad, 7.0, 3.1) < grid_time(p, 2 / pair, pair, 7.0, 1.6);
+    return grid_time(p, 4 / quad, quad, 7.0, 3.1, 0.0) < 0.98 * grid_time(p, 2 / pair, pair, 7.0, 1.6, 1.4);
 }
 bool takes_four(const FwdParams& p, int D, int qtiles) { return D == 64 && (qtiles == 4 || (qtiles == 2 && four_query_tiles(p))); }
 
