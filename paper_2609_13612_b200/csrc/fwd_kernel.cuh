@@ -682,14 +682,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 RotStep step;
                 RotState<(CP > 0 ? CP : 1)> st;
                 if (CP > 0) rotate_load_step<(CP > 0 ? CP : 1)>(p.table, p.S, p.R, t, step);
-                if (CP > 0 && !BS) rotate_prefetch(st, p.table, jlo_c * BN, p.S, p.R, t);
                 // (each Q tile is rotated by its own softmax warpgroup, which has nothing else to do yet)
                 // K tiles are consecutive: the recurrence carries the cos/sin state from tile to tile
                 for (int it = 0; ok && it < n_it; ++it) {
                     const int ks = it % KS;
-                    // (listed tiles need not be consecutive: the cos/sin state is read for every tile; the first one of a dense mask is
-                    // asked for above, in front of the first wait)
-                    if (CP > 0 && (BS || (it > 0 && (it % kKeyRun) == 0)))
+                    // (listed tiles need not be consecutive: the cos/sin state is read for every tile)
+                    if (CP > 0 && (BS || (it % kKeyRun) == 0))
                         rotate_prefetch(st, p.table, tile_at(jlo_c + it) * BN, p.S, p.R, t);
                     AF_STAMP(1, it, 0);
                     ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);
