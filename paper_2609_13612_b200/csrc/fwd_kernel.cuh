@@ -613,10 +613,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     // query tiles at D = 64, whose scores are short, between the halves of the first P V: 103.0 / 97.1 us in front / between
                     // (B = 3, 2 / 1 heads, S = 7552, no rotation), 43.2 / 41.4 us (B = 2, 4 heads, S = 3000); D = 128 the other way round, 104.0 /
                     // 105.1 us (8 / 2 heads, S = 7552) and 116.4 / 117.4 us (32 / 8 heads, S = 4096).
+                    // (The fence: a query tile that joins at this key tile has no wait for P in front of its scores.)
                     constexpr bool kBetween = D == 64 && NQ == 2;
                     bool k_waits = next;
                     const auto k_ready = [&] {
                         if (k_waits && !mbar_wait_warp_quick<kQuick>(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7)) return false;
+                        tc_fence_after_sync();
                         k_waits = false;
                         return true;
                     };
@@ -624,8 +626,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     if (!kBetween && !k_ready()) return;
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
-                        const bool now = active(q, j);
-                        if (now) {
+                        if (active(q, j)) {
                             const uint32_t d = tmem_base + NQ * BN + q * D, a = tmem_base + q * BN, v_lo = v_lo0 + vs * (TILE >> 4);
                             if (!mbar_wait_warp_quick<kQuick>(&bars[L::B_PREADY + 4 * q], cnt[q] & 1, abort_flag, 6)) return;
                             tc_fence_after_sync();
@@ -639,7 +640,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         }
                         if (next && active(q, j + 1)) {
                             if (kBetween && !k_ready()) return;
-                            if (!now) tc_fence_after_sync();   // (else the wait for P has one behind it)
                             issue_S(q, ks1);
                         }
                     }
