@@ -612,9 +612,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     // The next K is there already, as a rule.  It is taken while the pipe still works on the last scores, but with two
                     // query tiles at D = 64, whose scores are short, between the halves of the first P V: 103.0 / 97.1 us in front / between
                     // (B = 3, 2 / 1 heads, S = 7552, no rotation), 43.2 / 41.4 us (B = 2, 4 heads, S = 3000); D = 128 the other way round, 104.0 /
-                    // 105.1 us (8 / 2 heads, S = 7552) and 116.4 / 117.4 us (32 / 8 heads, S = 4096).
+                    // 105.1 us (8 / 2 heads, S = 7552) and 116.4 / 117.4 us (32 / 8 heads, S = 4096), and so keys that are rotated here, 17.4 /
+                    // 18.0 us (B = 8, 4 heads, S = 768, D = 64).
                     // (The fence: a query tile that joins at this key tile has no wait for P in front of its scores.)
-                    constexpr bool kBetween = D == 64 && NQ == 2;
+                    constexpr bool kBetween = D == 64 && NQ == 2 && !KROT;
                     bool k_waits = next;
                     const auto k_ready = [&] {
                         if (k_waits && !mbar_wait_warp_quick<kQuick>(&bars[B_KREADY + ks1], ((it + 1) / KS) & 1, abort_flag, 7)) return false;
