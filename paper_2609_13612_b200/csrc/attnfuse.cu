@@ -797,12 +797,6 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
     if (st != AF_OK) return st;
     p.delta = delta;
     const unsigned tiles = static_cast<unsigned>((sh->S + 127) / 128);
-#ifdef AF_TRACE
-    // tracing builds only: 1 = dK/dV kernel only, 2 = dQ kernel only (the skipped outputs stay unwritten)
-    const int only = getenv("AF_BWD_ONLY") ? atoi(getenv("AF_BWD_ONLY")) : 0;
-#else
-    constexpr int only = 0;
-#endif
     dim3 gkv(sh->B * sh->Hkv, tiles, 1), gq(sh->B * sh->Hq, tiles, 1);
     if (p.bias || p.relu) {
         // additive_bias / relu_attention: the both-caches set-up with rotation, the plain one without
@@ -818,7 +812,7 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
         p.out1 = dv; p.out2 = dk; p.out_f32 = dkv_f32; p.store_x = 0;
         return launch_bwd_gen<D, true, false>(tk, tv, tq, tdo, tk, p, gkv, stream);
     }
-    if (k_cached && only == 0) {
+    if (k_cached) {
         // both caches: K' by the set-up pass, Q' by the dQ kernel, no on-chip rotation in the dK/dV loop
         p.out1 = dq; p.out2 = nullptr; p.out_f32 = dq_f32; p.store_x = 1;
         role_lists(false);
@@ -827,13 +821,12 @@ af_status launch_bwd_mma(const af_shape* sh, const CUtensorMap& tq, const CUtens
         role_lists(true);
         return launch_bwd_variant<D, true, false, false>(*tkp, tv, *tqp, tdo, tk, p, gkv, stream);
     }
-    const bool cache = p.R > 0 && tkp != nullptr && only != 2;
+    const bool cache = p.R > 0 && tkp != nullptr;
     p.out1 = dv; p.out2 = dk; p.out_f32 = dkv_f32; p.store_x = cache ? 1 : 0;
     role_lists(true);
-    st = only == 2 ? AF_OK
-         : p.R > 0 ? launch_bwd_variant<D, true, true, true>(tk, tv, tq, tdo, cache ? *tkp : tk, p, gkv, stream)
-                   : launch_bwd_variant<D, true, false, false>(tk, tv, tq, tdo, tk, p, gkv, stream);
-    if (st != AF_OK || only == 1) return st;
+    st = p.R > 0 ? launch_bwd_variant<D, true, true, true>(tk, tv, tq, tdo, cache ? *tkp : tk, p, gkv, stream)
+                 : launch_bwd_variant<D, true, false, false>(tk, tv, tq, tdo, tk, p, gkv, stream);
+    if (st != AF_OK) return st;
     p.out1 = dq; p.out2 = nullptr; p.out_f32 = dq_f32; p.store_x = 0;
     role_lists(false);
     if (p.R == 0) return launch_bwd_variant<D, false, false, false>(tq, tdo, tk, tv, tk, p, gq, stream);
@@ -1111,10 +1104,6 @@ af_status fwd_impl(const af_shape* shape, const void* q, const void* k, const vo
     p.bias_sh = (bias && bias_H > 1) ? static_cast<long long>(shape->S) * shape->S : 0;
     p.bias_sb = (bias && bias_B > 1) ? static_cast<long long>(bias_H) * shape->S * shape->S : 0;
     p.relu = relu ? 1 : 0;
-#ifdef AF_TRACE
-    p.trace = reinterpret_cast<long long*>(getenv("AF_TRACE_PTR") ? strtoull(getenv("AF_TRACE_PTR"), nullptr, 0) : 0ull);
-    cudaMemcpyToSymbol(af::g_trace, &p.trace, sizeof(p.trace));
-#endif
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     if (bs_row_ptr)
         return shape->D == 128 ? launch_fwd_blocks<128>(tq, tk, tv, to, tt, p, two_tiles, stream)

@@ -73,16 +73,6 @@ struct BwdFusedSmem {
     static_assert(2 * 128 * STG_STRIDE * 4 <= OFF_STATS, "both staging buffers must fit in the operand tiles");
 };
 
-// timeline stamps for tuning (compiled out unless AF_TRACE): as AF_BSTAMP, with the buffer's address read once per
-// thread (`trc`) so that a stamp costs a clock read and a store
-#ifdef AF_TRACE
-#define AF_FSTAMP(role, it, ph)                                                                  \
-    do {                                                                                         \
-        if (trc && (threadIdx.x & 31) == 0 && (it) < 64) trc[((role) * 64 + (it)) * 8 + (ph)] = clock64(); \
-    } while (0)
-#else
-#define AF_FSTAMP(role, it, ph) do { } while (0)
-#endif
 
 // Registers: 768 threads at 80 give the six warpgroups 480 per thread slot to share; 48 + 48 + 4 x 96.
 constexpr int kFusedThreads = 768, kFusedGradThreads = 512;
@@ -263,12 +253,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = warp_uniform(*tmem_slot);
-#ifdef AF_TRACE
-    long long* const trc = (blockIdx.x == 0 && by == 0) ? g_trace : nullptr;
-#endif
     grid_dep_wait();     // delta, the RoPE passes and the zeroed accumulator precede this grid in the stream
     grid_dep_launch();
-    if (warp == 0) AF_FSTAMP(5, 0, 0);
 
     // register budgets per role: the gradient warpgroups keep 32 columns of probabilities next to 32 of dP^T
     if (warp < 4) setmaxnreg_dec<kFusedLightRegs>();
@@ -351,12 +337,10 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                 const bool next = n + 1 < n_it;
 #pragma unroll 1   // (rolled: half the issuer's loop code; the instruction path is the tightest resource of this kernel)
                 for (int hf = 0; hf < 2; ++hf) {
-                    AF_FSTAMP(who, n, hf * 4);
                     // issuer 0 goes on when P^T of the half is in TMEM, issuer 1 when dS^T is in shared memory
                     ok = wait_half(acc_stream, n, hf);
                     if (ok) ok = mbar_wait_warp_quick<D == 64>(&bars[(who == 0 ? L::B_PRDY : L::B_PDS) + hf], n & 1, abort_flag, 45);
                     if (!ok) break;
-                    AF_FSTAMP(who, n, hf * 4 + 1);
                     tc_fence_after_sync();
                     if (!elect_one()) {
                     } else if (who == 0) {
@@ -383,10 +367,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                         if (ok && who == 1 && !kOwnDq) ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_T2FREE + hf], n & 1, abort_flag, 46);
                         if (!ok) break;
                         tc_fence_after_sync();
-                        AF_FSTAMP(who, n, hf * 4 + 2);
                         issue_T(n + 1, hf);
                     }
-                    AF_FSTAMP(who, n, hf * 4 + 3);
                 }
                 if (!ok) break;
                 if (!next) elect_commit(&bars[L::B_DONE]);
@@ -401,13 +383,10 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             for (int n = 0; ok && n < n_it; ++n) {
 #pragma unroll 1   // (rolled: half the issuer's loop code; the instruction path is the tightest resource of this kernel)
                 for (int hf = 0; hf < 2; ++hf) {
-                    AF_FSTAMP(6, n, hf * 4);
                     ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_PDS + hf], n & 1, abort_flag, 48);
-                    AF_FSTAMP(6, n, hf * 4 + 1);
                     // (own buffers: the previous tile's partial of this half must have been read out)
                     if (ok && kOwnDq && n > 0) ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_T2FREE + hf], (n - 1) & 1, abort_flag, 54);
                     if (!ok) break;
-                    AF_FSTAMP(6, n, hf * 4 + 2);
                     tc_fence_after_sync();
                     if (elect_one()) {
                         const uint32_t b_lo = desc_lo(smem_u32(sDS + hf * L::DS_HALF), 16);
@@ -418,7 +397,6 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                         mma_commit(&bars[L::B_DQFULL + hf]);
                         mma_commit(&bars[L::B_DSFREE + hf]);
                     }
-                    AF_FSTAMP(6, n, hf * 4 + 3);
                 }
             }
         }
@@ -438,10 +416,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             advance(cur);
 #pragma unroll 1
             for (int hf = 0; hf < 2; ++hf) {
-                if (warp == 4) AF_FSTAMP(4, n, hf * 4);
                 ok = mbar_wait_warp_quick<D == 64>(&bars[L::B_DQFULL + hf], n & 1, abort_flag, 49);
                 if (!ok) break;
-                if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 1);
                 tc_fence_after_sync();
                 const int q0 = a0 + hf * 64, nq = min(64, p.S - q0);
                 float* dst = p.dq_acc + ((static_cast<size_t>(b) * p.Hq + ah) * p.S + q0) * D + d;
@@ -454,7 +430,6 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                         tc_fence_before_sync();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&bars[L::B_T2FREE + hf]);
-                        if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 2);
                     }
                     if (nq == 64) {
 #pragma unroll
@@ -467,7 +442,6 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                                 asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + (c * 32 + q) * D), "f"(__uint_as_float(v[q])) : "memory");
                     }
                 }
-                if (warp == 4) AF_FSTAMP(4, n, hf * 4 + 3);
             }
         }
     } else if (warp >= 8) {
@@ -530,10 +504,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             if (need_mask) kept_queries_of_key(ms, xrow, a0, mlo, mn);
             const float sb = -my_slope2;
             const float bias_base = sb * static_cast<float>(a0 - xrow);
-            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 0);
             ok = bar_all(ok && (!polls || mbar_wait(&bars[L::B_SFULL + hf], n & 1, abort_flag, 51)), wg_bar, 128);
             if (!ok) break;
-            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 1);
             tc_fence_after_sync();
             uint32_t pe_keep[32];
             tmem_ld32(tb + T1 + col0, pe_keep);
@@ -550,13 +522,11 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[L::B_PRDY + hf]);
-            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 2);
             // the previous tile's dS^T half must have been consumed by both MMAs that read it
             if (polls) ok = mbar_wait(&bars[L::B_DSFREE + hf], (n & 1) ^ 1, abort_flag, 50);
             // (the vote keeps the warpgroup together: a warp that gave up must not leave the others at the barrier above)
             ok = bar_all(ok && (!polls || mbar_wait(&bars[L::B_DPFULL + hf], n & 1, abort_flag, 53)), wg_bar, 128);
             if (!ok) break;
-            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 3);
             tc_fence_after_sync();
             uint32_t dp[32];
             tmem_ld32(tb + T2 + col0, dp);
@@ -566,7 +536,6 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[L::B_PDS + hf]);
-            if ((warp & 7) == 0) AF_FSTAMP(2 + hf, n, 4);
             if (n + 1 < n_it) store_stats(n + 1);   // (published by the named barrier at the top of the next iteration)
         }
         // (every thread of the four warpgroups takes this barrier, also after a wait that gave up in one of them:

@@ -436,16 +436,6 @@ __device__ __forceinline__ void grad_pass32_general(uint32_t t1, uint32_t t2, in
 //    runs without any on-chip rotation on (K', V) and streamed (Q', dO) - only its epilogue rotates dK' back;
 //  - K' cache only: the dK/dV role runs first (ROT_X, ROT_A, stores K'), the dQ role (ROT_X) streams K';
 //  - no cache: both roles rotate everything they touch.
-// timeline stamps for tuning (compiled out unless AF_TRACE): CTA (0, 0), lane 0 of each warp
-#ifdef AF_TRACE
-#define AF_BSTAMP(role, it, ph)                                                                          \
-    do {                                                                                                 \
-        if (g_trace && blockIdx.x == 0 && blockIdx.y == 0 && (threadIdx.x & 31) == 0 && (it) < 64)       \
-            g_trace[((role) * 64 + (it)) * 8 + (ph)] = clock64();                                        \
-    } while (0)
-#else
-#define AF_BSTAMP(role, it, ph) do { } while (0)
-#endif
 
 // GEN: the instantiation for additive_bias / relu_attention (grad_pass32_general), kept apart from the others.
 template <int D, bool DKV, bool ROT_X, bool ROT_A, bool BS = false, bool GEN = false>
@@ -536,7 +526,6 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
     // they wrote.  The next kernel of the sequence may in turn be scheduled from now on.
     grid_dep_wait();
     grid_dep_launch();
-    AF_BSTAMP(5, 0, 0);
 
     // (bias / relu, dK and dV) The general pass holds 32 scores, 32 dP, 32 biases and two rows of results at once, too much for
     // 128 registers: 80 + 40 + 2 x 192 of the 512 take 110 instead of 117 us at 8 / 4 heads, S = 1000, D = 128 (dQ: slower).
@@ -621,9 +610,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                 return r;
             };
             const bool has_acc = who == 0 || DKV;
-            AF_BSTAMP(who, 63, 0);   // stationary operand ready
             if (ok && n_it > 0) ok = wait_stream(0);
-            AF_BSTAMP(who, 63, 1);   // first streamed tile ready
             if (ok && n_it > 0) {
                 issue_T(0, 0);
                 issue_T(0, 1);
@@ -638,9 +625,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                 for (int hf = 0; hf < 2; ++hf) {
                     // this half: 4 K = 16 steps over its 64 streamed rows; the bf16 operands sit at the start of
                     // the half's own columns of T1 (issuer 0) or T2 (issuer 1)
-                    AF_BSTAMP(who, n, 3 * hf);
                     ok = mbar_wait_warp_quick(&bars[L::B_PDS + hf], n & 1, abort_flag, 26);
-                    AF_BSTAMP(who, n, 3 * hf + 1);
                     if (!ok) break;
                     tc_fence_after_sync();
                     if (has_acc && elect_one()) {
@@ -661,7 +646,6 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                         if (!ok) break;
                         issue_T(n + 1, hf);
                     }
-                    AF_BSTAMP(who, n, 3 * hf + 2);
                 }
                 if (!ok) break;
                 if (!next) {
@@ -690,15 +674,12 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     const int run_pos = DKV ? n % per_head : n;
                     // (listed tiles need not be consecutive: then the cos/sin state is read for every tile)
                     if (CP > 0 && (BS || (run_pos % kRotResync) == 0)) rotate_prefetch(st, p.table, a0, p.S, p.R, t);
-                    AF_BSTAMP(4, n, 0);
                     if (!mbar_wait_warp_quick(&bars[L::B_AFULL + sg], (n / NST) & 1, abort_flag, 28)) return;
-                    AF_BSTAMP(4, n, 1);
                     if (CP > 0) rotate_tile_fast(sA + sg * TILE, st, step, t);
                     else rotate_tile_smem(sA + sg * TILE, a0, p.S, p.R, p.table, t, 128);
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bars[L::B_AROT + sg]);
-                    AF_BSTAMP(4, n, 2);
                 }
             };
             if (p.R == 128) run(std::integral_constant<int, 8>{});
@@ -813,9 +794,7 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
             const float sb = DKV ? -my_slope2 : my_slope2;
             const float bias_base = sb * static_cast<float>(a0 - xrow);
             // this warpgroup's half of T1/T2; the barrier also publishes the statistics within the warpgroup
-            AF_BSTAMP(2 + hf, n, 0);
             ok = bar_all(mbar_wait(&bars[L::B_TFULL + hf], n & 1, abort_flag, 29), 1 + hf, 128);
-            AF_BSTAMP(2 + hf, n, 1);
             if (!ok) break;
             tc_fence_after_sync();
 #pragma unroll
@@ -846,20 +825,16 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
                     else grad_pass32<DKV, false, false>(tb + T1, tb + T2, col0, out_col, p.scale_log2, cbias, sb, sL2, sDl, my_l2, my_delta, mlo, mn);
                 }
             }
-            AF_BSTAMP(2 + hf, n, 2);
             tmem_wait_st();
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[L::B_PDS + hf]);
-            AF_BSTAMP(2 + hf, n, 3);
             if (DKV && n + 1 < n_it) store_stats(n + 1);   // (the named barrier at the top of the next iteration publishes it)
         }
         // epilogue: stage through shared memory (the stream stages are idle now), rotate back, store
-        AF_BSTAMP(2 + hf, 63, 0);
         // (every thread of both warpgroups takes this barrier, also after a wait that gave up in one of them:
         // a warpgroup that left its loop early must not leave the other alone at it)
         ok = wg_all(ok && (n_it <= 0 || mbar_wait(&bars[L::B_DONE], 0, abort_flag, 30)));
-        AF_BSTAMP(2 + hf, 63, 1);   // accumulators complete
         if (BS && ok && n_it <= 0) {
             // no active block for this stationary block: its gradient rows are zero
             const size_t row0 = (static_cast<size_t>(b) * xh_count + xh) * p.S + x0;
@@ -888,7 +863,6 @@ attn_bwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 
     tc_fence_before_sync();
     __syncthreads();
-    AF_BSTAMP(5, 0, 1);
     if (warp == 1) {
         __syncwarp();
         tmem_dealloc(tmem_base, TMEM_COLS);

@@ -50,9 +50,6 @@ struct FwdParams {
     int splits;            // SPLIT kernels: CTAs per cluster, the grid's z dimension
     int four_tiles;        // host-side choice of the kernel with four query tiles per CTA (fwd64_kernel.cuh): its heads per CTA
     long long heads;       // host side: heads (B * Hq) of the whole problem, of which this launch may be a part
-#ifdef AF_TRACE
-    long long* trace;
-#endif
 };
 
 template <int D, int NQ, int KS, int VS, bool TAB = false>
@@ -80,28 +77,6 @@ struct FwdSmem {
     static constexpr int BYTES = (HAS_AX ? OFF_AX + (NQ + 1) * AX_TILE : OFF_MISC + 16) + 1024;  // + alignment slack
 };
 
-// Optional timeline instrumentation for tuning (compiled out unless AF_TRACE is defined): one CTA
-// records SM-clock stamps per role, iteration and phase into a caller-provided buffer.
-#ifdef AF_TRACE
-#define AF_STAMP(role, it, ph)                                                                         \
-    do {                                                                                               \
-        if (p.trace && blockIdx.x == 0 && blockIdx.y == 0 && (threadIdx.x & 31) == 0 && (it) < 64)     \
-            p.trace[((role) * 64 + (it)) * 8 + (ph)] = clock64();                                      \
-    } while (0)
-// fine-grained stamps inside softmax_tile: slots 3..7 of role 2 (query tile 0, warp 8 lane 0 only)
-#define AF_STAMP_SM(ph)                                                                                \
-    do {                                                                                               \
-        if (g_trace && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 256 && n < 64)             \
-            g_trace[(2 * 64 + n) * 8 + (ph)] = clock64();                                              \
-    } while (0)
-#else
-#define AF_STAMP(role, it, ph) do { } while (0)
-#define AF_STAMP_SM(ph) do { } while (0)
-#endif
-
-#ifdef AF_TRACE
-__device__ long long* g_trace = nullptr;
-#endif
 constexpr int kFwdMaxSplits = 8;    // CTAs that share a query tile's key tiles, at most
 constexpr int kFwdMinTiles = 2;     // key tiles per CTA below which a query tile is not shared out further
 // What a forward kernel rotates on chip.  Kernels that rotate no key tiles have no rotation warpgroup and no code for it: its
@@ -139,7 +114,6 @@ __device__ __forceinline__ bool softmax_tile_halves(uint32_t tS, uint32_t tO, in
     tmem_ld32(tS + 64, v + 64);
     tmem_ld32(tS + 96, v + 96);
     tmem_wait_ld();
-    AF_STAMP_SM(3);
     float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
     for (int e = 0; e < BN; e += 2) {
@@ -155,7 +129,6 @@ __device__ __forceinline__ bool softmax_tile_halves(uint32_t tS, uint32_t tO, in
     }
     // scale > 0, so the max commutes with it
     const float mx = fmaf(fmax3(fmaxf(mx4[0], mx4[1]), mx4[2], mx4[3]), scale_log2, bias0);
-    AF_STAMP_SM(4);
     // lazy rescale: keep the old reference max unless it grew by more than the threshold
     const bool upd = mx > m_run + kRescaleThreshold;
     float alpha = 1.f;
@@ -200,10 +173,8 @@ __device__ __forceinline__ bool softmax_tile_halves(uint32_t tS, uint32_t tO, in
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&p_ready[pt]);
-        if (pt == 0) AF_STAMP_SM(5);
     }
     l_run = l_run * alpha + ((ps2[0].x + ps2[0].y) + (ps2[1].x + ps2[1].y));
-    AF_STAMP_SM(6);
     return true;
 }
 
@@ -460,7 +431,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     };
     auto is_last = [&](int q, int j) { return rowpair ? j == last_act[q] : j == jhi[q]; };
     const int n_it = jhi_c - jlo_c + 1;
-    AF_STAMP(0, 63, 0);  // kernel entry
 
     // Set-up, with as little as possible in a row (a CTA's first scores wait for it, and short key loops cannot hide it): the
     // lanes of warp 0 initialise a barrier each and the warp requests its first tiles at once, while warp 1 allocates
@@ -661,10 +631,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 bool ok = true;
                 for (int it = 0; ok && it < n_it; ++it) {
                     const int ks = it % KS;
-                    AF_STAMP(1, it, 0);
                     ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);
                     if (ok) ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_TFULL], it & 1, abort_flag, 13);
-                    AF_STAMP(1, it, 1);
                     if (!ok) break;
                     rotate_tile_tab<CP>(sK + ks * TILE, sT, t);
                     fence_proxy_async_smem();
@@ -673,7 +641,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         mbar_arrive(&bars[L::B_KROT + ks]);
                         mbar_arrive(&bars[L::B_TEMPTY]);
                     }
-                    AF_STAMP(1, it, 2);
                 }
             };
             // fp32 arithmetic from the fp32 table rows
@@ -690,16 +657,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     // (listed tiles need not be consecutive: the cos/sin state is read for every tile)
                     if (CP > 0 && (BS || (it % kKeyRun) == 0))
                         rotate_prefetch(st, p.table, tile_at(jlo_c + it) * BN, p.S, p.R, t);
-                    AF_STAMP(1, it, 0);
                     ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_KFULL + ks], (it / KS) & 1, abort_flag, 9);
-                    AF_STAMP(1, it, 1);
                     if (!ok) break;
                     if (CP > 0) rotate_tile_fast(sK + ks * TILE, st, step, t);
                     else rotate_tile_smem(sK + ks * TILE, tile_at(jlo_c + it) * BN, p.S, p.R, p.table, t, 128);
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bars[L::B_KROT + ks]);
-                    AF_STAMP(1, it, 2);
                 }
             };
             if constexpr (tab_tiles) {
@@ -760,7 +724,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         for (int j = jlo[q]; ok && j <= jhi[q]; ++j) {
             if (rowpair && !active(q, j)) continue;   // a listed block of the other row block only
             const int j0 = tile_at(j) * BN;
-            AF_STAMP(2 + q, n, 0);
             const bool need_mask = tile_needs_mask(ms, i0[q], j0);
             const float bias0 = slope2 * static_cast<float>(j0 - i);
             int mlo = 0;
@@ -785,7 +748,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (need_mask) ok = softmax_tile_halves<D, true, false, kQuick>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
                 else ok = softmax_tile_halves<D, false, false, kQuick>(tS, tO, n, p.scale_log2, kb, bias0, mlo, mn, sf, pr, n & 1, abort_flag, lane, m_run, l_run);
             }
-            AF_STAMP(2 + q, n, 2);
             ++n;
         }
         // epilogue (Section 4.4: save L = m + ln l, while the last products run)
@@ -795,7 +757,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             else p.lse[static_cast<size_t>(bh) * p.S + i] = l_run > 0.f ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
         }
         if (ok && jhi[q] >= jlo[q]) ok = mbar_wait_warp_quick<kQuick>(&bars[L::B_ODONE + q], 0, abort_flag, 11);
-        AF_STAMP(2 + q, 63, 0);  // O complete
         if (SPLIT && parts > 1 && ok) {
             // this CTA's share, unnormalised, over the operand tiles (idle now): rows of D + 4 floats, acc[D], m, l
             tc_fence_after_sync();
@@ -921,7 +882,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
     tc_fence_before_sync();
     __syncthreads();
-    AF_STAMP(0, 63, 1);  // all roles done
     if (warp == 1) {
         __syncwarp();
         tmem_dealloc(tmem_base, TMEM_COLS);
