@@ -49,17 +49,6 @@ __device__ __forceinline__ bool tile_needs_mask(const MaskSpec& m, int i0, int j
     return false;
 }
 
-__device__ __forceinline__ bool pair_kept(const MaskSpec& m, int i, int j) {
-    if (j >= m.S) return false;
-    int d = i - j;
-    if (m.causal && d < 0) return false;
-    if (m.window >= 0) {
-        if (d < 0) d = -d;
-        if (d > m.window) return false;
-    }
-    return true;
-}
-
 // For a fixed row of a tile pair the kept columns form one interval (causal, window and the sequence
 // end are all half-lines in the column index).  Returns lo and the width n: column e (0..127) is kept
 // iff (unsigned)(e - lo) < n.
@@ -138,7 +127,7 @@ __device__ __forceinline__ void rotate_tile_smem(uint8_t* tile, int row0, int S,
 // d = RP * theta_i, which the table carries as a trailer row.  The first-row read is split off
 // (rotate_prefetch) so that it can be issued before waiting for the tile to land.  After a tile the
 // state has advanced by 128 rows, i.e. to the thread's first row of the next consecutive tile, so a
-// run of consecutive tiles needs no table read at all; callers re-read the table every
+// run of consecutive tiles needs no table read at all; the backward's streamed tiles re-read the table every
 // kRotResync tiles to keep the accumulated rounding of the recurrence far below bf16 resolution.
 constexpr int kRotResync = 16;
 // The forward's key tiles re-read it every kKeyRun tiles, so that a pass over the keys ahead of the kernel can give the same

@@ -186,7 +186,8 @@ attn_fwd64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     grid_dep_launch();
     if (!hybrid) grid_dep_wait();
 
-    // 4 x 104 + 64 of 5 x 96 registers per thread slot; with the rotation warpgroup 4 x 88 + 80 + 48 of 6 x 80
+    // 4 x 104 + 64 of 5 x 96 registers per thread slot; with the rotation warpgroup 4 x 88 + 80 + 48 of 6 x 80, which spills (140 bytes
+    // per thread stored, 180 loaded): that kernel is left to windows, slopes and callers without scratch memory
     constexpr int kSoftmaxRegs = KROT ? 88 : 104, kLightRegs = KROT ? 48 : 64;
     if (warp < 4) setmaxnreg_dec<kLightRegs>();
     if (warp < NQ) {

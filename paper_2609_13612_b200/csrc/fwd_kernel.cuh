@@ -80,7 +80,8 @@ struct FwdSmem {
 constexpr int kFwdMaxSplits = 8;    // CTAs that share a query tile's key tiles, at most
 constexpr int kFwdMinTiles = 2;     // key tiles per CTA below which a query tile is not shared out further
 // What a forward kernel rotates on chip.  Kernels that rotate no key tiles have no rotation warpgroup and no code for it: its
-// registers go to the softmax warpgroups (176 -> 208 per thread, no spills), and a CTA's set-up starts four warps less.
+// registers go to the softmax warpgroups (176 -> 208 per thread; 8 bytes spilled by the kernels over block lists, none by the others), and
+// a CTA's set-up starts four warps less.
 // Against the same kernel with an idle rotation warpgroup: 179.0 -> 173.4 us (B = 4, 12 heads, S = 4096, D = 64, keys
 // rotated before), 141.4 -> 139.0 us (32 / 8 heads, S = 4096, D = 128, no rotation), both under sustained load.
 constexpr int kRotNone = 0, kRotAll = 1, kRotQueries = 2;
