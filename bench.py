@@ -37,10 +37,11 @@ from paper_2609_13612_b200 import shard, synth  # noqa: E402
 METRIC = "fused RoPE+causal attention TFLOP/s (bf16 fwd/bwd) and % of B200 tensor peak"
 UNIT = "TFLOP/s"
 L2_BYTES = 126 * 1024 * 1024
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture), by kernel and workload.
+# DRAM bytes per step (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of each launch), by kernel and workload.
 # A kernel or workload that has no entry reports "traffic": null instead of a figure that belongs to another one.
 KERNEL_TRAFFIC_BYTES = {
     ("attn_fwd_kernel<128,2,rope>", "c2_llama3_8b_fwd"): 55.1e6,
+    ("attn_fwd_kernel<128,2,queries>", "c2_llama3_8b_fwd"): 63.6e6,   # 8.5e6 of them by rope_key_tiles_kernel
 }
 RIDGE_CONTEXT = {"paper_ampere_flop_per_byte": 152, "paper_hopper_flop_per_byte": 300}
 PAPER_CONTEXT = {

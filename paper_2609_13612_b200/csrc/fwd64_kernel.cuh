@@ -6,7 +6,8 @@
 // (4 x (64 + 64) columns), and four softmax warps per SM sub-partition keep the unit busy.  K and V are read (and K tiles
 // rotated) half as often, too.
 //   Sustained, two -> four query tiles: 194 -> 185 us (B = 4, 12 heads, S = 4096, keys rotated on chip), 170 -> 157 us (rotated
-// before), 86 -> 75 us (the same with window 256 and ALiBi), 45 -> 37 us (B = 8, S = 1024).  With one issuing warp for all four
+// before), 86 -> 75 us (the same with window 256 and ALiBi), 45 -> 37 us (B = 8, S = 1024); all before the reference moved in
+// masked blocks (softmax_block64), which costs 1.4 to 1.9 %.  With one issuing warp for all four
 // tiles the issuer was the bound (3200 cycles per 64-key step, 188 us); with one per tile the rest of a step is MMAs of 64
 // columns, which read their whole A operand for half the work, and the special-function unit.
 // Warp roles: warps 0-3 issue the MMAs of a query tile each (warp 0 also all TMA loads), (kRotAll) warps 4-7 rotate the key
